@@ -35,6 +35,17 @@ namespace {
 constexpr int kHopThreads = 256;
 constexpr int kHopWarps = kHopThreads / 32;
 constexpr uint32_t kMinPerBlock = 512;       // live probes per active hop block
+// Batches of at most this many probes walk in one walk_thread_kernel launch
+// (indexed tables, tail hop left to the library).  Regrouping by switch costs
+// about 10 us of launches per hop and a table stage per occupied switch,
+// whatever the batch; the thread walk costs its L2 round trips.  Thread walk
+// against regrouped walk, us, at 1k / 100k / 800k / 1.6M / 3.2M probes:
+//   ring of 8, 64 rules       11/126   13/128   35/137   60/148  111/172
+//   mesh of 512, 1,000 rules  45/108   62/173  159/225  276/262  510/311
+//   fat tree, 2,000 rules     82/193  115/292  300/398  500/461  897/583
+// and compact flows of 512 switches at 1M: 223/231 (270/267 with policies).
+// The lines cross between 1M and 2M on the large tables.
+constexpr uint32_t kThreadWalkMax = 1u << 20;
 constexpr int kGridThreads = 256;
 constexpr uint32_t kSmemHistMax = 12288;     // switches for shared-memory histograms
 constexpr uint32_t kWaitLimit = 1u << 24;    // bounded mbarrier polls
@@ -1206,7 +1217,6 @@ struct HopArgs {
     const uint64_t *blob_offs;
     const uint8_t *region;
     const uint32_t *port_offs;
-    const int32_t *port_peer;
     const uint32_t *host_ip;
     const pv_probe *probes;
     const uint4 *recs;   // walk records (kRec kernels)
@@ -1510,44 +1520,19 @@ __device__ __forceinline__ uint32_t first_match_lane(const uint8_t *sm, const Bl
 constexpr uint32_t kAlive = 0xFFu;
 constexpr uint32_t kViolationNext = 0xFEu;
 
-__device__ __forceinline__ void hop_outcome(const HopArgs &g, uint32_t hop, uint32_t fm, uint32_t dst, uint32_t mask,
-                                            uint32_t pbase, uint32_t nports, uint32_t *status, uint32_t *next) {
+// Port p of the current switch comes as {peer, aux}, aux = the region of the
+// peer switch or the address of the attached host (port_stage_kernel builds
+// the table at load): the hop kernel stages the switch's ports in shared
+// memory, the thread walk reads them in place.
+__device__ __forceinline__ void hop_outcome(const HopArgs &g, const uint2 *ports, uint32_t hop, uint32_t fm, uint32_t dst,
+                                            uint32_t mask, uint32_t nports, uint32_t *status, uint32_t *next) {
     *next = 0;
     const uint32_t act = fm & 0xFFFFu;
     if (!(fm & kWinFound) || act == PV_DROP || act >= nports) {
         *status = PV_DROPPED;
         return;
     }
-    const int32_t peer = g.port_peer[pbase + act];
-    if (peer < 0) {
-        *status = PV_DROPPED;
-    } else if (peer & PV_PEER_HOST) {
-        const uint32_t q = (uint32_t)(peer & ~PV_PEER_HOST);
-        *status = (q < g.H && g.host_ip[q] == dst) ? PV_COMPLIANT : PV_MISDELIVERED;
-    } else if (hop + 1 >= g.cap) {
-        *status = PV_LOOP;
-    } else {
-        const uint32_t r2 = g.region[(uint32_t)peer >> 8];
-        *status = (r2 < 32 && ((mask >> r2) & 1u)) ? kAlive : kViolationNext;
-        *next = (uint32_t)peer;
-    }
-}
-
-// The hop kernel stages the current switch's ports once per table from the
-// port stage the table loader builds (port_stage_kernel): port p as {peer,
-// aux}, aux = the region of the peer switch, or the address of the attached
-// host, so a hop's outcome reads shared memory only.
-// hop_outcome with the port table staged in shared memory (same outcomes).
-__device__ __forceinline__ void hop_outcome_staged(const HopArgs &g, const uint2 *s_port, uint32_t hop, uint32_t fm,
-                                                   uint32_t dst, uint32_t mask, uint32_t nports, uint32_t *status,
-                                                   uint32_t *next) {
-    *next = 0;
-    const uint32_t act = fm & 0xFFFFu;
-    if (!(fm & kWinFound) || act == PV_DROP || act >= nports) {
-        *status = PV_DROPPED;
-        return;
-    }
-    const uint2 pe = s_port[act];
+    const uint2 pe = ports[act];
     const int32_t peer = (int32_t)pe.x;
     if (peer < 0) {
         *status = PV_DROPPED;
@@ -1699,7 +1684,7 @@ __global__ void __launch_bounds__(kHopThreads, 4) walk_hop_kernel(HopArgs g) {
                 const uint32_t fm = first_match_lane<kStats>(s_raw, L, act, pr.x, pr.y, pr.z & 0xFFFFu, e.y & 0xFFu,
                                                              stc[kStRuleTests], stc[kStLookups]);
                 my_fm = fm;
-                if (act) hop_outcome_staged(g, s_port, g.hop, fm, pr.y, pr.w, nports, &my_status, &my_next);
+                if (act) hop_outcome(g, s_port, g.hop, fm, pr.y, pr.w, nports, &my_status, &my_next);
             } else {
                 for (uint32_t j = 0; j < cnt; ++j) {
                     if ((fin_lanes >> j) & 1u) continue;
@@ -1713,7 +1698,7 @@ __global__ void __launch_bounds__(kHopThreads, 4) walk_hop_kernel(HopArgs g) {
                         kIndexed ? first_match_indexed<kStats>(s_raw, hdr, lane, src, dst, dport, in_port, tests, lookups)
                                  : first_match_linear<kStats>(s_raw, npad, lane, src, dst, dport, in_port, tests);
                     uint32_t status, next;
-                    hop_outcome_staged(g, s_port, g.hop, fm, dst, mask, nports, &status, &next);
+                    hop_outcome(g, s_port, g.hop, fm, dst, mask, nports, &status, &next);
                     if (lane == j) {
                         my_status = status;
                         my_next = next;
@@ -1849,88 +1834,162 @@ __device__ __forceinline__ uint32_t first_match_thread(const uint8_t *__restrict
     return 0u;
 }
 
-// The walk's last hops, first_hop .. cap - 1, in one launch: one thread per
-// probe still walking (the unsorted list the last hop kernel wrote, read
-// through its per-block slices), each thread taking its probe hop after hop
-// to the end with the tables read from L2.  Few probes are left by then, so
-// regrouping them by switch every hop would cost more in launches than the
-// table staging saves.  Results, cycle finishing, path constraints and the
-// per-hop live counts are those of walk_hop_kernel.
-template <bool kPolicy, bool kStats, bool kRec>
-__global__ void __launch_bounds__(256) walk_tail_kernel(HopArgs g, const uint2 *__restrict__ list,
-                                                        const uint2 *__restrict__ desc, uint32_t nslices,
-                                                        uint32_t first_hop) {
+// Whole walks, or a walk's last hops, in one launch: one thread per probe,
+// the tables read from L2, no regrouping.  Each block owns a contiguous share
+// of its input and its lanes draw probes from it as they finish the ones in
+// hand, so a warp is not held up by its longest walk.  Input (kSrc):
+//   kSrcProbes  the caller's probes, from their first visit (the checks of
+//               walk_init_kernel included);
+//   kSrcFlows   compact flows, bound as walk_init_kernel<., true> does, then
+//               the same;
+//   kSrcList /  the live list the last hop kernel wrote (block b reads slice
+//   kSrcListRec b), walked on from hop first_hop; records as load_header.
+// Results, cycle finishing, path constraints and visit counts are those of
+// walk_hop_kernel; a probe's cycle checkpoint and waypoint bits stay in
+// registers.
+// Bound by the chain of dependent L2 round trips of one first match (about
+// ten) times the visits of a lane; drawing new probes keeps the other lanes
+// at work meanwhile.  1,000 probes on the ring: 130 us as 27 launches, 11 us
+// as this one; 100,003 probes on 512 switches: 175 -> 62 us.
+enum { kSrcProbes = 0, kSrcFlows = 1, kSrcList = 2, kSrcListRec = 3 };
+
+struct ThreadWalkArgs {
+    uint32_t M;                    // probes (kSrcProbes, kSrcFlows)
+    const uint16_t *host_switch;
+    const uint2 *list, *desc;      // kSrcList, kSrcListRec
+    uint32_t first_hop;
+    BindArgs ba;                   // kSrcFlows
+    pv_probe *bound;               // kSrcFlows: the caller's copy of the bound records, or null
+    unsigned long long *visits;    // [gridDim.x]: visits each block made
+};
+
+template <bool kPolicy, bool kStats, int kSrc>
+__global__ void __launch_bounds__(256, !kStats && kSrc >= kSrcList ? 4 : 1) walk_thread_kernel(HopArgs g, ThreadWalkArgs w) {
+    constexpr bool kList = kSrc == kSrcList || kSrc == kSrcListRec;
+    __shared__ uint32_t s_next;
+    __shared__ unsigned long long s_visits;
     const uint32_t lane = threadIdx.x & 31;
+    uint32_t c0, c1;   // this block's share of the probes or of the list
+    if (kList) {
+        const uint2 d = w.desc[blockIdx.x];
+        c0 = d.x;
+        c1 = d.x + d.y;
+    } else {
+        c0 = (uint32_t)(((uint64_t)w.M * blockIdx.x) / gridDim.x);
+        c1 = (uint32_t)(((uint64_t)w.M * (blockIdx.x + 1)) / gridDim.x);
+    }
+    if (threadIdx.x == 0) {
+        s_next = 0;
+        s_visits = 0;
+    }
+    __syncthreads();
     uint32_t stc[kStCount] = {};
-    for (uint32_t sl = blockIdx.x; sl < nslices; sl += gridDim.x) {
-        const uint2 d = desc[sl];
-        for (uint32_t base = d.x; base < d.x + d.y; base += blockDim.x) {
-            const uint32_t i = base + threadIdx.x;
-            bool active = i < d.x + d.y;
-            uint2 e = make_uint2(0, 0);
-            uint4 pr = make_uint4(0, 0, 0, 0);
-            uint32_t pid = 0;
-            if (active) {
-                e = list[i];
-                pr = load_header<kRec>(g, e.x, &pid);
+    uint32_t visits = 0;
+    bool active = false, more = true;
+    uint4 pr = make_uint4(0, 0, 0, 0);
+    uint32_t pid = 0, loc = 0, h = 0, ck = 0, wp = 0;
+    uint4 ph = make_uint4(0, 0, 0, 0);
+    while (true) {
+        const uint32_t idle = __ballot_sync(PV_FULL_MASK, !active);
+        if (idle && more) {
+            uint32_t base = 0;
+            if (lane == 0) base = atomicAdd(&s_next, (uint32_t)__popc(idle));
+            base = __shfl_sync(PV_FULL_MASK, base, 0);
+            more = base + (uint32_t)__popc(idle) < c1 - c0;
+            const uint32_t k = base + __popc(idle & ((1u << lane) - 1u));
+            if (!active && k < c1 - c0) {
+                const uint32_t i = c0 + k;
+                wp = 0;
+                if (kList) {
+                    const uint2 e = w.list[i];
+                    pr = load_header<kSrc == kSrcListRec>(g, e.x, &pid);
+                    loc = e.y;
+                    h = w.first_hop;
+                    active = true;
+                    if (g.cycles && h >= kCycleCheckFrom) ck = g.ck[e.x];
+                    if (kPolicy) ph = policy_of(g.pa, pid);
+                } else {
+                    pid = i;
+                    h = 0;
+                    if (kSrc == kSrcFlows) {
+                        const uint32_t grp = i / w.ba.ppg;
+                        const uint32_t node = w.ba.assign[grp * w.ba.pods + (i - grp * w.ba.ppg) % w.ba.pods];
+                        const uint2 f = flow_at(w.ba, i);
+                        const bool placed = node < g.H;
+                        pr = make_uint4(placed ? w.ba.host_ip[node] : 0u, f.x,
+                                        (f.y & 0xFFFFu) | (placed ? node : (uint32_t)PV_NO_HOST) << 16,
+                                        w.ba.group_mask[grp]);
+                        if (w.bound) reinterpret_cast<uint4 *>(w.bound)[i] = pr;
+                    } else {
+                        pr = __ldg(reinterpret_cast<const uint4 *>(g.probes) + i);
+                    }
+                    if (kPolicy) ph = policy_of(g.pa, i);
+                    const uint32_t host = pr.z >> 16;
+                    if (host < g.H) {
+                        const uint32_t s = w.host_switch[host], reg = g.region[s];
+                        active = reg < 32 && ((pr.w >> reg) & 1u) &&
+                                 !(kPolicy && switch_listed(g.pa.sw + ph.x, ph.y, s));
+                        loc = s << 8 | __ldg(g.host_addr + host).y;
+                        if (!active) put_result(g.out, i, PV_VIOLATION, 1, s);
+                    } else {
+                        put_result(g.out, i, PV_NOSRC, 0, 0xFFFF);
+                    }
+                    if (kPolicy && !active) g.pa.hits[i] = 0;
+                }
             }
-            uint32_t loc = e.y;
-            for (uint32_t h = first_hop; h < g.cap; ++h) {
-                const uint32_t live = __ballot_sync(PV_FULL_MASK, active);
-                if (!live) break;
-                if (lane == 0) atomicAdd(&g.hop_live[h], (uint32_t)__popc(live));
-                if (!active) continue;
-                const uint32_t s = (loc >> 8) & 0xFFFFu, in_port = loc & 0xFFu, fin = loc_finish(loc);
-                uint32_t *out = reinterpret_cast<uint32_t *>(g.out) + pid;   // {status, hops, last_switch}
-                if (fin != 0 && fin - 1 == h) {   // finished at its cycle position
-                    *out = (uint32_t)PV_LOOP | g.cap << 8 | s << 16;
-                    active = false;
-                    continue;
-                }
-                const uint8_t *blob = g.blob + g.blob_offs[s];
-                const uint4 hdr = __ldg(reinterpret_cast<const uint4 *>(blob));
-                const BlobLayout L(hdr);
-                const uint32_t fm = first_match_thread<kStats>(blob, L, pr.x, pr.y, pr.z & 0xFFFFu, in_port,
-                                                               stc[kStRuleTests], stc[kStLookups]);
-                if (kStats) {
-                    uint32_t depth = 0;
-                    const uint32_t ref = scan_first_match(reinterpret_cast<const uint4 *>(blob + L.fa),
-                                                          reinterpret_cast<const uint2 *>(blob + L.fb),
-                                                          hdr.x & 0xFFFFu, pr.x, pr.y, pr.z & 0xFFFFu, in_port, &depth);
-                    ++stc[kStFirstMatches];
-                    stc[kStLinearDepth] += depth;
-                    stc[kStMismatch] += ref != fm ? 1u : 0u;
-                }
-                const uint32_t pbase = g.port_offs[s], nports = g.port_offs[s + 1] - pbase;
-                uint32_t status, next;
-                hop_outcome(g, h, fm, pr.y, pr.w, pbase, nports, &status, &next);
-                if (kPolicy) {
-                    const uint4 ph = policy_of(g.pa, pid);
-                    uint32_t bits = 0;
-                    for (uint32_t k = 0; k < ph.w; ++k)
-                        if (g.pa.sw[ph.z + k] == s) bits |= 1u << k;
-                    if (bits) g.pa.hits[pid] |= bits;
-                    if (status == kAlive && switch_listed(g.pa.sw + ph.x, ph.y, next >> 8)) status = kViolationNext;
-                }
-                if (status != kAlive) {
-                    const bool at_next = status == kViolationNext;
-                    *out = (at_next ? (uint32_t)PV_VIOLATION : status) | (h + (at_next ? 2u : 1u)) << 8 |
-                           (at_next ? (next >> 8) : s) << 16;
-                    active = false;
-                    continue;
-                }
-                const bool bounce = g.bounce && (fm & 0xFFFFu) == in_port;
-                if (bounce && (loc >> 24) == kBounced) {   // two bounces in a row: a two-switch cycle
-                    *out = (uint32_t)PV_LOOP | g.cap << 8 | (((g.cap - 1u - h) & 1u) ? (next >> 8) : s) << 16;
-                    active = false;
-                    continue;
-                }
+        }
+        if (!__any_sync(PV_FULL_MASK, active)) {
+            if (!more) break;
+            continue;
+        }
+        if (!active) continue;
+        // one visit
+        ++visits;
+        const uint32_t s = (loc >> 8) & 0xFFFFu, in_port = loc & 0xFFu, fin = loc_finish(loc);
+        uint32_t status = PV_LOOP, hops = g.cap, last = s;   // the walk's end, unless it goes on
+        if (fin != 0 && fin - 1 == h) {   // finished at its cycle position
+            active = false;
+        } else {
+            const uint8_t *blob = g.blob + g.blob_offs[s];
+            const uint4 hdr = __ldg(reinterpret_cast<const uint4 *>(blob));
+            const BlobLayout L(hdr);
+            const uint32_t fm = first_match_thread<kStats>(blob, L, pr.x, pr.y, pr.z & 0xFFFFu, in_port,
+                                                           stc[kStRuleTests], stc[kStLookups]);
+            if (kStats) {
+                uint32_t depth = 0;
+                const uint32_t ref = scan_first_match(reinterpret_cast<const uint4 *>(blob + L.fa),
+                                                      reinterpret_cast<const uint2 *>(blob + L.fb), hdr.x & 0xFFFFu,
+                                                      pr.x, pr.y, pr.z & 0xFFFFu, in_port, &depth);
+                ++stc[kStFirstMatches];
+                stc[kStLinearDepth] += depth;
+                stc[kStMismatch] += ref != fm ? 1u : 0u;
+            }
+            const uint32_t pbase = g.port_offs[s], nports = g.port_offs[s + 1] - pbase;
+            uint32_t next;
+            hop_outcome(g, g.port_stage + pbase, h, fm, pr.y, pr.w, nports, &status, &next);
+            if (kPolicy) {
+                for (uint32_t k = 0; k < ph.w; ++k)
+                    if (g.pa.sw[ph.z + k] == s) wp |= 1u << k;
+                if (status == kAlive && switch_listed(g.pa.sw + ph.x, ph.y, next >> 8)) status = kViolationNext;
+            }
+            const bool bounce = g.bounce && (fm & 0xFFFFu) == in_port;
+            if (status != kAlive) {
+                const bool at_next = status == kViolationNext;
+                status = at_next ? (uint32_t)PV_VIOLATION : status;
+                hops = h + (at_next ? 2u : 1u);
+                last = at_next ? (next >> 8) : s;
+                active = false;
+            } else if (bounce && (loc >> 24) == kBounced) {   // two bounces in a row: a two-switch cycle
+                status = PV_LOOP;
+                last = ((g.cap - 1u - h) & 1u) ? (next >> 8) : s;
+                active = false;
+            } else {
                 uint32_t nfin = fin;
                 const uint32_t h1 = h + 1;
                 if (g.cycles && nfin == 0 && h1 >= kCycleCheckFrom) {
                     if ((h1 & (h1 - 1u)) == 0) {
-                        g.ck[e.x] = next;
-                    } else if (g.ck[e.x] == next) {
+                        ck = next;
+                    } else if (ck == next) {
                         const uint32_t period = h1 - (1u << (31 - __clz(h1)));
                         nfin = h1 + (g.cap - 1u - h1) % period + 1u;
                         if (nfin >= g.cap) nfin = 0;
@@ -1938,10 +1997,22 @@ __global__ void __launch_bounds__(256) walk_tail_kernel(HopArgs g, const uint2 *
                 }
                 if (nfin == 0 && bounce) nfin = kBounced;
                 loc = next | (nfin << 24);
+                h = h1;
+            }
+        }
+        if (!active) {
+            put_result(g.out, pid, status, hops, last);
+            if (kPolicy) {
+                if (!kList) g.pa.hits[pid] = wp;
+                else if (wp) g.pa.hits[pid] |= wp;
             }
         }
     }
     if (kStats) flush_stats(g.stats, stc);
+    const uint32_t warp_visits = __reduce_add_sync(PV_FULL_MASK, visits);
+    if (lane == 0 && warp_visits) atomicAdd(&s_visits, (unsigned long long)warp_visits);
+    __syncthreads();
+    if (threadIdx.x == 0) w.visits[blockIdx.x] = s_visits;
 }
 
 inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
@@ -2373,7 +2444,7 @@ namespace {
 // The walk of pv_verify_probes; with pa, under the path constraints of
 // pv_verify_probes_constrained.
 using HopKernel = void (*)(HopArgs);
-using TailKernel = void (*)(HopArgs, const uint2 *, const uint2 *, uint32_t, uint32_t);
+using ThreadKernel = void (*)(HopArgs, ThreadWalkArgs);
 
 // first: the kernel for the walk's first hop (the statistics kernels serve
 // every hop with the general form)
@@ -2394,10 +2465,77 @@ HopKernel pick_hop(bool indexed, bool pol, bool stats, bool first) {
     return first ? pick_hop_form<kRec, true>(indexed, pol) : pick_hop_form<kRec, false>(indexed, pol);
 }
 
-template <bool kRec>
-TailKernel pick_tail(bool pol, bool stats) {
-    return pol ? (stats ? walk_tail_kernel<true, true, kRec> : walk_tail_kernel<true, false, kRec>)
-               : (stats ? walk_tail_kernel<false, true, kRec> : walk_tail_kernel<false, false, kRec>);
+template <int kSrc>
+ThreadKernel pick_thread(bool pol, bool stats) {
+    return pol ? (stats ? walk_thread_kernel<true, true, kSrc> : walk_thread_kernel<true, false, kSrc>)
+               : (stats ? walk_thread_kernel<false, true, kSrc> : walk_thread_kernel<false, false, kSrc>);
+}
+
+// What every walk kernel of a call is given: the loaded tables, the output,
+// the caller's constraints and the context's options.
+HopArgs walk_args(pv_ctx *ctx, uint32_t hop_cap, const pv_probe *d_probes, pv_result *d_out, const PolicyArgs *pa) {
+    const pv_table_state &t = ctx->tb;
+    HopArgs g = {};
+    g.cap = hop_cap;
+    g.S = t.num_switches;
+    g.H = t.num_hosts;
+    g.blob = t.d_blob;
+    g.blob_offs = t.d_blob_offs;
+    g.region = t.d_region;
+    g.port_offs = t.d_port_offs;
+    g.host_ip = t.d_host_ip;
+    g.probes = d_probes;
+    g.out = d_out;
+    g.status = ctx->d_status;
+    g.lane_max = (uint32_t)ctx->opt_walk_lane_max;
+    g.hop_live = ctx->d_walk_live;
+    g.cycles = ctx->opt_walk_cycles == 0 && hop_cap > kCycleCheckFrom ? 1u : 0u;
+    g.bounce = ctx->opt_walk_cycles == 0 && t.links_symmetric ? 1u : 0u;   // any cap: no checkpoints needed
+    if (pa) g.pa = *pa;
+    g.host_addr = t.d_host_addr;
+    g.port_stage = t.d_port_stage;
+    g.stats = ctx->d_walk_stats;
+    g.wait_extra = ctx->opt_test_stall_staging ? 16u : 0u;
+    g.wait_ns = ctx->opt_test_stall_staging ? 50ull * 1000 * 1000 : 2ull * 1000 * 1000 * 1000;
+    return g;
+}
+
+// Blocks of the thread walk over M probes: one thread per probe up to a full
+// device, in small blocks while they leave SMs idle.
+void thread_walk_grid(pv_ctx *ctx, ThreadKernel fn, uint32_t M, uint32_t *blocks, uint32_t *threads) {
+    *threads = M < (uint32_t)ctx->num_sms * 256u ? 64u : 256u;
+    const uint32_t per_sm = (uint32_t)std::max(1, pv_blocks_per_sm(ctx, (const void *)fn, (int)*threads, 0));
+    const uint32_t most = std::min<uint32_t>((uint32_t)ctx->num_sms * per_sm, ctx->walk_visit_slots);
+    *blocks = std::max(1u, (uint32_t)std::min<uint64_t>(((uint64_t)M + *threads - 1) / *threads, most));
+}
+
+// The whole walk in one walk_thread_kernel launch.
+int walk_by_thread(pv_ctx *ctx, uint32_t M, pv_probe *d_probes, uint32_t hop_cap, pv_result *d_out,
+                   const PolicyArgs *pa, cudaStream_t st, const BindArgs *ba) {
+    const bool stats = ctx->opt_walk_stats != 0;
+    const ThreadKernel fn = ba ? pick_thread<kSrcFlows>(pa != nullptr, stats) : pick_thread<kSrcProbes>(pa != nullptr, stats);
+    HopArgs g = walk_args(ctx, hop_cap, d_probes, d_out, pa);
+    ThreadWalkArgs w = {};
+    w.M = M;
+    w.host_switch = ctx->tb.d_host_switch;
+    if (ba) {
+        w.ba = *ba;
+        w.bound = d_probes;
+    }
+    w.visits = ctx->d_walk_visits;
+    uint32_t blocks, threads;
+    thread_walk_grid(ctx, fn, M, &blocks, &threads);
+    pv_use_begin(ctx, st);
+    if (stats)
+        PV_TRY_CUDA(ctx, cudaMemsetAsync(ctx->d_walk_stats, 0, PV_WALK_STATS * sizeof(unsigned long long), st),
+                    "walk statistics clear");
+    const int pr = pv_prof_start(ctx, st, PV_K_WALK_HOP);
+    fn<<<blocks, threads, 0, st>>>(g, w);
+    pv_prof_stop(ctx, st, pr, 1);
+    ctx->last_walk_hops = 0;
+    ctx->last_walk_blocks = blocks;
+    pv_mark_use(ctx, st);
+    return pv_check_launch(ctx, "thread walk kernel");
 }
 
 int walk_probes(pv_ctx *ctx, uint32_t M, const pv_probe *d_probes, uint32_t hop_cap, pv_result *d_out,
@@ -2416,6 +2554,15 @@ int walk_probes(pv_ctx *ctx, uint32_t M, const pv_probe *d_probes, uint32_t hop_
     if (which == 2 && !t.index_fits)
         return pv_fail(ctx, PV_EINVAL, "pv_verify_probes: the first-match index does not fit shared memory");
     const bool indexed = which == 2;
+    const uint64_t groups = ba ? ((uint64_t)M + ba->ppg - 1) / ba->ppg : 0;
+    const uint64_t G64 = groups * (ba ? ba->pods : 0);
+    // compact flows with one path constraint per group are placed directly
+    // (and walked through walk records)
+    const bool direct = ba && (!pol || (pa->probe_pol == nullptr && (pa->per == 0 || pa->per % ba->ppg == 0)));
+    if (direct && G64 > 0xFFFFFFFFull) return pv_fail(ctx, PV_EINVAL, "pv_verify_flows: too many (group, pod) pairs");
+    const uint32_t G = (uint32_t)G64;
+    if (indexed && M <= kThreadWalkMax && ctx->opt_walk_tail_hop < 0 && !ctx->opt_test_stall_staging)
+        return walk_by_thread(ctx, M, const_cast<pv_probe *>(d_probes), hop_cap, d_out, pa, (cudaStream_t)stream, ba);
     const size_t table_smem = indexed ? t.max_blob_bytes : t.max_linear_bytes;
     // the next hop's per-switch counts ride in the hop kernel's shared memory
     // after the staged table, when they fit
@@ -2428,16 +2575,14 @@ int walk_probes(pv_ctx *ctx, uint32_t M, const pv_probe *d_probes, uint32_t hop_
     const size_t hop_smem = port_off + port_bytes;
     int hop_blocks_per_sm = 0;
     const bool stats = ctx->opt_walk_stats != 0;
-    // compact flows with one path constraint per group are placed directly
-    // (and walked through walk records)
-    const bool direct = ba && (!pol || (pa->probe_pol == nullptr && (pa->per == 0 || pa->per % ba->ppg == 0)));
     const HopKernel hop_fn = direct ? pick_hop<true>(indexed, pol, stats, false) : pick_hop<false>(indexed, pol, stats, false);
     const HopKernel hop_fn0 = direct ? pick_hop<true>(indexed, pol, stats, true) : pick_hop<false>(indexed, pol, stats, true);
-    const TailKernel tail_fn = direct ? pick_tail<true>(pol, stats) : pick_tail<false>(pol, stats);
+    const ThreadKernel tail_fn = direct ? pick_thread<kSrcListRec>(pol, stats) : pick_thread<kSrcList>(pol, stats);
     if (int rc = pv_smem_limit(ctx, (const void *)hop_fn, "walk_hop_kernel smem")) return rc;
     if (int rc = pv_smem_limit(ctx, (const void *)hop_fn0, "walk_hop_kernel smem")) return rc;
     hop_blocks_per_sm = pv_blocks_per_sm(ctx, (const void *)hop_fn, kHopThreads, hop_smem);
-    const uint32_t hop_grid = (uint32_t)ctx->num_sms * (uint32_t)std::max(1, hop_blocks_per_sm);
+    const uint32_t hop_grid = std::min((uint32_t)ctx->num_sms * (uint32_t)std::max(1, hop_blocks_per_sm),
+                                       ctx->walk_visit_slots);
     const uint32_t init_grid = (uint32_t)ctx->num_sms * 8;
     const uint32_t max_desc = std::max(hop_grid, init_grid);
     const size_t o_a = 0, o_b = align256((size_t)M * 8), o_sorted = o_b + align256((size_t)M * 8);
@@ -2446,12 +2591,8 @@ int walk_probes(pv_ctx *ctx, uint32_t M, const pv_probe *d_probes, uint32_t hop_
     const size_t o_cur = o_seg + align256((size_t)(S + 2) * 4);
     const size_t o_desc = o_cur + align256((size_t)S * 4);
     const size_t o_ck = o_desc + 2 * align256((size_t)max_desc * 8);
-    const bool cycles = ctx->opt_walk_cycles == 0 && hop_cap > kCycleCheckFrom;
-    const uint64_t groups = ba ? ((uint64_t)M + ba->ppg - 1) / ba->ppg : 0;
-    const uint64_t G64 = groups * (ba ? ba->pods : 0);
-    if (direct && G64 > 0xFFFFFFFFull) return pv_fail(ctx, PV_EINVAL, "pv_verify_flows: too many (group, pod) pairs");
-    const uint32_t G = (uint32_t)G64;
-    const size_t o_pair = o_ck + (cycles ? align256((size_t)M * 4) : 0);
+    HopArgs g = walk_args(ctx, hop_cap, nullptr, d_out, pa);
+    const size_t o_pair = o_ck + (g.cycles ? align256((size_t)M * 4) : 0);
     // walk records (direct placement), or bound records the caller did not ask for
     const bool own_recs = direct || (ba && !d_probes);
     const size_t o_recs = o_pair + (direct ? align256((size_t)G * 4) : 0);
@@ -2490,7 +2631,6 @@ int walk_probes(pv_ctx *ctx, uint32_t M, const pv_probe *d_probes, uint32_t hop_
         const uint32_t groups32 = (uint32_t)groups;
         const size_t gsm = ba->ppg <= 0xFFFFu ? GroupInitSmem(ba->pods, ba->ppg, ba->dst_stride == 2).total : ~(size_t)0;
         const bool by_group = ba->pods <= kGroupInitMaxPods && gsm <= kGroupInitSmem && groups <= 0x7FFFFFFFull;
-        const uint64_t wait_ns = ctx->opt_test_stall_staging ? 50ull * 1000 * 1000 : 2ull * 1000 * 1000 * 1000;
         if (by_group) {
             const int rc2 = pol ? pv_smem_limit(ctx, (const void *)walk_init_group_kernel<true>, "walk_init_group_kernel smem")
                                 : pv_smem_limit(ctx, (const void *)walk_init_group_kernel<false>, "walk_init_group_kernel smem");
@@ -2499,11 +2639,11 @@ int walk_probes(pv_ctx *ctx, uint32_t M, const pv_probe *d_probes, uint32_t hop_
         if (by_group && pol)
             walk_init_group_kernel<true><<<groups32, kGroupInitThreads, gsm, st>>>(
                 M, probes_rw, t.num_hosts, t.d_host_switch, t.d_region, d_out, recs, seg,
-                pair_off, pa0, ba0, wait_ns, ctx->d_status);
+                pair_off, pa0, ba0, g.wait_ns, ctx->d_status);
         else if (by_group)
             walk_init_group_kernel<false><<<groups32, kGroupInitThreads, gsm, st>>>(
                 M, probes_rw, t.num_hosts, t.d_host_switch, t.d_region, d_out, recs, seg,
-                pair_off, pa0, ba0, wait_ns, ctx->d_status);
+                pair_off, pa0, ba0, g.wait_ns, ctx->d_status);
         else if (pol)
             walk_init_direct_kernel<true><<<init_grid, kGridThreads, 0, st>>>(
                 M, probes_rw, t.num_hosts, t.d_host_switch, t.d_region, d_out, recs, seg,
@@ -2531,37 +2671,12 @@ int walk_probes(pv_ctx *ctx, uint32_t M, const pv_probe *d_probes, uint32_t hop_
     pv_prof_stop(ctx, st, pr, direct ? 3 : 1);
     const size_t hist_smem = S <= kSmemHistMax ? (size_t)S * 4 : 0;
     const size_t scat_smem = S <= kSmemHistMax ? (size_t)S * 8 : 0;
-    HopArgs g;
-    g.cap = hop_cap;
     g.seg = seg;
-    g.S = S;
-    g.H = t.num_hosts;
-    g.blob = t.d_blob;
-    g.blob_offs = t.d_blob_offs;
-    g.region = t.d_region;
-    g.port_offs = t.d_port_offs;
-    g.port_peer = t.d_port_peer;
-    g.host_ip = t.d_host_ip;
     g.probes = probes_rw;
     g.recs = recs;
-    g.out = d_out;
-    g.status = ctx->d_status;
-    g.lane_max = (uint32_t)ctx->opt_walk_lane_max;
-    g.hop_live = ctx->d_walk_live;
     g.ck = (uint32_t *)(base + o_ck);
-    g.cycles = cycles ? 1u : 0u;
-    g.bounce = ctx->opt_walk_cycles == 0 && ctx->tb.links_symmetric ? 1u : 0u;   // any cap: no checkpoints needed
-    g.pa = pol ? *pa : no_policy;
-    g.hist_next = nullptr;
     g.hist_off = (uint32_t)hist_off;
     g.port_off = (uint32_t)port_off;
-    g.recs_at_position = 0;
-    g.host_addr = t.d_host_addr;
-    g.port_stage = t.d_port_stage;
-    g.stats = ctx->d_walk_stats;
-    ctx->last_walk_cap = hop_cap;
-    g.wait_extra = ctx->opt_test_stall_staging ? 16u : 0u;
-    g.wait_ns = ctx->opt_test_stall_staging ? 50ull * 1000 * 1000 : 2ull * 1000 * 1000 * 1000;
     uint32_t in_slices = init_grid;
     // hops from tail_hop on run in one walk_tail_kernel launch (indexed tables only)
     const uint32_t opt_tail = ctx->opt_walk_tail_hop < 0 ? t.tail_hop : (uint32_t)ctx->opt_walk_tail_hop;
@@ -2596,13 +2711,17 @@ int walk_probes(pv_ctx *ctx, uint32_t M, const pv_probe *d_probes, uint32_t hop_
         const uint32_t h = tail_hop - 1;   // the last regrouped hop wrote this list
         uint2 *lst = (h & 1) ? listA : listB;
         uint2 *dsc = (h & 1) ? descA : descB;
-        PV_TRY_CUDA(ctx, cudaMemsetAsync(ctx->d_walk_live + tail_hop, 0, (hop_cap - tail_hop) * sizeof(uint32_t), st),
-                    "tail live counts");
-        g.hop = tail_hop;
+        ThreadWalkArgs w = {};
+        w.list = lst;
+        w.desc = dsc;
+        w.first_hop = tail_hop;
+        w.visits = ctx->d_walk_visits;
         pr = pv_prof_start(ctx, st, PV_K_WALK_HOP);
-        tail_fn<<<hop_grid, 256, 0, st>>>(g, lst, dsc, hop_grid, tail_hop);
+        tail_fn<<<hop_grid, 256, 0, st>>>(g, w);
         pv_prof_stop(ctx, st, pr, 1);
     }
+    ctx->last_walk_hops = tail_hop;
+    ctx->last_walk_blocks = tail_hop < hop_cap ? hop_grid : 0u;
     pv_mark_use(ctx, st);
     return pv_check_launch(ctx, "probe walk kernels");
 }

@@ -257,6 +257,7 @@ extern "C" int pv_create(pv_ctx **out, int cuda_device) {
     int smem = 0;
     cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, cuda_device);
     ctx->max_smem_optin = (size_t)smem;
+    ctx->walk_visit_slots = (uint32_t)ctx->num_sms * 32u;   // most resident blocks
     cudaMemPoolProps props = {};
     props.allocType = cudaMemAllocationTypePinned;
     props.location.type = cudaMemLocationTypeDevice;
@@ -287,11 +288,14 @@ extern "C" int pv_create(pv_ctx **out, int cuda_device) {
                         "walk statistics") != PV_OK ||
         cudaMemset(ctx->d_walk_live, 0, (PV_MAX_HOP_CAP + 1) * sizeof(uint32_t)) != cudaSuccess ||
         pv_device_alloc(ctx, (void **)&ctx->d_reach_asym, sizeof(uint32_t), "reach symmetry flag") != PV_OK ||
+        pv_device_alloc(ctx, (void **)&ctx->d_walk_visits, ctx->walk_visit_slots * sizeof(unsigned long long),
+                        "walk visit counts") != PV_OK ||
         pv_device_alloc(ctx, (void **)&ctx->d_walk_stats, PV_WALK_STATS * sizeof(unsigned long long),
                         "walk statistics counters") != PV_OK ||
         cudaMemset(ctx->d_walk_stats, 0, PV_WALK_STATS * sizeof(unsigned long long)) != cudaSuccess) {
         pv_device_free(ctx->d_status);
         pv_device_free(ctx->d_walk_live);
+        pv_device_free(ctx->d_walk_visits);
         pv_device_free(ctx->d_walk_stats);
         pv_device_free(ctx->d_reach_asym);
         cudaEventDestroy(ctx->last_use);
@@ -329,6 +333,7 @@ extern "C" void pv_destroy(pv_ctx *ctx) {
     pv_device_free(ctx->scratch);
     pv_device_free(ctx->d_status);
     pv_device_free(ctx->d_walk_live);
+    pv_device_free(ctx->d_walk_visits);
     pv_device_free(ctx->d_walk_stats);
     pv_device_free(ctx->d_reach_asym);
     delete ctx;
@@ -409,12 +414,16 @@ extern "C" int pv_get_stat(const pv_ctx *ctx, int stat, int64_t *value) {
     case PV_STAT_WALK_INDEX_BYTES: *value = (int64_t)ctx->tb.max_blob_bytes; return PV_OK;
     case PV_STAT_WALK_LIVE_TOTAL: {
         uint32_t live[PV_MAX_HOP_CAP + 1];
-        const uint32_t cap = ctx->last_walk_cap;
-        if (cap && cudaMemcpy(live, ctx->d_walk_live, cap * sizeof(uint32_t), cudaMemcpyDeviceToHost) !=
-                       cudaSuccess)
+        const uint32_t hops = ctx->last_walk_hops, blocks = ctx->last_walk_blocks;
+        std::vector<unsigned long long> visits(blocks);
+        if (hops && cudaMemcpy(live, ctx->d_walk_live, hops * sizeof(uint32_t), cudaMemcpyDeviceToHost) != cudaSuccess)
+            return PV_ECUDA;
+        if (blocks && cudaMemcpy(visits.data(), ctx->d_walk_visits, blocks * sizeof(unsigned long long),
+                                 cudaMemcpyDeviceToHost) != cudaSuccess)
             return PV_ECUDA;
         int64_t sum = 0;
-        for (uint32_t h = 0; h < cap; ++h) sum += live[h];
+        for (uint32_t h = 0; h < hops; ++h) sum += live[h];
+        for (unsigned long long n : visits) sum += (int64_t)n;
         *value = sum;
         return PV_OK;
     }

@@ -129,7 +129,10 @@ struct pv_ctx {
     unsigned long long *d_walk_stats = nullptr;   // [PV_WALK_STATS] counters of the last statistics walk
     int opt_test_stall_staging = 0;   // failure test: staging waits expect bytes that never come
     uint32_t *d_walk_live = nullptr;  // [PV_MAX_HOP_CAP + 1] live probes per hop of the last walk
-    uint32_t last_walk_cap = 0;       // hop cap of the last walk
+    unsigned long long *d_walk_visits = nullptr;   // [walk_visit_slots] visits of the last walk's thread-walk blocks
+    uint32_t walk_visit_slots = 0;
+    uint32_t last_walk_hops = 0;      // entries of d_walk_live and of d_walk_visits that the last walk wrote
+    uint32_t last_walk_blocks = 0;
     int opt_reach = 0;                // 0: components on symmetric graphs, 1: sweeps only
     uint32_t *d_reach_asym = nullptr; // != 0: the last reach call's graph is not symmetric
     bool last_reach_comp = false;     // the last reach call launched the component path
