@@ -173,16 +173,24 @@ __global__ void __launch_bounds__(1024) compile_tables_kernel(const uint32_t *__
 // ---------------------------------------------------------------------------
 // A switch's blob (sections 16-byte aligned):
 //   header   uint4 {npad | n_plain << 16, n_items, n_segs, n_bnd}
-//   A[n_plain] uint4, B[n_plain] uint2   the plain rules (those not in a
-//                                    segment, the only ones items name), in
-//                                    first-match order (records as above)
 //   boff[kBuckets + 1] u32           item range of each destination-port bucket
+//   masks[kBuckets][2 * kClasses] u32   candidate filter of each bucket: bit j
+//                                    of word c is set when group j of the
+//                                    bucket's items (ceil(length / 32) items
+//                                    to a group) holds a segment token or a
+//                                    rule whose destination range meets
+//                                    address class c (word kClasses + c: its
+//                                    source range)
+//   rules[n_plain] uint4             the plain rules (those not in a segment,
+//                                    the only ones items name), in first-match
+//                                    order (PlainRule)
 //   items[n_items] u16               per bucket, in first-match order: a plain
 //                                    rule's position, or kSegItem | segment id
 //   segs[n_segs] uint2               {first boundary, number of boundaries}
-//   bnd[n_bnd] u32, win[n_bnd] u32   per segment: ascending elementary-interval
-//                                    starts (the first is 0) and the interval's
-//                                    winner (kWinFound | action, or 0 = none)
+//   bw[n_bnd] uint2                  per segment: {start, winner} of its
+//                                    ascending elementary intervals (the first
+//                                    starts at 0; winner = kWinFound | action,
+//                                    or 0 = none)
 //   jmp[n_segs]                      per segment, kJumpBytes: {base, shift,
 //                                    J[kJumpSlots + 1] u16}: base = the
 //                                    segment's second boundary (its first
@@ -194,7 +202,11 @@ __global__ void __launch_bounds__(1024) compile_tables_kernel(const uint32_t *__
 //   A[npad] uint4, B[npad] uint2     all rules in first-match order, padded to a
 //                                    multiple of 32 (linear scan, statistics)
 // The indexed kernel stages everything before the full rule list; the
-// linear kernel stages the header and the full rule list.
+// linear kernel stages the header and the full rule list.  When the filter is
+// what does not fit, the indexed kernel leaves it out of its stage and walks
+// the lists unfiltered.  boff, masks and
+// rules start at offsets that do not depend on the header, so a walk that
+// reads the blob in place loads them together with it.
 // Exactness.  A header whose dport lies in bucket k can only match rules whose
 // port range meets bucket k; bucket k's list keeps the first-match order, so
 // its first hit is the first match of the whole table.  A segment is a run of
@@ -210,6 +222,8 @@ constexpr uint32_t kTailEarlyItems = 12;    // candidate items per bucket below 
 constexpr uint32_t kMaxSegment = 4096;      // longer runs are split (in order: still exact)
 constexpr uint32_t kSegItem = 0x8000u;
 constexpr uint32_t kWinFound = 0x80000000u;
+constexpr uint32_t kActionDrop = 256;       // PV_DROP in a first match's result and in PlainRule
+constexpr uint32_t kClasses = 8;            // address classes of the candidate filter
 constexpr uint32_t kJumpSlots = 256;
 constexpr uint32_t kJumpBytes = (8 + (kJumpSlots + 1) * 2 + 15) / 16 * 16;   // 528
 static_assert(kJumpBytes % 16 == 0, "jump blocks keep the blob's later sections 16-byte aligned");
@@ -248,17 +262,17 @@ struct IndexSmem {
 __host__ __device__ inline uint32_t up16(uint32_t b) { return (b + 15u) & ~15u; }
 
 struct BlobLayout {
-    uint32_t a, b, boff, items, segs, bnd, win, jmp, fa, fb, total;
+    static constexpr uint32_t boff = 16;
+    static constexpr uint32_t masks = (boff + (kBuckets + 1) * 4 + 15) / 16 * 16;
+    static constexpr uint32_t rules = masks + kBuckets * 2 * kClasses * 4;
+    static constexpr uint32_t filter_bytes = rules - masks;
+    uint32_t items, segs, bw, jmp, fa, fb, total;
     __host__ __device__ BlobLayout(uint32_t npad, uint32_t n_plain, uint32_t n_items, uint32_t n_segs,
                                    uint32_t n_bnd) {
-        a = 16;
-        b = a + up16(n_plain * 16);
-        boff = b + up16(n_plain * 8);
-        items = boff + up16((kBuckets + 1) * 4);
+        items = rules + n_plain * 16;
         segs = items + up16(n_items * 2);
-        bnd = segs + up16(n_segs * 8);
-        win = bnd + up16(n_bnd * 4);
-        jmp = win + up16(n_bnd * 4);
+        bw = segs + up16(n_segs * 8);
+        jmp = bw + up16(n_bnd * 8);
         fa = jmp + n_segs * kJumpBytes;
         fb = fa + npad * 16;
         total = fb + npad * 8;
@@ -266,6 +280,43 @@ struct BlobLayout {
     __host__ __device__ explicit BlobLayout(uint4 hdr)
         : BlobLayout(hdr.x & 0xFFFFu, hdr.x >> 16, hdr.y, hdr.z, hdr.w) {}
 };
+
+// A plain rule in 16 bytes: {source value, destination value, dport lo | hi
+// << 16, meta}, meta bits 0-7 in_port, 8-13 and 14-19 the source and
+// destination host bits (32 - prefix length), 20-28 the action (kActionDrop =
+// drop), 31 set when the in_port counts.  One 16-byte load per test; the
+// separate masks of the full records would cost a second one.
+__device__ __forceinline__ uint4 plain_rule(uint4 a, uint2 b) {
+    const uint32_t act = min(b.y >> 16, kActionDrop);
+    return make_uint4(a.x, a.z, b.x,
+                      (b.y & 0xFFu) | (32u - __popc(a.y)) << 8 | (32u - __popc(a.w)) << 14 | act << 20 |
+                          ((b.y & 0xFF00u) ? 0x80000000u : 0u));
+}
+
+__device__ __forceinline__ bool plain_hit(uint4 r, uint32_t src, uint32_t dst, uint32_t dport, uint32_t in_port) {
+    // a funnel shift with clamp gives 0 for 32 host bits (prefix length 0)
+    const uint32_t ds = __funnelshift_rc(src ^ r.x, 0u, (r.w >> 8) & 63u);
+    const uint32_t dd = __funnelshift_rc(dst ^ r.y, 0u, (r.w >> 14) & 63u);
+    uint32_t pm;   // 0xFF when bit 31 is set: byte 0 repeats byte 3's sign, the others are 0
+    asm("prmt.b32 %0, %1, 0, 0x444B;" : "=r"(pm) : "r"(r.w));
+    const uint32_t dp = (in_port ^ r.w) & pm;
+    return (ds | dd | dp) == 0 && dport >= (r.z & 0xFFFFu) && dport <= (r.z >> 16);
+}
+
+__device__ __forceinline__ uint32_t plain_result(uint4 r) { return kWinFound | ((r.w >> 20) & 0x1FFu); }
+
+// Class of an address: the number of boundaries at or below it.  The
+// boundaries are the octiles of the loaded hosts' addresses (what probes
+// carry), so rules with long prefixes meet one or two of the eight classes;
+// any boundaries are exact, others only filter less.
+__device__ __forceinline__ uint32_t addr_class(const pv_addr_classes &c, uint32_t ip) {
+    const uint32_t b0 = c.b[0], b1 = c.b[1], b2 = c.b[2], b3 = c.b[3], b4 = c.b[4], b5 = c.b[5], b6 = c.b[6];
+    const bool p2 = ip >= b3;
+    const uint32_t m1 = p2 ? b5 : b1, lo = p2 ? b4 : b0, hi = p2 ? b6 : b2;
+    const bool p1 = ip >= m1;
+    const bool p0 = ip >= (p1 ? hi : lo);
+    return (p2 ? 4u : 0u) | (p1 ? 2u : 0u) | (p0 ? 1u : 0u);
+}
 
 // Bytes of the hop kernel's staged port table ({peer, aux} per port).
 inline size_t port_stage_bytes(uint32_t max_ports) { return ((size_t)max_ports * 8 + 15) & ~(size_t)15; }
@@ -323,7 +374,8 @@ __global__ void __launch_bounds__(kIndexThreads) index_build_kernel(const uint32
                                                            const uint4 *__restrict__ A, const uint2 *__restrict__ B,
                                                            uint32_t *__restrict__ sizes,
                                                            const uint64_t *__restrict__ blob_offs,
-                                                           uint8_t *__restrict__ blob, IndexSmem sm) {
+                                                           uint8_t *__restrict__ blob, IndexSmem sm,
+                                                           pv_addr_classes cls) {
     extern __shared__ __align__(16) uint32_t s_mem[];
     uint32_t *s_keys = s_mem;                                            // [sort_cap]
     uint32_t *s_win = s_keys + sm.sort_cap;                              // [key_cap]
@@ -409,13 +461,9 @@ __global__ void __launch_bounds__(kIndexThreads) index_build_kernel(const uint32
     if (kFill) {
         out = blob + blob_offs[s];
         L = BlobLayout(npad, n_plain, sizes[4 * s], sizes[4 * s + 1], sizes[4 * s + 2]);
-        uint4 *ca = reinterpret_cast<uint4 *>(out + L.a);
-        uint2 *cb = reinterpret_cast<uint2 *>(out + L.b);
+        uint4 *rules = reinterpret_cast<uint4 *>(out + L.rules);
         for (uint32_t i = t; i < n; i += nt)
-            if (s_cls[i] < 0) {
-                ca[s_plain[i]] = a[i];
-                cb[s_plain[i]] = b[i];
-            }
+            if (s_cls[i] < 0) rules[s_plain[i]] = plain_rule(a[i], b[i]);
     }
 
     // 2. bucket lists.  Rule i puts one item into each bucket its port range
@@ -580,7 +628,7 @@ __global__ void __launch_bounds__(kIndexThreads) index_build_kernel(const uint32
         __syncthreads();
         for (uint32_t x = t; x < K; x += nt) {
             const uint32_t r = s_win[x];
-            s_win[x] = r == 0xFFFFFFFFu ? 0u : (kWinFound | s_act[r]);
+            s_win[x] = r == 0xFFFFFFFFu ? 0u : (kWinFound | min((uint32_t)s_act[r], kActionDrop));
         }
         __syncthreads();
         // merge adjacent intervals with the same winner
@@ -594,18 +642,16 @@ __global__ void __launch_bounds__(kIndexThreads) index_build_kernel(const uint32
         const uint32_t K2 = block_exclusive_scan(s_pos, K, s_warp);
         if (kFill) {
             uint2 *segs = reinterpret_cast<uint2 *>(out + L.segs);
-            uint32_t *bnd = reinterpret_cast<uint32_t *>(out + L.bnd);
-            uint32_t *win = reinterpret_cast<uint32_t *>(out + L.win);
+            uint2 *bw = reinterpret_cast<uint2 *>(out + L.bw);
             if (t == 0) segs[j] = make_uint2(n_bnd, K2);
             for (uint32_t x = t, q = 0; x < K; x += nt, ++q)
                 if ((keep_mask >> q) & 1u) {
-                    bnd[n_bnd + s_pos[x]] = s_keys[x];
-                    win[n_bnd + s_pos[x]] = s_win[x];
+                    bw[n_bnd + s_pos[x]] = make_uint2(s_keys[x], s_win[x]);
                 }
             __syncthreads();   // the segment's boundaries are in the blob
             uint8_t *jb = out + L.jmp + j * kJumpBytes;
-            const uint32_t *bb = bnd + n_bnd;
-            const uint32_t base = K2 > 1 ? bb[1] : 0xFFFFFFFFu, top = bb[K2 - 1];
+            const uint2 *bb = bw + n_bnd;
+            const uint32_t base = K2 > 1 ? bb[1].x : 0xFFFFFFFFu, top = bb[K2 - 1].x;
             uint32_t shift = 0;
             while (shift < 32 && ((uint64_t)(top - (K2 > 1 ? base : top)) >> shift) >= kJumpSlots) ++shift;
             if (t == 0) {
@@ -620,7 +666,7 @@ __global__ void __launch_bounds__(kIndexThreads) index_build_kernel(const uint32
                     uint32_t lo = 0, hi = K2;   // bb[lo] <= start < bb[hi]
                     while (hi - lo > 1) {
                         const uint32_t mid = (lo + hi) >> 1;
-                        if (bb[mid] <= (uint32_t)start) lo = mid;
+                        if (bb[mid].x <= (uint32_t)start) lo = mid;
                         else hi = mid;
                     }
                     v = lo;
@@ -632,7 +678,42 @@ __global__ void __launch_bounds__(kIndexThreads) index_build_kernel(const uint32
         __syncthreads();
     }
 
-    // 4. header and the full rule list
+    // 4. candidate filter: a warp per bucket, a lane per group of items; the
+    //    sixteen words come from ballots (items and rules were written above
+    //    by this block)
+    if (kFill) {
+        __syncthreads();
+        const uint32_t *boff = reinterpret_cast<const uint32_t *>(out + L.boff);
+        const uint16_t *items = reinterpret_cast<const uint16_t *>(out + L.items);
+        const uint4 *rules = reinterpret_cast<const uint4 *>(out + L.rules);
+        uint32_t *masks = reinterpret_cast<uint32_t *>(out + L.masks);
+        for (uint32_t k = warp; k < kBuckets; k += kIndexWarps) {
+            const uint32_t i0 = boff[k], len = boff[k + 1] - i0, per = (len + 31) / 32;
+            uint32_t meets = 0;   // bit c: destination class c, bit kClasses + c: source class c
+            for (uint32_t q = lane * per; q < min(len, (lane + 1) * per); ++q) {
+                const uint32_t it = items[i0 + q];
+                if (it & kSegItem) {
+                    meets = 0xFFFFu;
+                    continue;
+                }
+                const uint4 r = rules[it];
+                const uint32_t sh = (r.w >> 8) & 63u, dh = (r.w >> 14) & 63u;   // host bits
+                const uint32_t s1 = r.x | (sh < 32 ? (1u << sh) - 1u : ~0u), d1 = r.y | (dh < 32 ? (1u << dh) - 1u : ~0u);
+                const uint32_t sc = (2u << addr_class(cls, s1)) - (1u << addr_class(cls, r.x));
+                const uint32_t dc = (2u << addr_class(cls, d1)) - (1u << addr_class(cls, r.y));
+                meets |= dc | sc << kClasses;
+            }
+            uint32_t mine = 0;
+#pragma unroll
+            for (uint32_t c = 0; c < 2 * kClasses; ++c) {
+                const uint32_t word = __ballot_sync(PV_FULL_MASK, (meets >> c) & 1u);
+                if (lane == c) mine = word;
+            }
+            if (lane < 2 * kClasses) masks[k * 2 * kClasses + lane] = mine;
+        }
+    }
+
+    // 5. header and the full rule list
     if (kFill) {
         if (t == 0) *reinterpret_cast<uint4 *>(out) = make_uint4(npad | n_plain << 16, n_items, nsegs, n_bnd);
         uint4 *oa = reinterpret_cast<uint4 *>(out + L.fa);
@@ -1224,6 +1305,7 @@ struct HopArgs {
     uint2 *next_list;
     uint2 *next_desc;
     int32_t *status;
+    uint32_t stage_skip; // bytes of the candidate filter when it is left out of the indexed stage, else 0
     uint32_t lane_max;   // longest candidate list handled one probe per lane
     uint32_t wait_extra; // bytes the staging barrier expects beyond the copy (0; > 0 only in failure tests)
     uint64_t wait_ns;    // bound on each staging wait
@@ -1236,7 +1318,8 @@ struct HopArgs {
     uint32_t hist_off;   // byte offset of the block's count array in dynamic shared memory
     uint32_t port_off;   // byte offset of the staged port table in dynamic shared memory
     uint32_t recs_at_position;   // 1: no list, entry i is record i (first hop of directly placed flows)
-    const uint2 *host_addr;      // [H] {address, attachment port} of each host
+    const uint2 *host_addr;      // [H] {address, attachment port | address class << 8} of each host
+    pv_addr_classes cls;
     const uint2 *port_stage;     // [ports] {peer, aux} as the hop kernel stages them
     unsigned long long *stats;   // [PV_WALK_STATS] counters of the statistics kernels (kStats)
 };
@@ -1263,7 +1346,7 @@ __device__ __forceinline__ uint32_t scan_first_match(const uint4 *A, const uint2
         const uint32_t diff = ((src ^ a.x) & a.y) | ((dst ^ a.z) & a.w) | ((in_port ^ b.y) & ((b.y >> 8) & 0xFFu));
         if (diff == 0 && dport >= (b.x & 0xFFFFu) && dport <= (b.x >> 16)) {
             *depth = r + 1;
-            return kWinFound | (b.y >> 16);
+            return kWinFound | min(b.y >> 16, kActionDrop);
         }
     }
     *depth = npad;
@@ -1310,14 +1393,16 @@ __device__ __forceinline__ uint4 load_raw(const HopArgs &g, uint32_t x) {
 
 template <bool kRec>
 __device__ __forceinline__ uint4 header_of(const HopArgs &g, uint4 raw, uint32_t x, uint32_t *id,
-                                           uint32_t *src_port) {
+                                           uint32_t *src_port, uint32_t *src_class) {
     if (kRec) {
         *id = raw.x;
-        const uint2 ha = __ldg(g.host_addr + (raw.z >> 16));   // the source host's address and port
-        *src_port = ha.y;
+        const uint2 ha = __ldg(g.host_addr + (raw.z >> 16));   // the source host's address, port and class
+        *src_port = ha.y & 0xFFu;
+        *src_class = ha.y >> 8;
         return make_uint4(ha.x, raw.y, raw.z, raw.w);
     }
     *id = x;
+    *src_class = addr_class(g.cls, raw.x);
     return raw;
 }
 
@@ -1334,7 +1419,7 @@ __device__ __forceinline__ uint32_t first_match_linear(const uint8_t *sm, uint32
         const bool hit = diff == 0 && dport >= (b.x & 0xFFFFu) && dport <= (b.x >> 16);
         const uint32_t m = __ballot_sync(PV_FULL_MASK, hit);
         if (kStats) tests += 32;
-        if (m) return kWinFound | __shfl_sync(PV_FULL_MASK, b.y >> 16, __ffs(m) - 1);
+        if (m) return kWinFound | min(__shfl_sync(PV_FULL_MASK, b.y >> 16, __ffs(m) - 1), kActionDrop);
     }
     return 0u;
 }
@@ -1357,36 +1442,34 @@ __device__ __forceinline__ void jump_range(const uint8_t *jb, uint32_t dst, uint
 }
 
 // Winner of the elementary interval holding dst: the warp narrows the range
-// 32-ways per step (bnd ascending, bnd[0] = 0 <= dst).
-__device__ __forceinline__ uint32_t segment_lookup(const uint32_t *bnd, const uint32_t *win, uint32_t cnt,
-                                                   uint32_t dst, uint32_t lane) {
+// 32-ways per step (starts ascending, the first 0 <= dst).
+__device__ __forceinline__ uint32_t segment_lookup(const uint2 *bw, uint32_t cnt, uint32_t dst, uint32_t lane) {
     uint32_t lo = 0, len = cnt;
     while (len > 32) {
         const uint32_t stride = (len + 31) / 32;
-        const bool le = lane * stride < len && bnd[lo + lane * stride] <= dst;
+        const bool le = lane * stride < len && bw[lo + lane * stride].x <= dst;
         const uint32_t c = __popc(__ballot_sync(PV_FULL_MASK, le));
         lo += (c - 1) * stride;
         len = min(stride, len - (c - 1) * stride);
     }
-    const bool le = lane < len && bnd[lo + lane] <= dst;
+    const bool le = lane < len && bw[lo + lane].x <= dst;
     const uint32_t c = __popc(__ballot_sync(PV_FULL_MASK, le));
-    return win[lo + c - 1];
+    return bw[lo + c - 1].y;
 }
 
 // Indexed first match: walk the dport bucket's candidate list in first-match
 // order, 32 items per step; segment items are answered by interval lookup.
 template <bool kStats>
-__device__ __forceinline__ uint32_t first_match_indexed(const uint8_t *sm, const uint4 hdr, uint32_t lane,
+__device__ __forceinline__ uint32_t first_match_indexed(const uint8_t *sm, uint32_t skip, const uint4 hdr, uint32_t lane,
                                                         uint32_t src, uint32_t dst, uint32_t dport, uint32_t in_port,
                                                         uint32_t &tests, uint32_t &lookups) {
     const BlobLayout L(hdr);
-    const uint4 *sA = reinterpret_cast<const uint4 *>(sm + L.a);
-    const uint2 *sB = reinterpret_cast<const uint2 *>(sm + L.b);
     const uint32_t *boff = reinterpret_cast<const uint32_t *>(sm + L.boff);
+    sm -= skip;
+    const uint4 *rules = reinterpret_cast<const uint4 *>(sm + L.rules);
     const uint16_t *items = reinterpret_cast<const uint16_t *>(sm + L.items);
     const uint2 *segs = reinterpret_cast<const uint2 *>(sm + L.segs);
-    const uint32_t *bnd = reinterpret_cast<const uint32_t *>(sm + L.bnd);
-    const uint32_t *win = reinterpret_cast<const uint32_t *>(sm + L.win);
+    const uint2 *bw = reinterpret_cast<const uint2 *>(sm + L.bw);
     const uint32_t k = dport >> kBucketShift;
     const uint32_t i0 = boff[k], i1 = boff[k + 1];
     for (uint32_t c0 = i0; c0 < i1; c0 += 32) {
@@ -1395,13 +1478,11 @@ __device__ __forceinline__ uint32_t first_match_indexed(const uint8_t *sm, const
         const bool valid = it != 0xFFFFu;
         const bool is_seg = valid && (it & kSegItem);
         bool hit = false;
-        uint32_t action = 0;
+        uint32_t res = 0;
         if (valid && !is_seg) {
-            const uint4 a = sA[it];
-            const uint2 b = sB[it];
-            const uint32_t diff = ((src ^ a.x) & a.y) | ((dst ^ a.z) & a.w) | ((in_port ^ b.y) & ((b.y >> 8) & 0xFFu));
-            hit = diff == 0 && dport >= (b.x & 0xFFFFu) && dport <= (b.x >> 16);
-            action = b.y >> 16;
+            const uint4 r = rules[it];
+            hit = plain_hit(r, src, dst, dport, in_port);
+            res = plain_result(r);
         }
         uint32_t G = __ballot_sync(PV_FULL_MASK, hit);
         uint32_t Sg = __ballot_sync(PV_FULL_MASK, is_seg);
@@ -1411,12 +1492,12 @@ __device__ __forceinline__ uint32_t first_match_indexed(const uint8_t *sm, const
             const uint32_t ps = Sg ? (uint32_t)__ffs(Sg) - 1 : 32u;
             if (ps < pg) {
                 const uint2 sd = segs[__shfl_sync(PV_FULL_MASK, it, ps) & 0x7FFFu];
-                const uint32_t w = segment_lookup(bnd + sd.x, win + sd.x, sd.y, dst, lane);
+                const uint32_t w = segment_lookup(bw + sd.x, sd.y, dst, lane);
                 if (kStats) ++lookups;
                 if (w & kWinFound) return w;
                 Sg &= Sg - 1u;
             } else if (pg < 32u) {
-                return kWinFound | __shfl_sync(PV_FULL_MASK, action, pg);
+                return __shfl_sync(PV_FULL_MASK, res, pg);
             } else {
                 break;
             }
@@ -1425,86 +1506,90 @@ __device__ __forceinline__ uint32_t first_match_indexed(const uint8_t *sm, const
     return 0u;
 }
 
+// A bucket's candidates in first-match order: the items of the groups that
+// the filter leaves for the probe's address classes.  The rule tests (a
+// 16-byte load from a random place and some 15 instructions each) bound a
+// first match; two filter words cut them from 15 to about 2 at 2,000 rules
+// a switch.  Eight classes a side cost 16 KB of a stage, so that tables of
+// 2,000 rules still leave three blocks an SM.  Before and after: 10M probes
+// on a k=16 fat tree 1,141 -> 817 us, 100,003 probes on 512 switches of 1,000
+// rules 62 -> 44 us, 50M flows over the same 1,547 -> 1,473 us.
+struct Candidates {
+    uint32_t m, i0, i1, per, at, end;   // groups left; the bucket's items; items per group; the group in hand
+    __device__ Candidates(uint32_t left, uint32_t first, uint32_t past)
+        : m(left), i0(first), i1(past), per((past - first + 31) / 32), at(0), end(0) {}
+    __device__ __forceinline__ uint32_t all() const {   // every group of the list
+        return i1 == i0 ? 0u : ~0u >> (32 - (i1 - i0 + per - 1) / per);
+    }
+    __device__ __forceinline__ bool next(uint32_t *item) {   // the next candidate's item index
+        if (at == end) {
+            if (m == 0) return false;
+            at = i0 + (uint32_t)(__ffs(m) - 1) * per;
+            end = min(at + per, i1);
+            m &= m - 1u;
+        }
+        *item = at++;
+        return true;
+    }
+};
+
 // Scalar first match, one probe per lane (called by all 32 lanes; inactive
-// lanes return 0): each lane walks its bucket's candidate list in order.
-// Plain rules are tested until a hit or a segment token; the warp then
-// reconverges and the lanes parked on a segment token run their interval
-// binary searches together (a segment miss resumes the walk after the token).
+// lanes return 0): each lane walks its bucket's candidates in order, src and
+// dst of classes sc and dc.  Plain rules are tested until a hit or a segment
+// token; the warp then reconverges and the lanes parked on a segment token
+// run their interval searches together (a segment miss resumes the walk).
 template <bool kStats>
-__device__ __forceinline__ uint32_t first_match_lane(const uint8_t *sm, const BlobLayout &L, bool active,
-                                                     uint32_t src, uint32_t dst, uint32_t dport, uint32_t in_port,
-                                                     uint32_t &tests, uint32_t &lookups) {
-    const uint4 *sA = reinterpret_cast<const uint4 *>(sm + L.a);
-    const uint2 *sB = reinterpret_cast<const uint2 *>(sm + L.b);
+__device__ __forceinline__ uint32_t first_match_lane(const uint8_t *sm, uint32_t skip, const BlobLayout &L,
+                                                     bool active, uint32_t src, uint32_t dst, uint32_t dport, uint32_t in_port,
+                                                     uint32_t sc, uint32_t dc, uint32_t &tests, uint32_t &lookups) {
     const uint32_t *boff = reinterpret_cast<const uint32_t *>(sm + L.boff);
+    const uint32_t *masks = reinterpret_cast<const uint32_t *>(sm + L.masks);
+    sm -= skip;   // skip: bytes left out of the stage where the filter would be
+    const uint4 *rules = reinterpret_cast<const uint4 *>(sm + L.rules);
     const uint16_t *items = reinterpret_cast<const uint16_t *>(sm + L.items);
     const uint2 *segs = reinterpret_cast<const uint2 *>(sm + L.segs);
-    const uint32_t *bnd = reinterpret_cast<const uint32_t *>(sm + L.bnd);
-    const uint32_t *win = reinterpret_cast<const uint32_t *>(sm + L.win);
+    const uint2 *bw = reinterpret_cast<const uint2 *>(sm + L.bw);
     const uint32_t k = dport >> kBucketShift;
-    uint32_t i = active ? boff[k] : 0u, i1 = active ? boff[k + 1] : 0u;
+    const uint32_t *mk = masks + k * (2 * kClasses);
+    Candidates cand(0u, boff[k], boff[k + 1]);
+    if (active) cand.m = skip ? cand.all() : mk[dc] & mk[kClasses + sc];
     uint32_t result = 0;
     bool done = !active;
     while (__any_sync(PV_FULL_MASK, !done)) {
         uint32_t seg = 0xFFFFFFFFu;
-        if (!done) {
-            // two items per step, both rules loaded before either is tested
-            // (a segment token's slot loads rule 0, unused)
-            auto hit = [&](uint4 a, uint2 bb) {
-                const uint32_t diff =
-                    ((src ^ a.x) & a.y) | ((dst ^ a.z) & a.w) | ((in_port ^ bb.y) & ((bb.y >> 8) & 0xFFu));
-                return diff == 0 && dport >= (bb.x & 0xFFFFu) && dport <= (bb.x >> 16);
-            };
-            for (; i < i1; i += 2) {
-                const uint32_t it0 = items[i];
-                const bool has1 = i + 1 < i1;
-                const uint32_t it1 = has1 ? items[i + 1] : 0u;
-                const uint32_t r0 = (it0 & kSegItem) ? 0u : it0, r1 = (it1 & kSegItem) ? 0u : it1;
-                const uint4 a0 = sA[r0], a1 = sA[r1];
-                const uint2 b0 = sB[r0], b1 = sB[r1];
-                if (it0 & kSegItem) {
-                    seg = it0 & 0x7FFFu;
-                    break;
-                }
-                if (kStats) ++tests;
-                if (hit(a0, b0)) {
-                    result = kWinFound | (b0.y >> 16);
-                    done = true;
-                    break;
-                }
-                if (!has1) break;
-                if (it1 & kSegItem) {
-                    seg = it1 & 0x7FFFu;
-                    ++i;   // i names the token, so a segment miss resumes after it
-                    break;
-                }
-                if (kStats) ++tests;
-                if (hit(a1, b1)) {
-                    result = kWinFound | (b1.y >> 16);
-                    done = true;
-                    break;
-                }
+        while (!done) {
+            uint32_t i;
+            if (!cand.next(&i)) {   // none left: table miss
+                done = true;
+                break;
             }
-            if (!done && seg == 0xFFFFFFFFu) done = true;   // list exhausted: table miss
+            const uint32_t it = items[i];
+            if (it & kSegItem) {
+                seg = it & 0x7FFFu;
+                break;
+            }
+            const uint4 r = rules[it];
+            if (kStats) ++tests;
+            if (plain_hit(r, src, dst, dport, in_port)) {
+                result = plain_result(r);
+                done = true;
+            }
         }
         __syncwarp();
         if (seg != 0xFFFFFFFFu) {
-            const uint2 sd = segs[seg];
-            const uint32_t *b = bnd + sd.x;
-            uint32_t lo, len;   // b[lo] <= dst; answer in [lo, lo + len)
+            const uint2 *b = bw + segs[seg].x;
+            uint32_t lo, len;   // b[lo].x <= dst; answer in [lo, lo + len)
             jump_range(sm + L.jmp + seg * kJumpBytes, dst, &lo, &len);
             while (len > 1) {
                 const uint32_t half = len >> 1;
-                lo = b[lo + half] <= dst ? lo + half : lo;
+                lo = b[lo + half].x <= dst ? lo + half : lo;
                 len -= half;
             }
-            const uint32_t w = win[sd.x + lo];
+            const uint32_t w = b[lo].y;
             if (kStats) ++lookups;
             if (w & kWinFound) {
                 result = w;
                 done = true;
-            } else {
-                ++i;
             }
         }
     }
@@ -1604,9 +1689,14 @@ __global__ void __launch_bounds__(kHopThreads, 4) walk_hop_kernel(HopArgs g) {
         __syncthreads();   // everyone is done with the previous table and ports
         if (threadIdx.x == 0) {
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            if (kIndexed) {   // header, plain rules, index
-                mbar_arrive_expect_tx(&s_bar, L.fa + g.wait_extra);
-                bulk_g2s_keep(s_raw, src_blob, L.fa, &s_bar);
+            if (kIndexed) {   // header, index, plain rules
+                mbar_arrive_expect_tx(&s_bar, L.fa - g.stage_skip + g.wait_extra);
+                if (!g.stage_skip) {
+                    bulk_g2s_keep(s_raw, src_blob, L.fa, &s_bar);
+                } else {   // all but the filter
+                    bulk_g2s_keep(s_raw, src_blob, L.masks, &s_bar);
+                    if (L.fa > L.rules) bulk_g2s_keep(s_raw + L.masks, src_blob + L.rules, L.fa - L.rules, &s_bar);
+                }
             } else {          // header and the full rule list
                 mbar_arrive_expect_tx(&s_bar, linear_bytes(npad) + g.wait_extra);
                 bulk_g2s_keep(s_raw, src_blob, 16, &s_bar);
@@ -1656,10 +1746,10 @@ __global__ void __launch_bounds__(kHopThreads, 4) walk_hop_kernel(HopArgs g) {
             if (wb + 2 * kStride + lane < seg_end)
                 e2 = at_pos ? make_uint2(wb + 2 * kStride + lane, 0) : g.sorted[wb + 2 * kStride + lane];
             uint4 pr = make_uint4(0, 0, 0, 0);   // {src_ip, dst_ip, dport | src_host << 16, allowed_mask}
-            uint32_t pid = 0;                     // probe id
+            uint32_t pid = 0, src_class = 0;      // probe id, class of its source address
             if (lane < cnt) {
                 uint32_t src_port = 0;
-                pr = header_of<kRec>(g, raw, e.x, &pid, &src_port);
+                pr = header_of<kRec>(g, raw, e.x, &pid, &src_port, &src_class);
                 if (at_pos) e.y = src_port;
             }
             // a probe in a known forwarding cycle that has reached its finish hop
@@ -1681,8 +1771,9 @@ __global__ void __launch_bounds__(kHopThreads, 4) walk_hop_kernel(HopArgs g) {
             }
             if (lane_mode) {
                 const bool act = lane < cnt && !fin_now;
-                const uint32_t fm = first_match_lane<kStats>(s_raw, L, act, pr.x, pr.y, pr.z & 0xFFFFu, e.y & 0xFFu,
-                                                             stc[kStRuleTests], stc[kStLookups]);
+                const uint32_t fm = first_match_lane<kStats>(s_raw, g.stage_skip, L, act, pr.x, pr.y, pr.z & 0xFFFFu, e.y & 0xFFu,
+                                                             src_class, addr_class(g.cls, pr.y), stc[kStRuleTests],
+                                                             stc[kStLookups]);
                 my_fm = fm;
                 if (act) hop_outcome(g, s_port, g.hop, fm, pr.y, pr.w, nports, &my_status, &my_next);
             } else {
@@ -1695,7 +1786,7 @@ __global__ void __launch_bounds__(kHopThreads, 4) walk_hop_kernel(HopArgs g) {
                     const uint32_t mask = __shfl_sync(PV_FULL_MASK, pr.w, j);
                     uint32_t tests = 0, lookups = 0;
                     const uint32_t fm =
-                        kIndexed ? first_match_indexed<kStats>(s_raw, hdr, lane, src, dst, dport, in_port, tests, lookups)
+                        kIndexed ? first_match_indexed<kStats>(s_raw, g.stage_skip, hdr, lane, src, dst, dport, in_port, tests, lookups)
                                  : first_match_linear<kStats>(s_raw, npad, lane, src, dst, dport, in_port, tests);
                     uint32_t status, next;
                     hop_outcome(g, s_port, g.hop, fm, dst, mask, nports, &status, &next);
@@ -1775,63 +1866,59 @@ __global__ void __launch_bounds__(kHopThreads, 4) walk_hop_kernel(HopArgs g) {
             if (s_hist[j]) atomicAdd(&g.hist_next[j], s_hist[j]);
 }
 
-// First match of one probe by one thread, reading the switch's blob from
-// global memory (L2-resident tables): the per-lane walk of first_match_lane
-// without its warp phases.  The candidate list is read four items at a time
-// and the four candidates' rules are loaded together before any is tested,
-// so a probe's chain of dependent L2 round trips per hop shrinks about as
-// many times (a tail walk is as long as its slowest probe's chain).
-constexpr uint32_t kTailBatch = 4;
-
+// First match of one probe by one thread, reading the switch's blob in place
+// (L2-resident tables).  Candidates are taken two at a time, both rules
+// loaded before either is tested: what a walk waits for here is the chain of
+// dependent L2 round trips.
 template <bool kStats>
 __device__ __forceinline__ uint32_t first_match_thread(const uint8_t *__restrict__ blob, const BlobLayout &L,
                                                        uint32_t src, uint32_t dst, uint32_t dport,
-                                                       uint32_t in_port, uint32_t &tests, uint32_t &lookups) {
-    const uint4 *A = reinterpret_cast<const uint4 *>(blob + L.a);
-    const uint2 *Bv = reinterpret_cast<const uint2 *>(blob + L.b);
+                                                       uint32_t in_port, uint32_t sc, uint32_t dc, uint32_t &tests,
+                                                       uint32_t &lookups) {
+    const uint4 *rules = reinterpret_cast<const uint4 *>(blob + L.rules);
     const uint32_t *boff = reinterpret_cast<const uint32_t *>(blob + L.boff);
+    const uint32_t *masks = reinterpret_cast<const uint32_t *>(blob + L.masks);
     const uint16_t *items = reinterpret_cast<const uint16_t *>(blob + L.items);
     const uint2 *segs = reinterpret_cast<const uint2 *>(blob + L.segs);
-    const uint32_t *bnd = reinterpret_cast<const uint32_t *>(blob + L.bnd);
-    const uint32_t *win = reinterpret_cast<const uint32_t *>(blob + L.win);
+    const uint2 *bw = reinterpret_cast<const uint2 *>(blob + L.bw);
     const uint32_t k = dport >> kBucketShift;
-    const uint32_t i1 = __ldg(boff + k + 1);
-    for (uint32_t i = __ldg(boff + k); i < i1; i += kTailBatch) {
-        uint32_t it[kTailBatch];
-        uint4 a[kTailBatch];
-        uint2 bb[kTailBatch];
+    const uint32_t *mk = masks + k * (2 * kClasses);
+    Candidates cand(__ldg(mk + dc) & __ldg(mk + kClasses + sc), __ldg(boff + k), __ldg(boff + k + 1));
+    constexpr uint32_t kNone = 0xFFFFu;
+    while (true) {
+        uint32_t it[2] = {kNone, kNone};
+        uint4 r[2];
 #pragma unroll
-        for (uint32_t j = 0; j < kTailBatch; ++j) it[j] = i + j < i1 ? __ldg(items + i + j) : 0xFFFFu;
-#pragma unroll
-        for (uint32_t j = 0; j < kTailBatch; ++j) {
-            const bool rule = it[j] != 0xFFFFu && !(it[j] & kSegItem);
-            a[j] = rule ? __ldg(A + it[j]) : make_uint4(0, 0, 0, 0);
-            bb[j] = rule ? __ldg(Bv + it[j]) : make_uint2(1u, 0u);   // lo 1 > hi 0: never matches
+        for (uint32_t j = 0; j < 2; ++j) {
+            uint32_t i;
+            if (cand.next(&i)) it[j] = __ldg(items + i);
         }
 #pragma unroll
-        for (uint32_t j = 0; j < kTailBatch; ++j) {
-            if (it[j] == 0xFFFFu) return 0u;   // past the list's end: table miss
+        for (uint32_t j = 0; j < 2; ++j) r[j] = (it[j] & kSegItem) ? make_uint4(0, 0, 0, 0) : __ldg(rules + it[j]);
+#pragma unroll
+        for (uint32_t j = 0; j < 2; ++j) {
+            if (it[j] == kNone) return 0u;   // no candidate left: table miss
             if (it[j] & kSegItem) {
                 const uint2 sd = __ldg(segs + (it[j] & 0x7FFFu));
-                uint32_t lo = 0, len = sd.y;   // bnd[sd.x] = 0 <= dst
+                uint32_t lo = 0, len = sd.y;   // the first interval starts at 0 <= dst
+                uint2 w = __ldg(bw + sd.x);
                 while (len > 1) {
                     const uint32_t half = len >> 1;
-                    lo = __ldg(bnd + sd.x + lo + half) <= dst ? lo + half : lo;
+                    const uint2 c = __ldg(bw + sd.x + lo + half);
+                    if (c.x <= dst) {
+                        lo += half;
+                        w = c;
+                    }
                     len -= half;
                 }
-                const uint32_t w = __ldg(win + sd.x + lo);
                 if (kStats) ++lookups;
-                if (w & kWinFound) return w;
+                if (w.y & kWinFound) return w.y;
                 continue;
             }
             if (kStats) ++tests;
-            const uint32_t diff = ((src ^ a[j].x) & a[j].y) | ((dst ^ a[j].z) & a[j].w) |
-                                  ((in_port ^ bb[j].y) & ((bb[j].y >> 8) & 0xFFu));
-            if (diff == 0 && dport >= (bb[j].x & 0xFFFFu) && dport <= (bb[j].x >> 16))
-                return kWinFound | (bb[j].y >> 16);
+            if (plain_hit(r[j], src, dst, dport, in_port)) return plain_result(r[j]);
         }
     }
-    return 0u;
 }
 
 // Whole walks, or a walk's last hops, in one launch: one thread per probe,
@@ -1887,7 +1974,7 @@ __global__ void __launch_bounds__(256, !kStats && kSrc >= kSrcList ? 4 : 1) walk
     uint32_t visits = 0;
     bool active = false, more = true;
     uint4 pr = make_uint4(0, 0, 0, 0);
-    uint32_t pid = 0, loc = 0, h = 0, ck = 0, wp = 0;
+    uint32_t pid = 0, loc = 0, h = 0, ck = 0, wp = 0, cls = 0;   // cls: source class | destination class << 8
     uint4 ph = make_uint4(0, 0, 0, 0);
     while (true) {
         const uint32_t idle = __ballot_sync(PV_FULL_MASK, !active);
@@ -1929,13 +2016,14 @@ __global__ void __launch_bounds__(256, !kStats && kSrc >= kSrcList ? 4 : 1) walk
                         const uint32_t s = w.host_switch[host], reg = g.region[s];
                         active = reg < 32 && ((pr.w >> reg) & 1u) &&
                                  !(kPolicy && switch_listed(g.pa.sw + ph.x, ph.y, s));
-                        loc = s << 8 | __ldg(g.host_addr + host).y;
+                        loc = s << 8 | (__ldg(g.host_addr + host).y & 0xFFu);
                         if (!active) put_result(g.out, i, PV_VIOLATION, 1, s);
                     } else {
                         put_result(g.out, i, PV_NOSRC, 0, 0xFFFF);
                     }
                     if (kPolicy && !active) g.pa.hits[i] = 0;
                 }
+                cls = addr_class(g.cls, pr.x) | addr_class(g.cls, pr.y) << 8;
             }
         }
         if (!__any_sync(PV_FULL_MASK, active)) {
@@ -1953,8 +2041,8 @@ __global__ void __launch_bounds__(256, !kStats && kSrc >= kSrcList ? 4 : 1) walk
             const uint8_t *blob = g.blob + g.blob_offs[s];
             const uint4 hdr = __ldg(reinterpret_cast<const uint4 *>(blob));
             const BlobLayout L(hdr);
-            const uint32_t fm = first_match_thread<kStats>(blob, L, pr.x, pr.y, pr.z & 0xFFFFu, in_port,
-                                                           stc[kStRuleTests], stc[kStLookups]);
+            const uint32_t fm = first_match_thread<kStats>(blob, L, pr.x, pr.y, pr.z & 0xFFFFu, in_port, cls & 0xFFu,
+                                                           cls >> 8, stc[kStRuleTests], stc[kStLookups]);
             if (kStats) {
                 uint32_t depth = 0;
                 const uint32_t ref = scan_first_match(reinterpret_cast<const uint4 *>(blob + L.fa),
@@ -2037,11 +2125,11 @@ __global__ void port_stage_kernel(uint32_t P, const int32_t *__restrict__ peer, 
     stage[p] = make_uint2((uint32_t)x, aux);
 }
 
-// addr[h] = {host_ip[h], host_port[h]}.
+// addr[h] = {host_ip[h], host_port[h] | class of host_ip[h] << 8}.
 __global__ void host_addr_kernel(uint32_t H, const uint32_t *__restrict__ ip, const uint16_t *__restrict__ port,
-                                 uint2 *__restrict__ addr) {
+                                 pv_addr_classes cls, uint2 *__restrict__ addr) {
     const uint32_t h = blockIdx.x * blockDim.x + threadIdx.x;
-    if (h < H) addr[h] = make_uint2(ip[h], port[h]);
+    if (h < H) addr[h] = make_uint2(ip[h], port[h] | addr_class(cls, ip[h]) << 8);
 }
 
 }  // namespace
@@ -2137,6 +2225,14 @@ int tables_begin(pv_ctx *ctx, pv_table_load &L, uint32_t S, const uint32_t *rule
     if (int rc0 = pv_load_begin(ctx)) return rc0;
     cudaStream_t ls = ctx->load_stream;
     pv_table_state &t = L.t;
+    // address classes: octiles of (at most 4,096 of) the hosts' addresses
+    if (H) {
+        const uint32_t step = (H + 4095) / 4096, n = (H + step - 1) / step;
+        std::vector<uint32_t> ips(n);
+        for (uint32_t i = 0; i < n; ++i) ips[i] = host_ip[i * step];
+        std::sort(ips.begin(), ips.end());
+        for (uint32_t j = 0; j + 1 < kClasses; ++j) t.cls.b[j] = ips[(size_t)(j + 1) * n / kClasses];
+    }
     const uint32_t T = tab[S];
     uint32_t *&d_rule_offs = L.d_rule_offs, *&d_tab_offs = L.d_tab_offs, *&d_sizes = L.d_sizes;
     uint4 *&d_rule_a = L.d_rule_a;
@@ -2172,7 +2268,7 @@ int tables_begin(pv_ctx *ctx, pv_table_load &L, uint32_t S, const uint32_t *rule
         e = e ? e : cudaMemcpyAsync(t.d_host_port, host_port, (size_t)H * 2, cudaMemcpyHostToDevice, ls);
         e = e ? e : cudaMemcpyAsync(t.d_host_ip, host_ip, (size_t)H * 4, cudaMemcpyHostToDevice, ls);
         if (e == cudaSuccess)
-            host_addr_kernel<<<(H + 255) / 256, 256, 0, ls>>>(H, t.d_host_ip, t.d_host_port, t.d_host_addr);
+            host_addr_kernel<<<(H + 255) / 256, 256, 0, ls>>>(H, t.d_host_ip, t.d_host_port, t.cls, t.d_host_addr);
         e = e ? e : cudaGetLastError();
     }
     if (P && e == cudaSuccess) {
@@ -2261,7 +2357,7 @@ int tables_begin(pv_ctx *ctx, pv_table_load &L, uint32_t S, const uint32_t *rule
         }
         if (e == cudaSuccess) {
             index_build_kernel<false><<<S, kIndexThreads, ism.bytes, ls>>>(d_rule_offs, d_tab_offs, d_rule_a,
-                                                                           d_rule_b, d_sizes, nullptr, nullptr, ism);
+                                                                           d_rule_b, d_sizes, nullptr, nullptr, ism, t.cls);
             e = cudaGetLastError();
         }
     }
@@ -2346,7 +2442,7 @@ int tables_end(pv_ctx *ctx, pv_table_load &L) {
             return rc;
         }
         index_build_kernel<true><<<S, kIndexThreads, ism.bytes, ls>>>(d_rule_offs, d_tab_offs, d_rule_a, d_rule_b,
-                                                                      d_sizes, t.d_blob_offs, t.d_blob, ism);
+                                                                      d_sizes, t.d_blob_offs, t.d_blob, ism, t.cls);
         e = cudaGetLastError();
     }
     free_temps();
@@ -2362,11 +2458,13 @@ int tables_end(pv_ctx *ctx, pv_table_load &L) {
     t.tail_hop = all_items <= (uint64_t)kTailEarlyItems * kBuckets * S ? 5u : 8u;
     t.max_rules_padded = max_pad;
     t.max_ports = L.max_ports;
-    t.max_blob_bytes = max_blob;
     t.max_linear_bytes = max_linear;
     // the hop kernel stages the port table after the table (16-byte aligned)
     const size_t smem_cap = ctx->max_smem_optin - 1024 - 16 - port_stage_bytes(t.max_ports);
-    t.index_fits = max_blob <= smem_cap;
+    // a filter that does not fit beside the rest is left out of the stage
+    if (max_blob > smem_cap) t.stage_skip = BlobLayout::filter_bytes;
+    t.max_blob_bytes = max_blob - t.stage_skip;
+    t.index_fits = t.max_blob_bytes <= smem_cap;
     if (max_linear > smem_cap) {
         pv_free_tables(ctx, t);
         return pv_fail(ctx, PV_EINVAL, "largest flow table needs %u bytes of shared memory", max_linear);
@@ -2493,6 +2591,8 @@ HopArgs walk_args(pv_ctx *ctx, uint32_t hop_cap, const pv_probe *d_probes, pv_re
     g.bounce = ctx->opt_walk_cycles == 0 && t.links_symmetric ? 1u : 0u;   // any cap: no checkpoints needed
     if (pa) g.pa = *pa;
     g.host_addr = t.d_host_addr;
+    g.cls = t.cls;
+    g.stage_skip = t.stage_skip;
     g.port_stage = t.d_port_stage;
     g.stats = ctx->d_walk_stats;
     g.wait_extra = ctx->opt_test_stall_staging ? 16u : 0u;

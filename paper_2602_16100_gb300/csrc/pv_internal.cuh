@@ -29,6 +29,12 @@ struct pv_cluster_state {
     uint32_t *d_rows = nullptr;       // [num_value_rows + K][row_words]
 };
 
+// Ascending boundaries of the eight address classes of the first-match
+// index's candidate filter (class = boundaries at or below the address).
+struct pv_addr_classes {
+    uint32_t b[7] = {~0u, ~0u, ~0u, ~0u, ~0u, ~0u, ~0u};
+};
+
 struct pv_table_state {
     bool loaded = false;
     uint32_t num_switches = 0, num_hosts = 0;
@@ -38,6 +44,7 @@ struct pv_table_state {
     uint8_t *d_blob = nullptr;
     uint64_t *d_blob_offs = nullptr;  // [S + 1] byte offsets
     uint32_t max_blob_bytes = 0;      // largest stage of the indexed kernel (all but the full rule list)
+    uint32_t stage_skip = 0;          // bytes of the candidate filter when the indexed kernel does not stage it
     uint32_t tail_hop = 8;            // default first tail hop for these tables (see walk_probes)
     uint32_t max_linear_bytes = 0;    // largest header + full rule list (linear-scan kernel)
     uint32_t max_ports = 0;           // most ports on one switch
@@ -47,7 +54,8 @@ struct pv_table_state {
     int32_t *d_port_peer = nullptr;   // [ports]
     uint16_t *d_host_switch = nullptr, *d_host_port = nullptr;
     uint32_t *d_host_ip = nullptr;
-    uint2 *d_host_addr = nullptr;     // [H] {address, attachment port}: one load for a walk's source host
+    pv_addr_classes cls;
+    uint2 *d_host_addr = nullptr;     // [H] {address, attachment port | address class << 8}: one load for a walk's source host
     uint2 *d_port_stage = nullptr;    // [ports] {peer, peer's region or host address}: the hop kernel's port stage
     // switch-to-switch links into each switch, sorted by (source switch,
     // source port): u << 16 | p << 8 | q for port p of u cabled to port q

@@ -12,6 +12,7 @@ import test_gpu_policies as TP
 import test_gpu_walk as TW
 from paper_2602_16100_gb300 import binding as B
 from paper_2602_16100_gb300 import workloads as W
+from netbuild import make_net
 
 pytestmark = pytest.mark.gpu
 
@@ -90,3 +91,64 @@ def test_forms_agree_at_the_changeover(validator, m):
     assert (auto == regrouped).all()
     idx = np.arange(0, m, 97)
     assert (auto[idx] == oracle.verify_probes(net, pr[idx], 32)).all()
+
+
+def _scattered_net(seed, n, hosts, wide):
+    """Four switches in a ring, n random rules each: prefixes of every length
+    0-32 of host and of arbitrary addresses, ports all `wide` or of mixed
+    widths; `hosts` hosts at addresses scattered over the whole range."""
+    r = np.random.default_rng(seed)
+    ips = np.unique(np.concatenate([[0, 0xFFFFFFFF], r.integers(0, 1 << 32, hosts)]))[:hosts] if hosts > 2 else \
+        r.integers(0, 1 << 32, hosts)
+    t = np.zeros((4, n), W.RULE_DTYPE)
+    t["priority"] = r.integers(0, 50, t.shape)            # many ties
+    t["in_port"] = np.where(r.random(t.shape) < 0.5, W.ANY_PORT, r.integers(0, 4, t.shape))
+    for a, ln in (("src_ip", "src_len"), ("dst_ip", "dst_len")):
+        t[a] = np.where(r.random(t.shape) < 0.8, r.choice(ips, t.shape), r.integers(0, 1 << 32, t.shape))
+        t[ln] = r.integers(0, 33, t.shape)
+    t["src_len"] = np.where(r.random(t.shape) < 0.5, 0, t["src_len"])
+    t["dport_lo"] = 0 if wide else r.integers(0, 65536, t.shape)
+    t["dport_hi"] = 65535 if wide else np.minimum(65535, t["dport_lo"].astype(np.int64)
+                                                  + (1 << r.integers(0, 17, t.shape)) - 1)
+    if wide:
+        t["in_port"] = np.where(t["src_len"] == 0, r.integers(0, 4, t.shape), t["in_port"])   # no segments
+    t["action"] = np.where(r.random(t.shape) < 0.1, W.DROP, r.integers(0, 4, t.shape))
+    nets = make_net([4] * 4, [(i, 2, (i + 1) % 4, 3) for i in range(4)], [(i % 4, i // 4 % 2, int(x)) for i, x in enumerate(ips)],
+                    [0, 1, 2, 3], [[x.reshape(1) for x in t[s]] for s in range(4)])
+    return nets
+
+
+@pytest.mark.parametrize("n,hosts,wide,lane_max", [(40, 2, False, 96), (40, 8, False, 0), (200, 8, False, 96),
+                                                   (600, 8, False, 65535), (31, 8, True, 96), (32, 8, True, 96),
+                                                   (33, 8, True, 96), (65, 8, True, 96), (400, 8, True, 65535),
+                                                   (400, 8, True, 96)])
+@pytest.mark.parametrize("tail", [-1, 0])
+def test_candidate_filter(validator, n, hosts, wide, lane_max, tail):
+    """The filter of the first-match index: addresses at class boundaries and
+    at both ends of the range, prefixes of every length, lists of 31 to 400
+    candidates (one and several per filter bit), fewer hosts than classes,
+    and tables whose filter does not fit the hop kernel's stage (400 rules of
+    every port: 205 KB of items)."""
+    net = _scattered_net(n + hosts, n, hosts, wide)
+    r = np.random.default_rng(n)
+    m = 3000
+    pr = np.zeros(m, W.PROBE_DTYPE)
+    ends = np.concatenate([net.host_ip, net.host_ip - np.uint32(1), net.host_ip + np.uint32(1)])
+    for f in ("src_ip", "dst_ip"):
+        pr[f] = np.where(r.random(m) < 0.8, r.choice(ends, m), r.integers(0, 1 << 32, m))
+    pr["src_host"] = r.integers(0, hosts, m)
+    pr["dport"] = r.integers(0, 65536, m)
+    pr["allowed_mask"] = r.integers(1, 16, m)
+    validator.set_option(B.PV_OPT_WALK_TAIL_HOP, tail)
+    validator.set_option(B.PV_OPT_WALK_LANE_MAX, lane_max)
+    validator.set_option(B.PV_OPT_WALK_STATS, 1)
+    try:
+        g = TW._gpu_walk(validator, net, pr, 20, 2)
+        assert B.pv_get_stat(validator.ctx, B.PV_STAT_WALK_INDEX_MISMATCHES) == 0
+        validator.set_option(B.PV_OPT_WALK_STATS, 0)
+        g2 = TW._gpu_walk(validator, net, pr, 20, 2)
+    finally:
+        for o, x in ((B.PV_OPT_WALK_TAIL_HOP, -1), (B.PV_OPT_WALK_LANE_MAX, 96), (B.PV_OPT_WALK_STATS, 0)):
+            validator.set_option(o, x)
+    o = oracle.verify_probes(net, pr, 20)
+    assert (g == o).all() and (g2 == o).all()
