@@ -535,9 +535,8 @@ int pv_install_path_rules(pv_ctx *ctx, uint32_t num_slots, const pv_rule *d_rule
  *   one on (0 = none) run in a single launch, one thread per probe still
  *   walking, tables read from L2 instead of staged per switch.  Same
  *   results.  Default (-1): batches of at most 2^20 probes walk every hop
- *   that way; for larger ones the hop is chosen by pv_load_flow_tables from
- *   the loaded index, hop 5 when its candidate lists hold at most 12 items
- *   per destination-port bucket on average, else hop 8.
+ *   that way, larger ones from a hop that grows with the batch (hop 2 at 3
+ *   million probes, hop 5 at 50 million).
  * PV_OPT_REACH_KERNEL: 0 = automatic (on a symmetric graph, rows are the
  *   connected components of the permitted subgraph; otherwise multi-source
  *   pull sweeps), 1 = sweeps always.  Both give the same rows.

@@ -46,6 +46,19 @@ constexpr uint32_t kMinPerBlock = 512;       // live probes per active hop block
 // and compact flows of 512 switches at 1M: 223/231 (270/267 with policies).
 // The lines cross between 1M and 2M on the large tables.
 constexpr uint32_t kThreadWalkMax = 1u << 20;
+// Larger batches: the hop from which the probes still walking finish in one
+// thread walk.  Live probes fall about 2.5 times a hop, and the thread walk
+// takes over best at some 400,000 of them, so one more hop is regrouped for
+// every factor 2.5 of the batch.  us at tail hop 1 / 2 / 3 / 4 / 5 / 6 / 8:
+//   mesh of 512, 3M probes    216  199  214  240  274  299  340
+//   fat tree, 10M probes      998  842  744  719  710  711  777
+//   compact flows, 3M         218  206  222  255  280  302  339
+//   compact flows, 50M       2207 1571 1410 1400 1411 1441 1490
+inline uint32_t auto_tail_hop(uint32_t M) {
+    uint32_t hop = 1;
+    for (uint64_t most = 1500000; M > most; most = most * 5 / 2) ++hop;
+    return hop;
+}
 constexpr int kGridThreads = 256;
 constexpr uint32_t kSmemHistMax = 12288;     // switches for shared-memory histograms
 constexpr uint32_t kWaitLimit = 1u << 24;    // bounded mbarrier polls
@@ -218,7 +231,6 @@ __global__ void __launch_bounds__(1024) compile_tables_kernel(const uint32_t *__
 constexpr uint32_t kBuckets = 256;          // dport >> kBucketShift
 constexpr uint32_t kBucketShift = 8;
 constexpr uint32_t kMinSegment = 4;         // shorter destination-only runs stay plain items
-constexpr uint32_t kTailEarlyItems = 12;    // candidate items per bucket below which the tail starts at hop 5
 constexpr uint32_t kMaxSegment = 4096;      // longer runs are split (in order: still exact)
 constexpr uint32_t kSegItem = 0x8000u;
 constexpr uint32_t kWinFound = 0x80000000u;
@@ -2422,11 +2434,9 @@ int tables_end(pv_ctx *ctx, pv_table_load &L) {
                        r.dport_lo, r.dport_hi);
     }
     uint32_t max_blob = 0, max_linear = 0;
-    uint64_t all_items = 0;
     if (e == cudaSuccess) {
         for (uint32_t s = 0; s < S; ++s) {
             const uint32_t npad = tab[s + 1] - tab[s];
-            all_items += sizes[4 * s];
             const BlobLayout L(npad, sizes[4 * s + 3], sizes[4 * s], sizes[4 * s + 1], sizes[4 * s + 2]);
             boffs[s + 1] = boffs[s] + L.total;
             max_blob = std::max(max_blob, L.fa);             // staged by the indexed kernel
@@ -2452,10 +2462,6 @@ int tables_end(pv_ctx *ctx, pv_table_load &L) {
     }
     t.num_switches = S;
     t.num_hosts = H;
-    // The tail launch walks each probe's candidate lists from L2, one thread
-    // per probe: with short lists (at most kTailEarlyItems items per bucket
-    // on average) it pays from hop 5 on, with long ones only from hop 8.
-    t.tail_hop = all_items <= (uint64_t)kTailEarlyItems * kBuckets * S ? 5u : 8u;
     t.max_rules_padded = max_pad;
     t.max_ports = L.max_ports;
     t.max_linear_bytes = max_linear;
@@ -2779,7 +2785,7 @@ int walk_probes(pv_ctx *ctx, uint32_t M, const pv_probe *d_probes, uint32_t hop_
     g.port_off = (uint32_t)port_off;
     uint32_t in_slices = init_grid;
     // hops from tail_hop on run in one walk_tail_kernel launch (indexed tables only)
-    const uint32_t opt_tail = ctx->opt_walk_tail_hop < 0 ? t.tail_hop : (uint32_t)ctx->opt_walk_tail_hop;
+    const uint32_t opt_tail = ctx->opt_walk_tail_hop < 0 ? auto_tail_hop(M) : (uint32_t)ctx->opt_walk_tail_hop;
     const uint32_t tail_hop = (indexed && opt_tail > 0 && opt_tail < hop_cap) ? opt_tail : hop_cap;
     for (uint32_t h = 0; h < tail_hop; ++h) {
         uint2 *cur = (h & 1) ? listB : listA;

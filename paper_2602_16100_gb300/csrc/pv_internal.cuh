@@ -45,7 +45,6 @@ struct pv_table_state {
     uint64_t *d_blob_offs = nullptr;  // [S + 1] byte offsets
     uint32_t max_blob_bytes = 0;      // largest stage of the indexed kernel (all but the full rule list)
     uint32_t stage_skip = 0;          // bytes of the candidate filter when the indexed kernel does not stage it
-    uint32_t tail_hop = 8;            // default first tail hop for these tables (see walk_probes)
     uint32_t max_linear_bytes = 0;    // largest header + full rule list (linear-scan kernel)
     uint32_t max_ports = 0;           // most ports on one switch
     bool index_fits = false;          // every blob fits shared memory
