@@ -510,11 +510,12 @@ int pv_install_path_rules(pv_ctx *ctx, uint32_t num_slots, const pv_rule *d_rule
  *   placement check.  Same results; pays off when lists repeat.  2 = the
  *   same with deliberately weak hashes (tests: every collision is resolved
  *   by comparing the lists).  Not used by pv_eval_selector_terms.
- * PV_OPT_SCHED_KERNEL: pv_schedule_paths' kernel (one block per request):
- *   0 = automatic (the links into each switch, with their weights, staged
- *   in shared memory when they fit, else read from global memory); 1 =
- *   links from global memory; 2 = staged (PV_EINVAL if they do not fit).
- *   Both give the same paths.
+ * PV_OPT_SCHED_KERNEL: pv_schedule_paths' kernel: 0 = automatic (a warp per
+ *   path segment when the links and at least four warps' state fit shared
+ *   memory, else a block per request); 1 = a block per request, links from
+ *   global memory; 2 = the same with the links into each switch, with their
+ *   weights, staged in shared memory (PV_EINVAL if they do not fit).  All
+ *   give the same paths.
  * PV_OPT_WALK_KERNEL: 0 = automatic, 1 = linear first-match scan of the
  *   staged table, 2 = indexed first match (per-dport-bucket candidate lists
  *   and destination-interval maps built by pv_load_flow_tables; needs every

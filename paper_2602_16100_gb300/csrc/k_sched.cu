@@ -217,6 +217,288 @@ __global__ void __launch_bounds__(kSchedThreads) sched_paths_kernel(SchedArgs a)
     }
 }
 
+// The same paths with a warp per path segment.  A request's segments (source
+// to first waypoint, and so on) do not depend on one another, so a block
+// takes a range of requests, its warps draw segments until none is left, and
+// a warp per request then joins the pieces.  A segment is searched from a
+// frontier: the switches lowered in one step are listed, and the next step
+// relaxes only their outgoing links (four lanes to a switch, atomicMin in
+// shared memory).  Labels count from 1; a switch that is not permitted holds
+// 0, which no label undercuts.  A label that does not stay below the target's
+// is dropped: every switch on a shortest path to the target lies nearer than
+// it, so those are exact at the end, and no other label can satisfy the
+// canonical walk back's equality.
+// A block per request swept every switch until a sweep changed nothing, and
+// waited at a block barrier each time: 10,000 weighted requests on 512
+// switches took 1,098 us with their rules, 165 us this way.  Bound by
+// instruction issue (about 3,900 warp instructions a segment, 41% of issue
+// slots) and, at a group's end, by its longest segments.  Tried: 32 segments
+// to a warp, one per lane (386 us: the union of their frontiers is every
+// switch), and a warp per whole request (375 us: as long as the requests with
+// the most waypoints).
+constexpr uint32_t kSegReqs = 128;               // most requests of a block's group
+constexpr uint32_t kSegTasks = 512;              // most segments of a group
+constexpr size_t kPieceBytes = 42 * 1024;        // pieces of a group's segments, max_len words each
+
+struct SegmentSmem {
+    uint32_t in_offs, in, out, in_w, region, pieces, tasks, warps, marks, list, per_warp, okw;
+    __host__ __device__ SegmentSmem(uint32_t S, uint32_t L, uint32_t max_len) {
+        // out_offs[S + 1] first
+        in_offs = (S + 1) * 4;
+        in = in_offs + (S + 1) * 4;              // in[L]: u << 16 | p << 8 | q, links into each switch
+        out = in + L * 4;                        // out[L]: v << 16 | weight, links out of each switch
+        pieces = out + L * 4;                    // pieces[tasks][max_len]: links of a segment, last first
+        tasks = kPieceBytes / 4 / max_len;       // at least the 33 segments of one request
+        tasks = tasks < kSegTasks ? tasks : kSegTasks;
+        in_w = pieces + tasks * max_len * 4;     // in_w[L]: weights of in[]
+        region = in_w + L * 2;                   // region[S]
+        warps = (region + S + 15) & ~15u;
+        // each warp: dist[S] first (the joined visits, max_len of them, later)
+        okw = (S + 31) / 32;
+        marks = ((S > max_len ? S : max_len) + 3) / 4 * 16;   // marks[okw]: switches listed for the next step
+        list = marks + okw * 4;                  // list[2][S]: the frontier and the next one
+        per_warp = (list + 2 * S * 2 + 15) & ~15u;
+    }
+    __host__ __device__ size_t total(uint32_t n) const { return (size_t)warps + (size_t)n * per_warp; }
+};
+static_assert(kPieceBytes / 4 / PV_MAX_HOP_CAP >= 33, "a request's segments fit one group");
+
+__global__ void __launch_bounds__(1024, 1) sched_segments_kernel(SchedArgs a) {
+    extern __shared__ __align__(16) uint8_t s_raw[];
+    __shared__ pv_path_req s_req[kSegReqs];
+    __shared__ uint4 s_pol[kSegReqs];
+    __shared__ uint32_t s_first[kSegReqs + 1], s_st[kSegReqs];
+    __shared__ uint8_t s_seg_st[kSegTasks], s_seg_len[kSegTasks];
+    __shared__ uint32_t s_next, s_group;
+    const uint32_t S = a.S, L = a.in_offs[S];
+    const SegmentSmem M(S, L, a.max_len);
+    uint32_t *out_offs = reinterpret_cast<uint32_t *>(s_raw), *in_offs = reinterpret_cast<uint32_t *>(s_raw + M.in_offs);
+    uint32_t *in = reinterpret_cast<uint32_t *>(s_raw + M.in), *out = reinterpret_cast<uint32_t *>(s_raw + M.out);
+    uint16_t *in_w = reinterpret_cast<uint16_t *>(s_raw + M.in_w);
+    uint8_t *region = s_raw + M.region;
+    const uint32_t t = threadIdx.x, nt = blockDim.x, lane = t & 31, warp = t >> 5, lt = (1u << lane) - 1u;
+    uint8_t *mine = s_raw + M.warps + warp * M.per_warp;
+    uint32_t *dist = reinterpret_cast<uint32_t *>(mine), *marks = reinterpret_cast<uint32_t *>(mine + M.marks);
+    uint16_t *list = reinterpret_cast<uint16_t *>(mine + M.list);
+    // the block's links: in-links as loaded, with weights, then out-links
+    // counted and placed by source (their order within a switch is free)
+    uint32_t *cursor = reinterpret_cast<uint32_t *>(s_raw + M.warps);   // warp 0's distances, free until the barrier below
+    for (uint32_t v = t; v <= S; v += nt) in_offs[v] = a.in_offs[v];
+    for (uint32_t v = t; v < S; v += nt) {
+        cursor[v] = 0;
+        region[v] = a.region[v];
+    }
+    __syncthreads();
+    for (uint32_t l = t; l < L; l += nt) {
+        const uint32_t x = a.in_links[l];
+        in[l] = x;
+        in_w[l] = (uint16_t)link_weight(a, x >> 16, (x >> 8) & 0xFFu);
+        atomicAdd(&cursor[x >> 16], 1u);
+    }
+    __syncthreads();
+    if (warp == 0) {
+        uint32_t run = 0;
+        for (uint32_t v0 = 0; v0 < S; v0 += 32) {
+            const uint32_t c = v0 + lane < S ? cursor[v0 + lane] : 0u;
+            uint32_t incl = c;
+            for (int d = 1; d < 32; d <<= 1) {
+                const uint32_t y = __shfl_up_sync(PV_FULL_MASK, incl, d);
+                if (lane >= (uint32_t)d) incl += y;
+            }
+            if (v0 + lane < S) {
+                out_offs[v0 + lane] = run + incl - c;
+                cursor[v0 + lane] = run + incl - c;
+            }
+            run += __shfl_sync(PV_FULL_MASK, incl, 31);
+        }
+        if (lane == 0) out_offs[S] = run;
+    }
+    __syncthreads();
+    for (uint32_t v = t; v < S; v += nt)
+        for (uint32_t l = in_offs[v]; l < in_offs[v + 1]; ++l) out[atomicAdd(&cursor[in[l] >> 16], 1u)] = v << 16 | in_w[l];
+    const uint32_t r_end = (uint32_t)(((uint64_t)a.R * (blockIdx.x + 1)) / gridDim.x);
+    for (uint32_t r0 = (uint32_t)(((uint64_t)a.R * blockIdx.x) / gridDim.x); r0 < r_end;) {
+        __syncthreads();   // the links are placed; the group before is done with the shared state
+        // the group: requests from r0 while their segments fit; refused ones have none
+        const uint32_t nreq = min(r_end - r0, kSegReqs);
+        if (t < nreq) {
+            const pv_path_req q = a.req[r0 + t];
+            uint4 ph = make_uint4(0, 0, 0, 0);
+            if (a.pol_hdr && q.policy < a.num_pol) ph = a.pol_hdr[q.policy];
+            auto permitted = [&](uint32_t s) {
+                if (s >= S) return false;   // a waypoint of policies loaded for other tables
+                bool fine = region[s] < 32 && ((q.allowed_mask >> region[s]) & 1u);
+                for (uint32_t i = 0; i < ph.y && fine; ++i) fine = a.pol_sw[ph.x + i] != s;
+                return fine;
+            };
+            uint32_t st = PV_PATH_NOSRC;
+            if (q.src_host < a.H && q.dst_host < a.H) {
+                bool fine = permitted(a.host_switch[q.src_host]) && permitted(a.host_switch[q.dst_host]);
+                for (uint32_t i = 0; i < ph.w && fine; ++i) fine = permitted(a.pol_sw[ph.z + i]);
+                st = fine ? PV_PATH_OK : PV_PATH_BLOCKED;
+            }
+            s_req[t] = q;
+            s_pol[t] = ph;
+            s_st[t] = st;
+            s_first[t + 1] = st == PV_PATH_OK ? ph.w + 1 : 0u;
+        }
+        __syncthreads();
+        if (t == 0) {
+            uint32_t g = 0, sum = 0;
+            s_first[0] = 0;
+            while (g < nreq && sum + s_first[g + 1] <= M.tasks) {
+                sum += s_first[g + 1];
+                s_first[++g] = sum;
+            }
+            s_group = g;
+            s_next = 0;
+        }
+        __syncthreads();
+        const uint32_t group = s_group, tasks = s_first[group];
+        while (true) {
+            uint32_t task = 0;
+            if (lane == 0) task = atomicAdd(&s_next, 1u);
+            task = __shfl_sync(PV_FULL_MASK, task, 0);
+            if (task >= tasks) break;
+            uint32_t slot = 0, len = group;   // the request with first[slot] <= task < first[slot + 1]
+            while (len > 1) {
+                const uint32_t half = len >> 1;
+                if (s_first[slot + half] <= task) slot += half;
+                len -= half;
+            }
+            const pv_path_req q = s_req[slot];
+            const uint4 ph = s_pol[slot];
+            const uint32_t i = task - s_first[slot];
+            const uint32_t cur = i == 0 ? a.host_switch[q.src_host] : a.pol_sw[ph.z + i - 1];
+            const uint32_t tgt = i < ph.w ? a.pol_sw[ph.z + i] : a.host_switch[q.dst_host];
+            uint32_t *piece = reinterpret_cast<uint32_t *>(s_raw + M.pieces) + (size_t)task * a.max_len;
+            uint32_t st = PV_PATH_OK, k = 0;
+            if (tgt != cur) {
+                for (uint32_t v = lane; v < S; v += 32) {
+                    const uint32_t reg = region[v];
+                    dist[v] = reg < 32 && ((q.allowed_mask >> reg) & 1u) ? kInf : 0u;
+                }
+                __syncwarp();
+                for (uint32_t f = lane; f < ph.y; f += 32) {
+                    const uint32_t v = a.pol_sw[ph.x + f];
+                    if (v < S) dist[v] = 0;
+                }
+                if (lane == 0) {
+                    dist[cur] = 1;
+                    list[0] = (uint16_t)cur;
+                }
+                uint16_t *from = list, *to = list + S;
+                for (uint32_t nf = 1; nf;) {
+                    for (uint32_t w = lane; w < M.okw; w += 32) marks[w] = 0;
+                    __syncwarp();
+                    uint32_t nn = 0;
+                    for (uint32_t b = 0; b < nf; b += 8) {
+                        const uint32_t bound = *(volatile uint32_t *)(dist + tgt);
+                        uint32_t du = 0, l = 0, l1 = 0;
+                        if (b + (lane >> 2) < nf) {
+                            const uint32_t u = from[b + (lane >> 2)];
+                            du = *(volatile uint32_t *)(dist + u);
+                            l = out_offs[u] + (lane & 3u);
+                            l1 = du < bound ? out_offs[u + 1] : 0u;
+                        }
+                        while (__any_sync(PV_FULL_MASK, l < l1)) {
+                            bool push = false;
+                            uint32_t v = 0;
+                            if (l < l1) {
+                                const uint32_t x = out[l], d = du + (x & 0xFFFFu);
+                                v = x >> 16;
+                                if (d < bound && d < atomicMin(dist + v, d)) {
+                                    const uint32_t bit = 1u << (v & 31u);
+                                    push = !(atomicOr(&marks[v >> 5], bit) & bit);
+                                }
+                                l += 4;
+                            }
+                            const uint32_t m = __ballot_sync(PV_FULL_MASK, push);
+                            if (push) to[nn + __popc(m & lt)] = (uint16_t)v;
+                            nn += __popc(m);
+                        }
+                    }
+                    __syncwarp();
+                    nf = nn;
+                    uint16_t *x = from;
+                    from = to;
+                    to = x;
+                }
+                if (dist[tgt] == kInf) st = PV_PATH_BLOCKED;
+                // canonical walk back from tgt: smallest (u, p) on a shortest path
+                for (uint32_t v = tgt; v != cur && st == PV_PATH_OK;) {
+                    const uint32_t dv = dist[v], l1 = in_offs[v + 1];
+                    uint32_t pick = kInf;
+                    for (uint32_t l0 = in_offs[v]; l0 < l1 && pick == kInf; l0 += 32) {
+                        const uint32_t l = min(l0 + lane, l1 - 1), x = in[l], du = dist[x >> 16];
+                        const uint32_t m = __ballot_sync(PV_FULL_MASK, l0 + lane < l1 && du - 1u < kInf - 1u && du + in_w[l] == dv);
+                        if (m) pick = __shfl_sync(PV_FULL_MASK, x, __ffs(m) - 1);
+                    }
+                    if (pick == kInf) {   // cannot happen once the distances are exact
+                        st = PV_PATH_BLOCKED;
+                    } else if (k + 1 >= a.max_len) {   // the source's visit and k + 1 more
+                        st = PV_PATH_TOO_LONG;
+                    } else {
+                        // {source port, switch v, its in_port}
+                        if (lane == 0) piece[k] = ((pick >> 8) & 0xFFu) << 24 | v << 8 | (pick & 0xFFu);
+                        ++k;
+                        v = pick >> 16;
+                    }
+                }
+                __syncwarp();   // the distances are rebuilt for the next segment
+            }
+            if (lane == 0) {
+                s_seg_st[task] = (uint8_t)st;
+                s_seg_len[task] = (uint8_t)k;
+            }
+        }
+        __syncthreads();
+        // a warp per request: its first failing segment decides, else the
+        // pieces in order are its visits
+        for (uint32_t g = warp; g < group; g += nt >> 5) {
+            const uint32_t r = r0 + g, r_tasks = s_first[g + 1] - s_first[g];
+            uint32_t *vis = dist, st = s_st[g], n = 1;
+            const pv_path_req q = s_req[g];
+            if (st == PV_PATH_OK && lane == 0)
+                vis[0] = (uint32_t)a.host_switch[q.src_host] << 16 | (uint32_t)a.host_port[q.src_host] << 8;
+            for (uint32_t i = 0; i < r_tasks && st == PV_PATH_OK; ++i) {
+                const uint32_t task = s_first[g] + i, k = s_seg_len[task];
+                st = s_seg_st[task];
+                if (st == PV_PATH_OK && n + k > a.max_len) st = PV_PATH_TOO_LONG;
+                if (st != PV_PATH_OK) break;
+                const uint32_t *piece = reinterpret_cast<const uint32_t *>(s_raw + M.pieces) + (size_t)task * a.max_len;
+                for (uint32_t j = lane; j < k; j += 32) {
+                    const uint32_t x = piece[k - 1 - j];
+                    vis[n + j] = ((x >> 8) & 0xFFFFu) << 16 | (x & 0xFFu) << 8;
+                }
+                __syncwarp();
+                for (uint32_t j = lane; j < k; j += 32) vis[n - 1 + j] |= piece[k - 1 - j] >> 24;   // out port toward the next switch
+                __syncwarp();
+                n += k;
+            }
+            __syncwarp();
+            if (st == PV_PATH_OK) {
+                if (lane == 0) vis[n - 1] |= a.host_port[q.dst_host];
+                __syncwarp();
+                // a recurring (switch, in_port) cannot be realised by header
+                // rules (a single segment is a simple path)
+                bool again = false;
+                if (r_tasks > 1)
+                    for (uint32_t x = lane; x < n; x += 32)
+                        for (uint32_t y = x + 1; y < n; ++y) again = again || (vis[x] >> 8) == (vis[y] >> 8);
+                if (__any_sync(PV_FULL_MASK, again)) st = PV_PATH_REPEAT;
+            }
+            for (uint32_t x = lane; x < n && st == PV_PATH_OK; x += 32) a.visits[(size_t)r * a.max_len + x] = vis[x];
+            if (lane == 0) {
+                a.status[r] = (uint8_t)st;
+                a.len[r] = (uint8_t)(st == PV_PATH_OK ? n : 0);
+            }
+            __syncwarp();
+        }
+        r0 += group;
+    }
+}
+
 // Visit i of an OK request becomes, at its switch, the rule {priority,
 // in_port, src /32, dst /32, any destination port, output port}, in slot
 // r * max_len + i; unused slots get rule_switch 0xFFFF.
@@ -292,26 +574,37 @@ extern "C" int pv_schedule_paths(pv_ctx *ctx, uint32_t num_requests, const pv_pa
     // the links (with weights) and the predecessors staged when they fit
     const uint32_t L = t.num_links;
     const size_t staged_smem = base_smem + ((size_t)a.S + (size_t)a.S + 1 + L) * 4 + ((size_t)L * 2 + 15) / 16 * 16;
-    const int force = ctx->opt_sched_kernel;   // 0 automatic, 1 links from global memory, 2 staged
+    // 0 automatic: a warp per segment when at least four warps' state fits,
+    // else a block per request; 1 block per request, links from global memory;
+    // 2 staged
+    const int force = ctx->opt_sched_kernel;
+    const SegmentSmem W(a.S, L, max_len);
+    const size_t smem_cap = ctx->max_smem_optin - 8 * 1024;   // less the kernel's static arrays
+    const uint32_t warps = W.warps < smem_cap ? (uint32_t)std::min<size_t>(32, (smem_cap - W.warps) / W.per_warp) : 0u;
+    const bool by_warp = force == 0 && warps >= 4;
     const bool staged_fits = staged_smem <= std::min<size_t>(96 * 1024, ctx->max_smem_optin - 1024);
     if (force == 2 && !staged_fits)
         return pv_fail(ctx, PV_EINVAL, "pv_schedule_paths: the staged links do not fit shared memory");
     const bool staged = force == 2 || (force == 0 && staged_fits);
-    const size_t smem = staged ? staged_smem : base_smem;
-    const void *fn = staged ? (const void *)sched_paths_kernel<true> : (const void *)sched_paths_kernel<false>;
-    PV_TRY_CUDA(ctx, cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem), "sched smem");
-    int per_sm = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kSchedThreads, smem);
-    const uint32_t grid = std::min<uint32_t>(num_requests, (uint32_t)std::max(per_sm, 1) * ctx->num_sms);
+    const size_t smem = by_warp ? W.total(warps) : staged ? staged_smem : base_smem;
+    const void *fn = by_warp  ? (const void *)sched_segments_kernel
+                     : staged ? (const void *)sched_paths_kernel<true>
+                              : (const void *)sched_paths_kernel<false>;
+    if (int rc = pv_smem_limit(ctx, fn, "path scheduler shared memory")) return rc;
+    const int threads = by_warp ? (int)warps * 32 : kSchedThreads;
+    const uint32_t resident = (uint32_t)std::max(pv_blocks_per_sm(ctx, fn, threads, smem), 1) * ctx->num_sms;
+    const uint32_t grid = std::min<uint32_t>(num_requests, resident);
     pv_use_begin(ctx, (cudaStream_t)stream);
     const int pr = pv_prof_start(ctx, (cudaStream_t)stream, PV_K_SCHEDULE);
-    if (staged)
-        sched_paths_kernel<true><<<grid, kSchedThreads, smem, (cudaStream_t)stream>>>(a);
+    if (by_warp)
+        sched_segments_kernel<<<grid, threads, smem, (cudaStream_t)stream>>>(a);
+    else if (staged)
+        sched_paths_kernel<true><<<grid, threads, smem, (cudaStream_t)stream>>>(a);
     else
-        sched_paths_kernel<false><<<grid, kSchedThreads, smem, (cudaStream_t)stream>>>(a);
+        sched_paths_kernel<false><<<grid, threads, smem, (cudaStream_t)stream>>>(a);
     pv_prof_stop(ctx, (cudaStream_t)stream, pr, 1);
     pv_mark_use(ctx, (cudaStream_t)stream);
-    return pv_check_launch(ctx, "sched_paths_kernel");
+    return pv_check_launch(ctx, "path scheduler kernel");
 }
 
 extern "C" int pv_compile_path_rules(pv_ctx *ctx, uint32_t num_requests, const pv_path_req *d_requests,

@@ -12,6 +12,7 @@ import oracle
 from paper_2602_16100_gb300 import binding as B
 from paper_2602_16100_gb300 import workloads as W
 from paper_2602_16100_gb300.validator import empty_device, to_device, to_numpy
+from netbuild import ip, make_net
 from test_oracle_policies import _backup_switch_net, _policies
 
 pytestmark = pytest.mark.gpu
@@ -142,3 +143,28 @@ def test_end_to_end_network_10000_requests(validator):
         if o_st[k] == W.PATH_OK:
             assert (g_vis[r, : o_ln[k]] == o_vis[k, : o_ln[k]]).all()
     assert (g_st == W.PATH_OK).sum() > 1000
+
+
+@pytest.mark.parametrize("requests,must_max,max_len", [(1, 3, 64), (17, 3, 1), (311, 32, 255), (311, 32, 40),
+                                                       (152 * 2 * 16 + 5, 2, 64)])
+def test_warp_per_request_edges(validator, requests, must_max, max_len):
+    """The automatic kernel, a warp per request: one request, paths of one
+    visit, requests of up to 33 segments, paths longer than max_len in a later
+    segment, and more requests than resident warps."""
+    e = W.end_to_end(seed=90, num_switches=70, num_intents=4, probes_per_intent=4, rules_per_switch=80)
+    net = e.network
+    pol = W.path_policies(requests, net, 80, forbid_max=3, must_max=must_max, hubs=40)
+    req = W.path_requests(requests, net, requests, num_policies=80, extra_regions=(8, 14), bad_hosts=requests // 9)
+    weights = W.Stream(5, "segment-weights").ints(0, 65535, int(net.port_offs[-1])).astype(np.uint16)
+    _run(validator, net, req, pol, weights, max_len)
+
+
+@pytest.mark.parametrize("S", [700, 1900, 2500, 6000])
+def test_networks_around_the_kernels_shared_memory(validator, S):
+    """Rings of more and more switches: two blocks an SM, one with fewer warps, a block per request."""
+    net = make_net([3] * S, [(i, 1, (i + 1) % S, 2) for i in range(S)], [(i * (S // 50), 0, ip(10, 0, i, 1)) for i in range(50)],
+                   [i % 5 for i in range(S)], [[] for _ in range(S)])
+    req = np.zeros(40, W.PATH_REQ_DTYPE)
+    req["src_host"], req["dst_host"] = np.arange(40), (np.arange(40) * 7 + 1) % 50
+    req["allowed_mask"], req["policy"] = 31, W.NO_POLICY
+    _run(validator, net, req, None, None, 255)
