@@ -19,10 +19,19 @@
 // and v lie in the same connected component of the subgraph induced by the
 // permitted vertices, so R(s, m) is that component (or empty when s itself
 // is not permitted).  One block labels the components of one mask with a
-// lock-free union-find in shared memory, materialises the bitset of each
-// component its sources fall in, and copies those rows out: the output
-// write is the whole cost.  A device-side check decides per call which of
+// lock-free union-find in shared memory and writes the bitset of each to a
+// table; a source's row is then a copy of its component's.  A device-side check decides per call which of
 // the two paths runs; both are launched and the other one returns at once.
+//
+// Other graphs seldom need a search per source either: most permitted
+// vertices lie in one strongly connected component.  Per mask, a hub vertex h
+// is taken and its forward set F and backward set B are searched once; a
+// source in F and B has R(s, m) = F, and only the others are searched (those
+// in B from F on: F is part of their sets).
+//
+// A row of a source that is not permitted is empty on either path, so those
+// rows are cleared by blocks of their own in the check's and the labels'
+// launches.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -41,28 +50,40 @@ inline size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 // A CSR whose offsets are malformed (some row with offs[u + 1] < offs[u] or
 // offs[u + 1] > E) counts as having no edges at all: its well-formed rows
 // could overlap, so their lengths could add up past E, the size of every
-// edge-indexed scratch array.  indeg[V] (cleared with the counts, never
-// counted into) is that per-call flag; every later kernel of the call reads
-// it before it touches an edge.
+// edge-indexed scratch array.  A per-call flag says so (kBadOffs of the
+// context's flags; the no-allocation call's is indeg[V]); every later kernel
+// of the call reads it before it touches an edge.
+enum { kAsym = 0, kBadOffs = 1, kPairs = 2, kReachFlags = 3 };   // words of pv_ctx::d_reach_flags
+
+// The call's rows come from components: the graph is symmetric (no edges at
+// all included).
+__device__ __forceinline__ bool component_path(const uint32_t *flags) {
+    const volatile uint32_t *f = flags;
+    return f[kAsym] == 0 || f[kBadOffs] != 0;
+}
+
 __device__ __forceinline__ bool csr_offsets_bad(const uint32_t *bad) {
     return *(volatile const uint32_t *)bad != 0;
 }
 
-// In-degree count with validation of the caller's CSR.  An out-of-range
-// column skips that edge; malformed offsets set the flag at indeg[V] (the
-// counts of this pass are then unused).
+// In-degree count with validation of the caller's CSR, eight lanes to a
+// vertex (a vertex's loads then overlap).  An out-of-range column skips that
+// edge; malformed offsets set the flag at indeg[V] (the counts of this pass
+// are then unused).
+constexpr uint32_t kEdgeLanes = 8;
 __global__ void reach_indeg_kernel(uint32_t V, uint32_t E, const uint32_t *__restrict__ offs,
                                    const uint32_t *__restrict__ cols, const uint8_t *__restrict__ region,
                                    uint32_t *__restrict__ indeg, int32_t *status) {
-    for (uint32_t u = blockIdx.x * blockDim.x + threadIdx.x; u < V; u += gridDim.x * blockDim.x) {
-        if (region[u] >= 32) pv_device_error(status, PV_EINVAL);
+    const uint32_t sub = threadIdx.x % kEdgeLanes, groups = gridDim.x * blockDim.x / kEdgeLanes;
+    for (uint32_t u = (blockIdx.x * blockDim.x + threadIdx.x) / kEdgeLanes; u < V; u += groups) {
+        if (sub == 0 && region[u] >= 32) pv_device_error(status, PV_EINVAL);
         const uint32_t a = offs[u], b = offs[u + 1];
         if (b < a || b > E) {
             pv_device_error(status, PV_EINVAL);
             atomicOr(&indeg[V], 1u);
             continue;
         }
-        for (uint32_t e = a; e < b; ++e) {
+        for (uint32_t e = a + sub; e < b; e += kEdgeLanes) {
             const uint32_t v = cols[e];
             if (v >= V) {
                 pv_device_error(status, PV_EINVAL);
@@ -73,15 +94,23 @@ __global__ void reach_indeg_kernel(uint32_t V, uint32_t E, const uint32_t *__res
     }
 }
 
+// indeg and the call's flags cleared in one launch.
+__global__ void reach_clear_kernel(uint32_t V, uint32_t *__restrict__ indeg, uint32_t *__restrict__ flags) {
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < V) indeg[i] = 0;
+    if (i < kReachFlags) flags[i] = 0;
+}
+
 // Single block: in_offs = exclusive scan of indeg (V+1 entries); cursor copy.
 // With malformed offsets every in-edge list is empty.
 __global__ void __launch_bounds__(1024) reach_scan_kernel(uint32_t V, const uint32_t *__restrict__ indeg,
                                                           uint32_t *__restrict__ in_offs,
-                                                          uint32_t *__restrict__ cursor, const uint32_t *asym) {
-    if (asym && *(volatile const uint32_t *)asym == 0) return;   // symmetric: in-edges unused
+                                                          uint32_t *__restrict__ cursor, const uint32_t *flags,
+                                                          const uint32_t *bad_offs) {
+    if (flags && component_path(flags)) return;   // in-edges unused
     __shared__ uint32_t s_warp[32];
     __shared__ uint32_t s_carry;
-    const bool bad = csr_offsets_bad(indeg + V);
+    const bool bad = csr_offsets_bad(bad_offs);
     const uint32_t t = threadIdx.x, lane = t & 31, warp = t >> 5;
     if (t == 0) s_carry = 0;
     __syncthreads();
@@ -118,68 +147,122 @@ __global__ void __launch_bounds__(1024) reach_scan_kernel(uint32_t V, const uint
 
 __global__ void reach_fill_kernel(uint32_t V, uint32_t E, const uint32_t *__restrict__ offs,
                                   const uint32_t *__restrict__ cols, uint32_t *__restrict__ cursor,
-                                  uint32_t *__restrict__ in_cols, const uint32_t *asym, const uint32_t *bad) {
-    if (asym && *(volatile const uint32_t *)asym == 0) return;   // symmetric: in-edges unused
-    if (csr_offsets_bad(bad)) return;                            // no edges
-    for (uint32_t u = blockIdx.x * blockDim.x + threadIdx.x; u < V; u += gridDim.x * blockDim.x) {
+                                  uint32_t *__restrict__ in_cols, const uint32_t *flags, const uint32_t *bad) {
+    if (flags && component_path(flags)) return;   // in-edges unused
+    if (csr_offsets_bad(bad)) return;             // no edges
+    const uint32_t sub = threadIdx.x % kEdgeLanes, groups = gridDim.x * blockDim.x / kEdgeLanes;
+    for (uint32_t u = (blockIdx.x * blockDim.x + threadIdx.x) / kEdgeLanes; u < V; u += groups) {
         const uint32_t a = offs[u], b = offs[u + 1];
         if (b < a || b > E) continue;
-        for (uint32_t e = a; e < b; ++e) {
+        for (uint32_t e = a + sub; e < b; e += kEdgeLanes) {
             const uint32_t v = cols[e];
             if (v < V) in_cols[atomicAdd(&cursor[v], 1u)] = u;
         }
     }
 }
 
-// Symmetry check of the caller's out-edge CSR, one warp per vertex:
-// *asym != 0 unless every edge u -> v (v < V, both lists well formed) has
-// its reverse v -> u.  Vertices whose list is longer than kSymScanMax make
-// the graph count as asymmetric (the sweep path then runs; still exact).
-// With malformed offsets (flag set by the in-degree pass) the graph has no
-// edges, which is symmetric: nothing is listed.
-// The same pass lists each undirected edge once, as pairs[] = u << 16 | v
-// with v < u (*npairs of them, in no particular order).
+__device__ __forceinline__ bool source_permitted(uint32_t s, uint32_t V, const uint8_t *__restrict__ region,
+                                                 uint32_t mask) {
+    const uint32_t r = s < V ? region[s] : 32u;
+    return r < 32 && ((mask >> r) & 1u);
+}
+
+// Rows of the sources that are not permitted or out of range (empty on either
+// path), a warp to 32 (mask, source) rows at a time.  Two thirds of a WAN's
+// rows are, and checking and labelling the graph leave most SMs and the memory
+// idle, so blocks of their own in those two launches write them.  [lo, hi):
+// this launch's share of the rows.
+struct ClearArgs {
+    const uint32_t *masks, *src;
+    uint32_t num_src, W;
+    uint32_t *reach;
+    uint64_t lo, hi;
+};
+__device__ __forceinline__ void clear_rows(const ClearArgs &c, uint32_t block, uint32_t blocks, uint32_t V,
+                                           const uint8_t *__restrict__ region) {
+    const uint32_t lane = threadIdx.x & 31, warps = blockDim.x / 32;
+    for (uint64_t i0 = c.lo + ((uint64_t)block * warps + threadIdx.x / 32) * 32; i0 < c.hi;
+         i0 += (uint64_t)blocks * warps * 32) {
+        const uint64_t i = i0 + lane;
+        const uint32_t m = (uint32_t)(i / c.num_src);
+        const bool clear = i < c.hi && !source_permitted(c.src[i - (uint64_t)m * c.num_src], V, region, c.masks[m]);
+        for (uint32_t todo = __ballot_sync(PV_FULL_MASK, clear); todo; todo &= todo - 1u) {
+            uint4 *out = reinterpret_cast<uint4 *>(c.reach + (i0 + (uint32_t)(__ffs(todo) - 1)) * c.W);
+            for (uint32_t q = lane; q < c.W / 4; q += 32) out[q] = make_uint4(0, 0, 0, 0);
+        }
+    }
+}
+
+// Validation, in-degrees and symmetry of the caller's out-edge CSR in one
+// pass, one warp per vertex.  kAsym is set unless every edge u -> v (v < V)
+// has its reverse v -> u; vertices whose list is longer than kSymScanMax make
+// the graph count as asymmetric (the search path then runs; still exact).
+// Each undirected edge is listed once, as pairs[] = u << 16 | v with v < u, in
+// no particular order.  With malformed offsets the counts and pairs of this
+// pass are unused (rows that overlap could list more than E pairs: those past
+// the array are dropped).
 constexpr uint32_t kSymScanMax = 64;
 
-__global__ void reach_symcheck_kernel(uint32_t V, uint32_t E, const uint32_t *__restrict__ offs,
-                                      const uint32_t *__restrict__ cols, uint32_t *asym, uint32_t *pairs,
-                                      uint32_t *npairs, const uint32_t *bad) {
-    if (csr_offsets_bad(bad)) return;   // no edges: symmetric, no pairs
+__global__ void reach_check_kernel(uint32_t V, uint32_t E, const uint32_t *__restrict__ offs,
+                                   const uint32_t *__restrict__ cols, const uint8_t *__restrict__ region,
+                                   uint32_t *__restrict__ indeg, uint32_t *flags, uint32_t *__restrict__ pairs,
+                                   int32_t *status, uint32_t check_blocks, ClearArgs clear) {
+    if (blockIdx.x >= check_blocks) {
+        clear_rows(clear, blockIdx.x - check_blocks, gridDim.x - check_blocks, V, region);
+        return;
+    }
     const uint32_t lane = threadIdx.x & 31;
-    const uint32_t nwarps = gridDim.x * (blockDim.x / 32);
+    const uint32_t nwarps = check_blocks * (blockDim.x / 32);
     for (uint32_t u = blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32; u < V; u += nwarps) {
-        // warp-uniform early exit (lane 0's read decides for the warp)
-        if (__shfl_sync(PV_FULL_MASK, *(volatile uint32_t *)asym, 0)) return;
         const uint32_t a = offs[u], b = offs[u + 1];
-        if (b < a || b > E) continue;
-        if (b - a > kSymScanMax) {
-            if (lane == 0) atomicOr(asym, 1u);
-            return;
+        if (lane == 0 && region[u] >= 32) pv_device_error(status, PV_EINVAL);
+        if (b < a || b > E) {
+            if (lane == 0) {
+                pv_device_error(status, PV_EINVAL);
+                atomicOr(flags + kBadOffs, 1u);
+            }
+            continue;
+        }
+        // once the graph is known to be asymmetric only the counts matter
+        // (warp-uniform: lane 0's read decides)
+        bool sym = __shfl_sync(PV_FULL_MASK, *(volatile uint32_t *)(flags + kAsym), 0) == 0;
+        if (sym && b - a > kSymScanMax) {
+            if (lane == 0) atomicOr(flags + kAsym, 1u);
+            sym = false;
         }
         for (uint32_t e0 = a; e0 < b; e0 += 32) {
             const uint32_t e = e0 + lane;
             uint32_t v = V;
-            bool ok = true;
             if (e < b) {
                 v = cols[e];
-                if (v < V && v != u) {
-                    const uint32_t c = offs[v], d = offs[v + 1];
-                    bool found = false;
-                    if (!(d < c || d > E) && d - c <= kSymScanMax)
-                        for (uint32_t f = c; f < d && !found; ++f) found = cols[f] == u;
-                    ok = found;
-                }
+                if (v < V) atomicAdd(&indeg[v], 1u);
+                else pv_device_error(status, PV_EINVAL);
+            }
+            if (!sym) continue;
+            bool ok = true;
+            if (v < V && v != u) {
+                const uint32_t c = offs[v], d = offs[v + 1];
+                bool found = false;
+                if (!(d < c || d > E) && d - c <= kSymScanMax)
+                    for (uint32_t f = c; f < d && !found; f += 4) {   // four columns in flight
+                        uint32_t x[4];
+#pragma unroll
+                        for (uint32_t j = 0; j < 4; ++j) x[j] = f + j < d ? cols[f + j] : V;
+                        found = x[0] == u || x[1] == u || x[2] == u || x[3] == u;
+                    }
+                ok = found;
             }
             if (__any_sync(PV_FULL_MASK, !ok)) {
-                if (lane == 0) atomicOr(asym, 1u);
-                return;
+                if (lane == 0) atomicOr(flags + kAsym, 1u);
+                sym = false;
+                continue;
             }
             const bool keep = v < u;   // v < V too
             const uint32_t bal = __ballot_sync(PV_FULL_MASK, keep);
             uint32_t base = 0;
-            if (lane == 0 && bal) base = atomicAdd(npairs, (uint32_t)__popc(bal));
-            base = __shfl_sync(PV_FULL_MASK, base, 0);
-            if (keep) pairs[base + __popc(bal & ((1u << lane) - 1u))] = (u << 16) | v;
+            if (lane == 0 && bal) base = atomicAdd(flags + kPairs, (uint32_t)__popc(bal));
+            base = __shfl_sync(PV_FULL_MASK, base, 0) + __popc(bal & ((1u << lane) - 1u));
+            if (keep && base < E) pairs[base] = (u << 16) | v;
         }
     }
 }
@@ -217,10 +300,8 @@ __device__ __forceinline__ void uf_union(volatile uint32_t *parent, uint32_t a, 
     pv_device_error(status, PV_ETIMEOUT);
 }
 
-constexpr int kCompThreads = 512;
-constexpr uint32_t kNoComp = 0xFFFFFFFFu;
 constexpr uint16_t kNoLabel = 0xFFFF;
-constexpr uint16_t kSlotNone = 0xFFFF, kSlotWanted = 0xFFFE, kSlotOverflow = 0xFFFD;
+constexpr uint16_t kSlotNone = 0xFFFF, kSlotOverflow = 0xFFFE, kSlotSingle = 0xFFFD;   // table rows stay below these
 
 __host__ __device__ inline uint32_t up16u(uint32_t x) { return (x + 15u) & ~15u; }
 
@@ -231,7 +312,11 @@ __host__ __device__ inline uint32_t up16u(uint32_t x) { return (x + 15u) & ~15u;
 // it (a valid forest of the same components, so most unions then find one
 // root) and copies the pairs inside the permitted subgraph, usually a small
 // share of them, to shared memory; the union pass then runs over that
-// compact list (over the whole list again when it did not fit).
+// compact list (over the whole list again when it did not fit).  Each
+// component of several vertices then takes the next row of the mask's table,
+// if one is left: slots[m][v] = v's row, kSlotOverflow past the table,
+// kSlotSingle for a vertex alone in its component, kSlotNone for one that is
+// not permitted.
 constexpr int kLabelThreads = 1024;
 constexpr size_t kLabelSmemTarget = 100 * 1024;   // two label blocks per SM
 
@@ -250,12 +335,17 @@ struct LabelSmem {
 };
 
 __global__ void __launch_bounds__(kLabelThreads) reach_labels_kernel(
-    uint32_t V, const uint32_t *__restrict__ pairs, const uint32_t *__restrict__ npairs,
-    const uint8_t *__restrict__ region, const uint32_t *__restrict__ masks, uint16_t *__restrict__ lab,
-    const uint32_t *asym, int32_t *status) {
-    if (*(volatile const uint32_t *)asym) return;       // not symmetric: the sweep kernel runs
+    uint32_t V, const uint32_t *__restrict__ pairs, const uint8_t *__restrict__ region,
+    const uint32_t *__restrict__ masks, uint16_t *__restrict__ lab, uint16_t *__restrict__ slots,
+    uint32_t *__restrict__ table, uint32_t cap, uint32_t W, const uint32_t *flags, int32_t *status,
+    uint32_t num_masks, ClearArgs clear) {
+    if (blockIdx.x >= num_masks) {
+        clear_rows(clear, blockIdx.x - num_masks, gridDim.x - num_masks, V, region);
+        return;
+    }
+    if (!component_path(flags)) return;       // the search path runs
     extern __shared__ __align__(16) uint8_t s_dyn[];
-    __shared__ uint32_t s_np;                                                      // compact pairs
+    __shared__ uint32_t s_np, s_comps;                                             // compact pairs, components
     const LabelSmem L(V);
     volatile uint32_t *parent = reinterpret_cast<uint32_t *>(s_dyn);              // [V]
     uint32_t *s_allow = reinterpret_cast<uint32_t *>(s_dyn + L.allow);            // [ceil(V / 32)]
@@ -275,11 +365,11 @@ __global__ void __launch_bounds__(kLabelThreads) reach_labels_kernel(
         const uint32_t bal = __ballot_sync(PV_FULL_MASK, ok);
         if (lane == 0 && v0 + warp * 32 < V) s_allow[(v0 >> 5) + warp] = bal;
     }
-    if (t == 0) s_np = 0;
+    if (t == 0) s_np = s_comps = 0;
     __syncthreads();
     // each permitted vertex under its smallest permitted neighbour; the
     // pairs inside the permitted subgraph copied to the compact list
-    const uint32_t np = *npairs;
+    const uint32_t np = csr_offsets_bad(flags + kBadOffs) ? 0u : flags[kPairs];
     for (uint32_t i0 = 0; i0 < np; i0 += 4 * nt) {
         const uint32_t i = i0 + 4 * t;
         uint32_t pq[4] = {0, 0, 0, 0};
@@ -324,23 +414,39 @@ __global__ void __launch_bounds__(kLabelThreads) reach_labels_kernel(
         }
     }
     __syncthreads();
-    uint16_t *out = lab + (size_t)m * V;
-    for (uint32_t v = t; v < V; v += nt) out[v] = allowed(v) ? (uint16_t)uf_find(parent, v) : kNoLabel;
+    uint16_t *s_slot = reinterpret_cast<uint16_t *>(s_pairs);   // [V]: the pairs are done with
+    for (uint32_t v = t; v < V; v += nt) s_slot[v] = 0;
+    __syncthreads();
+    for (uint32_t v = t; v < V; v += nt) {
+        const uint32_t r = uf_find(parent, v);
+        lab[(size_t)m * V + v] = allowed(v) ? (uint16_t)r : kNoLabel;
+        if (r != v) s_slot[r] = 1;   // r has company
+    }
+    __syncthreads();
+    for (uint32_t v = t; v < V; v += nt)
+        if (parent[v] == v && allowed(v)) {
+            const uint32_t k = s_slot[v] ? atomicAdd(&s_comps, 1u) : 0u;
+            s_slot[v] = !s_slot[v] ? kSlotSingle : k < cap ? (uint16_t)k : kSlotOverflow;
+        }
+    __syncthreads();
+    // the table's rows: cleared, then every word written once, by the first
+    // of the component's vertices among its 32
+    const uint32_t rows = min(s_comps, cap);
+    uint32_t *tab = table + (size_t)m * cap * W;
+    for (uint32_t q = t; q < rows * (W / 4); q += nt) reinterpret_cast<uint4 *>(tab)[q] = make_uint4(0, 0, 0, 0);
+    __syncthreads();
+    for (uint32_t v0 = warp * 32; v0 < V; v0 += nt) {
+        const uint32_t v = v0 + lane;
+        const uint32_t k = v < V && allowed(v) ? s_slot[uf_find(parent, v)] : kSlotNone;
+        if (v < V) slots[(size_t)m * V + v] = (uint16_t)k;
+        const uint32_t peers = __match_any_sync(PV_FULL_MASK, k);
+        if (k < cap && lane == (uint32_t)(__ffs(peers) - 1)) tab[(size_t)k * W + (v0 >> 5)] = peers;
+    }
 }
 
-struct RowSmem {   // dynamic shared-memory layout of reach_rows_kernel
-    uint32_t slot, slot_comp, rows, total;
-    __host__ __device__ RowSmem(uint32_t V, uint32_t W, uint32_t cap) {
-        slot = up16u(V * 4);
-        slot_comp = slot + up16u(V * 2);
-        rows = slot_comp + up16u(cap * 4);
-        total = rows + cap * W * 4;
-    }
-};
-
 // The bitset row of component c (all v < V with lab[v] == c; words past V
-// are zero), W / 4 uint4s written by one warp to dst (shared or global).
-__device__ __forceinline__ void comp_row(const uint32_t *lab, uint32_t V, uint32_t W, uint32_t c, uint4 *dst,
+// are zero), written by one warp: for components past the table.
+__device__ __forceinline__ void comp_row(const uint16_t *lab, uint32_t V, uint32_t W, uint32_t c, uint4 *dst,
                                          uint32_t lane) {
     const uint32_t groups = W / 4;
     for (uint32_t g0 = 0; g0 < groups; g0 += 32) {
@@ -352,7 +458,7 @@ __device__ __forceinline__ void comp_row(const uint32_t *lab, uint32_t V, uint32
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const uint32_t v = base + 32 * k;
-                bits[k] = __ballot_sync(PV_FULL_MASK, v < V && lab[v] == c);
+                bits[k] = __ballot_sync(PV_FULL_MASK, v < V && __ldg(lab + v) == c);
             }
             if (lane == i) mine = make_uint4(bits[0], bits[1], bits[2], bits[3]);
         }
@@ -360,108 +466,102 @@ __device__ __forceinline__ void comp_row(const uint32_t *lab, uint32_t V, uint32
     }
 }
 
-// Rows of one mask for a slice of sources: R(s, m) = the bitset of s's
-// component (empty when s is not permitted or out of range).  The
-// components the slice's sources fall in get a shared-memory row each
-// (first come, up to cap), built in one pass over the vertices; each output
-// row is then a 128-bit copy, or, past cap, built from ballots directly.
-__global__ void __launch_bounds__(kCompThreads) reach_rows_kernel(
-    uint32_t V, const uint16_t *__restrict__ lab_all, uint32_t num_src, const uint32_t *__restrict__ src,
-    uint32_t *__restrict__ reach, uint32_t W, uint32_t src_per_block, uint32_t cap, const uint32_t *asym) {
-    if (*(volatile const uint32_t *)asym) return;
-    extern __shared__ __align__(16) uint8_t s_dyn[];
-    const RowSmem L(V, W, cap);
-    uint32_t *s_lab = reinterpret_cast<uint32_t *>(s_dyn);
-    uint16_t *s_slot = reinterpret_cast<uint16_t *>(s_dyn + L.slot);
-    uint32_t *s_slot_comp = reinterpret_cast<uint32_t *>(s_dyn + L.slot_comp);
-    uint4 *s_rows = reinterpret_cast<uint4 *>(s_dyn + L.rows);
-    __shared__ uint32_t s_nslots;
-    const uint32_t t = threadIdx.x, lane = t & 31, warp = t >> 5, nt = blockDim.x, nw = nt / 32;
-    const uint32_t m = blockIdx.y;
-    const uint32_t j0 = blockIdx.x * src_per_block, j1 = min(num_src, j0 + src_per_block);
-    const uint16_t *lab = lab_all + (size_t)m * V;
-    for (uint32_t v = t; v < V; v += nt) {
-        const uint16_t l = lab[v];
-        s_lab[v] = l == kNoLabel ? kNoComp : l;
-        s_slot[v] = kSlotNone;
-    }
-    if (t == 0) s_nslots = 0;
-    __syncthreads();
-    for (uint32_t j = j0 + t; j < j1; j += nt) {
-        const uint32_t s = src[j];
-        if (s < V && s_lab[s] != kNoComp) s_slot[s_lab[s]] = kSlotWanted;
-    }
-    __syncthreads();
-    for (uint32_t v = t; v < V; v += nt)
-        if (s_slot[v] == kSlotWanted) {
-            const uint32_t k = atomicAdd(&s_nslots, 1u);
-            s_slot[v] = k < cap ? (uint16_t)k : kSlotOverflow;
-            if (k < cap) s_slot_comp[k] = v;
+// R(s, m) = the row of s's component (clear_rows writes the rows
+// of the other sources): a warp takes 32 (mask, source) rows, finds their
+// table rows at once and copies them one after the other from L2.
+// Bound by the row writes.  A block per mask and slice of sources used to
+// rebuild the labels and the rows of its components, up to 90 of them, in
+// shared memory (a 4,096-vertex WAN has some 150 a mask, so that many rows
+// came from ballots): 22-32 us of the call's 70.
+constexpr int kRowThreads = 256;
+__global__ void __launch_bounds__(kRowThreads) reach_rows_kernel(
+    uint32_t V, const uint16_t *__restrict__ lab, const uint16_t *__restrict__ slots,
+    const uint32_t *__restrict__ table, uint32_t cap, uint32_t num_masks, uint32_t num_src,
+    const uint32_t *__restrict__ src, uint32_t *__restrict__ reach, uint32_t W, const uint32_t *flags) {
+    if (!component_path(flags)) return;
+    const uint32_t lane = threadIdx.x & 31, warps = kRowThreads / 32;
+    const uint64_t rows = (uint64_t)num_masks * num_src, step = (uint64_t)gridDim.x * warps * 32;
+    for (uint64_t i0 = ((uint64_t)blockIdx.x * warps + threadIdx.x / 32) * 32; i0 < rows; i0 += step) {
+        const uint64_t i = i0 + lane;
+        const uint32_t m = (uint32_t)(i / num_src);
+        const uint32_t s = i < rows ? src[i - (uint64_t)m * num_src] : V;
+        const uint32_t slot = s < V ? __ldg(slots + (size_t)m * V + s) : kSlotNone;
+        // four rows in flight
+        for (uint32_t todo = __ballot_sync(PV_FULL_MASK, slot < kSlotSingle); todo;) {
+            const uint4 *row[4];
+            uint4 *out[4];
+#pragma unroll
+            for (uint32_t r = 0; r < 4; ++r) {
+                out[r] = nullptr;
+                row[r] = nullptr;
+                if (todo) {   // warp-uniform
+                    const uint32_t j = (uint32_t)(__ffs(todo) - 1);
+                    todo &= todo - 1u;
+                    out[r] = reinterpret_cast<uint4 *>(reach + (i0 + j) * W);
+                    row[r] = reinterpret_cast<const uint4 *>(
+                        table + ((size_t)__shfl_sync(PV_FULL_MASK, m, j) * cap + __shfl_sync(PV_FULL_MASK, slot, j)) * W);
+                }
+            }
+            for (uint32_t q = lane; q < W / 4; q += 32) {
+                uint4 x[4];
+#pragma unroll
+                for (uint32_t r = 0; r < 4; ++r) x[r] = row[r] ? __ldg(row[r] + q) : make_uint4(0, 0, 0, 0);
+#pragma unroll
+                for (uint32_t r = 0; r < 4; ++r)
+                    if (out[r]) out[r][q] = x[r];
+            }
         }
-    __syncthreads();
-    const uint32_t nsl = min(s_nslots, cap);
-    // slot rows: cleared, then every word written once by the lanes of the
-    // slot's component among its 32 vertices
-    for (uint32_t q = t; q < nsl * (W / 4); q += nt) s_rows[q] = make_uint4(0, 0, 0, 0);
-    __syncthreads();
-    uint32_t *s_words = reinterpret_cast<uint32_t *>(s_rows);
-    for (uint32_t v0 = warp * 32; v0 < V; v0 += nt) {
-        const uint32_t v = v0 + lane;
-        const uint32_t c = v < V ? s_lab[v] : kNoComp;
-        const uint32_t k = c != kNoComp ? s_slot[c] : kSlotNone;
-        const uint32_t peers = __match_any_sync(PV_FULL_MASK, k);
-        if (k < cap && lane == (uint32_t)(__ffs(peers) - 1)) s_words[(size_t)k * W + (v0 >> 5)] = peers;
-    }
-    __syncthreads();
-    for (uint32_t j = j0 + warp; j < j1; j += nw) {
-        const uint32_t s = src[j];
-        const uint32_t c = s < V ? s_lab[s] : kNoComp;
-        uint4 *out = reinterpret_cast<uint4 *>(reach + ((size_t)m * num_src + j) * W);
-        if (c == kNoComp) {
-            for (uint32_t q = lane; q < W / 4; q += 32) out[q] = make_uint4(0, 0, 0, 0);
-        } else if (s_slot[c] < cap) {
-            const uint4 *row = s_rows + (size_t)s_slot[c] * (W / 4);
-            for (uint32_t q = lane; q < W / 4; q += 32) out[q] = row[q];
-        } else {
-            comp_row(s_lab, V, W, c, out, lane);
+        for (uint32_t todo = __ballot_sync(PV_FULL_MASK, slot == kSlotSingle); todo; todo &= todo - 1u) {
+            const uint32_t j = (uint32_t)(__ffs(todo) - 1), v = __shfl_sync(PV_FULL_MASK, s, j), bit = 1u << (v & 31);
+            uint4 *out = reinterpret_cast<uint4 *>(reach + (i0 + j) * W);
+            for (uint32_t q = lane; q < W / 4; q += 32) {
+                const uint32_t w = q == v >> 7 ? (v >> 5) & 3u : 4u;
+                out[q] = make_uint4(w == 0 ? bit : 0u, w == 1 ? bit : 0u, w == 2 ? bit : 0u, w == 3 ? bit : 0u);
+            }
+        }
+        for (uint32_t todo = __ballot_sync(PV_FULL_MASK, slot == kSlotOverflow); todo; todo &= todo - 1u) {
+            const uint32_t j = (uint32_t)(__ffs(todo) - 1);
+            const uint16_t *l = lab + (size_t)__shfl_sync(PV_FULL_MASK, m, j) * V;
+            comp_row(l, V, W, __ldg(l + __shfl_sync(PV_FULL_MASK, s, j)),
+                     reinterpret_cast<uint4 *>(reach + (i0 + j) * W), lane);
         }
     }
 }
 
-// One work item of the sweep kernel: mask m, sources j0 .. j0 + 63.
-__device__ __forceinline__ void msbfs_item(uint32_t V, const uint32_t *__restrict__ in_offs,
-                                           const uint32_t *__restrict__ in_cols, const uint8_t *__restrict__ region,
-                                           uint32_t num_src, const uint32_t *__restrict__ src, uint32_t mask,
-                                           uint32_t *__restrict__ reach, uint32_t W, uint32_t m, uint32_t j0,
-                                           uint64_t *s_vis, uint32_t *s_allow) {
+// Permitted-vertex bitmap of a mask, by the whole block.
+__device__ __forceinline__ void block_allow(uint32_t V, const uint8_t *__restrict__ region, uint32_t mask,
+                                            uint32_t *s_allow) {
     const uint32_t t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const uint32_t nb = min(64u, num_src - j0);
-    volatile uint64_t *vis = s_vis;
-    for (uint32_t v0 = 0; v0 < V; v0 += kReachThreads) {
-        const uint32_t v = v0 + t;
-        bool ok = false;
-        if (v < V) {
-            const uint32_t r = region[v];
-            ok = r < 32 && ((mask >> r) & 1u);
-            s_vis[v] = 0;
-        }
-        const uint32_t b = __ballot_sync(PV_FULL_MASK, ok);
+    for (uint32_t v0 = 0; v0 < V; v0 += blockDim.x) {
+        const uint32_t b = __ballot_sync(PV_FULL_MASK, source_permitted(v0 + t, V, region, mask));
         if (lane == 0 && v0 + warp * 32 < V) s_allow[(v0 >> 5) + warp] = b;
     }
-    __syncthreads();
-    if (t < nb) {
-        const uint32_t s = src[j0 + t];
-        if (s < V && ((s_allow[s >> 5] >> (s & 31)) & 1u)) atomicOr((unsigned long long *)&s_vis[s], 1ull << t);
-    }
-    __syncthreads();
+}
+
+// Sweeps of up to 64 sources to the fixpoint from the words in s_vis (bit j of
+// s_vis[v]: v is known to be in source j's set; all: the bits in use), then
+// source j's row to row_of(j).
+template <typename RowOf>
+__device__ __forceinline__ void msbfs_sweeps(uint32_t V, const uint32_t *__restrict__ in_offs,
+                                             const uint32_t *__restrict__ in_cols, uint32_t nb, uint32_t W,
+                                             uint64_t *s_vis, const uint32_t *s_allow, RowOf row_of) {
+    const uint32_t t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const uint64_t all = nb == 64 ? ~0ull : (1ull << nb) - 1ull;
+    volatile uint64_t *vis = s_vis;
     for (uint32_t iter = 0; iter <= V; ++iter) {
         int changed = 0;
         for (uint32_t v = t; v < V; v += kReachThreads) {
             if (!((s_allow[v >> 5] >> (v & 31)) & 1u)) continue;
             const uint64_t old = vis[v];
+            if (old == all) continue;
             uint64_t acc = old;
             const uint32_t a = __ldg(in_offs + v), b = __ldg(in_offs + v + 1);
-            for (uint32_t e = a; e < b; ++e) acc |= vis[__ldg(in_cols + e)];
+            for (uint32_t e = a; e < b; e += 4) {   // four in-edges in flight (v itself adds nothing)
+                uint32_t x[4];
+#pragma unroll
+                for (uint32_t j = 0; j < 4; ++j) x[j] = e + j < b ? __ldg(in_cols + e + j) : v;
+                acc |= vis[x[0]] | vis[x[1]] | vis[x[2]] | vis[x[3]];
+            }
             if (acc != old) {
                 vis[v] = acc;
                 changed = 1;
@@ -479,7 +579,7 @@ __device__ __forceinline__ void msbfs_item(uint32_t V, const uint32_t *__restric
             x[i] = v < V ? vis[v] : 0ull;
         }
         uint4 lo = make_uint4(0, 0, 0, 0), hi = make_uint4(0, 0, 0, 0);
-        for (uint32_t j = 0; j < 64; ++j) {
+        for (uint32_t j = 0; j < nb; ++j) {
             uint32_t b[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) b[i] = __ballot_sync(PV_FULL_MASK, (x[i] >> j) & 1ull);
@@ -488,33 +588,311 @@ __device__ __forceinline__ void msbfs_item(uint32_t V, const uint32_t *__restric
                 else hi = make_uint4(b[0], b[1], b[2], b[3]);
             }
         }
-        if (lane < nb)
-            reinterpret_cast<uint4 *>(reach + ((size_t)m * num_src + j0 + lane) * W)[q] = lo;
-        if (lane + 32 < nb)
-            reinterpret_cast<uint4 *>(reach + ((size_t)m * num_src + j0 + lane + 32) * W)[q] = hi;
+        if (lane < nb) reinterpret_cast<uint4 *>(row_of(lane))[q] = lo;
+        if (lane + 32 < nb) reinterpret_cast<uint4 *>(row_of(lane + 32))[q] = hi;
     }
 }
-
 
 __global__ void __launch_bounds__(kReachThreads) reach_msbfs_kernel(
     uint32_t V, const uint32_t *__restrict__ in_offs, const uint32_t *__restrict__ in_cols,
     const uint8_t *__restrict__ region, uint32_t num_src, const uint32_t *__restrict__ src, uint32_t num_masks,
-    const uint32_t *__restrict__ masks, uint32_t *__restrict__ reach, uint32_t W, const uint32_t *asym) {
-    // the component path has written the rows of a symmetric graph
-    if (asym && *(volatile const uint32_t *)asym == 0) return;
+    const uint32_t *__restrict__ masks, uint32_t *__restrict__ reach, uint32_t W, const uint32_t *flags) {
+    if (flags && component_path(flags)) return;
     extern __shared__ uint64_t s_vis[];                 // [V]
     __shared__ uint32_t s_allow[kReachMaxV / 32];
-    const uint32_t nbatch = (num_src + 63) / 64;
+    const uint32_t nbatch = (num_src + 63) / 64, t = threadIdx.x;
     const uint64_t items = (uint64_t)nbatch * num_masks;   // (mask, source batch) pairs
     for (uint64_t item = blockIdx.x; item < items; item += gridDim.x) {
-        const uint32_t m = (uint32_t)(item / nbatch);
-        msbfs_item(V, in_offs, in_cols, region, num_src, src, masks[m], reach, W, m,
-                   (uint32_t)(item % nbatch) * 64, s_vis, s_allow);
+        const uint32_t m = (uint32_t)(item / nbatch), j0 = (uint32_t)(item % nbatch) * 64;
+        const uint32_t nb = min(64u, num_src - j0);
+        block_allow(V, region, masks[m], s_allow);
+        for (uint32_t v = t; v < V; v += kReachThreads) s_vis[v] = 0;
+        __syncthreads();
+        if (t < nb) {
+            const uint32_t s = src[j0 + t];
+            if (s < V && ((s_allow[s >> 5] >> (s & 31)) & 1u)) atomicOr((unsigned long long *)&s_vis[s], 1ull << t);
+        }
+        __syncthreads();
+        msbfs_sweeps(V, in_offs, in_cols, nb, W, s_vis, s_allow,
+                     [&](uint32_t j) { return reach + ((size_t)m * num_src + j0 + j) * W; });
         __syncthreads();
     }
 }
 
-// The dynamic shared-memory limits of the three block-wide kernels are
+// Hub of a mask (search path, one block per mask): the permitted vertex with
+// the most edges both in and out inside the permitted subgraph (the smaller of
+// the two counts; ties to the lower id) and the vertices it reaches and is
+// reached from there, searched level by level, half of the block each way.
+// Any hub is exact; one inside the largest strongly connected component
+// leaves the fewest sources to search, so a second is tried when the first
+// one's component holds less than a quarter of the permitted vertices (and the
+// sets themselves did not both hold one), and the better is kept.  Last, the permitted sources outside the kept component are
+// listed: rest[m][0 .. rest_n[m]), in no particular order.
+constexpr int kHubThreads = 1024;
+constexpr uint32_t kHubTries = 2;
+
+struct HubSmem {   // two visited bitmaps, the permitted bitmap, two queues
+    uint32_t allow, queue, total;
+    __host__ __device__ explicit HubSmem(uint32_t V) {
+        const uint32_t words = (V + 31) / 32;
+        allow = 2 * words * 4;
+        queue = allow + words * 4;
+        total = queue + 2 * V * 2;
+    }
+};
+
+__global__ void __launch_bounds__(kHubThreads) reach_hub_kernel(
+    uint32_t V, const uint32_t *__restrict__ offs, const uint32_t *__restrict__ cols,
+    const uint32_t *__restrict__ in_offs, const uint32_t *__restrict__ in_cols, const uint8_t *__restrict__ region,
+    const uint32_t *__restrict__ masks, uint32_t *__restrict__ sets,
+    uint32_t num_src, const uint32_t *__restrict__ src, uint32_t *__restrict__ rest, uint2 *__restrict__ rest_n,
+    const uint32_t *flags) {
+    if (component_path(flags)) return;
+    extern __shared__ __align__(16) uint8_t s_dyn[];
+    __shared__ uint32_t s_best, s_tail[2], s_core, s_all, s_rest;
+    const HubSmem L(V);
+    const uint32_t words = (V + 31) / 32, t = threadIdx.x, way = t / (kHubThreads / 2), m = blockIdx.x;
+    uint32_t *s_sets = reinterpret_cast<uint32_t *>(s_dyn), *s_seen = s_sets + way * words;   // this half's visited set
+    uint32_t *s_allow = reinterpret_cast<uint32_t *>(s_dyn + L.allow);
+    uint16_t *queue = reinterpret_cast<uint16_t *>(s_dyn + L.queue) + way * V;
+    const uint32_t *o = way ? in_offs : offs, *c = way ? in_cols : cols;
+    if (t == 0) s_all = s_rest = 0;
+    block_allow(V, region, masks[m], s_allow);
+    __syncthreads();
+    auto allowed = [&](uint32_t v) { return v < V && ((s_allow[v >> 5] >> (v & 31)) & 1u); };
+    auto degree = [&](const uint32_t *off, const uint32_t *col, uint32_t v) {   // inside the permitted subgraph
+        uint32_t n = 0;
+        for (uint32_t e = __ldg(off + v), e1 = __ldg(off + v + 1); e < e1; e += 8) {   // eight columns in flight
+            uint32_t x[8];
+#pragma unroll
+            for (uint32_t j = 0; j < 8; ++j) x[j] = e + j < e1 ? __ldg(col + e + j) : V;
+#pragma unroll
+            for (uint32_t j = 0; j < 8; ++j) n += allowed(x[j]) ? 1u : 0u;
+        }
+        return n;
+    };
+    for (uint32_t w = t; w < words; w += kHubThreads)
+        if (s_allow[w]) atomicAdd(&s_all, (uint32_t)__popc(s_allow[w]));
+    uint32_t tried[kHubTries], kept = 0;
+    for (uint32_t attempt = 0; attempt < kHubTries; ++attempt) {
+        if (t == 0) s_best = s_core = 0;
+        __syncthreads();
+        uint32_t best = 0;
+        for (uint32_t v = t; v < V; v += kHubThreads) {
+            bool skip = !allowed(v);
+            for (uint32_t i = 0; i < attempt; ++i) skip = skip || v == tried[i];
+            if (!skip)
+                best = max(best, (min(min(degree(offs, cols, v), degree(in_offs, in_cols, v)), 0xFFFEu) + 1u) << 16 |
+                                     (0xFFFFu - v));
+        }
+        best = __reduce_max_sync(PV_FULL_MASK, best);
+        if ((t & 31) == 0) atomicMax(&s_best, best);
+        // a vertex that is not permitted counts as seen
+        for (uint32_t w = t; w < 2 * words; w += kHubThreads) s_sets[w] = ~s_allow[w < words ? w : w - words];
+        __syncthreads();
+        const uint32_t hub = 0xFFFFu - (s_best & 0xFFFFu);
+        tried[attempt] = hub;
+        if (t % (kHubThreads / 2) == 0) {
+            s_tail[way] = s_best != 0 ? 1u : 0u;   // 0: no permitted vertex is left to try
+            if (s_best != 0) {
+                queue[0] = (uint16_t)hub;
+                s_seen[hub >> 5] |= 1u << (hub & 31);
+            }
+        }
+        __syncthreads();
+        uint32_t head = 0;
+        const uint32_t sub = t % kEdgeLanes, lane8 = t % (kHubThreads / 2) / kEdgeLanes;
+        while (true) {
+            const uint32_t tail = *(volatile uint32_t *)&s_tail[way];
+            if (!__syncthreads_or(head < tail)) break;   // also: everyone has read the tail before it moves
+            for (uint32_t i = head + lane8; i < tail; i += kHubThreads / 2 / kEdgeLanes) {
+                const uint32_t u = queue[i], b = __ldg(o + u + 1);
+                for (uint32_t e = __ldg(o + u) + sub; e < b; e += kEdgeLanes) {
+                    const uint32_t v = __ldg(c + e);
+                    if (v >= V) continue;
+                    const uint32_t bit = 1u << (v & 31);
+                    if (!(*(volatile uint32_t *)&s_seen[v >> 5] & bit) && !(atomicOr(&s_seen[v >> 5], bit) & bit))
+                        queue[atomicAdd(&s_tail[way], 1u)] = (uint16_t)v;
+                }
+            }
+            head = tail;
+            __syncthreads();
+        }
+        for (uint32_t w = t; w < words; w += kHubThreads) {
+            const uint32_t n = __popc(s_sets[w] & s_sets[words + w] & s_allow[w]);
+            if (n) atomicAdd(&s_core, n);
+        }
+        __syncthreads();
+        const uint32_t core = s_core;
+        if (attempt == 0 || core > kept) {   // sets[m]: forward, then backward, words each
+            for (uint32_t w = t; w < 2 * words; w += kHubThreads)
+                sets[(size_t)m * 2 * words + w] = s_sets[w] & s_allow[w < words ? w : w - words];
+            kept = core;
+        }
+        __syncthreads();
+        // (block-uniform) large enough, or both sets large and yet little in
+        // common: no large component is near
+        if (kept * 4 >= s_all || min(s_tail[0], s_tail[1]) * 4 >= s_all) break;
+        __syncthreads();
+    }
+    const uint32_t lane = t & 31;
+    const uint32_t *fwd = sets + (size_t)m * 2 * words, *bwd = fwd + words;   // written by this block
+    for (uint32_t b = t - lane; b < num_src; b += kHubThreads) {
+        const uint32_t s = b + lane < num_src ? src[b + lane] : V;
+        const bool listed = allowed(s) && !((fwd[s >> 5] & bwd[s >> 5]) >> (s & 31) & 1u);
+        const uint32_t bal = __ballot_sync(PV_FULL_MASK, listed);
+        uint32_t base = 0;
+        if (lane == 0 && bal) base = atomicAdd(&s_rest, (uint32_t)__popc(bal));
+        base = __shfl_sync(PV_FULL_MASK, base, 0) + __popc(bal & ((1u << lane) - 1u));
+        if (listed) rest[(size_t)m * num_src + base] = b + lane;
+    }
+    __syncthreads();
+    if (t == 0) rest_n[m] = make_uint2(s_rest, kept * 4 >= s_all ? 1u : 0u);   // y: the component is large
+}
+
+// Rows of the search path.  Item (m, x) copies the hub's forward set to the
+// rows of those of sources 64 x .. 64 x + 63 that lie in its strongly connected
+// component, then takes 64 of the listed others.  When the component is large
+// they are few and what they reach outside it is little: a warp searches each
+// from its own queue, a source that reaches the hub over the forward set it
+// starts with.  Searches past kOwnQueue vertices, and all of them when the
+// component is small, are swept together.
+// (3,001 vertices, 18,006 one-way edges, 24 masks, all sources: sweeps for
+// every 64 sources took 311 of the call's 330 us; hub and rows take 60 of its
+// 100, most of it the hub's levels.)
+constexpr uint32_t kOwnQueue = 128;
+struct HubRowSmem {   // vis[V] first
+    uint32_t sets, allow, seen, queue, total;
+    __host__ __device__ explicit HubRowSmem(uint32_t V) {
+        const uint32_t words = (V + 31) / 32;
+        sets = V * 8;
+        allow = sets + 2 * words * 4;
+        seen = allow + words * 4;                             // a warp's own set each
+        queue = seen + kReachThreads / 32 * words * 4;        // and queue
+        total = queue + kReachThreads / 32 * kOwnQueue * 2;
+    }
+};
+
+__global__ void __launch_bounds__(kReachThreads) reach_hub_rows_kernel(
+    uint32_t V, const uint32_t *__restrict__ offs, const uint32_t *__restrict__ cols,
+    const uint32_t *__restrict__ in_offs, const uint32_t *__restrict__ in_cols, const uint8_t *__restrict__ region,
+    uint32_t num_src, const uint32_t *__restrict__ src, uint32_t num_masks, const uint32_t *__restrict__ masks,
+    const uint32_t *__restrict__ sets, const uint32_t *__restrict__ rest, const uint2 *__restrict__ rest_n,
+    uint32_t *__restrict__ reach, uint32_t W, uint32_t per_block, const uint32_t *flags) {
+    if (component_path(flags)) return;
+    extern __shared__ uint64_t s_vis[];
+    __shared__ uint32_t s_list[64], s_sweep;   // sources (as row numbers) to sweep
+    __shared__ uint64_t s_back;
+    const HubRowSmem L(V);
+    uint8_t *s_dyn = reinterpret_cast<uint8_t *>(s_vis);
+    const uint32_t words = (V + 31) / 32, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    uint32_t *fwd = reinterpret_cast<uint32_t *>(s_dyn + L.sets), *bwd = fwd + words;
+    uint32_t *s_allow = reinterpret_cast<uint32_t *>(s_dyn + L.allow);
+    uint32_t *seen = reinterpret_cast<uint32_t *>(s_dyn + L.seen) + warp * words;
+    uint16_t *queue = reinterpret_cast<uint16_t *>(s_dyn + L.queue) + warp * kOwnQueue;
+    const uint32_t batches = (num_src + 63) / 64;
+    const uint64_t i1 = min((uint64_t)(blockIdx.x + 1) * per_block, (uint64_t)batches * num_masks);
+    for (uint64_t item = (uint64_t)blockIdx.x * per_block; item < i1; ++item) {
+        const uint32_t m = (uint32_t)(item / batches), x = (uint32_t)(item % batches);
+        __syncthreads();   // the item before is done with the shared state
+        uint32_t *rows = reach + (size_t)m * num_src * W;
+        const uint2 listed = rest_n[m];
+        const uint32_t j0 = x * 64, n = j0 < listed.x ? min(64u, listed.x - j0) : 0u;
+        const uint32_t *list = rest + (size_t)m * num_src + j0;
+        if (t == 0) {
+            s_sweep = 0;
+            s_back = 0;
+        }
+        for (uint32_t w = t; w < 2 * words; w += kReachThreads) fwd[w] = sets[(size_t)m * 2 * words + w];
+        if (n) block_allow(V, region, masks[m], s_allow);
+        __syncthreads();
+        auto in = [](const uint32_t *set, uint32_t v) { return (set[v >> 5] >> (v & 31)) & 1u; };
+        if (warp < 2) {
+            const uint32_t j = j0 + warp * 32 + lane, s = j < num_src ? src[j] : V;
+            uint32_t todo = __ballot_sync(PV_FULL_MASK, s < V && in(fwd, s) && in(bwd, s));
+            if (lane == 0) s_list[warp] = todo;
+        }
+        __syncthreads();
+        for (uint32_t half = 0; half < 2; ++half) {
+            uint32_t todo = s_list[half];
+            for (uint32_t i = 0; todo; ++i, todo &= todo - 1u) {
+                uint32_t *row = rows + (size_t)(j0 + half * 32 + (uint32_t)(__ffs(todo) - 1)) * W;
+                if (i % (kReachThreads / 32) == warp)
+                    for (uint32_t w = lane; w < W; w += 32) row[w] = w < words ? fwd[w] : 0u;
+            }
+        }
+        if (n == 0) continue;   // block-uniform
+        __syncthreads();        // s_list is free
+        if (!listed.y) {
+            if (t < n) s_list[t] = list[t];
+            if (t == 0) s_sweep = n;
+        } else {
+            const uint32_t sub = lane % kEdgeLanes, lt = (1u << lane) - 1u;
+            for (uint32_t i = warp; i < n; i += kReachThreads / 32) {
+                const uint32_t j = list[i], s = src[j];
+                const bool back = in(bwd, s) != 0;
+                for (uint32_t w = lane; w < words; w += 32) seen[w] = back ? fwd[w] : 0u;
+                __syncwarp();
+                if (lane == 0) {
+                    seen[s >> 5] |= 1u << (s & 31);
+                    queue[0] = (uint16_t)s;
+                }
+                __syncwarp();
+                uint32_t head = 0, tail = 1;
+                bool over = false;
+                while (head < tail && !over) {
+                    // four vertices of the queue, eight lanes to each
+                    const uint32_t q = head + lane / kEdgeLanes;
+                    uint32_t e = 0, e1 = 0;
+                    if (q < tail) {
+                        const uint32_t u = queue[q];
+                        e = __ldg(offs + u) + sub;
+                        e1 = __ldg(offs + u + 1);
+                    }
+                    head = min(head + 32 / kEdgeLanes, tail);
+                    while (__any_sync(PV_FULL_MASK, e < e1) && !over) {
+                        bool push = false;
+                        uint32_t v = 0;
+                        if (e < e1) {
+                            v = __ldg(cols + e);
+                            e += kEdgeLanes;
+                            if (v < V && in(s_allow, v)) {
+                                const uint32_t bit = 1u << (v & 31);
+                                push = !(atomicOr(&seen[v >> 5], bit) & bit);
+                            }
+                        }
+                        const uint32_t pushed = __ballot_sync(PV_FULL_MASK, push);
+                        over = tail + __popc(pushed) > kOwnQueue;
+                        if (push && !over) queue[tail + __popc(pushed & lt)] = (uint16_t)v;
+                        tail += over ? 0u : __popc(pushed);
+                        __syncwarp();
+                    }
+                }
+                if (over) {
+                    if (lane == 0) s_list[atomicAdd(&s_sweep, 1u)] = j;
+                } else {
+                    uint32_t *row = rows + (size_t)j * W;
+                    for (uint32_t w = lane; w < W; w += 32) row[w] = w < words ? seen[w] : 0u;
+                }
+                __syncwarp();
+            }
+        }
+        __syncthreads();
+        const uint32_t nb = s_sweep;
+        if (nb == 0) continue;   // block-uniform
+        // a source that reaches the hub starts with the hub's whole forward set
+        if (t < nb && in(bwd, src[s_list[t]])) atomicOr((unsigned long long *)&s_back, 1ull << t);
+        __syncthreads();
+        const uint64_t back = s_back;
+        for (uint32_t v = t; v < V; v += kReachThreads) s_vis[v] = in(fwd, v) ? back : 0ull;
+        __syncthreads();
+        if (t < nb) atomicOr((unsigned long long *)&s_vis[src[s_list[t]]], 1ull << t);
+        __syncthreads();
+        msbfs_sweeps(V, in_offs, in_cols, nb, W, s_vis, s_allow, [&](uint32_t j) { return rows + (size_t)s_list[j] * W; });
+    }
+}
+
+// The dynamic shared-memory limits of the block-wide kernels are
 // process-wide settings per device.  They are raised once per device to the
 // largest size any call can ask for (under a mutex), so that no call lowers
 // the limit between another thread's setting and launch.
@@ -533,13 +911,15 @@ cudaError_t reach_smem_limits() {
     if (e != cudaSuccess) return e;
     const int rows_max = optin - 1024;
     const int lab_max = (int)LabelSmem(kReachMaxV).total;
-    const int bfs_max = (int)(kReachMaxV * 8);
-    if ((e = cudaFuncSetAttribute(reach_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_max)) !=
-            cudaSuccess ||
-        (e = cudaFuncSetAttribute(reach_labels_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    const int bfs_max = (int)(kReachMaxV * 8), hub_max = (int)HubSmem(kReachMaxV).total;
+    if ((e = cudaFuncSetAttribute(reach_labels_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   std::min(lab_max, rows_max))) != cudaSuccess ||
         (e = cudaFuncSetAttribute(reach_msbfs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  std::min(bfs_max, rows_max))) != cudaSuccess)
+                                  std::min(bfs_max, rows_max))) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(reach_hub_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  std::min(hub_max, rows_max))) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(reach_hub_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_max)) !=
+            cudaSuccess)
         return e;
     g_smem_attr_set[dev] = true;
     return cudaSuccess;
@@ -563,98 +943,108 @@ extern "C" int pv_compliant_reach(pv_ctx *ctx, uint32_t V, const uint32_t *d_off
     const size_t o_indeg = 0, o_in_offs = align256((size_t)(V + 1) * 4);
     const size_t o_cursor = o_in_offs + align256((size_t)(V + 1) * 4);
     const size_t o_cols = o_cursor + align256((size_t)V * 4);
-    const size_t o_pairs = o_cols + align256((size_t)num_edges * 4 + 4);   // undirected pairs (+ count)
-    const size_t o_lab = o_pairs + align256((size_t)num_edges * 4 + 16) + 256;   // component labels
+    const size_t o_pairs = o_cols + align256((size_t)num_edges * 4 + 4);   // undirected pairs
+    const size_t o_lab = o_pairs + align256((size_t)num_edges * 4 + 16);   // component labels, or the hubs' sets
     const bool comp = ctx->opt_reach == 0;
-    const size_t total = o_lab + (comp ? align256((size_t)num_masks * V * 2) : 0);
+    const size_t set_words = 2 * (((size_t)V + 31) / 32);                  // a hub's two sets
+    const size_t o_slots = o_lab + align256((size_t)num_masks * std::max<size_t>((size_t)V * 2, set_words * 4));
+    const size_t o_table = o_slots + align256((size_t)num_masks * V * 2);
+    // table rows a mask: every component's when that takes 64 MB or a quarter
+    // of the caller's rows at most
+    const size_t mask_row = (size_t)num_masks * words_per_row * 4;
+    const uint32_t cap = (uint32_t)std::min<size_t>(V, std::max<size_t>(((size_t)64 << 20) / mask_row, num_src / 4));
+    // search path: the sources to search of every mask and their counts, in the table's place
+    const size_t o_rest_n = o_table + align256((size_t)num_masks * num_src * 4);
+    const size_t total = comp ? std::max(o_table + cap * mask_row, o_rest_n + (size_t)num_masks * 8) : o_lab;
     uint8_t *base = (uint8_t *)pv_scratch(ctx, total);
     if (!base) return PV_ENOMEM;
     uint32_t *indeg = (uint32_t *)(base + o_indeg), *in_offs = (uint32_t *)(base + o_in_offs);
     uint32_t *cursor = (uint32_t *)(base + o_cursor), *in_cols = (uint32_t *)(base + o_cols);
     uint32_t *pairs = (uint32_t *)(base + o_pairs);
-    uint32_t *npairs = (uint32_t *)(base + o_pairs + align256((size_t)num_edges * 4 + 16));
     cudaStream_t st = (cudaStream_t)stream;
-    // component path: row-slot cache sized to keep 3 blocks per SM when the
-    // fixed part allows it, at least one slot otherwise, none if even that
-    // does not fit (rows then come straight from the ballots)
-    uint32_t cap = 0;
-    size_t rows_smem = 0;
-    const size_t lab_smem = LabelSmem(V).total;
-    const size_t limit = ctx->max_smem_optin - 1024;
-    if (comp) {
-        const size_t fixed = RowSmem(V, words_per_row, 0).total;
-        const size_t row = (size_t)words_per_row * 4 + 4;
-        const size_t budget = std::max<size_t>(72 * 1024, fixed + 16 * row);
-        if (fixed + row <= limit) cap = (uint32_t)std::min<size_t>((std::min(budget, limit) - fixed) / row, 0xFFF0);
-        rows_smem = RowSmem(V, words_per_row, cap).total;
-        if (rows_smem > limit) {
-            cap = 0;
-            rows_smem = RowSmem(V, words_per_row, 0).total;
-        }
-        if (rows_smem > limit) return pv_fail(ctx, PV_EINVAL, "pv_compliant_reach: words_per_row too large");
-    }
-    uint16_t *lab = (uint16_t *)(base + o_lab);   // [num_masks][V] (component path only)
+    uint16_t *lab = (uint16_t *)(base + o_lab);     // [num_masks][V] (component path)
+    uint32_t *sets = (uint32_t *)(base + o_lab);    // [num_masks][2][ceil(V / 32)] (search path): never both
+    uint16_t *slots = (uint16_t *)(base + o_slots);   // [num_masks][V]
+    uint32_t *table = (uint32_t *)(base + o_table);   // [num_masks][cap][words_per_row]
+    uint32_t *rest = (uint32_t *)(base + o_table);    // [num_masks][num_src] (search path)
+    uint2 *rest_n = (uint2 *)(base + o_rest_n);       // [num_masks] (search path)
     PV_TRY_CUDA(ctx, reach_smem_limits(), "reach shared-memory limits");
-    if (comp && !ctx->reach_side) {   // first call: the sweep path's side stream
+    if (comp && !ctx->reach_side) {   // first call: the search path's side stream
         PV_TRY_CUDA(ctx, cudaStreamCreateWithFlags(&ctx->reach_side, cudaStreamNonBlocking), "reach side stream");
         PV_TRY_CUDA(ctx, cudaEventCreateWithFlags(&ctx->reach_fork, cudaEventDisableTiming), "reach fork event");
         PV_TRY_CUDA(ctx, cudaEventCreateWithFlags(&ctx->reach_join, cudaEventDisableTiming), "reach join event");
     }
-    PV_TRY_CUDA(ctx, cudaMemsetAsync(indeg, 0, (size_t)(V + 1) * 4, st), "indeg clear");
-    if (comp) {
-        PV_TRY_CUDA(ctx, cudaMemsetAsync(ctx->d_reach_asym, 0, 4, st), "symmetry flag clear");
-        PV_TRY_CUDA(ctx, cudaMemsetAsync(npairs, 0, 4, st), "pair count clear");
-    }
     ctx->last_reach_comp = comp;
-    const uint32_t *sym_flag = comp ? ctx->d_reach_asym : nullptr;
-    const uint32_t grid = std::min<uint32_t>((V + kGridThreads - 1) / kGridThreads, (uint32_t)ctx->num_sms * 8);
+    uint32_t *flags = ctx->d_reach_flags;
+    const uint32_t sms = (uint32_t)ctx->num_sms;
+    const uint32_t egrid = std::min<uint32_t>((V * kEdgeLanes + kGridThreads - 1) / kGridThreads, sms * 8);
     const int pr = pv_prof_start(ctx, st, PV_K_REACH);
-    uint32_t launches = 4;
-    reach_indeg_kernel<<<grid, kGridThreads, 0, st>>>(V, num_edges, d_offs, d_cols, d_region, indeg, ctx->d_status);
-    if (comp) {
-        const uint32_t wgrid = std::min<uint32_t>((V + kGridThreads / 32 - 1) / (kGridThreads / 32),
-                                                  (uint32_t)ctx->num_sms * 8);
-        reach_symcheck_kernel<<<wgrid, kGridThreads, 0, st>>>(V, num_edges, d_offs, d_cols, ctx->d_reach_asym, pairs,
-                                                              npairs, indeg + V);
-        launches += 3;
-        // Both paths are launched and the symmetry flag picks the one that
-        // works: on the component path's calls the sweep path's kernels go to
-        // the side stream (they need only the in-degrees and the flag), so
-        // their launches overlap the labels and rows kernels instead of
-        // queueing behind them; the caller's stream joins it at the end.
-        PV_TRY_CUDA(ctx, cudaEventRecord(ctx->reach_fork, st), "reach fork");
-        PV_TRY_CUDA(ctx, cudaStreamWaitEvent(ctx->reach_side, ctx->reach_fork, 0), "reach fork");
+    reach_clear_kernel<<<(V + 255) / 256, 256, 0, st>>>(V, indeg, flags);
+    if (!comp) {
+        // the counts, and the flag at flags[kBadOffs], as the no-allocation call
+        const uint32_t wgrid = std::min<uint32_t>((V + kGridThreads / 32 - 1) / (kGridThreads / 32), sms * 8);
+        reach_check_kernel<<<wgrid, kGridThreads, 0, st>>>(V, num_edges, d_offs, d_cols, d_region, indeg, flags, pairs,
+                                                           ctx->d_status, wgrid, ClearArgs{});
+        reach_scan_kernel<<<1, 1024, 0, st>>>(V, indeg, in_offs, cursor, nullptr, flags + kBadOffs);
+        reach_fill_kernel<<<egrid, kGridThreads, 0, st>>>(V, num_edges, d_offs, d_cols, cursor, in_cols, nullptr,
+                                                          flags + kBadOffs);
+        const size_t smem = (size_t)V * 8;
+        const int per_sm = std::max(1, pv_blocks_per_sm(ctx, (const void *)reach_msbfs_kernel, kReachThreads, smem));
+        const uint64_t items = (uint64_t)((num_src + 63) / 64) * num_masks;
+        reach_msbfs_kernel<<<(uint32_t)std::min<uint64_t>(items, (uint64_t)per_sm * sms), kReachThreads, smem, st>>>(
+            V, in_offs, in_cols, d_region, num_src, d_src, num_masks, d_masks, d_reach, words_per_row, nullptr);
+        pv_prof_stop(ctx, st, pr, 5);
+        return pv_check_launch(ctx, "reach kernels");
     }
-    cudaStream_t sw = comp ? ctx->reach_side : st;   // the sweep path's stream
-    reach_scan_kernel<<<1, 1024, 0, sw>>>(V, indeg, in_offs, cursor, sym_flag);
-    reach_fill_kernel<<<grid, kGridThreads, 0, sw>>>(V, num_edges, d_offs, d_cols, cursor, in_cols, sym_flag,
-                                                     indeg + V);
-    if (comp) {
-        reach_labels_kernel<<<num_masks, kLabelThreads, lab_smem, st>>>(V, pairs, npairs, d_region, d_masks, lab,
-                                                                         ctx->d_reach_asym, ctx->d_status);
-        int per_sm = 1;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, reach_rows_kernel, kCompThreads, rows_smem);
-        // one wave of resident blocks over masks x source slices
-        const uint64_t want = (uint64_t)std::max(per_sm, 1) * ctx->num_sms;
-        const uint32_t slices = (uint32_t)std::max<uint64_t>(1, std::min<uint64_t>(num_src, want / num_masks));
-        const uint32_t spb = (num_src + slices - 1) / slices;
-        dim3 gc((num_src + spb - 1) / spb, num_masks);
-        reach_rows_kernel<<<gc, kCompThreads, rows_smem, st>>>(V, lab, num_src, d_src, d_reach, words_per_row, spb,
-                                                               cap, ctx->d_reach_asym);
-    }
-    const size_t smem = (size_t)V * 8;
-    int bfs_per_sm = 1;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bfs_per_sm, reach_msbfs_kernel, kReachThreads, smem);
+    const uint32_t wgrid = std::min<uint32_t>((V + kGridThreads / 32 - 1) / (kGridThreads / 32), sms * 8);
+    // the empty rows: a third beside the check, the rest beside the labels,
+    // about as their times are
+    const uint64_t all_rows = (uint64_t)num_masks * num_src;
+    ClearArgs clear = {d_masks, d_src, num_src, words_per_row, d_reach, 0, all_rows / 96 * 32};
+    reach_check_kernel<<<wgrid + 2 * sms, kGridThreads, 0, st>>>(V, num_edges, d_offs, d_cols, d_region, indeg, flags,
+                                                                 pairs, ctx->d_status, wgrid, clear);
+    clear.lo = clear.hi;
+    clear.hi = all_rows;
+    // Both paths are launched and the flags pick the one that works: the
+    // search path's kernels go to the side stream, so on a symmetric graph
+    // their launches overlap the labels and rows kernels instead of queueing
+    // behind them; the caller's stream joins it at the end.
+    PV_TRY_CUDA(ctx, cudaEventRecord(ctx->reach_fork, st), "reach fork");
+    PV_TRY_CUDA(ctx, cudaStreamWaitEvent(ctx->reach_side, ctx->reach_fork, 0), "reach fork");
+    cudaStream_t sw = ctx->reach_side;
+    reach_scan_kernel<<<1, 1024, 0, sw>>>(V, indeg, in_offs, cursor, flags, flags + kBadOffs);
+    reach_fill_kernel<<<egrid, kGridThreads, 0, sw>>>(V, num_edges, d_offs, d_cols, cursor, in_cols, flags,
+                                                      flags + kBadOffs);
+    // A hub and its two sets take some 25 us a mask before the first row: more
+    // than sweeps while every (mask, 64 sources) item has a block of its own
+    // (16 masks: 500 vertices 49 us against 66; 3,000, of which no component is
+    // large, 265 against 221; 8,000 with a large one 1,642 against 188).
     const uint64_t items = (uint64_t)((num_src + 63) / 64) * num_masks;
-    const uint32_t g2 = (uint32_t)std::min<uint64_t>(items, (uint64_t)std::max(bfs_per_sm, 1) * ctx->num_sms);
-    reach_msbfs_kernel<<<g2, kReachThreads, smem, sw>>>(V, in_offs, in_cols, d_region, num_src, d_src, num_masks,
-                                                       d_masks, d_reach, words_per_row,
-                                                       comp ? ctx->d_reach_asym : nullptr);
-    if (comp) {
-        PV_TRY_CUDA(ctx, cudaEventRecord(ctx->reach_join, ctx->reach_side), "reach join");
-        PV_TRY_CUDA(ctx, cudaStreamWaitEvent(st, ctx->reach_join, 0), "reach join");
+    const bool by_hub = items > 4ull * sms;
+    if (by_hub) {
+        reach_hub_kernel<<<num_masks, kHubThreads, HubSmem(V).total, sw>>>(V, d_offs, d_cols, in_offs, in_cols, d_region,
+                                                                          d_masks, sets, num_src, d_src, rest, rest_n,
+                                                                          flags);
+        // at most sixteen blocks an SM: on a symmetric graph they all start and return
+        const uint32_t per = (uint32_t)((items + 16ull * sms - 1) / (16ull * sms));
+        reach_hub_rows_kernel<<<(uint32_t)((items + per - 1) / per), kReachThreads, HubRowSmem(V).total, sw>>>(
+            V, d_offs, d_cols, in_offs, in_cols, d_region, num_src, d_src, num_masks, d_masks, sets, rest, rest_n,
+            d_reach, words_per_row, per, flags);
+    } else {
+        reach_msbfs_kernel<<<(uint32_t)std::min<uint64_t>(items, 0x7FFFFFFFull), kReachThreads, (size_t)V * 8, sw>>>(
+            V, in_offs, in_cols, d_region, num_src, d_src, num_masks, d_masks, d_reach, words_per_row, flags);
     }
-    pv_prof_stop(ctx, st, pr, launches);
+    reach_labels_kernel<<<num_masks + sms, kLabelThreads, LabelSmem(V).total, st>>>(
+        V, pairs, d_region, d_masks, lab, slots, table, cap, words_per_row, flags, ctx->d_status, num_masks, clear);
+    {
+        const uint64_t warps = ((uint64_t)num_masks * num_src + 31) / 32;
+        const uint32_t rgrid = (uint32_t)std::min<uint64_t>((warps + kRowThreads / 32 - 1) / (kRowThreads / 32), sms * 8);
+        reach_rows_kernel<<<rgrid, kRowThreads, 0, st>>>(V, lab, slots, table, cap, num_masks, num_src, d_src, d_reach,
+                                                         words_per_row, flags);
+    }
+    PV_TRY_CUDA(ctx, cudaEventRecord(ctx->reach_join, sw), "reach join");
+    PV_TRY_CUDA(ctx, cudaStreamWaitEvent(st, ctx->reach_join, 0), "reach join");
+    pv_prof_stop(ctx, st, pr, by_hub ? 8 : 7);
     return pv_check_launch(ctx, "reach kernels");
 }
 
@@ -731,9 +1121,9 @@ extern "C" int pv_compliant_reach_noalloc(uint32_t V, const uint32_t *d_offs, ui
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return PV_ECUDA;
-    const uint32_t grid = std::min<uint32_t>((V + kGridThreads - 1) / kGridThreads, (uint32_t)sms * 8);
+    const uint32_t grid = std::min<uint32_t>((V * kEdgeLanes + kGridThreads - 1) / kGridThreads, (uint32_t)sms * 8);
     reach_indeg_kernel<<<grid, kGridThreads, 0, st>>>(V, num_edges, d_offs, d_cols, d_region, indeg, status);
-    reach_scan_kernel<<<1, 1024, 0, st>>>(V, indeg, in_offs, cursor, nullptr);
+    reach_scan_kernel<<<1, 1024, 0, st>>>(V, indeg, in_offs, cursor, nullptr, indeg + V);
     reach_fill_kernel<<<grid, kGridThreads, 0, st>>>(V, num_edges, d_offs, d_cols, cursor, in_cols, nullptr,
                                                      indeg + V);
     const size_t smem = (size_t)V * 8;

@@ -287,7 +287,7 @@ extern "C" int pv_create(pv_ctx **out, int cuda_device) {
         pv_device_alloc(ctx, (void **)&ctx->d_walk_live, (PV_MAX_HOP_CAP + 1) * sizeof(uint32_t),
                         "walk statistics") != PV_OK ||
         cudaMemset(ctx->d_walk_live, 0, (PV_MAX_HOP_CAP + 1) * sizeof(uint32_t)) != cudaSuccess ||
-        pv_device_alloc(ctx, (void **)&ctx->d_reach_asym, sizeof(uint32_t), "reach symmetry flag") != PV_OK ||
+        pv_device_alloc(ctx, (void **)&ctx->d_reach_flags, 4 * sizeof(uint32_t), "reach flags") != PV_OK ||
         pv_device_alloc(ctx, (void **)&ctx->d_walk_visits, ctx->walk_visit_slots * sizeof(unsigned long long),
                         "walk visit counts") != PV_OK ||
         pv_device_alloc(ctx, (void **)&ctx->d_walk_stats, PV_WALK_STATS * sizeof(unsigned long long),
@@ -297,7 +297,7 @@ extern "C" int pv_create(pv_ctx **out, int cuda_device) {
         pv_device_free(ctx->d_walk_live);
         pv_device_free(ctx->d_walk_visits);
         pv_device_free(ctx->d_walk_stats);
-        pv_device_free(ctx->d_reach_asym);
+        pv_device_free(ctx->d_reach_flags);
         cudaEventDestroy(ctx->last_use);
         cudaEventDestroy(ctx->load_done);
         cudaEventDestroy(ctx->retire_from);
@@ -335,7 +335,7 @@ extern "C" void pv_destroy(pv_ctx *ctx) {
     pv_device_free(ctx->d_walk_live);
     pv_device_free(ctx->d_walk_visits);
     pv_device_free(ctx->d_walk_stats);
-    pv_device_free(ctx->d_reach_asym);
+    pv_device_free(ctx->d_reach_flags);
     delete ctx;
 }
 
@@ -428,11 +428,10 @@ extern "C" int pv_get_stat(const pv_ctx *ctx, int stat, int64_t *value) {
         return PV_OK;
     }
     case PV_STAT_REACH_COMPONENTS: {
-        uint32_t asym = 1;
-        if (ctx->last_reach_comp &&
-            cudaMemcpy(&asym, ctx->d_reach_asym, sizeof asym, cudaMemcpyDeviceToHost) != cudaSuccess)
+        uint32_t f[2] = {1, 0};   // not symmetric, malformed offsets (no edges, so symmetric)
+        if (ctx->last_reach_comp && cudaMemcpy(f, ctx->d_reach_flags, sizeof f, cudaMemcpyDeviceToHost) != cudaSuccess)
             return PV_ECUDA;
-        *value = (ctx->last_reach_comp && asym == 0) ? 1 : 0;
+        *value = (ctx->last_reach_comp && (f[0] == 0 || f[1] != 0)) ? 1 : 0;
         return PV_OK;
     }
     case PV_STAT_WALK_FIRST_MATCHES:

@@ -141,7 +141,7 @@ struct pv_ctx {
     uint32_t last_walk_hops = 0;      // entries of d_walk_live and of d_walk_visits that the last walk wrote
     uint32_t last_walk_blocks = 0;
     int opt_reach = 0;                // 0: components on symmetric graphs, 1: sweeps only
-    uint32_t *d_reach_asym = nullptr; // != 0: the last reach call's graph is not symmetric
+    uint32_t *d_reach_flags = nullptr; // [4] the last reach call's {not symmetric, malformed offsets, listed pairs}
     bool last_reach_comp = false;     // the last reach call launched the component path
     void *scratch = nullptr;
     size_t scratch_bytes = 0;

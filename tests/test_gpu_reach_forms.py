@@ -1,0 +1,105 @@
+"""Compliant reach where the library's choice of kernel changes: the hub search
+of directed graphs (taken when there are more (mask, 64 sources) items than
+blocks fit the GPU at once) and the component table of symmetric ones, against
+the oracle."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2602_16100_gb300 import binding as B
+from paper_2602_16100_gb300 import workloads as W
+from paper_2602_16100_gb300.validator import to_device, to_numpy
+
+pytestmark = pytest.mark.gpu
+
+ITEMS = 4 * 152   # more than this many (mask, 64 sources) items: hub search
+
+
+def _graph(V, a, b, regions, seed):
+    o = np.lexsort((b, a))
+    a, b = np.asarray(a)[o], np.asarray(b)[o]
+    offs = np.zeros(V + 1, np.int64)
+    np.add.at(offs, a + 1, 1)
+    return W.Graph(V, np.cumsum(offs).astype(np.uint32), b.astype(np.uint32),
+                   np.random.default_rng(seed).integers(0, regions, V).astype(np.uint8))
+
+
+def _check(v, g, src, masks, components):
+    out = v.compliant_reach(v.upload_graph(g), len(src), to_device(src.astype(np.uint32), v.device), len(masks),
+                            to_device(masks.astype(np.uint32), v.device))
+    v.sync()
+    assert B.pv_get_stat(v.ctx, B.PV_STAT_REACH_COMPONENTS) == components
+    want = oracle.compliant_reach(g, src.astype(np.uint32), masks.astype(np.uint32))
+    assert (to_numpy(out, np.uint32, want.shape) == want).all()
+
+
+def _edges(kind, V, r):
+    if kind == "giant":          # one large strongly connected component and tendrils
+        return r.integers(0, V, 6 * V), r.integers(0, V, 6 * V)
+    if kind == "dag":            # none: every source is swept
+        a, b = r.integers(0, V, 4 * V), r.integers(0, V, 4 * V)
+        return np.minimum(a, b), np.maximum(a, b)
+    if kind == "tail":           # a component whose sources outside it reach more than a queue holds
+        core, n = V // 2, 6 * (V // 2)
+        path = np.arange(core, V - 1)
+        return np.concatenate([r.integers(0, core, n), path, path[-1:] + 1]), \
+            np.concatenate([r.integers(0, core, n), path + 1, [0]])
+    if kind == "two":            # two components, the first hub may sit in the smaller
+        h = V // 3
+        return np.concatenate([r.integers(0, h, 8 * h), r.integers(h, V, 5 * (V - h))]), \
+            np.concatenate([r.integers(0, h, 8 * h), r.integers(h, V, 5 * (V - h))])
+    a = np.arange(V - 1)         # a long path: as many levels as vertices
+    return a, a + 1
+
+
+@pytest.mark.parametrize("kind", ["giant", "dag", "tail", "two", "path"])
+@pytest.mark.parametrize("V,num_masks", [(700, 64), (321, 120)])
+def test_hub_search(validator, kind, V, num_masks):
+    r = np.random.default_rng(V + len(kind))
+    g = _graph(V, *_edges(kind, V, r), 5, 3)
+    src = np.concatenate([np.arange(V), [0, V - 1, V, 0xFFFFFFFF]])      # duplicates, out of range
+    masks = r.integers(0, 32, num_masks)
+    masks[:3] = [31, 0, 1]
+    assert (len(src) + 63) // 64 * num_masks > ITEMS
+    _check(validator, g, src, masks, 0)
+
+
+@pytest.mark.parametrize("masks", [ITEMS // 2, ITEMS // 2 + 1])
+def test_either_side_of_the_item_limit(validator, masks):
+    r = np.random.default_rng(masks)
+    g = _graph(130, *_edges("giant", 130, r), 4, 1)
+    _check(validator, g, np.arange(128), r.integers(1, 16, masks), 0)
+
+
+@pytest.mark.parametrize("bad", ["offsets", "columns"])
+def test_hub_search_malformed(validator, bad):
+    """Malformed offsets (no edges) and columns out of range (skipped), reported by the next sync."""
+    r = np.random.default_rng(9)
+    g = _graph(400, *_edges("giant", 400, r), 3, 2)
+    if bad == "offsets":
+        g.offs[200] = g.offs[-1] + 7
+    else:
+        g.cols[::9] = 400 + np.arange(len(g.cols[::9]))
+    src, masks = np.arange(400), r.integers(0, 8, 100)
+    v = validator
+    out = v.compliant_reach(v.upload_graph(g), 400, to_device(src.astype(np.uint32), v.device), 100,
+                            to_device(masks.astype(np.uint32), v.device))
+    with pytest.raises(B.PVError) as e:
+        v.sync()
+    assert e.value.code == B.PV_EINVAL
+    assert B.pv_get_stat(v.ctx, B.PV_STAT_REACH_COMPONENTS) == (1 if bad == "offsets" else 0)
+    want = oracle.compliant_reach(g, src.astype(np.uint32), masks.astype(np.uint32))
+    assert (to_numpy(out, np.uint32, want.shape) == want).all()
+
+
+@pytest.mark.parametrize("group,num_masks", [(1, 7), (2, 2000), (5, 2000), (2, 7)])
+def test_component_table(validator, group, num_masks):
+    """Vertices alone, and components of `group`: fewer and more of them than
+    the mask's table holds (2,000 masks leave it 131 rows)."""
+    V = 2003
+    v = np.arange(V)
+    a = v[(v % group != group - 1) & (v + 1 < V)] if group > 1 else v[:0]
+    g = _graph(V, np.concatenate([a, a + 1]), np.concatenate([a + 1, a]), 3, 4)
+    r = np.random.default_rng(group)
+    src = np.concatenate([r.integers(0, V, 5), [V - 1, 0, V]])
+    _check(validator, g, src, r.integers(0, 8, num_masks), 1)
