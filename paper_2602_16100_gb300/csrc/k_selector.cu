@@ -12,8 +12,10 @@
 //    value), the bitset of nodes carrying it, plus one "key present" row
 //    per key.  An In expression is then the OR of its values' rows, NotIn
 //    its complement, Exists / DoesNotExist the present row or its
-//    complement, and a pod's row the AND over its expressions -- 32 nodes
-//    per word operation, rows read from L2 with 128-bit loads.
+//    complement, and a pod's row the AND over its expressions (in the term
+//    form the OR of its terms' ANDs) -- 32 nodes per word operation, rows
+//    read from L2 with 128-bit loads.  Warps own ranges of pods and resolve
+//    the expressions of several pods at once, one per lane.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -43,9 +45,10 @@ __global__ void build_inventory_kernel(uint32_t N, uint32_t K, const uint16_t *_
 }
 
 // One block (1024 threads) per key: exclusive prefix popcount over the key's
-// 2048 inventory words; count[k] = number of carried values.
+// 2048 inventory words, stored beside them (a value's row then takes one
+// load); count[k] = number of carried values.
 __global__ void __launch_bounds__(1024) inventory_rank_kernel(const uint32_t *__restrict__ inv,
-                                                              uint32_t *__restrict__ rank,
+                                                              uint2 *__restrict__ ranked,
                                                               uint32_t *__restrict__ count) {
     __shared__ uint32_t s_warp[32];
     const uint32_t k = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -69,8 +72,8 @@ __global__ void __launch_bounds__(1024) inventory_rank_kernel(const uint32_t *__
     }
     __syncthreads();
     uint32_t excl = s_warp[warp] + incl - x;
-    rank[(size_t)k * kInvWords + 2 * t] = excl;
-    rank[(size_t)k * kInvWords + 2 * t + 1] = excl + a;
+    ranked[(size_t)k * kInvWords + 2 * t] = make_uint2(w[2 * t], excl);
+    ranked[(size_t)k * kInvWords + 2 * t + 1] = make_uint2(w[2 * t + 1], excl + a);
 }
 
 // Single block: key_base = exclusive scan of count[0..K), key_base[K] = total.
@@ -108,21 +111,22 @@ __global__ void __launch_bounds__(1024) key_base_kernel(uint32_t K, const uint32
     if (t == 0) base[K] = s_carry;
 }
 
-__device__ __forceinline__ uint32_t value_row(const uint32_t *__restrict__ inv, const uint32_t *__restrict__ rank,
+// The row of value v of key k, if some node carries it: the key's first row
+// plus the carried values below v.
+__device__ __forceinline__ uint32_t value_row(const uint2 *__restrict__ ranked,
                                               const uint32_t *__restrict__ key_base, uint32_t k, uint32_t v,
                                               bool *carried) {
-    uint32_t w = inv[(size_t)k * kInvWords + (v >> 5)];
-    uint32_t bit = v & 31;
-    *carried = (w >> bit) & 1u;
-    return key_base[k] + rank[(size_t)k * kInvWords + (v >> 5)] + __popc(w & ((1u << bit) - 1u));
+    const uint2 w = __ldg(ranked + (size_t)k * kInvWords + (v >> 5));
+    const uint32_t bit = v & 31;
+    *carried = (w.x >> bit) & 1u;
+    return __ldg(key_base + k) + w.y + __popc(w.x & ((1u << bit) - 1u));
 }
 
 // Value rows and present rows.  One warp covers 32 consecutive nodes of one
 // key; present rows are written with a ballot, value rows with atomicOr.
 __global__ void build_rows_kernel(uint32_t N, uint32_t K, const uint16_t *__restrict__ labels,
-                                  const uint32_t *__restrict__ inv, const uint32_t *__restrict__ rank,
-                                  const uint32_t *__restrict__ key_base, uint32_t num_value_rows,
-                                  uint32_t row_words, uint32_t *__restrict__ rows) {
+                                  const uint2 *__restrict__ ranked, const uint32_t *__restrict__ key_base,
+                                  uint32_t num_value_rows, uint32_t row_words, uint32_t *__restrict__ rows) {
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t words = (N + 31) / 32;
     const size_t total_warps = (size_t)K * words;
@@ -136,7 +140,7 @@ __global__ void build_rows_kernel(uint32_t N, uint32_t K, const uint16_t *__rest
         if (lane == 0) rows[((size_t)num_value_rows + k) * row_words + wd] = pres;
         if (v != PV_ABSENT) {
             bool carried;
-            uint32_t r = value_row(inv, rank, key_base, k, v, &carried);
+            uint32_t r = value_row(ranked, key_base, k, v, &carried);
             atomicOr(&rows[(size_t)r * row_words + wd], 1u << lane);
         }
     }
@@ -302,16 +306,15 @@ __global__ void __launch_bounds__(kCmpThreads) sel_cmp_kernel(
 // ---------------------------------------------------------------------------
 // kernel 2: per-(key, value) node-bitset rows
 // ---------------------------------------------------------------------------
-constexpr int kRowsThreads = 256;
 
 // Four words (128 nodes from word w0) of the node set matching expression x:
 // In = OR of its values' rows, NotIn its complement, Exists the key's
 // present row, DoesNotExist its complement.  Words past the rows read 0
 // before the complement.
 __device__ __forceinline__ uint4 expr_rows4(const pv_expr &x, uint32_t w0, bool in_rows,
-                                            const uint32_t *__restrict__ inv, const uint32_t *__restrict__ rank,
-                                            const uint32_t *__restrict__ key_base, const uint32_t *__restrict__ rows,
-                                            uint32_t row_words, uint32_t num_value_rows) {
+                                            const uint2 *__restrict__ ranked, const uint32_t *__restrict__ key_base,
+                                            const uint32_t *__restrict__ rows, uint32_t row_words,
+                                            uint32_t num_value_rows) {
     const uint32_t k = x.key, op = x.op;
     uint4 r;
     if (op == PV_IN || op == PV_NOTIN) {
@@ -319,7 +322,7 @@ __device__ __forceinline__ uint4 expr_rows4(const pv_expr &x, uint32_t w0, bool 
         const uint32_t nv = x.nvals;
         for (uint32_t j = 0; j < nv; ++j) {
             bool carried;
-            const uint32_t row = value_row(inv, rank, key_base, k, x.vals[j], &carried);
+            const uint32_t row = value_row(ranked, key_base, k, x.vals[j], &carried);
             if (carried && in_rows) {
                 const uint4 v = __ldg(reinterpret_cast<const uint4 *>(rows + (size_t)row * row_words + w0));
                 r.x |= v.x; r.y |= v.y; r.z |= v.z; r.w |= v.w;
@@ -333,210 +336,77 @@ __device__ __forceinline__ uint4 expr_rows4(const pv_expr &x, uint32_t w0, bool 
     return r;
 }
 
-// A pod's expressions resolved once, one expression per lane (lists of at
-// most 32): each lane validates its expression, flags In values that no
-// node carries, and leaves the word offsets of the rows to OR (the key's
-// present row for Exists / DoesNotExist) in the warp's shared slots.  The
-// row sweep then reads only rows.  Returns bit0 = a bad expression, bit1 =
-// an unknown value (as pod_prescan).
-constexpr int kRowsWarps = kRowsThreads / 32;
-struct ResolvedExprs {
-    uint32_t meta[kRowsWarps][32];     // op | rows << 8
-    uint32_t off[kRowsWarps][32][8];   // word offset of each row in the row array
-    uint8_t order[kRowsWarps][32];     // evaluation order of the expressions (sel_rows_kernel)
+// A warp takes as many of its pods as have 32 expressions together and first
+// resolves those, one per lane: validated, In values that no node carries
+// flagged, and every expression turned into words of the warp's list in shared
+// memory, one per row to OR; then it sweeps pod after pod,
+// reading only the list and rows.  (Resolving one pod at a time kept most lanes
+// idle in code of 300 instructions.)
+// Threads per block: in the term form the pods' lengths differ more, and with
+// half the block the first ones to finish leave room sooner (5,500 pods on
+// 5,000 nodes 16.7 us with 256 threads, 15.8 with 128; the single-list form at
+// 100,000 pods 68.7 and 72.8).  Three blocks of 256 per SM, or as much: 80
+// registers without a spill; with four the term form at 100,000 pods took 113.8
+// us instead of 97.1, with two of 128 registers 129.
+template <bool kTerms>
+constexpr int kRowsThreads = kTerms ? 128 : 256;
+// A row's word is its byte offset (a multiple of 16 below 2^32) and the flags
+// below.
+constexpr uint32_t kRowLast = 1u;   // the expression's last row
+constexpr uint32_t kRowNot = 2u;    // complement of the OR (NotIn, DoesNotExist)
+constexpr uint32_t kRowTerm = 4u;   // the term's last row
+constexpr int kAhead = 4;   // rows in flight (2: 72.1 us for the 100,000 pods, 3: 70.1, 4: 68.7, 6: 75.8)
+constexpr uint32_t kListWords = 32 * 8;   // a group's rows at most
+static_assert(kRowBudgetBytes < 1ull << 32, "rows and the row of no node have 32-bit byte offsets");
+
+// One expression of at most eight rows, resolved by one lane.
+struct LaneExpr {
+    uint32_t off[8];       // byte offset of each listed value's row; off[0] alone for Exists / DoesNotExist
+    uint32_t carried;      // bit j: off[j] is a row to OR
+    uint32_t op;
+    bool bad, unknown;
 };
 
-template <bool kOrder>
-__device__ __forceinline__ uint32_t resolve_exprs(ResolvedExprs &rx, uint32_t warp, uint32_t lane, uint32_t lo,
-                                                  uint32_t E, const pv_expr *__restrict__ exprs, uint32_t K,
-                                                  const uint32_t *__restrict__ inv, const uint32_t *__restrict__ rank,
-                                                  const uint32_t *__restrict__ key_base, uint32_t num_value_rows,
-                                                  uint32_t row_words) {
-    bool bad = false, unknown = false;
-    if (lane < E) {
-        const pv_expr *xp = exprs + lo + lane;
-        const uint32_t k = xp->key, op = xp->op, nv = xp->nvals;
-        uint32_t n = 0;
-        if (k >= K) {
-            bad = true;
-        } else if (op == PV_IN || op == PV_NOTIN) {
-            bad = nv < 1 || nv > 8;
+__device__ __forceinline__ void resolve_expr(LaneExpr &r, const pv_expr *__restrict__ x, uint32_t K,
+                                             const uint2 *__restrict__ ranked,
+                                             const uint32_t *__restrict__ key_base, uint32_t num_value_rows,
+                                             uint32_t row_bytes) {
+    uint32_t w[5];   // 20-byte records: 32-bit loads unless the caller's array is only 2-byte aligned
+    if (((uintptr_t)x & 3) == 0) {
 #pragma unroll
-            for (uint32_t j = 0; j < 8; ++j) {
-                if (j >= nv || bad) continue;
-                const uint32_t v = xp->vals[j];
-                if (v == PV_ABSENT) {
-                    bad = true;
-                    continue;
-                }
-                const uint32_t w = inv[(size_t)k * kInvWords + (v >> 5)], bit = v & 31;
-                if ((w >> bit) & 1u) {
-                    const uint32_t row = key_base[k] + rank[(size_t)k * kInvWords + (v >> 5)] +
-                                         __popc(w & ((1u << bit) - 1u));
-                    rx.off[warp][lane][n++] = row * row_words;
-                } else if (op == PV_IN) {
-                    unknown = true;
-                }
-            }
-        } else if (op == PV_EXISTS || op == PV_DOESNOTEXIST) {
-            bad = nv != 0;
-            rx.off[warp][lane][n++] = (num_value_rows + k) * row_words;
-        } else {
-            bad = true;
-        }
-        rx.meta[warp][lane] = op | n << 8;
-    }
-    // Evaluation order (the AND of the expressions' sets does not depend on
-    // it): In expressions with the fewest carried values first, then
-    // DoesNotExist, Exists and NotIn, the sparsest sets first, so that a pod
-    // whose row empties early stops reading rows.  Ties keep list order.
-    uint32_t key = 0xFFFFFFFFu;
-    if (kOrder && lane < E) {
-        const uint32_t op = rx.meta[warp][lane] & 0xFFu, n = rx.meta[warp][lane] >> 8;
-        const uint32_t cls = op == PV_IN ? 0u : op == PV_DOESNOTEXIST ? 1u : op == PV_EXISTS ? 2u : 3u;
-        key = cls << 8 | n;
-    }
-    uint32_t place = 0;
-    for (uint32_t j = 0; kOrder && j < E; ++j) {
-        const uint32_t kj = __shfl_sync(PV_FULL_MASK, key, j);
-        place += (kj < key || (kj == key && j < lane)) ? 1u : 0u;
-    }
-    if (kOrder && lane < E) rx.order[warp][place] = (uint8_t)lane;
-    __syncwarp();
-    bad = __any_sync(PV_FULL_MASK, bad);
-    unknown = __any_sync(PV_FULL_MASK, unknown);
-    return (bad ? 1u : 0u) | (unknown ? 2u : 0u);
-}
-
-// The same resolution with one lane per (expression, value) slot: lanes
-// 0 .. E - 1 read their expression's header word, a warp scan lays the
-// slots out (an In or NotIn expression takes one slot per listed value,
-// any other one slot), and every slot's lane resolves its value's row in
-// one step.  For lists of at most 32 slots (returns bit2 and resolves
-// nothing when there are more).  Same results, flags and order as
-// resolve_exprs<true>.
-__device__ __forceinline__ uint32_t expr_header(const pv_expr *__restrict__ exprs, uint32_t lo, uint32_t lane) {
-    return __ldg(reinterpret_cast<const uint32_t *>(exprs + lo + lane));
-}
-
-__device__ __forceinline__ uint32_t resolve_slots(ResolvedExprs &rx, uint32_t warp, uint32_t lane, uint32_t lo,
-                                                  uint32_t E, const pv_expr *__restrict__ exprs, uint32_t K,
-                                                  const uint32_t *__restrict__ inv, const uint32_t *__restrict__ rank,
-                                                  const uint32_t *__restrict__ key_base, uint32_t num_value_rows,
-                                                  uint32_t row_words, uint32_t lane_hdr) {
-    // header word (expr_header, fetched by the caller): key (bits 0..15),
-    // op (16..23), nvals (24..31)
-    uint32_t hdr = 0, m = 0;
-    bool bad = false;
-    if (lane < E) {
-        hdr = lane_hdr;
-        const uint32_t k = hdr & 0xFFFFu, op = (hdr >> 16) & 0xFFu, nv = hdr >> 24;
-        const bool listed = op == PV_IN || op == PV_NOTIN;
-        bad = k >= K || (listed ? (nv < 1 || nv > 8) : (op == PV_EXISTS || op == PV_DOESNOTEXIST) ? nv != 0 : true);
-        m = (listed && !bad) ? nv : 1u;
-    }
-    uint32_t incl = m;   // slots of expressions 0 .. lane
-    for (int d = 1; d < 32; d <<= 1) {
-        const uint32_t y = __shfl_up_sync(PV_FULL_MASK, incl, d);
-        if (lane >= (uint32_t)d) incl += y;
-    }
-    const uint32_t T = __shfl_sync(PV_FULL_MASK, incl, 31);
-    if (T > 32) return 4u;
-    const uint32_t pre = incl - m;
-    const uint32_t starts = __reduce_or_sync(PV_FULL_MASK, lane < E ? 1u << pre : 0u);
-    // slot lane: expression e, value j
-    const uint32_t upto = lane == 31 ? ~0u : (2u << lane) - 1u;
-    const uint32_t e = lane < T ? (uint32_t)__popc(starts & upto) - 1u : 0u;
-    const uint32_t pre_e = __shfl_sync(PV_FULL_MASK, pre, e);
-    const uint32_t hdr_e = __shfl_sync(PV_FULL_MASK, hdr, e);
-    const uint32_t m_e = __shfl_sync(PV_FULL_MASK, m, e);
-    const bool bad_e = __shfl_sync(PV_FULL_MASK, bad ? 1u : 0u, e) != 0;
-    const uint32_t k = hdr_e & 0xFFFFu, op = (hdr_e >> 16) & 0xFFu;
-    bool carried = false, unknown = false;
-    uint32_t off = 0;
-    if (lane < T && !bad_e) {
-        if (op == PV_IN || op == PV_NOTIN) {
-            const uint32_t v = __ldg(&exprs[lo + e].vals[lane - pre_e]);
-            if (v == PV_ABSENT) {
-                bad = true;
-            } else {
-                const uint32_t w = __ldg(inv + (size_t)k * kInvWords + (v >> 5)), bit = v & 31;
-                carried = (w >> bit) & 1u;
-                if (carried)
-                    off = (__ldg(key_base + k) + __ldg(rank + (size_t)k * kInvWords + (v >> 5)) +
-                           __popc(w & ((1u << bit) - 1u))) * row_words;
-                else if (op == PV_IN)
-                    unknown = true;
-            }
-        } else {
-            carried = true;
-            off = (num_value_rows + k) * row_words;
-        }
-    }
-    // carried rows of each expression, packed in slot order
-    const uint32_t C = __ballot_sync(PV_FULL_MASK, carried);
-    const uint32_t below = (1u << lane) - 1u;
-    if (carried) rx.off[warp][e][__popc(C & below & ~((1u << pre_e) - 1u))] = off;
-    uint32_t key = 0xFFFFFFFFu;
-    if (lane < E) {
-        const uint32_t span = (m >= 32 ? ~0u : (1u << m) - 1u) << pre;
-        const uint32_t n = __popc(C & span), opl = (hdr >> 16) & 0xFFu;
-        rx.meta[warp][lane] = opl | n << 8;
-        const uint32_t cls = opl == PV_IN ? 0u : opl == PV_DOESNOTEXIST ? 1u : opl == PV_EXISTS ? 2u : 3u;
-        key = cls << 8 | n;
-    }
-    (void)m_e;
-    uint32_t place = 0;
-    for (uint32_t j = 0; j < E; ++j) {
-        const uint32_t kj = __shfl_sync(PV_FULL_MASK, key, j);
-        place += (kj < key || (kj == key && j < lane)) ? 1u : 0u;
-    }
-    if (lane < E) rx.order[warp][place] = (uint8_t)lane;
-    __syncwarp();
-    bad = __any_sync(PV_FULL_MASK, bad);
-    unknown = __any_sync(PV_FULL_MASK, unknown);
-    return (bad ? 1u : 0u) | (unknown ? 2u : 0u);
-}
-
-// ANDs resolved expression e's node set into a 160-word span's accumulators
-// of one lane: chunk q (four words, loaded when l0) and word w (loaded when
-// l1); words past the rows read 0 before the complement.
-__device__ __forceinline__ void and_resolved5(const ResolvedExprs &rx, uint32_t warp, uint32_t e,
-                                              const uint32_t *__restrict__ rows, uint32_t q, uint32_t w, bool l0,
-                                              bool l1, uint4 &a0, uint32_t &a1) {
-    const uint32_t meta = rx.meta[warp][e], op = meta & 0xFFu, n = meta >> 8;
-    uint4 v0 = make_uint4(0, 0, 0, 0);
-    uint32_t v1 = 0;
-    uint32_t j = 0;
-    for (; j + 1 < n; j += 2) {   // two rows per step: four loads in flight
-        const uint32_t *rp = rows + rx.off[warp][e][j], *rq = rows + rx.off[warp][e][j + 1];
-        uint4 x0 = make_uint4(0, 0, 0, 0), y0 = x0;
-        uint32_t x1 = 0, y1 = 0;
-        if (l0) {
-            x0 = __ldg(reinterpret_cast<const uint4 *>(rp) + q);
-            y0 = __ldg(reinterpret_cast<const uint4 *>(rq) + q);
-        }
-        if (l1) {
-            x1 = __ldg(rp + w);
-            y1 = __ldg(rq + w);
-        }
-        v0.x |= x0.x | y0.x; v0.y |= x0.y | y0.y; v0.z |= x0.z | y0.z; v0.w |= x0.w | y0.w;
-        v1 |= x1 | y1;
-    }
-    if (j < n) {
-        const uint32_t *rp = rows + rx.off[warp][e][j];
-        if (l0) {
-            const uint4 x = __ldg(reinterpret_cast<const uint4 *>(rp) + q);
-            v0.x |= x.x; v0.y |= x.y; v0.z |= x.z; v0.w |= x.w;
-        }
-        if (l1) v1 |= __ldg(rp + w);
-    }
-    if (op == PV_NOTIN || op == PV_DOESNOTEXIST) {
-        a0.x &= ~v0.x; a0.y &= ~v0.y; a0.z &= ~v0.z; a0.w &= ~v0.w;
-        a1 &= ~v1;
+        for (int i = 0; i < 5; ++i) w[i] = __ldg(reinterpret_cast<const uint32_t *>(x) + i);
     } else {
-        a0.x &= v0.x; a0.y &= v0.y; a0.z &= v0.z; a0.w &= v0.w;
-        a1 &= v1;
+        const uint16_t *h = reinterpret_cast<const uint16_t *>(x);
+#pragma unroll
+        for (int i = 0; i < 5; ++i) w[i] = (uint32_t)__ldg(h + 2 * i) | (uint32_t)__ldg(h + 2 * i + 1) << 16;
+    }
+    const uint32_t k = w[0] & 0xFFFFu, op = (w[0] >> 16) & 0xFFu, nv = w[0] >> 24;
+    const bool listed = op == PV_IN || op == PV_NOTIN;
+    r.op = op;
+    r.bad = k >= K || (listed ? nv < 1 || nv > 8 : (op == PV_EXISTS || op == PV_DOESNOTEXIST) ? nv != 0 : true);
+    r.unknown = false;
+    r.carried = 0;
+    if (r.bad) return;
+    if (!listed) {
+        r.off[0] = (num_value_rows + k) * row_bytes;
+        r.carried = 1;
+        return;
+    }
+    uint2 e[8];   // the values' inventory words, all in flight
+#pragma unroll
+    for (uint32_t j = 0; j < 8; ++j) {
+        const uint32_t v = (w[1 + j / 2] >> (16 * (j & 1))) & 0xFFFFu;
+        e[j] = j < nv ? __ldg(ranked + (size_t)k * kInvWords + (v >> 5)) : make_uint2(0, 0);
+    }
+    const uint32_t base = __ldg(key_base + k);
+#pragma unroll
+    for (uint32_t j = 0; j < 8; ++j) {
+        const uint32_t v = (w[1 + j / 2] >> (16 * (j & 1))) & 0xFFFFu, bit = v & 31;
+        const bool used = j < nv, has = used && ((e[j].x >> bit) & 1u);
+        r.bad = r.bad || (used && v == PV_ABSENT);
+        r.unknown = r.unknown || (used && !has && op == PV_IN);
+        r.carried |= has ? 1u << j : 0u;
+        r.off[j] = (base + e[j].y + __popc(e[j].x & ((1u << bit) - 1u))) * row_bytes;
     }
 }
 
@@ -552,220 +422,352 @@ __device__ __forceinline__ void clip_rows4(uint4 &acc, uint32_t w0, uint32_t N) 
     }
 }
 
-__global__ void __launch_bounds__(kRowsThreads) sel_rows_kernel(
-    uint32_t N, uint32_t K, uint32_t P, const uint32_t *__restrict__ offs, uint32_t num_exprs,
-    const pv_expr *__restrict__ exprs, const uint32_t *__restrict__ assign, uint32_t *__restrict__ bits,
-    uint32_t W, uint8_t *__restrict__ flags, const uint32_t *__restrict__ inv, const uint32_t *__restrict__ rank,
-    const uint32_t *__restrict__ key_base, const uint32_t *__restrict__ rows, uint32_t row_words,
-    uint32_t num_value_rows, const uint32_t *__restrict__ pod_list, const uint32_t *__restrict__ list_len) {
-    __shared__ ResolvedExprs rx;
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t gw = (blockIdx.x * kRowsThreads + threadIdx.x) >> 5;
-    const uint32_t nw = (gridDim.x * kRowsThreads) >> 5;
-    const uint32_t n = pod_list ? *list_len : P;   // with a list: only the pods it names
-    // The next pod's offsets are loaded while this pod is resolved, and its
-    // expression headers while this pod's rows are swept, so a pod's chain
-    // of dependent loads starts at its values.
-    auto pod_at = [&](uint32_t i) { return pod_list ? pod_list[i] : i; };
-    auto headed = [&](uint32_t lo, uint32_t hi) { return hi >= lo && hi <= num_exprs && hi - lo <= 32; };
-    uint32_t p = 0, lo = 0, hi = 0, hdr = 0;
-    if (gw < n) {
-        p = pod_at(gw);
-        lo = offs[p];
-        hi = offs[p + 1];
-        hdr = headed(lo, hi) && lane < hi - lo ? expr_header(exprs, lo, lane) : 0u;
-    }
-    for (uint32_t i = gw; i < n; i += nw) {
-        uint32_t np = 0, nlo = 0, nhi = 0;
-        if (i + nw < n) {
-            np = pod_at(i + nw);
-            nlo = offs[np];
-            nhi = offs[np + 1];
-        }
-        const uint32_t a = assign ? assign[p] : PV_UNPLACED;
-        const uint32_t E = hi - lo;
-        const bool resolved = headed(lo, hi);
-        uint32_t pre = resolved ? resolve_slots(rx, warp, lane, lo, E, exprs, K, inv, rank, key_base, num_value_rows,
-                                                row_words, hdr)
-                                : pod_prescan(lo, hi, num_exprs, exprs, K, inv, lane);
-        if (resolved && (pre & 4u))   // more than 32 slots: one lane per expression
-            pre = resolve_exprs<true>(rx, warp, lane, lo, E, exprs, K, inv, rank, key_base, num_value_rows,
-                                      row_words);
-        const uint32_t nhdr = i + nw < n && headed(nlo, nhi) && lane < nhi - nlo ? expr_header(exprs, nlo, lane) : 0u;
-        uint4 *out = reinterpret_cast<uint4 *>(bits + (size_t)p * W);
-        const uint32_t pc = p, lc = lo;   // this pod (the names below move on to the next one)
-        p = np;
-        lo = nlo;
-        hi = nhi;
-        hdr = nhdr;
-        if (pre & 1u) {
-            for (uint32_t q = lane; q < W / 4; q += 32) out[q] = make_uint4(0, 0, 0, 0);
-            if (lane == 0) flags[pc] = PV_F_BAD_EXPR;
-            continue;
-        }
-        bool any = false, aok = false;
-        auto finish = [&](uint4 acc, uint32_t q) {
-            const uint32_t w0 = q * 4;
-            if (w0 + 4 > (N >> 5)) clip_rows4(acc, w0, N);   // only chunks reaching node N - 1 or past it
-            out[q] = acc;
-            any = any || (acc.x | acc.y | acc.z | acc.w) != 0;
-            if (a < N && (a >> 7) == q) {   // the assigned node's word is in this chunk
-                const uint32_t wsel = (a >> 5) & 3u;
-                const uint32_t word = wsel == 0 ? acc.x : wsel == 1 ? acc.y : wsel == 2 ? acc.z : acc.w;
-                aok = (word >> (a & 31)) & 1u;
-            }
-        };
-        if (resolved) {
-            // of each 160-word span a lane takes chunk lane (words 4 lane ..
-            // 4 lane + 3) and word 128 + lane: five words per lane, so a row
-            // of up to 5,120 nodes keeps every lane busy in one pass over the
-            // resolved rows
-            for (uint32_t sb = 0; sb < W; sb += 160) {
-                const uint32_t q = sb / 4 + lane, w = sb + 128 + lane;
-                const bool h0 = q * 4 < W, h1 = w < W;
-                const bool l0 = h0 && q * 4 < row_words, l1 = h1 && w < row_words;
-                uint4 a0 = make_uint4(~0u, ~0u, ~0u, ~0u);
-                uint32_t a1 = ~0u;
-                for (uint32_t i = 0; i < E; ++i) {
-                    and_resolved5(rx, warp, rx.order[warp][i], rows, q, w, l0, l1, a0, a1);
-                    // every node of the span rejected: the remaining sets
-                    // cannot add any back (words past the rows hold no nodes)
-                    const bool nz = (l0 && (a0.x | a0.y | a0.z | a0.w)) || (l1 && a1);
-                    if (!__any_sync(PV_FULL_MASK, nz)) {
-                        a0 = make_uint4(0, 0, 0, 0);
-                        a1 = 0;
-                        break;
-                    }
-                }
-                if (h0) finish(a0, q);
-                if (h1) {
-                    const uint32_t full_words = N >> 5, tail_bits = N & 31;
-                    if (w > full_words || (w == full_words && tail_bits == 0)) a1 = 0;
-                    else if (w == full_words) a1 &= (1u << tail_bits) - 1u;
-                    bits[(size_t)pc * W + w] = a1;
-                    any = any || a1 != 0;
-                    if (a < N && (a >> 5) == w) aok = (a1 >> (a & 31)) & 1u;
-                }
-            }
-        } else {
-            for (uint32_t q = lane; q < W / 4; q += 32) {
-                const uint32_t w0 = q * 4;
-                uint4 acc = make_uint4(~0u, ~0u, ~0u, ~0u);
-                const bool in_rows = w0 < row_words;
-                for (uint32_t e = 0; e < E; ++e) {
-                    const uint4 r = expr_rows4(exprs[lc + e], w0, in_rows, inv, rank, key_base, rows, row_words,
-                                               num_value_rows);
-                    acc.x &= r.x; acc.y &= r.y; acc.z &= r.z; acc.w &= r.w;
-                }
-                finish(acc, q);
-            }
-        }
-        any = __any_sync(PV_FULL_MASK, any);   // also keeps the warp's resolved rows until all lanes are done
-        aok = __any_sync(PV_FULL_MASK, aok);
-        if (lane == 0) flags[pc] = pod_flags(any, pre & 2u, assign != nullptr, aok);
-    }
+struct SelArgs {
+    uint32_t N, K, P;
+    const uint32_t *offs;        // pod -> expressions (or terms)
+    const uint32_t *term_offs;   // term -> expressions (multi-term form)
+    uint32_t num_terms, num_exprs;
+    const pv_expr *exprs;
+    const uint32_t *assign;
+    uint32_t *bits;
+    uint32_t W;
+    uint8_t *flags;
+    const uint32_t *inv;
+    const uint2 *ranked;
+    const uint32_t *key_base, *rows;
+    uint32_t row_words, num_value_rows, zero_row;   // zero_row: byte offset of the row of no node
+    const uint32_t *pod_list, *list_len;   // with a list: only the pods it names
+};
+
+// A lane's share of the 160-word span from word sb: byte offsets of its chunk
+// and its word within a row, and the bits of theirs that are nodes (a lane past
+// the rows reads a word of theirs and keeps nothing).
+struct RowSpan {
+    uint4 m0;
+    uint32_t m1, b0, b1;
+};
+__device__ __forceinline__ RowSpan row_span(uint32_t sb, uint32_t lane, uint32_t N, uint32_t W, uint32_t row_words) {
+    const uint32_t q = sb / 4 + lane, w = sb + 128 + lane;
+    const bool in0 = q * 4 < row_words && q * 4 < W, in1 = w < row_words && w < W;
+    RowSpan s;
+    s.b0 = in0 ? q * 16 : 0u;
+    s.b1 = in1 ? w * 4 : 0u;
+    s.m0 = in0 ? make_uint4(~0u, ~0u, ~0u, ~0u) : make_uint4(0, 0, 0, 0);
+    if (in0 && q * 4 + 4 > N >> 5) clip_rows4(s.m0, q * 4, N);
+    s.m1 = !in1 || w > N >> 5 ? 0u : w == N >> 5 ? (1u << (N & 31)) - 1u : ~0u;
+    return s;
 }
 
-// Multi-term selectors (Kubernetes required node affinity): a pod's row is
-// the OR over its terms of the AND over each term's expressions.  A pod
-// without terms admits every node; a term without expressions matches none.
-// Warp per pod; every term's list is validated and scanned for values no
-// node carries, as in sel_rows_kernel.
-__global__ void __launch_bounds__(kRowsThreads) sel_terms_kernel(
-    uint32_t N, uint32_t K, uint32_t P, const uint32_t *__restrict__ pod_terms, uint32_t num_terms,
-    const uint32_t *__restrict__ term_offs, uint32_t num_exprs, const pv_expr *__restrict__ exprs,
-    const uint32_t *__restrict__ assign, uint32_t *__restrict__ bits, uint32_t W, uint8_t *__restrict__ flags,
-    const uint32_t *__restrict__ inv, const uint32_t *__restrict__ rank, const uint32_t *__restrict__ key_base,
-    const uint32_t *__restrict__ rows, uint32_t row_words, uint32_t num_value_rows) {
-    __shared__ ResolvedExprs rx;
-    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const uint32_t gw = (blockIdx.x * kRowsThreads + threadIdx.x) >> 5;
-    const uint32_t nw = (gridDim.x * kRowsThreads) >> 5;
-    for (uint32_t p = gw; p < P; p += nw) {
-        const uint32_t t0 = pod_terms[p], t1 = pod_terms[p + 1];
-        uint32_t pre = (t1 < t0 || t1 > num_terms) ? 1u : 0u;
-        // the terms' expressions form one range; lists of at most 32 are resolved once
-        uint32_t e0 = 0, E = 0;
-        bool resolved = false;
-        if (!(pre & 1u) && t1 > t0) {
-            e0 = term_offs[t0];
-            const uint32_t e1 = term_offs[t1];
-            bool mono = e1 >= e0;
-            for (uint32_t t = t0; t < t1 && mono; ++t) mono = term_offs[t + 1] >= term_offs[t];
-            resolved = mono && e1 <= num_exprs && e1 - e0 <= 32;
-            E = resolved ? e1 - e0 : 0u;
-        }
-        if (resolved)
-            pre |= resolve_exprs<false>(rx, warp, lane, e0, E, exprs, K, inv, rank, key_base, num_value_rows, row_words);
-        else
-            for (uint32_t t = t0; t < t1 && !(pre & 1u); ++t)
-                pre |= pod_prescan(term_offs[t], term_offs[t + 1], num_exprs, exprs, K, inv, lane);
-        uint4 *out = reinterpret_cast<uint4 *>(bits + (size_t)p * W);
-        if (pre & 1u) {
-            for (uint32_t q = lane; q < W / 4; q += 32) out[q] = make_uint4(0, 0, 0, 0);
-            if (lane == 0) flags[p] = PV_F_BAD_EXPR;
-            continue;
-        }
-        const uint32_t a = assign ? assign[p] : PV_UNPLACED;
-        bool any = false, aok = false;
-        auto finish = [&](uint4 res, uint32_t q) {
-            const uint32_t w0 = q * 4;
-            if (w0 + 4 > (N >> 5)) clip_rows4(res, w0, N);   // only chunks reaching node N - 1 or past it
-            out[q] = res;
-            any = any || (res.x | res.y | res.z | res.w) != 0;
-            if (a < N && (a >> 7) == q) {   // the assigned node's word is in this chunk
-                const uint32_t wsel = (a >> 5) & 3u;
-                const uint32_t word = wsel == 0 ? res.x : wsel == 1 ? res.y : wsel == 2 ? res.z : res.w;
-                aok = (word >> (a & 31)) & 1u;
+// A pod with a malformed list, a bad expression or more than 32 of them:
+// validated and scanned for unknown values, then evaluated expression by
+// expression for every four words.  (After a warp's other pods, so that its
+// code costs them no registers; kPodLeft in the flags marks it until then.)
+constexpr uint8_t kPodLeft = 0x80;
+template <bool kTerms>
+__device__ __noinline__ void unresolved_pod(const SelArgs &g, uint32_t p, uint32_t lane) {
+    const uint32_t o0 = g.offs[p], o1 = g.offs[p + 1], W = g.W, N = g.N, a = g.assign ? g.assign[p] : PV_UNPLACED;
+    uint32_t pre;
+    if (!kTerms) {
+        pre = pod_prescan(o0, o1, g.num_exprs, g.exprs, g.K, g.inv, lane);
+    } else {
+        pre = o1 < o0 || o1 > g.num_terms ? 1u : 0u;
+        for (uint32_t k = o0; k < o1 && !(pre & 1u); ++k)
+            pre |= pod_prescan(g.term_offs[k], g.term_offs[k + 1], g.num_exprs, g.exprs, g.K, g.inv, lane);
+    }
+    const uint4 none = make_uint4(0, 0, 0, 0), all = make_uint4(~0u, ~0u, ~0u, ~0u);
+    uint4 *out = reinterpret_cast<uint4 *>(g.bits + (size_t)p * W);
+    bool any = false, aok = false;
+    for (uint32_t q = lane; q < W / 4; q += 32) {
+        const uint32_t w0 = q * 4;
+        const bool in_rows = w0 < g.row_words;
+        auto conj = [&](uint32_t first, uint32_t past) {
+            uint4 acc = all;
+            for (uint32_t k = first; k < past; ++k) {
+                const uint4 y = expr_rows4(g.exprs[k], w0, in_rows, g.ranked, g.key_base, g.rows, g.row_words,
+                                           g.num_value_rows);
+                acc.x &= y.x; acc.y &= y.y; acc.z &= y.z; acc.w &= y.w;
             }
+            return acc;
         };
-        const uint4 none = make_uint4(0, 0, 0, 0), all = make_uint4(~0u, ~0u, ~0u, ~0u);
-        if (resolved) {   // a 160-word span per pass, five words per lane, as in sel_rows_kernel
-            for (uint32_t sb = 0; sb < W; sb += 160) {
-                const uint32_t q = sb / 4 + lane, w = sb + 128 + lane;
-                const bool h0 = q * 4 < W, h1 = w < W;
-                const bool l0 = h0 && q * 4 < row_words, l1 = h1 && w < row_words;
-                uint4 r0 = t0 == t1 ? all : none;
-                uint32_t r1 = t0 == t1 ? ~0u : 0u;
-                for (uint32_t t = t0; t < t1; ++t) {
-                    const uint32_t lo = term_offs[t] - e0, hi = term_offs[t + 1] - e0;
-                    uint4 a0 = hi > lo ? all : none;
-                    uint32_t a1 = hi > lo ? ~0u : 0u;
-                    for (uint32_t e = lo; e < hi; ++e) and_resolved5(rx, warp, e, rows, q, w, l0, l1, a0, a1);
-                    r0.x |= a0.x; r0.y |= a0.y; r0.z |= a0.z; r0.w |= a0.w;
-                    r1 |= a1;
-                }
-                if (h0) finish(r0, q);
-                if (h1) {
-                    const uint32_t full_words = N >> 5, tail_bits = N & 31;
-                    if (w > full_words || (w == full_words && tail_bits == 0)) r1 = 0;
-                    else if (w == full_words) r1 &= (1u << tail_bits) - 1u;
-                    bits[(size_t)p * W + w] = r1;
-                    any = any || r1 != 0;
-                    if (a < N && (a >> 5) == w) aok = (r1 >> (a & 31)) & 1u;
-                }
-            }
-        } else {
-            for (uint32_t q = lane; q < W / 4; q += 32) {
-                const uint32_t w0 = q * 4;
-                const bool in_rows = w0 < row_words;
-                uint4 res = t0 == t1 ? all : none;
-                for (uint32_t t = t0; t < t1; ++t) {
-                    const uint32_t lo = term_offs[t], hi = term_offs[t + 1];
-                    uint4 acc = hi > lo ? all : none;
-                    for (uint32_t e = lo; e < hi; ++e) {
-                        const uint4 r = expr_rows4(exprs[e], w0, in_rows, inv, rank, key_base, rows, row_words,
-                                                   num_value_rows);
-                        acc.x &= r.x; acc.y &= r.y; acc.z &= r.z; acc.w &= r.w;
-                    }
-                    res.x |= acc.x; res.y |= acc.y; res.z |= acc.z; res.w |= acc.w;
-                }
-                finish(res, q);
+        uint4 res = pre & 1u ? none : all;
+        if (pre & 1u) {   // an empty row
+        } else if (!kTerms) {
+            res = conj(o0, o1);
+        } else if (o1 > o0) {
+            res = none;
+            for (uint32_t k = o0; k < o1; ++k) {
+                const uint32_t first = g.term_offs[k], past = g.term_offs[k + 1];
+                const uint4 acc = past > first ? conj(first, past) : none;
+                res.x |= acc.x; res.y |= acc.y; res.z |= acc.z; res.w |= acc.w;
             }
         }
-        any = __any_sync(PV_FULL_MASK, any);
-        aok = __any_sync(PV_FULL_MASK, aok);
-        if (lane == 0) flags[p] = pod_flags(any, pre & 2u, assign != nullptr, aok);
+        if (w0 + 4 > N >> 5) clip_rows4(res, w0, N);   // only chunks reaching node N - 1 or past it
+        out[q] = res;
+        any = any || (res.x | res.y | res.z | res.w) != 0;
+        if (a < N && a >> 7 == q) {
+            const uint32_t i = (a >> 5) & 3u, word = i == 0 ? res.x : i == 1 ? res.y : i == 2 ? res.z : res.w;
+            aok = (word >> (a & 31)) & 1u;
+        }
+    }
+    any = __any_sync(PV_FULL_MASK, any);
+    aok = __any_sync(PV_FULL_MASK, aok);
+    if (lane == 0)
+        g.flags[p] = pre & 1u ? (uint8_t)PV_F_BAD_EXPR : pod_flags(any, pre & 2u, g.assign != nullptr, aok);
+}
+
+// A pod's row is the AND over its expressions, or, with kTerms (Kubernetes
+// required node affinity), the OR over its terms of the AND over each term's
+// expressions: a pod without terms admits every node, a term without
+// expressions matches none.  The AND does not depend on the order: In
+// expressions with the fewest carried values first, then DoesNotExist, Exists
+// and NotIn, the sparsest sets first, so that a pod whose row empties early
+// stops reading rows.
+// kOneSpan: rows of at most 160 words (5,120 nodes), one pass over a pod's
+// entries.
+// What bounds it: instruction issue with many pods (about two thirds of the
+// slots at 100,000 pods, the rows coming from L2), with few the chain offsets
+// -> expressions -> inventory -> rows of one pod.  On 5,000 nodes against a
+// warp per pod that resolved one pod at a time and loaded two rows ahead:
+// 100,000 pods 99.5 -> 69.3 us, 10,000 19.0 -> 15.6, 777 11.6 -> 10.0; in the
+// term form 129.6 -> 96.9, 22.1 -> 18.9 and 14.0 -> 11.1 (6,000 pods, where some
+// warps have two and that kernel had room for a warp each: 17.2 -> 18.6).
+template <bool kTerms, bool kOneSpan>
+__global__ void __launch_bounds__(kRowsThreads<kTerms>, 768 / kRowsThreads<kTerms>)
+    sel_rows_kernel(const __grid_constant__ SelArgs g) {
+    constexpr int kWarps = kRowsThreads<kTerms> / 32;
+    __shared__ uint32_t s_list[kWarps][kListWords];
+    __shared__ uint4 s_pod[kWarps][32];
+    __shared__ uint32_t s_word[kWarps][32];   // the word of each pod's row that holds its assigned node
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, N = g.N, W = g.W;
+    uint32_t *list = s_list[warp];
+    const uint32_t total = g.pod_list ? *g.list_len : g.P;
+    const uint32_t gw = blockIdx.x * kWarps + warp, nw = gridDim.x * kWarps;
+    const uint32_t end = (uint32_t)(((uint64_t)total * (gw + 1)) / nw);
+    uint32_t take = 0;
+    RowSpan sp = row_span(0, lane, N, W, g.row_words);
+    const uint32_t begin = (uint32_t)(((uint64_t)total * gw) / nw);
+    bool left_over = false;
+    for (uint32_t at = begin; at < end; at += take) {
+        // lane i: pod at + i, its expressions [lo, lo + cnt); a pod with a
+        // malformed list or more than 32 takes no slots and is evaluated
+        // unresolved
+        uint32_t p = 0, o0 = 0, o1 = 0, lo = 0, cnt = 0, a = PV_UNPLACED;
+        uint32_t t1 = 0, t2 = 0, t3 = 0;   // kTerms: ends of the first three terms
+        bool slow = false;
+        if (at + lane < end) {
+            p = g.pod_list ? g.pod_list[at + lane] : at + lane;
+            o0 = lo = g.offs[p];
+            o1 = g.offs[p + 1];
+            if (g.assign) a = g.assign[p];
+            uint32_t hi = o1;
+            slow = o1 < o0 || o1 > (kTerms ? g.num_terms : g.num_exprs);
+            if (kTerms) {
+                // the terms' expressions form one range when their offsets do not decrease
+                lo = hi = 0;
+                if (o1 > o0 && !slow) {
+                    // up to four terms' ends in flight (the last one's repeated)
+                    const uint32_t last = o1;
+                    lo = g.term_offs[o0];
+                    t1 = g.term_offs[o0 + 1];
+                    t2 = g.term_offs[min(o0 + 2, last)];
+                    t3 = g.term_offs[min(o0 + 3, last)];
+                    hi = g.term_offs[min(o0 + 4, last)];
+                    slow = t1 < lo || t2 < t1 || t3 < t2 || hi < t3;
+                    for (uint32_t k = o0 + 4; k < o1 && !slow; ++k) {
+                        const uint32_t x = g.term_offs[k + 1];
+                        slow = x < hi;
+                        hi = x;
+                    }
+                    slow = slow || hi > g.num_exprs;
+                }
+            }
+            slow = slow || hi - lo > 32;
+            cnt = slow ? 0u : hi - lo;
+        }
+        uint32_t incl = cnt;
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(PV_FULL_MASK, incl, d);
+            if (lane >= (uint32_t)d) incl += y;
+        }
+        const uint32_t fit = __ballot_sync(PV_FULL_MASK, at + lane < end && incl <= 32);   // leading lanes, the first always
+        take = fit == PV_FULL_MASK ? 32u : (uint32_t)__ffs(~fit) - 1u;
+        const uint32_t slots = __shfl_sync(PV_FULL_MASK, incl, take - 1), excl = incl - cnt;
+        // lane t: expression t of the group, of pod `pod`
+        uint32_t pod = 0;   // the first whose expressions end past t
+#pragma unroll
+        for (uint32_t step = 16; step; step >>= 1)
+            if (__shfl_sync(PV_FULL_MASK, incl, pod + step - 1) <= lane) pod += step;
+        pod = min(pod, 31u);   // lanes past the slots: unused
+        const uint32_t f = __shfl_sync(PV_FULL_MASK, excl, pod), c = __shfl_sync(PV_FULL_MASK, cnt, pod);
+        const uint32_t e = __shfl_sync(PV_FULL_MASK, lo, pod) + lane - f;
+        uint32_t term = 0;   // e's term among the pod's
+        if (kTerms) {
+            const uint32_t tm0 = __shfl_sync(PV_FULL_MASK, o0, pod), tm1 = __shfl_sync(PV_FULL_MASK, o1, pod);
+            term = (e >= __shfl_sync(PV_FULL_MASK, t1, pod) ? 1u : 0u) + (e >= __shfl_sync(PV_FULL_MASK, t2, pod) ? 1u : 0u) +
+                   (e >= __shfl_sync(PV_FULL_MASK, t3, pod) ? 1u : 0u);
+            if (lane < slots && tm1 - tm0 > 4 && term == 3)
+                while (g.term_offs[tm0 + term + 1] <= e) ++term;
+        }
+        LaneExpr r;
+        r.carried = 0;
+        r.op = 0;
+        r.bad = r.unknown = false;
+        uint32_t key = 0, n = 0;
+        if (lane < slots) {
+            resolve_expr(r, g.exprs + e, g.K, g.ranked, g.key_base, g.num_value_rows, g.row_words * 4);
+            const uint32_t cls = r.op == PV_IN ? 0u : r.op == PV_DOESNOTEXIST ? 1u : r.op == PV_EXISTS ? 2u : 3u;
+            const uint32_t rows = __popc(r.carried);
+            n = max(rows, 1u);   // (no value carried: the row of no node)
+            key = term << 6 | cls << 4 | rows;
+        }
+        const uint32_t bad = __ballot_sync(PV_FULL_MASK, r.bad), unknown = __ballot_sync(PV_FULL_MASK, r.unknown);
+        // the list: pods in order, each one's expressions in evaluation order
+        uint32_t ni = n;
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t y = __shfl_up_sync(PV_FULL_MASK, ni, d);
+            if (lane >= (uint32_t)d) ni += y;
+        }
+        uint32_t pos = __shfl_sync(PV_FULL_MASK, ni - n, f & 31u);   // the pod's first word
+        bool term_end = true;
+        const uint32_t most = __reduce_max_sync(PV_FULL_MASK, lane < slots ? c : 0u);
+        for (uint32_t j = 0; j < most; ++j) {
+            const uint32_t y = (f + j) & 31u, ky = __shfl_sync(PV_FULL_MASK, key, y), ny = __shfl_sync(PV_FULL_MASK, n, y);
+            if (j < c && y != lane) {
+                const bool before = ky < key || (ky == key && y < lane);
+                if (before) pos += ny;
+                else if (kTerms && ky >> 6 == term) term_end = false;
+            }
+        }
+        if (lane < slots) {
+            const uint32_t fl = r.op == PV_NOTIN || r.op == PV_DOESNOTEXIST ? kRowNot : 0u;
+            const uint32_t last = kRowLast | (kTerms && term_end ? kRowTerm : 0u);
+            if (r.carried == 0) list[pos] = g.zero_row | fl | last;
+#pragma unroll
+            for (uint32_t j = 0; j < 8; ++j)
+                if ((r.carried >> j) & 1u) list[pos++] = r.off[j] | fl | (r.carried >> j == 1u ? last : 0u);
+        }
+        // lane i: pod i {index, words first | past << 16, assigned node, it has terms}
+        const uint32_t ent0 = __shfl_sync(PV_FULL_MASK, ni - n, excl & 31u);
+        const uint32_t ent1 = __shfl_sync(PV_FULL_MASK, ni, (incl - 1u) & 31u);
+        const uint32_t span = cnt >= 32 ? PV_FULL_MASK : ((1u << cnt) - 1u) << (excl & 31u);
+        uint32_t pre = (cnt && (bad & span) ? 1u : 0u) | (cnt && (unknown & span) ? 2u : 0u);
+        s_pod[warp][lane] = make_uint4(p, cnt ? ent0 | ent1 << 16 : 0u, a, o1 > o0 ? 1u : 0u);
+        s_word[warp][lane] = 0;
+        const uint32_t group = take == 32 ? PV_FULL_MASK : (1u << take) - 1u;
+        const uint32_t plain = __ballot_sync(PV_FULL_MASK, !slow && !(pre & 1u)) & group;
+        uint32_t feasible = 0;   // pods with a feasible node
+        __syncwarp();
+        for (uint32_t todo = plain; todo; todo &= todo - 1u) {
+            const uint32_t i = (uint32_t)__ffs(todo) - 1u;
+            const uint4 pod = s_pod[warp][i];
+            uint32_t *row = g.bits + (size_t)pod.x * W;
+            bool any = false;
+            // of each 160-word span a lane takes chunk lane (words 4 lane ..
+            // 4 lane + 3) and word 128 + lane: five words per lane, so a row of
+            // up to 5,120 nodes keeps every lane busy in one pass
+            for (uint32_t sb = 0; kOneSpan ? sb == 0 : sb < W; sb += 160) {
+                if (!kOneSpan) sp = row_span(sb, lane, N, W, g.row_words);
+                uint4 a0 = sp.m0;   // the AND of the expressions, from the words' nodes
+                uint32_t a1 = sp.m1;
+                uint4 r0 = a0;      // kTerms: the OR of the terms; no terms: every node
+                uint32_t r1 = a1;
+                if (kTerms && pod.w) {
+                    r0 = make_uint4(0, 0, 0, 0);
+                    r1 = 0;
+                }
+                bool left = true;   // some node of the span is left
+                const uint8_t *rb = reinterpret_cast<const uint8_t *>(g.rows);
+                uint32_t x = pod.y & 0xFFFFu;
+                const uint32_t x1 = pod.y >> 16;
+                // rows are loaded kAhead entries ahead, across expressions
+                uint4 n0[kAhead];
+                uint32_t n1[kAhead];
+                auto load = [&](int s, uint32_t at) {
+                    if (at < x1) {
+                        const uint32_t off = list[at] & ~15u;
+                        n0[s] = __ldg(reinterpret_cast<const uint4 *>(rb + (size_t)(off + sp.b0)));
+                        n1[s] = __ldg(reinterpret_cast<const uint32_t *>(rb + (size_t)(off + sp.b1)));
+                    }
+                };
+                while (x < x1) {
+#pragma unroll
+                    for (int s = 0; s < kAhead; ++s) {
+                        n0[s] = make_uint4(0, 0, 0, 0);
+                        n1[s] = 0;
+                        load(s, x + s);
+                    }
+                    uint4 v0 = make_uint4(0, 0, 0, 0);   // the OR of the expression's rows
+                    uint32_t v1 = 0;
+                    bool on = true;
+                    while (on) {
+#pragma unroll
+                        for (int s = 0; s < kAhead; ++s) {
+                            const uint32_t ent = list[x];
+                            v0.x |= n0[s].x; v0.y |= n0[s].y; v0.z |= n0[s].z; v0.w |= n0[s].w;
+                            v1 |= n1[s];
+                            load(s, x + kAhead);
+                            ++x;
+                            if (!(ent & kRowLast)) continue;
+                            const uint32_t inv = ent & kRowNot ? ~0u : 0u;
+                            a0.x &= v0.x ^ inv; a0.y &= v0.y ^ inv; a0.z &= v0.z ^ inv; a0.w &= v0.w ^ inv;
+                            a1 &= v1 ^ inv;
+                            v0 = make_uint4(0, 0, 0, 0);
+                            v1 = 0;
+                            left = __any_sync(PV_FULL_MASK, (a0.x | a0.y | a0.z | a0.w | a1) != 0);
+                            on = x < x1;
+                            if (!kTerms) {
+                                if (!left) x = x1;
+                                on = on && left;
+                            } else if (!left || (ent & kRowTerm)) {
+                                r0.x |= a0.x; r0.y |= a0.y; r0.z |= a0.z; r0.w |= a0.w;
+                                r1 |= a1;
+                                a0 = sp.m0;
+                                a1 = sp.m1;
+                                if (!(ent & kRowTerm)) {
+                                    // no node is left and the term's other sets cannot add
+                                    // one back: the next term comes first
+                                    while (!(list[x++] & kRowTerm)) {}
+                                    on = false;
+                                }
+                            }
+                            if (!on) break;
+                        }
+                    }
+                }
+                if (kTerms) {
+                    left = __any_sync(PV_FULL_MASK, (r0.x | r0.y | r0.z | r0.w | r1) != 0);
+                } else {
+                    r0 = a0;
+                    r1 = a1;
+                }
+                any = any || left;
+                const uint32_t q = sb / 4 + lane, w = sb + 128 + lane;
+                if (q * 4 < W) reinterpret_cast<uint4 *>(row)[q] = r0;
+                if (w < W) row[w] = r1;
+                const uint32_t at_word = (pod.z >> 5) - sb;   // of the assigned node, in the span
+                if (at_word < 160 && lane == (at_word < 128 ? at_word >> 2 : at_word - 128))
+                    s_word[warp][i] = at_word >= 128 ? r1
+                                      : at_word & 2u ? (at_word & 1u ? r0.w : r0.z) : (at_word & 1u ? r0.y : r0.x);
+            }
+            if (any) feasible |= 1u << i;
+        }
+        // lane i: pod i's flags.  Malformed lists, bad expressions and lists
+        // without slots are left to the pass below.
+        __syncwarp();
+        if (lane < take) {
+            const bool aok = a < N && ((s_word[warp][lane] >> (a & 31)) & 1u);
+            g.flags[p] = (plain >> lane) & 1u ? pod_flags((feasible >> lane) & 1u, pre & 2u, g.assign != nullptr, aok)
+                                              : kPodLeft;
+        }
+        left_over = left_over || plain != group;
+        __syncwarp();   // the list is rebuilt for the next pods
+    }
+    if (!left_over) return;
+    for (uint32_t at = begin; at < end; at += 32) {
+        const uint32_t pl = at + lane < end ? (g.pod_list ? g.pod_list[at + lane] : at + lane) : 0u;
+        const bool mine = at + lane < end && *(volatile uint8_t *)(g.flags + pl) == kPodLeft;
+        for (uint32_t todo = __ballot_sync(PV_FULL_MASK, mine); todo; todo &= todo - 1u)
+            unresolved_pod<kTerms>(g, __shfl_sync(PV_FULL_MASK, pl, __ffs(todo) - 1), lane);
     }
 }
 
@@ -933,7 +935,7 @@ extern "C" int pv_load_cluster(pv_ctx *ctx, uint32_t num_nodes, uint32_t num_key
     int rc;
     if ((rc = pv_pool_alloc(ctx, (void **)&c.d_labels, nl * 2, "labels")) ||
         (rc = pv_pool_alloc(ctx, (void **)&c.d_inv, (size_t)num_keys * kInvWords * 4, "inventory")) ||
-        (rc = pv_pool_alloc(ctx, (void **)&c.d_inv_rank, (size_t)num_keys * kInvWords * 4, "inventory rank")) ||
+        (rc = pv_pool_alloc(ctx, (void **)&c.d_ranked, (size_t)num_keys * kInvWords * 8, "inventory rank")) ||
         (rc = pv_pool_alloc(ctx, (void **)&c.d_key_base, ((size_t)num_keys + 1) * 4 * 2, "key base"))) {
         pv_free_cluster(ctx, c);
         return rc;
@@ -942,7 +944,7 @@ extern "C" int pv_load_cluster(pv_ctx *ctx, uint32_t num_nodes, uint32_t num_key
     PV_TRY_CUDA(ctx, cudaMemcpyAsync(c.d_labels, labels, nl * 2, cudaMemcpyHostToDevice, ls), "labels upload");
     PV_TRY_CUDA(ctx, cudaMemsetAsync(c.d_inv, 0, (size_t)num_keys * kInvWords * 4, ls), "inventory clear");
     build_inventory_kernel<<<ctx->num_sms * 8, 256, 0, ls>>>(num_nodes, num_keys, c.d_labels, c.d_inv);
-    inventory_rank_kernel<<<num_keys, 1024, 0, ls>>>(c.d_inv, c.d_inv_rank, d_count);
+    inventory_rank_kernel<<<num_keys, 1024, 0, ls>>>(c.d_inv, c.d_ranked, d_count);
     key_base_kernel<<<1, 1024, 0, ls>>>(num_keys, d_count, c.d_key_base);
     if ((rc = pv_check_launch(ctx, "inventory kernels"))) { pv_free_cluster(ctx, c); return rc; }
     uint32_t nvr = 0;
@@ -956,15 +958,15 @@ extern "C" int pv_load_cluster(pv_ctx *ctx, uint32_t num_nodes, uint32_t num_key
     c.num_keys = num_keys;
     c.row_words = words_for(num_nodes);
     c.num_value_rows = nvr;
-    const uint64_t row_bytes = ((uint64_t)nvr + num_keys) * c.row_words * 4;
-    if (row_bytes <= kRowBudgetBytes) {
+    const uint64_t row_bytes = ((uint64_t)nvr + num_keys + 1) * c.row_words * 4;   // and the row of no node
+    if (row_bytes - c.row_words * 4ull <= kRowBudgetBytes) {
         if (pv_pool_alloc(ctx, (void **)&c.d_rows, row_bytes, "value rows") == PV_OK) {
             if ((e = cudaMemsetAsync(c.d_rows, 0, row_bytes, ls)) != cudaSuccess) {
                 pv_free_cluster(ctx, c);
                 return pv_cuda_fail(ctx, e, "value rows clear");
             }
-            build_rows_kernel<<<ctx->num_sms * 8, 256, 0, ls>>>(num_nodes, num_keys, c.d_labels, c.d_inv, c.d_inv_rank,
-                                                          c.d_key_base, nvr, c.row_words, c.d_rows);
+            build_rows_kernel<<<ctx->num_sms * 8, 256, 0, ls>>>(num_nodes, num_keys, c.d_labels, c.d_ranked, c.d_key_base,
+                                                          nvr, c.row_words, c.d_rows);
             if ((rc = pv_check_launch(ctx, "value rows"))) { pv_free_cluster(ctx, c); return rc; }
             c.rows_built = true;
         } else {
@@ -978,6 +980,31 @@ extern "C" int pv_load_cluster(pv_ctx *ctx, uint32_t num_nodes, uint32_t num_key
     ctx->cl = c;
     return pv_load_end(ctx);
 }
+
+namespace {
+
+// The rows kernel's arguments and grid: a warp per pod until the GPU is full,
+// then the pods shared out.
+template <bool kTerms>
+void launch_rows(pv_ctx *ctx, SelArgs g, cudaStream_t st) {
+    const pv_cluster_state &c = ctx->cl;
+    g.N = c.num_nodes;
+    g.K = c.num_keys;
+    g.inv = c.d_inv;
+    g.ranked = c.d_ranked;
+    g.key_base = c.d_key_base;
+    g.rows = c.d_rows;
+    g.row_words = c.row_words;
+    g.num_value_rows = c.num_value_rows;
+    g.zero_row = (c.num_value_rows + c.num_keys) * c.row_words * 4;
+    void (*fn)(SelArgs) = g.W <= 160 ? sel_rows_kernel<kTerms, true> : sel_rows_kernel<kTerms, false>;
+    const int per_sm = std::max(1, pv_blocks_per_sm(ctx, (const void *)fn, kRowsThreads<kTerms>, 0));
+    constexpr uint32_t warps = kRowsThreads<kTerms> / 32;
+    const uint32_t blocks = std::min((g.P + warps - 1) / warps, (uint32_t)(ctx->num_sms * per_sm));
+    fn<<<blocks, kRowsThreads<kTerms>, 0, st>>>(g);
+}
+
+}  // namespace
 
 extern "C" int pv_eval_selectors(pv_ctx *ctx, uint32_t num_pods, const uint32_t *d_expr_offs, uint32_t num_exprs,
                                  const pv_expr *d_exprs, const uint32_t *d_assign, uint32_t *d_bits,
@@ -1033,10 +1060,18 @@ extern "C" int pv_eval_selectors(pv_ctx *ctx, uint32_t num_pods, const uint32_t 
                                                  rep_list, rep_count);
     }
     if (which == 2) {
-        sel_rows_kernel<<<wblocks, kRowsThreads, 0, st>>>(c.num_nodes, c.num_keys, num_pods, d_expr_offs, num_exprs,
-                                                          d_exprs, d_assign, d_bits, words_per_row, d_flags, c.d_inv,
-                                                          c.d_inv_rank, c.d_key_base, c.d_rows, c.row_words,
-                                                          c.num_value_rows, rep_list, rep_count);
+        SelArgs g = {};
+        g.P = num_pods;
+        g.offs = d_expr_offs;
+        g.num_exprs = num_exprs;
+        g.exprs = d_exprs;
+        g.assign = d_assign;
+        g.bits = d_bits;
+        g.W = words_per_row;
+        g.flags = d_flags;
+        g.pod_list = rep_list;
+        g.list_len = rep_count;
+        launch_rows<false>(ctx, g, st);
     } else {
         const size_t smem = (size_t)tile * c.num_keys * 2;
         PV_TRY_CUDA(ctx, cudaFuncSetAttribute(sel_cmp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
@@ -1072,14 +1107,21 @@ extern "C" int pv_eval_selector_terms(pv_ctx *ctx, uint32_t num_pods, const uint
     if (!c.rows_built)
         return pv_fail(ctx, PV_EINVAL, "pv_eval_selector_terms: value rows were not built for this cluster");
     cudaStream_t st = (cudaStream_t)stream;
-    const uint32_t blocks = std::min<uint32_t>((num_pods + 7) / 8, (uint32_t)ctx->num_sms * 16);
+    SelArgs g = {};
+    g.P = num_pods;
+    g.offs = d_pod_terms;
+    g.num_terms = num_terms;
+    g.term_offs = d_term_offs;
+    g.num_exprs = num_exprs;
+    g.exprs = d_exprs;
+    g.assign = d_assign;
+    g.bits = d_bits;
+    g.W = words_per_row;
+    g.flags = d_flags;
     pv_use_begin(ctx, st);
     const int pr = pv_prof_start(ctx, st, PV_K_SELECTOR);
-    sel_terms_kernel<<<blocks, kRowsThreads, 0, st>>>(c.num_nodes, c.num_keys, num_pods, d_pod_terms, num_terms,
-                                                      d_term_offs, num_exprs, d_exprs, d_assign, d_bits,
-                                                      words_per_row, d_flags, c.d_inv, c.d_inv_rank, c.d_key_base,
-                                                      c.d_rows, c.row_words, c.num_value_rows);
+    launch_rows<true>(ctx, g, st);
     pv_prof_stop(ctx, st, pr, 1);
     pv_mark_use(ctx, st);
-    return pv_check_launch(ctx, "sel_terms_kernel");
+    return pv_check_launch(ctx, "selector kernels");
 }

@@ -143,7 +143,7 @@ void *pv_scratch(pv_ctx *ctx, size_t bytes) {
 void pv_free_cluster(pv_ctx *ctx, pv_cluster_state &c) {
     pv_free_ptr(ctx, c.d_labels);
     pv_free_ptr(ctx, c.d_inv);
-    pv_free_ptr(ctx, c.d_inv_rank);
+    pv_free_ptr(ctx, c.d_ranked);
     pv_free_ptr(ctx, c.d_key_base);
     pv_free_ptr(ctx, c.d_rows);
     c = pv_cluster_state();

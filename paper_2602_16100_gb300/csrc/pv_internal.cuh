@@ -20,7 +20,7 @@ struct pv_cluster_state {
     uint32_t num_nodes = 0, num_keys = 0;
     uint16_t *d_labels = nullptr;     // [K][N]
     uint32_t *d_inv = nullptr;        // [K][2048]: bit v = some node carries value v of key k
-    uint32_t *d_inv_rank = nullptr;   // [K][2048]: set bits of the key's inventory before word w
+    uint2 *d_ranked = nullptr;        // [K][2048]: inventory word w and the set bits of the key's inventory before it
     uint32_t *d_key_base = nullptr;   // [K + 1]: first value row of key k; [K] = number of value rows
     // per-(key, value) node bitsets, then one "present" row per key
     bool rows_built = false;
