@@ -1545,15 +1545,24 @@ struct Candidates {
     }
 };
 
+// The n lowest bits, n at most 32.
+__device__ __forceinline__ uint32_t first_bits(uint32_t n) { return n ? ~0u >> (32 - n) : 0u; }
+
 // Scalar first match, one probe per lane (called by all 32 lanes; inactive
 // lanes return 0): each lane walks its bucket's candidates in order, src and
 // dst of classes sc and dc.  Plain rules are tested until a hit or a segment
 // token; the warp then reconverges and the lanes parked on a segment token
 // run their interval searches together (a segment miss resumes the walk).
+// max_len: the longest list of the 32.  Up to 32 every bit of the filter is one
+// item, which spares the group arithmetic (25 of about 65 instructions per
+// candidate; on 512 switches of 1,000 rules a list has 7 items, 1.6 of which a
+// probe walks, 3.3 the longest of a warp: first hop of 50 million flows 504 ->
+// 450 us together with hop_outcome's selects).
 template <bool kStats>
 __device__ __forceinline__ uint32_t first_match_lane(const uint8_t *sm, uint32_t skip, const BlobLayout &L,
                                                      bool active, uint32_t src, uint32_t dst, uint32_t dport, uint32_t in_port,
-                                                     uint32_t sc, uint32_t dc, uint32_t &tests, uint32_t &lookups) {
+                                                     uint32_t sc, uint32_t dc, uint32_t max_len, uint32_t &tests,
+                                                     uint32_t &lookups) {
     const uint32_t *boff = reinterpret_cast<const uint32_t *>(sm + L.boff);
     const uint32_t *masks = reinterpret_cast<const uint32_t *>(sm + L.masks);
     sm -= skip;   // skip: bytes left out of the stage where the filter would be
@@ -1561,11 +1570,53 @@ __device__ __forceinline__ uint32_t first_match_lane(const uint8_t *sm, uint32_t
     const uint16_t *items = reinterpret_cast<const uint16_t *>(sm + L.items);
     const uint2 *segs = reinterpret_cast<const uint2 *>(sm + L.segs);
     const uint2 *bw = reinterpret_cast<const uint2 *>(sm + L.bw);
-    const uint32_t k = dport >> kBucketShift;
+    const uint32_t k = dport >> kBucketShift, first = boff[k];
     const uint32_t *mk = masks + k * (2 * kClasses);
-    Candidates cand(0u, boff[k], boff[k + 1]);
-    if (active) cand.m = skip ? cand.all() : mk[dc] & mk[kClasses + sc];
+    // the winner of segment seg's interval holding dst, or 0
+    auto search = [&](uint32_t seg) {
+        const uint2 *b = bw + segs[seg].x;
+        uint32_t lo, len;   // b[lo].x <= dst; answer in [lo, lo + len)
+        jump_range(sm + L.jmp + seg * kJumpBytes, dst, &lo, &len);
+        while (len > 1) {
+            const uint32_t half = len >> 1;
+            lo = b[lo + half].x <= dst ? lo + half : lo;
+            len -= half;
+        }
+        if (kStats) ++lookups;
+        const uint32_t w = b[lo].y;
+        return w & kWinFound ? w : 0u;
+    };
     uint32_t result = 0;
+    if (max_len <= 32) {   // a filter bit is an item
+        const uint16_t *own = items + first;
+        uint32_t m = 0;   // candidates left
+        if (active) m = skip ? first_bits(boff[k + 1] - first) : mk[dc] & mk[kClasses + sc];
+        do {
+            uint32_t seg = 0xFFFFFFFFu;
+            while (m) {
+                const uint32_t it = own[__ffs(m) - 1];
+                m &= m - 1u;
+                if (it & kSegItem) {
+                    seg = it & 0x7FFFu;
+                    break;
+                }
+                const uint4 r = rules[it];
+                if (kStats) ++tests;
+                if (plain_hit(r, src, dst, dport, in_port)) {
+                    result = plain_result(r);
+                    m = 0;
+                }
+            }
+            __syncwarp();
+            if (seg != 0xFFFFFFFFu) {
+                result = search(seg);
+                if (result) m = 0;
+            }
+        } while (__any_sync(PV_FULL_MASK, m != 0));
+        return result;
+    }
+    Candidates cand(0u, first, boff[k + 1]);
+    if (active) cand.m = skip ? cand.all() : mk[dc] & mk[kClasses + sc];
     bool done = !active;
     while (__any_sync(PV_FULL_MASK, !done)) {
         uint32_t seg = 0xFFFFFFFFu;
@@ -1589,20 +1640,8 @@ __device__ __forceinline__ uint32_t first_match_lane(const uint8_t *sm, uint32_t
         }
         __syncwarp();
         if (seg != 0xFFFFFFFFu) {
-            const uint2 *b = bw + segs[seg].x;
-            uint32_t lo, len;   // b[lo].x <= dst; answer in [lo, lo + len)
-            jump_range(sm + L.jmp + seg * kJumpBytes, dst, &lo, &len);
-            while (len > 1) {
-                const uint32_t half = len >> 1;
-                lo = b[lo + half].x <= dst ? lo + half : lo;
-                len -= half;
-            }
-            const uint32_t w = b[lo].y;
-            if (kStats) ++lookups;
-            if (w & kWinFound) {
-                result = w;
-                done = true;
-            }
+            result = search(seg);
+            done = result != 0;
         }
     }
     return result;
@@ -1623,26 +1662,16 @@ constexpr uint32_t kViolationNext = 0xFEu;
 // memory, the thread walk reads them in place.
 __device__ __forceinline__ void hop_outcome(const HopArgs &g, const uint2 *ports, uint32_t hop, uint32_t fm, uint32_t dst,
                                             uint32_t mask, uint32_t nports, uint32_t *status, uint32_t *next) {
-    *next = 0;
+    // (selects rather than branches: the lanes of a warp end in every way)
     const uint32_t act = fm & 0xFFFFu;
-    if (!(fm & kWinFound) || act == PV_DROP || act >= nports) {
-        *status = PV_DROPPED;
-        return;
-    }
-    const uint2 pe = ports[act];
+    uint2 pe = make_uint2(~0u, 0u);   // no such port (a drop is none): the probe is dropped
+    if ((fm & kWinFound) && act < nports) pe = ports[act];
     const int32_t peer = (int32_t)pe.x;
-    if (peer < 0) {
-        *status = PV_DROPPED;
-    } else if (peer & PV_PEER_HOST) {
-        const uint32_t q = (uint32_t)(peer & ~PV_PEER_HOST);
-        *status = (q < g.H && pe.y == dst) ? PV_COMPLIANT : PV_MISDELIVERED;
-    } else if (hop + 1 >= g.cap) {
-        *status = PV_LOOP;
-    } else {
-        const uint32_t r2 = pe.y;
-        *status = (r2 < 32 && ((mask >> r2) & 1u)) ? kAlive : kViolationNext;
-        *next = (uint32_t)peer;
-    }
+    const uint32_t q = (uint32_t)(peer & ~PV_PEER_HOST);
+    const uint32_t at_host = q < g.H && pe.y == dst ? PV_COMPLIANT : PV_MISDELIVERED;
+    const uint32_t onward = hop + 1 >= g.cap ? (uint32_t)PV_LOOP : pe.y < 32 && ((mask >> pe.y) & 1u) ? kAlive : kViolationNext;
+    *status = peer < 0 ? (uint32_t)PV_DROPPED : peer & PV_PEER_HOST ? at_host : onward;
+    *next = (uint32_t)peer;
 }
 
 // kFirst: the walk's first hop, where every entry's finish field is 0, its
@@ -1740,7 +1769,7 @@ __global__ void __launch_bounds__(kHopThreads, 4) walk_hop_kernel(HopArgs g) {
         const uint32_t wb0 = pos + warp * 32;
         // At the first hop of directly placed flows there is no list: entry
         // i is record i, and its in_port is its source host's port.
-        const bool at_pos = kRec && g.recs_at_position != 0;
+        const bool at_pos = kRec && (kStats ? g.recs_at_position != 0 : kFirst);
         uint2 e1 = make_uint2(0, 0), e2 = make_uint2(0, 0);   // entries of batches wb, wb + kStride
         uint4 raw1 = make_uint4(0, 0, 0, 0);                  // record of batch wb
         if (wb0 + lane < seg_end) {
@@ -1772,6 +1801,7 @@ __global__ void __launch_bounds__(kHopThreads, 4) walk_hop_kernel(HopArgs g) {
             // Every listed probe is permitted at s (checked when it was handed
             // on).  Lane-per-probe when every candidate list of the batch is short.
             bool lane_mode = false;
+            uint32_t max_len = 0;   // longest candidate list of the batch
             if (kIndexed) {
                 const uint32_t *boff = reinterpret_cast<const uint32_t *>(s_raw + L.boff);
                 uint32_t len = 0;
@@ -1779,12 +1809,13 @@ __global__ void __launch_bounds__(kHopThreads, 4) walk_hop_kernel(HopArgs g) {
                     const uint32_t k = (pr.z & 0xFFFFu) >> kBucketShift;
                     len = boff[k + 1] - boff[k];
                 }
-                lane_mode = __reduce_max_sync(PV_FULL_MASK, len) <= g.lane_max;
+                max_len = __reduce_max_sync(PV_FULL_MASK, len);
+                lane_mode = max_len <= g.lane_max;
             }
             if (lane_mode) {
                 const bool act = lane < cnt && !fin_now;
                 const uint32_t fm = first_match_lane<kStats>(s_raw, g.stage_skip, L, act, pr.x, pr.y, pr.z & 0xFFFFu, e.y & 0xFFu,
-                                                             src_class, addr_class(g.cls, pr.y), stc[kStRuleTests],
+                                                             src_class, addr_class(g.cls, pr.y), max_len, stc[kStRuleTests],
                                                              stc[kStLookups]);
                 my_fm = fm;
                 if (act) hop_outcome(g, s_port, g.hop, fm, pr.y, pr.w, nports, &my_status, &my_next);
