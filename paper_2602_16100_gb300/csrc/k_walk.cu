@@ -187,7 +187,9 @@ __global__ void __launch_bounds__(1024) compile_tables_kernel(const uint32_t *__
 // A switch's blob (sections 16-byte aligned):
 //   header   uint4 {npad | n_plain << 16, n_items, n_segs, n_bnd}
 //   boff[kBuckets + 1] u32           item range of each destination-port bucket
-//   masks[kBuckets][2 * kClasses] u32   candidate filter of each bucket: bit j
+//   masks[2 * kClasses][kBuckets] u32   candidate filter of each bucket (by class
+//                                    first: a warp's lanes look up one class in
+//                                    many buckets, in different banks): bit j
 //                                    of word c is set when group j of the
 //                                    bucket's items (ceil(length / 32) items
 //                                    to a group) holds a segment token or a
@@ -721,7 +723,7 @@ __global__ void __launch_bounds__(kIndexThreads) index_build_kernel(const uint32
                 const uint32_t word = __ballot_sync(PV_FULL_MASK, (meets >> c) & 1u);
                 if (lane == c) mine = word;
             }
-            if (lane < 2 * kClasses) masks[k * 2 * kClasses + lane] = mine;
+            if (lane < 2 * kClasses) masks[lane * kBuckets + k] = mine;
         }
     }
 
@@ -819,10 +821,6 @@ __device__ __forceinline__ uint2 flow_at(const BindArgs &ba, uint32_t i) {
     return make_uint2(__ldg(ba.dst + (size_t)i * ba.dst_stride), __ldg(ba.dport + (size_t)i * ba.dport_stride));
 }
 
-__device__ __forceinline__ uint32_t flow_dport(const BindArgs &ba, uint32_t i) {
-    return __ldg(ba.dport + (size_t)i * ba.dport_stride);
-}
-
 template <bool kPolicy, bool kBind>
 __global__ void __launch_bounds__(kGridThreads) walk_init_kernel(
     uint32_t M, pv_probe *__restrict__ probes, uint32_t H, const uint16_t *__restrict__ host_switch,
@@ -898,11 +896,16 @@ __global__ void __launch_bounds__(kGridThreads) walk_init_kernel(
 // record straight to its slot in the first hop's switch order (switch start
 // + pair offset + rank within the pair), so the first hop needs neither a
 // regroup nor a list: it reads records by position and takes each in_port
-// from the record's source host.  walk_init_group_kernel (below) does so one group per
-// block with each pair's run in bucket order; walk_init_direct_kernel is the
-// grid-stride form for groups too large for its shared memory.  Probe i
-// belongs to group i / ppg and pod (i mod ppg) mod pods; the caller
-// guarantees one path constraint per group.
+// from the record's source host.  Probe i belongs to group i / ppg and pod
+// (i mod ppg) mod pods; the caller guarantees one path constraint per group.
+// What bounds it: memory (50 million flows: 300 MB of columns in, 570 MB of
+// records and results out).  Blocks take consecutive probes.  (Ordering each
+// pair's run by destination-port bucket, so that a first-hop warp shared its
+// candidate lists, cost 73 us here and made the first hop write its results one
+// word to a sector: with the matching left out it still took 459 us, without
+// the order 246.)
+constexpr uint32_t kNoRun = 0xFFFFFFFFu;   // pair_off of a pair that is not listed
+
 template <bool kPolicy>
 __device__ __forceinline__ bool first_switch_permitted(const PolicyArgs &pa, uint32_t k, uint32_t s, uint32_t reg,
                                                        uint32_t mask) {
@@ -925,7 +928,7 @@ __global__ void __launch_bounds__(kGridThreads) flow_groups_kernel(uint32_t M, u
         const uint32_t first = grp * ba.ppg, len = min(ba.ppg, M - first);
         const uint32_t cnt = len > q ? (len - q + ba.pods - 1) / ba.pods : 0u;
         const uint32_t node = ba.assign[g];
-        uint32_t off = 0;
+        uint32_t off = kNoRun;
         if (cnt && node < H) {
             const uint32_t s = host_switch[node];
             if (first_switch_permitted<kPolicy>(pa, first + q, s, region[s], ba.group_mask[grp]))
@@ -938,58 +941,73 @@ __global__ void __launch_bounds__(kGridThreads) flow_groups_kernel(uint32_t M, u
 template <bool kPolicy>
 __global__ void __launch_bounds__(kGridThreads) walk_init_direct_kernel(
     uint32_t M, pv_probe *__restrict__ probes, uint32_t H, const uint16_t *__restrict__ host_switch,
-    const uint8_t *__restrict__ region, pv_result *__restrict__ out, uint4 *__restrict__ recs,
-    const uint32_t *__restrict__ seg,
+    pv_result *__restrict__ out, uint4 *__restrict__ recs, const uint32_t *__restrict__ seg,
     const uint32_t *__restrict__ pair_off, PolicyArgs pa, BindArgs ba) {
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < M; i += gridDim.x * blockDim.x) {
-        const uint32_t grp = i / ba.ppg, r = i - grp * ba.ppg, g = grp * ba.pods + r % ba.pods;
-        const uint32_t node = ba.assign[g];
-        const uint2 f = flow_at(ba, i);
+    constexpr uint32_t stride = kGridThreads;
+    // consecutive probes per block, so that its pairs stay in L1
+    const uint32_t P = ba.pods, ppg = ba.ppg, end = (uint32_t)(((uint64_t)M * (blockIdx.x + 1)) / gridDim.x);
+    uint32_t i = (uint32_t)(((uint64_t)M * blockIdx.x) / gridDim.x) + threadIdx.x;
+    if (i >= end) return;
+    // probe i is probe r of group grp, and that is number run of pod q: r =
+    // run * P + q, carried along without further divisions
+    uint32_t grp = i / ppg, r = i - grp * ppg, run = r / P, q = r - run * P;
+    const uint32_t dgrp = stride / ppg, dr = stride - dgrp * ppg, drun = dr / P, dq = dr - drun * P;
+    const uint32_t wrun = ppg / P, wq = ppg - wrun * P;
+    uint2 next = flow_at(ba, i);
+    while (true) {
+        const uint2 f = next;
+        if (end - i > stride) next = flow_at(ba, i + stride);
+        const uint32_t g = grp * P + q, node = __ldg(ba.assign + g), off = __ldg(pair_off + g);
         const bool placed = node < H;
-        const uint32_t mask = ba.group_mask[grp];
+        const uint32_t s = placed ? __ldg(host_switch + node) : 0u, mask = __ldg(ba.group_mask + grp);
         const uint32_t z = (f.y & 0xFFFFu) | (placed ? node : (uint32_t)PV_NO_HOST) << 16;
         if (probes)   // the caller's copy of the bound record {src_ip, dst_ip, dport | src_host << 16, mask}
             reinterpret_cast<uint4 *>(probes)[i] = make_uint4(placed ? ba.host_ip[node] : 0u, f.x, z, mask);
         if (kPolicy) pa.hits[i] = 0;
-        if (!placed) {
-            put_result(out, i, PV_NOSRC, 0, 0xFFFF);
-            continue;
+        if (off != kNoRun) recs[__ldg(seg + s) + off + run] = make_uint4(i, f.x, z, mask);
+        else put_result(out, i, placed ? PV_VIOLATION : PV_NOSRC, placed ? 1u : 0u, placed ? s : 0xFFFFu);
+        if (end - i <= stride) break;
+        i += stride;
+        grp += dgrp;
+        r += dr;
+        run += drun;
+        q += dq;
+        if (q >= P) {
+            q -= P;
+            ++run;
         }
-        const uint32_t s = host_switch[node];
-        if (first_switch_permitted<kPolicy>(pa, i, s, region[s], mask)) {
-            const uint32_t slot = seg[s] + pair_off[g] + r / ba.pods;
-            recs[slot] = make_uint4(i, f.x, z, mask);
-        } else {
-            put_result(out, i, PV_VIOLATION, 1, s);
+        if (r >= ppg) {
+            r -= ppg;
+            ++grp;
+            run -= wrun;
+            if (q < wq) {
+                q += P;
+                --run;
+            }
+            q -= wq;
         }
     }
 }
 
-// The same placement by one block per group, with each pair's run ordered
-// by destination-port bucket of the first-match index, so the lanes of a
-// first-hop warp mostly read the same few candidate lists.  The block brings
-// its group's slice of the flows into shared memory with bulk copies (one
-// per column, or one for records; the few elements outside the copies'
-// 16-byte-aligned middles by plain loads), counts its probes per (pod,
-// bucket), binds and judges them in one pass that drops each listed probe's
-// rank into its pod's run (the next slot of its bucket), then writes every
-// run out whole as walk records, so each sector of the records is written
-// at once.  Used when the counts, ranks and flow slices fit
-// kGroupInitSmem.
+// The same by one block per group, whose flows come into shared memory by
+// bulk copies (one per column, or one for records; the few elements outside
+// the copies' 16-byte-aligned middles by plain loads).  For large groups: a
+// block costs about 1 us whatever it does, the form above more instructions per
+// probe.  us by group / by range: 5 million flows in groups of 333 91/21, 1,000
+// 31/21, 2,000 22.1/20.2, 6 million of 3,000 21.5/23.5, 50 million of 4,999
+// 148/199.
 constexpr uint32_t kGroupInitMaxPods = 16;
 constexpr uint32_t kGroupInitThreads = 512;
-constexpr size_t kGroupInitSmem = 64 * 1024;   // ppg <= 65535 also fits the rank's 16 bits
+constexpr uint32_t kGroupInitMin = 2560;   // smallest groups that take a block
+constexpr size_t kGroupInitSmem = 64 * 1024;
 
-// Shared-memory layout of walk_init_group_kernel: bucket counts / run
-// slots [pods][kBuckets], ranks [ppg], then the destination slice and the
-// port slice (the same slice for records), each with 16 bytes of slack so
-// that its elements keep their global address modulo 16.
+// Shared-memory layout of walk_init_group_kernel: the destination slice and
+// the port slice (one slice for records), each with 16 bytes of slack so that
+// its elements keep their global address modulo 16.
 struct GroupInitSmem {
-    uint32_t rank, dst, dport, total;
-    __host__ __device__ GroupInitSmem(uint32_t pods, uint32_t ppg, bool records) {
-        rank = pods * kBuckets * 4;
-        dst = rank + ((ppg * 2 + 15) & ~15u);
-        dport = dst + (records ? 0u : ((ppg * 4 + 16 + 15) & ~15u));
+    uint32_t dport, total;
+    __host__ __device__ GroupInitSmem(uint32_t ppg, bool records) {
+        dport = records ? 0u : ((ppg * 4 + 16 + 15) & ~15u);
         total = dport + (records ? ppg * 8 + 16 : ((ppg * 2 + 16 + 15) & ~15u));
     }
 };
@@ -1044,17 +1062,15 @@ __device__ __forceinline__ void slice_edges(const Slice &sl, uint8_t *s_base) {
 template <bool kPolicy>
 __global__ void __launch_bounds__(kGroupInitThreads) walk_init_group_kernel(
     uint32_t M, pv_probe *__restrict__ probes, uint32_t H, const uint16_t *__restrict__ host_switch,
-    const uint8_t *__restrict__ region, pv_result *__restrict__ out, uint4 *__restrict__ recs,
+    pv_result *__restrict__ out, uint4 *__restrict__ recs,
     const uint32_t *__restrict__ seg,
     const uint32_t *__restrict__ pair_off, PolicyArgs pa, BindArgs ba, uint64_t wait_ns, int32_t *status) {
     extern __shared__ __align__(16) uint8_t s_raw[];
-    __shared__ uint32_t s_pair[kGroupInitMaxPods][3];   // per pod: {node, switch, listed}
+    __shared__ uint4 s_pair[kGroupInitMaxPods];   // per pod: {node, switch, listed, its run's first record}
     __shared__ uint64_t s_bar;
-    const uint32_t grp = blockIdx.x, P = ba.pods, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const uint32_t grp = blockIdx.x, P = ba.pods, t = threadIdx.x;
     const bool records = ba.dst_stride == 2;
-    const GroupInitSmem L(P, ba.ppg, records);
-    uint32_t *s_cur = reinterpret_cast<uint32_t *>(s_raw);                  // [pods][kBuckets] counts, then slots
-    uint16_t *s_rank = reinterpret_cast<uint16_t *>(s_raw + L.rank);        // pod runs: ranks in the group
+    const GroupInitSmem L(ba.ppg, records);
     const uint32_t first = grp * ba.ppg, len = min(ba.ppg, M - first);
     // the group's flows: destination and port slices (one slice for records)
     const Slice sa = records ? Slice(ba.dst + (size_t)first * 2, len, 8) : Slice(ba.dst + first, len, 4);
@@ -1063,24 +1079,20 @@ __global__ void __launch_bounds__(kGroupInitThreads) walk_init_group_kernel(
         mbar_init(&s_bar, 1);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         mbar_arrive_expect_tx(&s_bar, sa.bulk_bytes() + sb.bulk_bytes());
-        slice_copy(sa, s_raw + L.dst, &s_bar);
+        slice_copy(sa, s_raw, &s_bar);
         slice_copy(sb, s_raw + L.dport, &s_bar);
     }
-    slice_edges(sa, s_raw + L.dst);
+    slice_edges(sa, s_raw);
     slice_edges(sb, s_raw + L.dport);
-    const uint32_t *s_dst = reinterpret_cast<const uint32_t *>(sa.staged(s_raw + L.dst));
+    const uint32_t *s_dst = reinterpret_cast<const uint32_t *>(sa.staged(s_raw));
     const uint16_t *s_dport = records ? reinterpret_cast<const uint16_t *>(s_dst) + 2
                                       : reinterpret_cast<const uint16_t *>(sb.staged(s_raw + L.dport));
     const uint32_t ds = records ? 2u : 1u, ps = records ? 4u : 1u;
     const uint32_t mask = ba.group_mask[grp];
-    for (uint32_t x = t; x < P * kBuckets; x += kGroupInitThreads) s_cur[x] = 0;
     if (t < P) {
-        const uint32_t node = ba.assign[grp * P + t];
-        const bool placed = node < H;
-        const uint32_t sw = placed ? host_switch[node] : 0u;
-        s_pair[t][0] = node;
-        s_pair[t][1] = sw;
-        s_pair[t][2] = placed && t < len && first_switch_permitted<kPolicy>(pa, first + t, sw, region[sw], mask);
+        const uint32_t node = ba.assign[grp * P + t], off = pair_off[grp * P + t];
+        const uint32_t sw = node < H ? host_switch[node] : 0u;
+        s_pair[t] = make_uint4(node, sw, off != kNoRun, off != kNoRun ? seg[sw] + off : 0u);
     }
     __syncthreads();   // barrier initialised before anyone waits on it
     const bool ok = mbar_wait_bounded(&s_bar, 0, wait_ns);
@@ -1093,63 +1105,25 @@ __global__ void __launch_bounds__(kGroupInitThreads) walk_init_group_kernel(
         s_dst = records ? ba.dst + (size_t)first * 2 : ba.dst + first;
         s_dport = records ? ba.dport + (size_t)first * 4 : ba.dport + first;
     }
-    for (uint32_t r = t; r < len; r += kGroupInitThreads)
-        atomicAdd(&s_cur[(r % P) * kBuckets + (s_dport[r * ps] >> kBucketShift)], 1u);
-    __syncthreads();
-    // exclusive scan of each pod's buckets, offset by the runs of the pods
-    // before it (pod q holds probes q, q + P, ...: ceil((len - q) / P) of them)
-    for (uint32_t q = warp; q < P; q += kGroupInitThreads / 32) {
-        uint32_t *c = s_cur + q * kBuckets;
-        constexpr uint32_t kPer = kBuckets / 32;
-        uint32_t v[kPer], sum = 0;
-        for (uint32_t j = 0; j < kPer; ++j) {
-            v[j] = c[lane * kPer + j];
-            sum += v[j];
-        }
-        uint32_t incl = sum;
-        for (int d = 1; d < 32; d <<= 1) {
-            const uint32_t y = __shfl_up_sync(PV_FULL_MASK, incl, d);
-            if (lane >= (uint32_t)d) incl += y;
-        }
-        uint32_t before = 0;   // probes of pods 0 .. q - 1
-        for (uint32_t q2 = 0; q2 < q; ++q2) before += len > q2 ? (len - q2 + P - 1) / P : 0u;
-        uint32_t run = before + incl - sum;
-        for (uint32_t j = 0; j < kPer; ++j) {
-            c[lane * kPer + j] = run;
-            run += v[j];
-        }
-    }
-    __syncthreads();
+    // probe r of the group is number run of pod q, carried along without dividing
+    uint32_t run = t / P, q = t - run * P;
+    const uint32_t drun = kGroupInitThreads / P, dq = kGroupInitThreads - drun * P;
     for (uint32_t r = t; r < len; r += kGroupInitThreads) {
-        const uint32_t i = first + r, q = r % P;
-        const uint32_t node = s_pair[q][0], sw = s_pair[q][1];
-        const bool placed = node < H;
-        const uint32_t dport = s_dport[r * ps];
+        const uint4 pair = s_pair[q];
+        const uint32_t i = first + r, dst = s_dst[r * ds], dport = s_dport[r * ps];
+        const bool placed = pair.x < H;
         if (probes)   // the caller's copy of the bound record {src_ip, dst_ip, dport | src_host << 16, mask}
-            reinterpret_cast<uint4 *>(probes)[i] = make_uint4(placed ? ba.host_ip[node] : 0u, s_dst[r * ds],
-                                                              dport | (placed ? node : (uint32_t)PV_NO_HOST) << 16,
-                                                              mask);
+            reinterpret_cast<uint4 *>(probes)[i] = make_uint4(placed ? ba.host_ip[pair.x] : 0u, dst,
+                                                              dport | (placed ? pair.x : (uint32_t)PV_NO_HOST) << 16, mask);
         if (kPolicy) pa.hits[i] = 0;
-        if (s_pair[q][2]) {
-            s_rank[atomicAdd(&s_cur[q * kBuckets + (dport >> kBucketShift)], 1u)] = (uint16_t)r;
-        } else {
-            put_result(out, i, placed ? PV_VIOLATION : PV_NOSRC, placed ? 1u : 0u, placed ? sw : 0xFFFFu);
+        if (pair.z) recs[pair.w + run] = make_uint4(i, dst, dport | pair.x << 16, mask);
+        else put_result(out, i, placed ? PV_VIOLATION : PV_NOSRC, placed ? 1u : 0u, placed ? pair.y : 0xFFFFu);
+        run += drun;
+        q += dq;
+        if (q >= P) {
+            q -= P;
+            ++run;
         }
-    }
-    __syncthreads();
-    uint32_t before = 0;
-    for (uint32_t q = 0; q < P && q < len; ++q) {
-        const uint32_t n = (len - q + P - 1) / P;
-        if (s_pair[q][2]) {
-            const uint32_t sw = s_pair[q][1];
-            const uint32_t node = s_pair[q][0];
-            const uint32_t base = seg[sw] + pair_off[grp * P + q];
-            for (uint32_t k = t; k < n; k += kGroupInitThreads) {
-                const uint32_t r = s_rank[before + k];
-                recs[base + k] = make_uint4(first + r, s_dst[r * ds], s_dport[r * ps] | node << 16, mask);
-            }
-        }
-        before += n;
     }
 }
 
@@ -1571,7 +1545,7 @@ __device__ __forceinline__ uint32_t first_match_lane(const uint8_t *sm, uint32_t
     const uint2 *segs = reinterpret_cast<const uint2 *>(sm + L.segs);
     const uint2 *bw = reinterpret_cast<const uint2 *>(sm + L.bw);
     const uint32_t k = dport >> kBucketShift, first = boff[k];
-    const uint32_t *mk = masks + k * (2 * kClasses);
+    const uint32_t *mk = masks + k;
     // the winner of segment seg's interval holding dst, or 0
     auto search = [&](uint32_t seg) {
         const uint2 *b = bw + segs[seg].x;
@@ -1590,7 +1564,7 @@ __device__ __forceinline__ uint32_t first_match_lane(const uint8_t *sm, uint32_t
     if (max_len <= 32) {   // a filter bit is an item
         const uint16_t *own = items + first;
         uint32_t m = 0;   // candidates left
-        if (active) m = skip ? first_bits(boff[k + 1] - first) : mk[dc] & mk[kClasses + sc];
+        if (active) m = skip ? first_bits(boff[k + 1] - first) : mk[dc * kBuckets] & mk[(kClasses + sc) * kBuckets];
         do {
             uint32_t seg = 0xFFFFFFFFu;
             while (m) {
@@ -1616,7 +1590,7 @@ __device__ __forceinline__ uint32_t first_match_lane(const uint8_t *sm, uint32_t
         return result;
     }
     Candidates cand(0u, first, boff[k + 1]);
-    if (active) cand.m = skip ? cand.all() : mk[dc] & mk[kClasses + sc];
+    if (active) cand.m = skip ? cand.all() : mk[dc * kBuckets] & mk[(kClasses + sc) * kBuckets];
     bool done = !active;
     while (__any_sync(PV_FULL_MASK, !done)) {
         uint32_t seg = 0xFFFFFFFFu;
@@ -1678,7 +1652,7 @@ __device__ __forceinline__ void hop_outcome(const HopArgs &g, const uint2 *ports
 // in_port is the source host's port (so a live probe never bounces) and no
 // cycle check is due, so all of that is left out.
 template <bool kIndexed, bool kPolicy, bool kStats, bool kRec, bool kFirst>
-__global__ void __launch_bounds__(kHopThreads, 4) walk_hop_kernel(HopArgs g) {
+__global__ void __launch_bounds__(kHopThreads, kFirst ? 4 : 4) walk_hop_kernel(HopArgs g) {
     extern __shared__ __align__(128) uint8_t s_raw[];
     __shared__ uint64_t s_bar;
     __shared__ uint32_t s_count;
@@ -1925,8 +1899,8 @@ __device__ __forceinline__ uint32_t first_match_thread(const uint8_t *__restrict
     const uint2 *segs = reinterpret_cast<const uint2 *>(blob + L.segs);
     const uint2 *bw = reinterpret_cast<const uint2 *>(blob + L.bw);
     const uint32_t k = dport >> kBucketShift;
-    const uint32_t *mk = masks + k * (2 * kClasses);
-    Candidates cand(__ldg(mk + dc) & __ldg(mk + kClasses + sc), __ldg(boff + k), __ldg(boff + k + 1));
+    const uint32_t *mk = masks + k;
+    Candidates cand(__ldg(mk + dc * kBuckets) & __ldg(mk + (kClasses + sc) * kBuckets), __ldg(boff + k), __ldg(boff + k + 1));
     constexpr uint32_t kNone = 0xFFFFu;
     while (true) {
         uint32_t it[2] = {kNone, kNone};
@@ -2765,30 +2739,26 @@ int walk_probes(pv_ctx *ctx, uint32_t M, const pv_probe *d_probes, uint32_t hop_
             flow_groups_kernel<false><<<gb, kGridThreads, 0, st>>>(M, t.num_hosts, t.d_host_switch, t.d_region, pa0,
                                                                   ba0, G, hist, pair_off);
         walk_scan_kernel<<<1, 1024, 0, st>>>(S, hist, seg, cursor);
-        const uint32_t groups32 = (uint32_t)groups;
-        const size_t gsm = ba->ppg <= 0xFFFFu ? GroupInitSmem(ba->pods, ba->ppg, ba->dst_stride == 2).total : ~(size_t)0;
-        const bool by_group = ba->pods <= kGroupInitMaxPods && gsm <= kGroupInitSmem && groups <= 0x7FFFFFFFull;
+        // (ppg is bounded first: the layout's sizes are 32-bit)
+        const size_t gsm = ba->ppg <= 0xFFFFu ? GroupInitSmem(ba->ppg, ba->dst_stride == 2).total : ~(size_t)0;
+        const bool by_group = ba->ppg >= kGroupInitMin && ba->pods <= kGroupInitMaxPods && gsm <= kGroupInitSmem;
         if (by_group) {
             const int rc2 = pol ? pv_smem_limit(ctx, (const void *)walk_init_group_kernel<true>, "walk_init_group_kernel smem")
                                 : pv_smem_limit(ctx, (const void *)walk_init_group_kernel<false>, "walk_init_group_kernel smem");
             if (rc2) return rc2;
         }
         if (by_group && pol)
-            walk_init_group_kernel<true><<<groups32, kGroupInitThreads, gsm, st>>>(
-                M, probes_rw, t.num_hosts, t.d_host_switch, t.d_region, d_out, recs, seg,
-                pair_off, pa0, ba0, g.wait_ns, ctx->d_status);
+            walk_init_group_kernel<true><<<(uint32_t)groups, kGroupInitThreads, gsm, st>>>(
+                M, probes_rw, t.num_hosts, t.d_host_switch, d_out, recs, seg, pair_off, pa0, ba0, g.wait_ns, ctx->d_status);
         else if (by_group)
-            walk_init_group_kernel<false><<<groups32, kGroupInitThreads, gsm, st>>>(
-                M, probes_rw, t.num_hosts, t.d_host_switch, t.d_region, d_out, recs, seg,
-                pair_off, pa0, ba0, g.wait_ns, ctx->d_status);
+            walk_init_group_kernel<false><<<(uint32_t)groups, kGroupInitThreads, gsm, st>>>(
+                M, probes_rw, t.num_hosts, t.d_host_switch, d_out, recs, seg, pair_off, pa0, ba0, g.wait_ns, ctx->d_status);
         else if (pol)
             walk_init_direct_kernel<true><<<init_grid, kGridThreads, 0, st>>>(
-                M, probes_rw, t.num_hosts, t.d_host_switch, t.d_region, d_out, recs, seg,
-                pair_off, pa0, ba0);
+                M, probes_rw, t.num_hosts, t.d_host_switch, d_out, recs, seg, pair_off, pa0, ba0);
         else
             walk_init_direct_kernel<false><<<init_grid, kGridThreads, 0, st>>>(
-                M, probes_rw, t.num_hosts, t.d_host_switch, t.d_region, d_out, recs, seg,
-                pair_off, pa0, ba0);
+                M, probes_rw, t.num_hosts, t.d_host_switch, d_out, recs, seg, pair_off, pa0, ba0);
     } else if (pol && ba)
         walk_init_kernel<true, true><<<init_grid, kGridThreads, init_smem, st>>>(
             M, probes_rw, t.num_hosts, t.d_host_switch, t.d_host_port, t.d_region, d_out, listA, descA, pa0, S, hist,
