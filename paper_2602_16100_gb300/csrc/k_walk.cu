@@ -35,6 +35,7 @@ namespace {
 constexpr int kHopThreads = 256;
 constexpr int kHopWarps = kHopThreads / 32;
 constexpr uint32_t kMinPerBlock = 512;       // live probes per active hop block
+constexpr uint32_t kHopShare = 20480;        // probes per hop block before there are more blocks than fit at once
 // Batches of at most this many probes walk in one walk_thread_kernel launch
 // (indexed tables, tail hop left to the library).  Regrouping by switch costs
 // about 10 us of launches per hop and a table stage per occupied switch,
@@ -2692,8 +2693,14 @@ int walk_probes(pv_ctx *ctx, uint32_t M, const pv_probe *d_probes, uint32_t hop_
     if (int rc = pv_smem_limit(ctx, (const void *)hop_fn, "walk_hop_kernel smem")) return rc;
     if (int rc = pv_smem_limit(ctx, (const void *)hop_fn0, "walk_hop_kernel smem")) return rc;
     hop_blocks_per_sm = pv_blocks_per_sm(ctx, (const void *)hop_fn, kHopThreads, hop_smem);
-    const uint32_t hop_grid = std::min((uint32_t)ctx->num_sms * (uint32_t)std::max(1, hop_blocks_per_sm),
-                                       ctx->walk_visit_slots);
+    // hop blocks: the resident ones, or up to four times as many when each
+    // still has kHopShare probes, because shares of equal size take unequal time
+    // (50 million flows, 1 / 2 / 4 / 8 times: first hop 486 / 475 / 465 / 469 us,
+    // regroup after it 72 / 53 / 48 / 47, whole pass 1338 / 1308 / 1280 / -; 20
+    // million 606 / 613 / 616, 10 million probes on a fat tree 691 / 714 / 760)
+    const uint32_t resident = (uint32_t)ctx->num_sms * (uint32_t)std::max(1, hop_blocks_per_sm);
+    const uint32_t shares = std::min(4u, std::max(1u, M / (resident * kHopShare)));
+    const uint32_t hop_grid = std::min(resident * shares, ctx->walk_visit_slots);
     const uint32_t init_grid = (uint32_t)ctx->num_sms * 8;
     const uint32_t max_desc = std::max(hop_grid, init_grid);
     const size_t o_a = 0, o_b = align256((size_t)M * 8), o_sorted = o_b + align256((size_t)M * 8);
