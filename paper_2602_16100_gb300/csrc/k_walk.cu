@@ -251,6 +251,7 @@ static_assert(kIndexThreads / 32 == 16, "bucket fill counts are laid out for 16 
 // rule classes, segment bounds, one segment's prefixes and actions, and the
 // bucket fill's per-warp counts and cursors.
 constexpr uint32_t kIndexWarps = 512 / 32;
+constexpr uint32_t kSortMin = 64;           // smallest block_sort
 static_assert(PV_MAX_RULES * 4 <= kMaxSegment * 10, "plain-rule ranks overlay one segment's staging area");
 static_assert(PV_MAX_RULES < kSegItem, "plain-rule positions fit an item below the segment flag");
 struct IndexSmem {
@@ -261,7 +262,7 @@ struct IndexSmem {
         const uint32_t n = max_rules < 1 ? 1 : max_rules;
         seg_cap = n < kMaxSegment ? n : kMaxSegment;
         const uint32_t need = 2 * seg_cap + 1 > n ? 2 * seg_cap + 1 : n;
-        sort_cap = 1;
+        sort_cap = kSortMin;
         while (sort_cap < need) sort_cap <<= 1;
         key_cap = 2 * seg_cap + 8 > kBuckets + 8 ? 2 * seg_cap + 8 : kBuckets + 8;
         key_cap = (key_cap + 1) & ~1u;
@@ -381,6 +382,72 @@ __device__ uint32_t block_exclusive_scan(uint32_t *v, uint32_t n, uint32_t *s_wa
     return total;
 }
 
+// Ascending bitonic sort of n keys (a power of two from kSortMin) by the block.
+// Steps between elements less than 64 apart run in a warp's registers, two
+// neighbours per lane, so that only the wide ones go through shared memory and
+// a barrier: 10 of 55 for 1,024 keys.
+__device__ __forceinline__ void block_sort(uint32_t *keys, uint32_t n) {
+    const uint32_t t = threadIdx.x, nt = blockDim.x, lane = t & 31;
+    // for every 64 keys: the steps of stage kk from distance 32 (or kk / 2) down
+    auto stage = [&](uint2 &e, uint32_t i, uint32_t kk) {
+        const bool up = (i & kk) == 0;
+#pragma unroll
+        for (uint32_t d = 16; d; d >>= 1) {
+            if (2 * d >= kk) continue;
+            const uint32_t x = __shfl_xor_sync(PV_FULL_MASK, e.x, d), y = __shfl_xor_sync(PV_FULL_MASK, e.y, d);
+            const bool low = ((lane & d) == 0) == up;
+            e.x = low ? min(e.x, x) : max(e.x, x);
+            e.y = low ? min(e.y, y) : max(e.y, y);
+        }
+        const uint32_t lo = min(e.x, e.y), hi = max(e.x, e.y);
+        e = up ? make_uint2(lo, hi) : make_uint2(hi, lo);
+    };
+    uint2 *pairs = reinterpret_cast<uint2 *>(keys);
+    for (uint32_t p = t; p < n / 2; p += nt) {   // whole warps: n / 2 is a multiple of 32
+        uint2 e = pairs[p];
+#pragma unroll
+        for (uint32_t kk = 2; kk <= 64; kk <<= 1) stage(e, 2 * p, kk);
+        pairs[p] = e;
+    }
+    __syncthreads();
+    for (uint32_t kk = 128; kk <= n; kk <<= 1) {
+        for (uint32_t jj = kk >> 1; jj >= 64; jj >>= 1) {
+            for (uint32_t p = t; p < n / 2; p += nt) {
+                const uint32_t i = 2 * (p & ~(jj - 1)) | (p & (jj - 1));
+                const uint32_t a = keys[i], b = keys[i + jj];
+                if ((a > b) == ((i & kk) == 0)) {
+                    keys[i] = b;
+                    keys[i + jj] = a;
+                }
+            }
+            __syncthreads();
+        }
+        for (uint32_t p = t; p < n / 2; p += nt) {
+            uint2 e = pairs[p];
+            stage(e, 2 * p, kk);
+            pairs[p] = e;
+        }
+        __syncthreads();
+    }
+}
+
+// Transposes a 32 x 32 bit matrix, a row per lane (bit c of lane r becomes bit
+// r of lane c): five exchanges of half of every row.
+__device__ __forceinline__ uint32_t transpose_bits(uint32_t x, uint32_t lane) {
+    uint32_t low = 0x0000FFFFu;   // columns without bit d
+#pragma unroll
+    for (uint32_t d = 16; d; d >>= 1) {
+        const uint32_t y = __shfl_xor_sync(PV_FULL_MASK, x, d);
+        x = lane & d ? (x & ~low) | ((y & ~low) >> d) : (x & low) | ((y & low) << d);
+        low ^= low << (d >> 1);
+    }
+    return x;
+}
+
+// What bounds it: instruction issue (four blocks per SM).  512 switches of 1,000
+// rules, pass 1 / pass 2: 79 / 162 us with a sort step per barrier, sixteen
+// ballots per bucket for the filter and an atomic per bucket of every rule; 40 /
+// 82 with block_sort, transpose_bits and differences.
 // Pass 1 (kFill = false) writes sizes[4s..4s+3] = {n_items, n_segs, n_bnd,
 // n_plain}; pass 2 writes the blob at blob_offs[s].  One kIndexThreads-thread block per switch.
 template <bool kFill>
@@ -498,16 +565,27 @@ __global__ void __launch_bounds__(kIndexThreads) index_build_kernel(const uint32
         return ((pr >> 16) >> kBucketShift) - *b0 + 1u;
     };
     uint32_t *s_poff = s_win;   // [n]: first pair of rule i (s_win is free until step 3)
-    for (uint32_t k = t; k < kBuckets; k += nt) s_pos[k] = 0;
+    for (uint32_t k = t; k <= kBuckets; k += nt) s_pos[k] = 0;
     for (uint32_t x = t; x < kIndexWarps * kBuckets; x += nt) s_wcnt[x] = 0;
     __syncthreads();
     for (uint32_t i = t; i < n; i += nt) {
         uint32_t b0;
         const uint32_t nb = bucket_range(i, &b0);
         s_poff[i] = nb;
-        for (uint32_t k = b0; k < b0 + nb; ++k) atomicAdd(&s_pos[k], 1u);
+        if (nb) {   // items per bucket: the sums of these
+            atomicAdd(&s_pos[b0], 1u);
+            atomicSub(&s_pos[b0 + nb], 1u);
+        }
     }
     __syncthreads();
+    block_exclusive_scan(s_pos, kBuckets + 1, s_warp);   // s_pos[k + 1] = items of bucket k
+    {
+        static_assert(kBuckets <= kIndexThreads, "a thread per bucket");
+        const uint32_t mine = t < kBuckets ? s_pos[t + 1] : 0u;
+        __syncthreads();
+        if (t < kBuckets) s_pos[t] = mine;
+        __syncthreads();
+    }
     const uint32_t n_items = block_exclusive_scan(s_pos, kBuckets, s_warp);   // s_pos[k] = first item of bucket k
     if (kFill) {
         uint32_t *boff = reinterpret_cast<uint32_t *>(out + L.boff);
@@ -558,12 +636,58 @@ __global__ void __launch_bounds__(kIndexThreads) index_build_kernel(const uint32
     }
     __syncthreads();
 
+    __syncthreads();
+
+    // candidate filter: each plain rule's classes once, then a warp per bucket
+    // and a lane per group of items, whose class bits are transposed into the
+    // sixteen words (two buckets at once; the items were written above by this
+    // block, four buckets' are read together)
+    if (kFill) {
+        uint32_t *s_meets = s_keys;   // [n_plain] bit c: destination class c, bit kClasses + c: source class c
+        for (uint32_t i = t; i < n; i += nt) {
+            if (s_cls[i] >= 0) continue;
+            const uint4 r = a[i];   // {src, its mask, dst, its mask}
+            const uint32_t sc = (2u << addr_class(cls, r.x | ~r.y)) - (1u << addr_class(cls, r.x));
+            const uint32_t dc = (2u << addr_class(cls, r.z | ~r.w)) - (1u << addr_class(cls, r.z));
+            s_meets[s_plain[i]] = dc | sc << kClasses;
+        }
+        __syncthreads();
+        const uint16_t *items = reinterpret_cast<const uint16_t *>(out + L.items);
+        uint32_t *masks = reinterpret_cast<uint32_t *>(out + L.masks);
+        constexpr uint32_t kAtOnce = 4;
+        for (uint32_t k0 = warp * kAtOnce; k0 < kBuckets; k0 += kIndexWarps * kAtOnce) {
+            uint32_t it[kAtOnce], i0[kAtOnce], len[kAtOnce], meets[kAtOnce];
+#pragma unroll
+            for (uint32_t j = 0; j < kAtOnce; ++j) {
+                i0[j] = s_pos[k0 + j];
+                len[j] = (k0 + j + 1 < kBuckets ? s_pos[k0 + j + 1] : n_items) - i0[j];
+                it[j] = lane < len[j] ? items[i0[j] + lane] : 0u;
+            }
+#pragma unroll
+            for (uint32_t j = 0; j < kAtOnce; ++j) {
+                const uint32_t per = (len[j] + 31) / 32;
+                meets[j] = 0;
+                for (uint32_t q = lane * per; q < min(len[j], (lane + 1) * per); ++q) {
+                    const uint32_t x = per == 1 ? it[j] : items[i0[j] + q];
+                    meets[j] |= x & kSegItem ? 0xFFFFu : s_meets[x];
+                }
+            }
+            // lane c of the first half: class c of the first of two buckets
+            const uint32_t m0 = transpose_bits(meets[0] | meets[1] << 16, lane);
+            const uint32_t m1 = transpose_bits(meets[2] | meets[3] << 16, lane);
+            uint32_t *w = masks + (lane & 15u) * kBuckets + k0 + (lane >> 4);
+            w[0] = m0;
+            w[2] = m1;
+        }
+        __syncthreads();
+    }
+
     // 3. per segment: sorted unique boundaries, interval winners, merged runs
     uint32_t n_bnd = 0;
     for (uint32_t j = 0; j < nsegs; ++j) {
         const uint32_t k0 = s_segs[2 * j], k1 = s_segs[2 * j + 1], m = k1 - k0;
         const uint32_t nk = 2 * m + 1;
-        uint32_t npow = 1;
+        uint32_t npow = kSortMin;
         while (npow < nk) npow <<= 1;
         for (uint32_t x = t; x < npow; x += nt) {
             uint32_t key = 0xFFFFFFFFu;
@@ -581,20 +705,7 @@ __global__ void __launch_bounds__(kIndexThreads) index_build_kernel(const uint32
             s_keys[x] = key;
         }
         __syncthreads();
-        for (uint32_t kk = 2; kk <= npow; kk <<= 1)
-            for (uint32_t jj = kk >> 1; jj > 0; jj >>= 1) {
-                for (uint32_t i = t; i < npow; i += nt) {
-                    const uint32_t ixj = i ^ jj;
-                    if (ixj > i) {
-                        const uint32_t p = s_keys[i], q = s_keys[ixj];
-                        if ((p > q) == ((i & kk) == 0)) {
-                            s_keys[i] = q;
-                            s_keys[ixj] = p;
-                        }
-                    }
-                }
-                __syncthreads();
-            }
+        block_sort(s_keys, npow);
         for (uint32_t x = t; x < nk; x += nt) s_pos[x] = (x == 0 || s_keys[x] != s_keys[x - 1]) ? 1u : 0u;
         __syncthreads();
         for (uint32_t x = t; x < nk; x += nt) s_win[x] = s_keys[x];   // keep sorted copy
@@ -693,42 +804,7 @@ __global__ void __launch_bounds__(kIndexThreads) index_build_kernel(const uint32
         __syncthreads();
     }
 
-    // 4. candidate filter: a warp per bucket, a lane per group of items; the
-    //    sixteen words come from ballots (items and rules were written above
-    //    by this block)
-    if (kFill) {
-        __syncthreads();
-        const uint32_t *boff = reinterpret_cast<const uint32_t *>(out + L.boff);
-        const uint16_t *items = reinterpret_cast<const uint16_t *>(out + L.items);
-        const uint4 *rules = reinterpret_cast<const uint4 *>(out + L.rules);
-        uint32_t *masks = reinterpret_cast<uint32_t *>(out + L.masks);
-        for (uint32_t k = warp; k < kBuckets; k += kIndexWarps) {
-            const uint32_t i0 = boff[k], len = boff[k + 1] - i0, per = (len + 31) / 32;
-            uint32_t meets = 0;   // bit c: destination class c, bit kClasses + c: source class c
-            for (uint32_t q = lane * per; q < min(len, (lane + 1) * per); ++q) {
-                const uint32_t it = items[i0 + q];
-                if (it & kSegItem) {
-                    meets = 0xFFFFu;
-                    continue;
-                }
-                const uint4 r = rules[it];
-                const uint32_t sh = (r.w >> 8) & 63u, dh = (r.w >> 14) & 63u;   // host bits
-                const uint32_t s1 = r.x | (sh < 32 ? (1u << sh) - 1u : ~0u), d1 = r.y | (dh < 32 ? (1u << dh) - 1u : ~0u);
-                const uint32_t sc = (2u << addr_class(cls, s1)) - (1u << addr_class(cls, r.x));
-                const uint32_t dc = (2u << addr_class(cls, d1)) - (1u << addr_class(cls, r.y));
-                meets |= dc | sc << kClasses;
-            }
-            uint32_t mine = 0;
-#pragma unroll
-            for (uint32_t c = 0; c < 2 * kClasses; ++c) {
-                const uint32_t word = __ballot_sync(PV_FULL_MASK, (meets >> c) & 1u);
-                if (lane == c) mine = word;
-            }
-            if (lane < 2 * kClasses) masks[lane * kBuckets + k] = mine;
-        }
-    }
-
-    // 5. header and the full rule list
+    // 4. header and the full rule list
     if (kFill) {
         if (t == 0) *reinterpret_cast<uint4 *>(out) = make_uint4(npad | n_plain << 16, n_items, nsegs, n_bnd);
         uint4 *oa = reinterpret_cast<uint4 *>(out + L.fa);
