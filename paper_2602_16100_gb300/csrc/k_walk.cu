@@ -119,17 +119,75 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t *bar, uint32_t parity
 }
 
 // ---------------------------------------------------------------------------
+// load: sorting
+// ---------------------------------------------------------------------------
+constexpr uint32_t kSortMin = 64;   // smallest block_sort
+
+// Ascending bitonic sort of n keys (a power of two from kSortMin) by the block.
+// Steps between elements less than 64 apart run in a warp's registers, two
+// neighbours per lane, so that only the wide ones go through shared memory and
+// a barrier: 10 of 55 for 1,024 keys.
+__device__ __forceinline__ void block_sort(uint32_t *keys, uint32_t n) {
+    const uint32_t t = threadIdx.x, nt = blockDim.x, lane = t & 31;
+    // for every 64 keys: the steps of stage kk from distance 32 (or kk / 2) down
+    auto stage = [&](uint2 &e, uint32_t i, uint32_t kk) {
+        const bool up = (i & kk) == 0;
+#pragma unroll
+        for (uint32_t d = 16; d; d >>= 1) {
+            if (2 * d >= kk) continue;
+            const uint32_t x = __shfl_xor_sync(PV_FULL_MASK, e.x, d), y = __shfl_xor_sync(PV_FULL_MASK, e.y, d);
+            const bool low = ((lane & d) == 0) == up;
+            e.x = low ? min(e.x, x) : max(e.x, x);
+            e.y = low ? min(e.y, y) : max(e.y, y);
+        }
+        const uint32_t lo = min(e.x, e.y), hi = max(e.x, e.y);
+        e = up ? make_uint2(lo, hi) : make_uint2(hi, lo);
+    };
+    uint2 *pairs = reinterpret_cast<uint2 *>(keys);
+    for (uint32_t p = t; p < n / 2; p += nt) {   // whole warps: n / 2 is a multiple of 32
+        uint2 e = pairs[p];
+#pragma unroll
+        for (uint32_t kk = 2; kk <= 64; kk <<= 1) stage(e, 2 * p, kk);
+        pairs[p] = e;
+    }
+    __syncthreads();
+    for (uint32_t kk = 128; kk <= n; kk <<= 1) {
+        for (uint32_t jj = kk >> 1; jj >= 64; jj >>= 1) {
+            for (uint32_t p = t; p < n / 2; p += nt) {
+                const uint32_t i = 2 * (p & ~(jj - 1)) | (p & (jj - 1));
+                const uint32_t a = keys[i], b = keys[i + jj];
+                if ((a > b) == ((i & kk) == 0)) {
+                    keys[i] = b;
+                    keys[i + jj] = a;
+                }
+            }
+            __syncthreads();
+        }
+        for (uint32_t p = t; p < n / 2; p += nt) {
+            uint2 e = pairs[p];
+            stage(e, 2 * p, kk);
+            pairs[p] = e;
+        }
+        __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------------------
 // load: per-switch stable priority sort + compile
 // ---------------------------------------------------------------------------
 // Also validates every rule of the switch against its port count; the lowest
 // offending global rule index goes to *bad (0xFFFFFFFF when all are valid).
-__global__ void __launch_bounds__(1024) compile_tables_kernel(const uint32_t *__restrict__ rule_offs,
+// 512 threads: four blocks per SM, so 512 switches run at once.  Bound by
+// instruction issue, most of it the sort (512 switches of 1,000 rules
+// 37 us with 1,024 threads and a barrier per sort step, 16 now).
+constexpr int kCompileThreads = 512;
+__global__ void __launch_bounds__(kCompileThreads) compile_tables_kernel(const uint32_t *__restrict__ rule_offs,
                                                               const pv_rule *__restrict__ raw,
                                                               const uint32_t *__restrict__ port_offs,
                                                               const uint32_t *__restrict__ tab_offs,
                                                               uint4 *__restrict__ A, uint2 *__restrict__ B,
                                                               uint32_t *__restrict__ bad) {
-    extern __shared__ uint32_t s_keys[];
+    extern __shared__ __align__(16) uint32_t s_keys[];
     const uint32_t s = blockIdx.x, t = threadIdx.x;
     const uint32_t base = rule_offs[s], n = rule_offs[s + 1] - base;
     const uint32_t nports = port_offs[s + 1] - port_offs[s];
@@ -140,26 +198,12 @@ __global__ void __launch_bounds__(1024) compile_tables_kernel(const uint32_t *__
                         r.dport_lo <= r.dport_hi;
         if (!ok) atomicMin(bad, base + i);
     }
-    uint32_t npow = 1;
+    uint32_t npow = kSortMin;
     while (npow < n) npow <<= 1;
     for (uint32_t i = t; i < npow; i += blockDim.x)
         s_keys[i] = i < n ? ((uint32_t)(65535u - raw[base + i].priority) << 16) | i : 0xFFFFFFFFu;
     __syncthreads();
-    for (uint32_t k = 2; k <= npow; k <<= 1)
-        for (uint32_t j = k >> 1; j > 0; j >>= 1) {
-            for (uint32_t i = t; i < npow; i += blockDim.x) {
-                uint32_t ixj = i ^ j;
-                if (ixj > i) {
-                    uint32_t a = s_keys[i], b = s_keys[ixj];
-                    bool up = (i & k) == 0;
-                    if ((a > b) == up) {
-                        s_keys[i] = b;
-                        s_keys[ixj] = a;
-                    }
-                }
-            }
-            __syncthreads();
-        }
+    block_sort(s_keys, npow);
     const uint32_t out = tab_offs[s], npad = tab_offs[s + 1] - out;
     for (uint32_t i = t; i < npad; i += blockDim.x) {
         uint4 a;
@@ -251,7 +295,6 @@ static_assert(kIndexThreads / 32 == 16, "bucket fill counts are laid out for 16 
 // rule classes, segment bounds, one segment's prefixes and actions, and the
 // bucket fill's per-warp counts and cursors.
 constexpr uint32_t kIndexWarps = 512 / 32;
-constexpr uint32_t kSortMin = 64;           // smallest block_sort
 static_assert(PV_MAX_RULES * 4 <= kMaxSegment * 10, "plain-rule ranks overlay one segment's staging area");
 static_assert(PV_MAX_RULES < kSegItem, "plain-rule positions fit an item below the segment flag");
 struct IndexSmem {
@@ -380,55 +423,6 @@ __device__ uint32_t block_exclusive_scan(uint32_t *v, uint32_t n, uint32_t *s_wa
     const uint32_t total = s_warp[32];
     __syncthreads();
     return total;
-}
-
-// Ascending bitonic sort of n keys (a power of two from kSortMin) by the block.
-// Steps between elements less than 64 apart run in a warp's registers, two
-// neighbours per lane, so that only the wide ones go through shared memory and
-// a barrier: 10 of 55 for 1,024 keys.
-__device__ __forceinline__ void block_sort(uint32_t *keys, uint32_t n) {
-    const uint32_t t = threadIdx.x, nt = blockDim.x, lane = t & 31;
-    // for every 64 keys: the steps of stage kk from distance 32 (or kk / 2) down
-    auto stage = [&](uint2 &e, uint32_t i, uint32_t kk) {
-        const bool up = (i & kk) == 0;
-#pragma unroll
-        for (uint32_t d = 16; d; d >>= 1) {
-            if (2 * d >= kk) continue;
-            const uint32_t x = __shfl_xor_sync(PV_FULL_MASK, e.x, d), y = __shfl_xor_sync(PV_FULL_MASK, e.y, d);
-            const bool low = ((lane & d) == 0) == up;
-            e.x = low ? min(e.x, x) : max(e.x, x);
-            e.y = low ? min(e.y, y) : max(e.y, y);
-        }
-        const uint32_t lo = min(e.x, e.y), hi = max(e.x, e.y);
-        e = up ? make_uint2(lo, hi) : make_uint2(hi, lo);
-    };
-    uint2 *pairs = reinterpret_cast<uint2 *>(keys);
-    for (uint32_t p = t; p < n / 2; p += nt) {   // whole warps: n / 2 is a multiple of 32
-        uint2 e = pairs[p];
-#pragma unroll
-        for (uint32_t kk = 2; kk <= 64; kk <<= 1) stage(e, 2 * p, kk);
-        pairs[p] = e;
-    }
-    __syncthreads();
-    for (uint32_t kk = 128; kk <= n; kk <<= 1) {
-        for (uint32_t jj = kk >> 1; jj >= 64; jj >>= 1) {
-            for (uint32_t p = t; p < n / 2; p += nt) {
-                const uint32_t i = 2 * (p & ~(jj - 1)) | (p & (jj - 1));
-                const uint32_t a = keys[i], b = keys[i + jj];
-                if ((a > b) == ((i & kk) == 0)) {
-                    keys[i] = b;
-                    keys[i + jj] = a;
-                }
-            }
-            __syncthreads();
-        }
-        for (uint32_t p = t; p < n / 2; p += nt) {
-            uint2 e = pairs[p];
-            stage(e, 2 * p, kk);
-            pairs[p] = e;
-        }
-        __syncthreads();
-    }
 }
 
 // Transposes a 32 x 32 bit matrix, a row per lane (bit c of lane r becomes bit
@@ -2433,12 +2427,12 @@ int tables_begin(pv_ctx *ctx, pv_table_load &L, uint32_t S, const uint32_t *rule
     L.max_rules = maxn;
     const IndexSmem ism(maxn);
     if (e == cudaSuccess) {
-        uint32_t npow = 1;
+        uint32_t npow = kSortMin;
         while (npow < maxn) npow <<= 1;
         uint32_t *d_bad = d_sizes + (size_t)S * 4;   // lowest invalid rule index
         e = cudaMemsetAsync(d_bad, 0xFF, 4, ls);
         if (e == cudaSuccess) {
-            compile_tables_kernel<<<S, 1024, npow * 4, ls>>>(d_rule_offs, t.d_raw, t.d_port_offs, d_tab_offs,
+            compile_tables_kernel<<<S, kCompileThreads, npow * 4, ls>>>(d_rule_offs, t.d_raw, t.d_port_offs, d_tab_offs,
                                                              d_rule_a, d_rule_b, d_bad);
             e = cudaGetLastError();
         }
