@@ -8,10 +8,13 @@
 // shortest segments, each made canonical: walking back from the segment's
 // end, every switch takes the predecessor link with the smallest (source
 // switch, source port) among those on a shortest path.  Any exact shortest-
-// path algorithm therefore yields the same path; one block per request runs
-// in-place Bellman-Ford pull sweeps over the links into each switch (every
-// sweep only lowers upper bounds, so the fixpoint is exact), all in shared
-// memory, and one thread walks the predecessors back.
+// path algorithm therefore yields the same path.  A warp per segment searches
+// from the frontier of switches whose distance fell, bounded by the target's
+// (sched_segments_kernel); networks whose state does not fit, and the options,
+// run one block per request with in-place Bellman-Ford pull sweeps over the
+// links into each switch (every sweep only lowers upper bounds, so the fixpoint
+// is exact), all in shared memory, and one thread walks the predecessors back
+// (sched_paths_kernel).
 #include <cuda_runtime.h>
 
 #include <algorithm>

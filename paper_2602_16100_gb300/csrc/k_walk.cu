@@ -13,16 +13,21 @@
 // so a rule matches iff ((src^A.x)&A.y | (dst^A.z)&A.w | (in^B.y)&mask) == 0
 // and lo <= dport <= hi.
 //
-// A walk runs one hop for all live probes per step:
-//   regroup  : histogram of live probes by current switch, exclusive scan,
-//              block-aggregated scatter into switch-contiguous order;
+// Small batches walk in one launch, a thread per probe over the tables in L2
+// (walk_thread_kernel).  Larger ones run one hop for all live probes per step:
+//   regroup  : counts of live probes by current switch (from the kernel that
+//              listed them), exclusive scan, block-aggregated scatter into
+//              switch-contiguous order; compact flows start in that order;
 //   hop      : each block takes a contiguous range of that order, stages
 //              the range's switch tables into shared memory with a
 //              (non-multicast) cp.async.bulk copy completed on an mbarrier,
-//              and each warp resolves first-match for one probe at a time,
-//              32 rules per step, with __ballot_sync / __ffs.  Terminated
-//              probes write their result; live ones are appended (block-
-//              aggregated) to the next hop's list.
+//              and each warp resolves 32 probes' first matches, one per lane
+//              over the first-match index (one probe at a time, 32 items per
+//              step, where lists are long; 32 rules per step over the full
+//              list where the index does not fit).  Terminated probes write
+//              their result; live ones are appended (block-aggregated) to the
+//              next hop's list;
+// and the few probes left after some hops finish in one thread walk.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -40,17 +45,20 @@ constexpr uint32_t kHopShare = 20480;        // probes per hop block before ther
 // (indexed tables, tail hop left to the library).  Regrouping by switch costs
 // about 10 us of launches per hop and a table stage per occupied switch,
 // whatever the batch; the thread walk costs its L2 round trips.  Thread walk
-// against regrouped walk, us, at 1k / 100k / 800k / 1.6M / 3.2M probes:
-//   ring of 8, 64 rules       11/126   13/128   35/137   60/148  111/172
-//   mesh of 512, 1,000 rules  45/108   62/173  159/225  276/262  510/311
-//   fat tree, 2,000 rules     82/193  115/292  300/398  500/461  897/583
-// and compact flows of 512 switches at 1M: 223/231 (270/267 with policies).
-// The lines cross between 1M and 2M on the large tables.
+// against regrouped walk, us, at 200k / 400k / 600k / 800k / 1M probes:
+//   mesh of 512, 1,000 rules   59/94   72/108   84/109  101/117  119/127
+//   mesh of 64, 200 rules      33/69   40/71    49/71    56/76    66/82
+//   fat tree, 1,000 rules      65/111  84/115  105/121  126/133  150/145
+//   fat tree, 2,000 rules      82/132 103/134  135/149  154/167  181/182
+//   flows of 512 switches      81/105  95/104  118/114  128/120  144/132
+//   the same with policies     84/112 107/119  127/128  141/135  156/150
+// (a ring of 8 at 1k: 11/126).  The lines cross between 0.5M and 1.2M.
 constexpr uint32_t kThreadWalkMax = 1u << 20;
 // Larger batches: the hop from which the probes still walking finish in one
 // thread walk.  Live probes fall about 2.5 times a hop, and the thread walk
 // takes over best at some 400,000 of them, so one more hop is regrouped for
-// every factor 2.5 of the batch.  us at tail hop 1 / 2 / 3 / 4 / 5 / 6 / 8:
+// every factor 2.5 of the batch.  us at tail hop 1 / 2 / 3 / 4 / 5 / 6 / 8 (the hop
+// kernels have become about a tenth faster since, at every tail hop):
 //   mesh of 512, 3M probes    216  199  214  240  274  299  340
 //   fat tree, 10M probes      998  842  744  719  710  711  777
 //   compact flows, 3M         218  206  222  255  280  302  339
