@@ -45,14 +45,14 @@ constexpr uint32_t kHopShare = 20480;        // probes per hop block before ther
 // (indexed tables, tail hop left to the library).  Regrouping by switch costs
 // about 10 us of launches per hop and a table stage per occupied switch,
 // whatever the batch; the thread walk costs its L2 round trips.  Thread walk
-// against regrouped walk, us, at 200k / 400k / 600k / 800k / 1M probes:
-//   mesh of 512, 1,000 rules   59/94   72/108   84/109  101/117  119/127
-//   mesh of 64, 200 rules      33/69   40/71    49/71    56/76    66/82
-//   fat tree, 1,000 rules      65/111  84/115  105/121  126/133  150/145
-//   fat tree, 2,000 rules      82/132 103/134  135/149  154/167  181/182
-//   flows of 512 switches      81/105  95/104  118/114  128/120  144/132
-//   the same with policies     84/112 107/119  127/128  141/135  156/150
-// (a ring of 8 at 1k: 11/126).  The lines cross between 0.5M and 1.2M.
+// against regrouped walk, us, at 1.1M / 1.4M / 1.7M / 2M / 2.5M probes:
+//   mesh of 512, 1,000 rules   91/109 108/123 127/144 142/157 176/173
+//   mesh of 64, 200 rules      58/78   68/84   78/106  91/111 108/127
+//   fat tree, 1,000 rules     135/137 165/157 192/169 222/185 264/216
+//   fat tree, 2,000 rules     161/176 193/200 227/214 257/233 314/274
+//   flows of 512 switches     115/113 143/122 146/137 177/143 199/160
+//   the same with policies    128/135 159/135 162/155 199/165 222/186
+// (a ring of 8 at 1k: 11/126).  The lines cross between 1.1M and 2.4M.
 constexpr uint32_t kThreadWalkMax = 1u << 20;
 // Larger batches: the hop from which the probes still walking finish in one
 // thread walk.  Live probes fall about 2.5 times a hop, and the thread walk
@@ -1965,7 +1965,12 @@ __global__ void __launch_bounds__(kHopThreads, kFirst ? 4 : 4) walk_hop_kernel(H
 // First match of one probe by one thread, reading the switch's blob in place
 // (L2-resident tables).  Candidates are taken two at a time, both rules
 // loaded before either is tested: what a walk waits for here is the chain of
-// dependent L2 round trips.
+// dependent L2 round trips.  So does a
+// segment's jump block, from kJumpFrom boundaries on: two loads side by side and
+// two or three more where a search of 512 boundaries has ten in a row (100,000
+// probes on 512 switches 41.5 -> 32.3 us, 1 million 112 -> 85, 1 million flows
+// with policies 144 -> 117).
+constexpr uint32_t kJumpFrom = 16;
 template <bool kStats>
 __device__ __forceinline__ uint32_t first_match_thread(const uint8_t *__restrict__ blob, const BlobLayout &L,
                                                        uint32_t src, uint32_t dst, uint32_t dport,
@@ -1995,9 +2000,20 @@ __device__ __forceinline__ uint32_t first_match_thread(const uint8_t *__restrict
         for (uint32_t j = 0; j < 2; ++j) {
             if (it[j] == kNone) return 0u;   // no candidate left: table miss
             if (it[j] & kSegItem) {
+                const uint8_t *jb = blob + L.jmp + (it[j] & 0x7FFFu) * kJumpBytes;
                 const uint2 sd = __ldg(segs + (it[j] & 0x7FFFu));
+                const uint2 bs = __ldg(reinterpret_cast<const uint2 *>(jb));   // {base, shift}
                 uint32_t lo = 0, len = sd.y;   // the first interval starts at 0 <= dst
-                uint2 w = __ldg(bw + sd.x);
+                if (len > kJumpFrom) {
+                    if (dst < bs.x) {
+                        len = 1;
+                    } else {
+                        const uint16_t *J = reinterpret_cast<const uint16_t *>(jb + 8) + min((dst - bs.x) >> bs.y, kJumpSlots - 1);
+                        lo = __ldg(J);
+                        len = __ldg(J + 1) - lo + 1;
+                    }
+                }
+                uint2 w = __ldg(bw + sd.x + lo);
                 while (len > 1) {
                     const uint32_t half = len >> 1;
                     const uint2 c = __ldg(bw + sd.x + lo + half);
