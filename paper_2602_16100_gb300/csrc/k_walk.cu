@@ -2886,7 +2886,7 @@ int walk_probes(pv_ctx *ctx, uint32_t M, const pv_probe *d_probes, uint32_t hop_
     g.hist_off = (uint32_t)hist_off;
     g.port_off = (uint32_t)port_off;
     uint32_t in_slices = init_grid;
-    // hops from tail_hop on run in one walk_tail_kernel launch (indexed tables only)
+    // hops from tail_hop on run in one walk_thread_kernel launch (indexed tables only)
     const uint32_t opt_tail = ctx->opt_walk_tail_hop < 0 ? auto_tail_hop(M) : (uint32_t)ctx->opt_walk_tail_hop;
     const uint32_t tail_hop = (indexed && opt_tail > 0 && opt_tail < hop_cap) ? opt_tail : hop_cap;
     for (uint32_t h = 0; h < tail_hop; ++h) {
