@@ -1985,51 +1985,51 @@ __device__ __forceinline__ uint32_t first_match_thread(const uint8_t *__restrict
     const uint32_t k = dport >> kBucketShift;
     const uint32_t *mk = masks + k;
     Candidates cand(__ldg(mk + dc * kBuckets) & __ldg(mk + (kClasses + sc) * kBuckets), __ldg(boff + k), __ldg(boff + k + 1));
-    constexpr uint32_t kNone = 0xFFFFu;
-    while (true) {
-        uint32_t it[2] = {kNone, kNone};
-        uint4 r[2];
-#pragma unroll
-        for (uint32_t j = 0; j < 2; ++j) {
-            uint32_t i;
-            if (cand.next(&i)) it[j] = __ldg(items + i);
-        }
-#pragma unroll
-        for (uint32_t j = 0; j < 2; ++j) r[j] = (it[j] & kSegItem) ? make_uint4(0, 0, 0, 0) : __ldg(rules + it[j]);
-#pragma unroll
-        for (uint32_t j = 0; j < 2; ++j) {
-            if (it[j] == kNone) return 0u;   // no candidate left: table miss
-            if (it[j] & kSegItem) {
-                const uint8_t *jb = blob + L.jmp + (it[j] & 0x7FFFu) * kJumpBytes;
-                const uint2 sd = __ldg(segs + (it[j] & 0x7FFFu));
-                const uint2 bs = __ldg(reinterpret_cast<const uint2 *>(jb));   // {base, shift}
-                uint32_t lo = 0, len = sd.y;   // the first interval starts at 0 <= dst
-                if (len > kJumpFrom) {
-                    if (dst < bs.x) {
-                        len = 1;
-                    } else {
-                        const uint16_t *J = reinterpret_cast<const uint16_t *>(jb + 8) + min((dst - bs.x) >> bs.y, kJumpSlots - 1);
-                        lo = __ldg(J);
-                        len = __ldg(J + 1) - lo + 1;
-                    }
+    constexpr uint32_t kNone = 0xFFFFu, kOn = 1u;
+    // one candidate: the first match's result, 0 for a table miss, or kOn
+    auto decide = [&](uint32_t it, uint4 r) -> uint32_t {
+        if (it == kNone) return 0u;   // no candidate left
+        if (it & kSegItem) {
+            const uint8_t *jb = blob + L.jmp + (it & 0x7FFFu) * kJumpBytes;
+            const uint2 sd = __ldg(segs + (it & 0x7FFFu));
+            const uint2 bs = __ldg(reinterpret_cast<const uint2 *>(jb));   // {base, shift}
+            uint32_t lo = 0, len = sd.y;   // the first interval starts at 0 <= dst
+            if (len > kJumpFrom) {
+                if (dst < bs.x) {
+                    len = 1;
+                } else {
+                    const uint16_t *J = reinterpret_cast<const uint16_t *>(jb + 8) + min((dst - bs.x) >> bs.y, kJumpSlots - 1);
+                    lo = __ldg(J);
+                    len = __ldg(J + 1) - lo + 1;
                 }
-                uint2 w = __ldg(bw + sd.x + lo);
-                while (len > 1) {
-                    const uint32_t half = len >> 1;
-                    const uint2 c = __ldg(bw + sd.x + lo + half);
-                    if (c.x <= dst) {
-                        lo += half;
-                        w = c;
-                    }
-                    len -= half;
-                }
-                if (kStats) ++lookups;
-                if (w.y & kWinFound) return w.y;
-                continue;
             }
-            if (kStats) ++tests;
-            if (plain_hit(r[j], src, dst, dport, in_port)) return plain_result(r[j]);
+            uint2 w = __ldg(bw + sd.x + lo);
+            while (len > 1) {
+                const uint32_t half = len >> 1;
+                const uint2 c = __ldg(bw + sd.x + lo + half);
+                if (c.x <= dst) {
+                    lo += half;
+                    w = c;
+                }
+                len -= half;
+            }
+            if (kStats) ++lookups;
+            return w.y & kWinFound ? w.y : kOn;
         }
+        if (kStats) ++tests;
+        return plain_hit(r, src, dst, dport, in_port) ? plain_result(r) : kOn;
+    };
+    while (true) {
+        // (two named candidates: as arrays their rules went to local memory)
+        uint32_t i, it0 = kNone, it1 = kNone;
+        if (cand.next(&i)) it0 = __ldg(items + i);
+        if (cand.next(&i)) it1 = __ldg(items + i);
+        const uint4 none = make_uint4(0, 0, 0, 0);
+        const uint4 r0 = it0 & kSegItem ? none : __ldg(rules + it0), r1 = it1 & kSegItem ? none : __ldg(rules + it1);
+        uint32_t w = decide(it0, r0);
+        if (w != kOn) return w;
+        w = decide(it1, r1);
+        if (w != kOn) return w;
     }
 }
 
@@ -2049,7 +2049,8 @@ __device__ __forceinline__ uint32_t first_match_thread(const uint8_t *__restrict
 // Bound by the chain of dependent L2 round trips of one first match (about
 // ten) times the visits of a lane; drawing new probes keeps the other lanes
 // at work meanwhile.  1,000 probes on the ring: 130 us as 27 launches, 11 us
-// as this one; 100,003 probes on 512 switches: 175 -> 62 us.
+// as this one; 100,003 probes on 512 switches: 175 -> 32 us with the filter and
+// the jump blocks.
 enum { kSrcProbes = 0, kSrcFlows = 1, kSrcList = 2, kSrcListRec = 3 };
 
 struct ThreadWalkArgs {
