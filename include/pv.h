@@ -535,9 +535,10 @@ int pv_install_path_rules(pv_ctx *ctx, uint32_t num_slots, const pv_rule *d_rule
  * PV_OPT_WALK_TAIL_HOP: with the indexed kernel, the walk's hops from this
  *   one on (0 = none) run in a single launch, one thread per probe still
  *   walking, tables read from L2 instead of staged per switch.  Same
- *   results.  Default (-1): batches of at most 2^20 probes walk every hop
- *   that way, larger ones from a hop that grows with the batch (hop 2 at 3
- *   million probes, hop 5 at 50 million).
+ *   results.  Default (-1): batches of at most 2^20 probes (tables with a
+ *   list of 3,000 candidate rules: all batches) walk every hop that way,
+ *   larger ones from a hop that grows with the batch (hop 2 at 3 million
+ *   probes, hop 5 at 50 million).
  * PV_OPT_REACH_KERNEL: 0 = automatic (on a symmetric graph, rows are the
  *   connected components of the permitted subgraph; otherwise multi-source
  *   pull sweeps), 1 = sweeps always.  Both give the same rows.

@@ -68,6 +68,27 @@ inline uint32_t auto_tail_hop(uint32_t M) {
     for (uint64_t most = 1500000; M > most; most = most * 5 / 2) ++hop;
     return hop;
 }
+// The thread walk's form for long candidate lists (kLong), by the longest of the
+// tables: it costs the ordinary one's batches some 15% (a ballot and two
+// registers a visit), so it is taken where a lane's own list would hold the walk
+// up: from 96 items while the batch leaves lanes idle, from 256 while it fits one
+// launch, from 300 in the last hops of a regrouped walk.  Ordinary / long form, us,
+// host pairs that match late in ACLs of one port bucket:
+//   longest list     117       157       257        337        936       1,932
+//     1,000 probes   317/82    397/77    758/133    818/116  1839/198  2477/181
+//   100,000          391/390   683/436  1067/559   1425/623  3419/846  4307/878
+//   1 million       1886/2951 2425/3233 3701/3796  4523/4288 7672/4952 10732/5169
+//   4 million (the regrouped walk's last hops)
+//                   7240/9475 8516/10453 10982/12417 12786/13987 18444/16647 24530/19248
+// (matches early in the lists: 4 million at 337 4954/4567, at 936 4881/4195.)
+inline bool long_form(uint32_t longest, uint32_t M) {
+    return longest >= (M <= 1u << 17 ? 96u : M <= kThreadWalkMax ? 256u : 300u);
+}
+// Tables with a list this long walk in one launch whatever the batch: the hop
+// kernels scan such lists whole (fat tree of 80, lists of 6,950, 1.5 million probes
+// 55.9 ms regrouped, 30.7 with the long form after the first hop; one launch takes
+// 7.1 a million), from about 2,000 on one launch is no slower.
+constexpr uint32_t kThreadWalkList = 3000;
 constexpr int kGridThreads = 256;
 constexpr uint32_t kSmemHistMax = 12288;     // switches for shared-memory histograms
 constexpr uint32_t kWaitLimit = 1u << 24;    // bounded mbarrier polls
@@ -305,6 +326,7 @@ static_assert(kIndexThreads / 32 == 16, "bucket fill counts are laid out for 16 
 constexpr uint32_t kIndexWarps = 512 / 32;
 static_assert(PV_MAX_RULES * 4 <= kMaxSegment * 10, "plain-rule ranks overlay one segment's staging area");
 static_assert(PV_MAX_RULES < kSegItem, "plain-rule positions fit an item below the segment flag");
+static_assert(2 * PV_MAX_RULES < 1 << 16, "a bucket's item count fits 16 bits");
 struct IndexSmem {
     uint32_t sort_cap, key_cap, rules_cap, segs_cap, seg_cap;
     size_t bytes;
@@ -451,7 +473,7 @@ __device__ __forceinline__ uint32_t transpose_bits(uint32_t x, uint32_t lane) {
 // ballots per bucket for the filter and an atomic per bucket of every rule; 40 /
 // 82 with block_sort, transpose_bits and differences.
 // Pass 1 (kFill = false) writes sizes[4s..4s+3] = {n_items, n_segs, n_bnd,
-// n_plain}; pass 2 writes the blob at blob_offs[s].  One kIndexThreads-thread block per switch.
+// n_plain | longest bucket's items << 16}; pass 2 writes the blob at blob_offs[s].  One kIndexThreads-thread block per switch.
 template <bool kFill>
 __global__ void __launch_bounds__(kIndexThreads) index_build_kernel(const uint32_t *__restrict__ rule_offs,
                                                            const uint32_t *__restrict__ tab_offs,
@@ -473,8 +495,9 @@ __global__ void __launch_bounds__(kIndexThreads) index_build_kernel(const uint32
                         (size_t)sm.segs_cap * 8 + (size_t)sm.seg_cap * 10 + 15) & ~(size_t)15);
     uint16_t *s_wcnt = reinterpret_cast<uint16_t *>(s_tail);                        // [16][kBuckets]
     uint32_t *s_cur = reinterpret_cast<uint32_t *>(s_tail + kIndexWarps * kBuckets * 2);  // [kBuckets]
-    __shared__ uint32_t s_warp[33];
+    __shared__ uint32_t s_warp[33], s_longest;
     const uint32_t s = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5, nt = blockDim.x;
+    if (t == 0) s_longest = 0;
     const uint32_t n = rule_offs[s + 1] - rule_offs[s];
     const uint32_t t0 = tab_offs[s], npad = tab_offs[s + 1] - t0;
     const uint4 *a = A + t0;
@@ -584,6 +607,10 @@ __global__ void __launch_bounds__(kIndexThreads) index_build_kernel(const uint32
     {
         static_assert(kBuckets <= kIndexThreads, "a thread per bucket");
         const uint32_t mine = t < kBuckets ? s_pos[t + 1] : 0u;
+        if (!kFill) {
+            const uint32_t most = __reduce_max_sync(PV_FULL_MASK, mine);
+            if (lane == 0 && most) atomicMax(&s_longest, most);
+        }
         __syncthreads();
         if (t < kBuckets) s_pos[t] = mine;
         __syncthreads();
@@ -819,7 +846,7 @@ __global__ void __launch_bounds__(kIndexThreads) index_build_kernel(const uint32
         sizes[4 * s] = n_items;
         sizes[4 * s + 1] = nsegs;
         sizes[4 * s + 2] = n_bnd;
-        sizes[4 * s + 3] = n_plain;
+        sizes[4 * s + 3] = n_plain | s_longest << 16;
     }
 }
 
@@ -1970,8 +1997,13 @@ __global__ void __launch_bounds__(kHopThreads, kFirst ? 4 : 4) walk_hop_kernel(H
 // two or three more where a search of 512 boundaries has ten in a row (100,000
 // probes on 512 switches 41.5 -> 32.3 us, 1 million 112 -> 85, 1 million flows
 // with policies 144 -> 117).
+// kLong: gives up after kLanePairs pairs, with kDeep as the result (100,000 probes
+// on 512 switches with lists of 337 items: 859 us with 32 pairs, 685 with 16, 625
+// with 8; of 1,932: 1035, 928, 881).
 constexpr uint32_t kJumpFrom = 16;
-template <bool kStats>
+constexpr uint32_t kLanePairs = 8;
+constexpr uint32_t kDeep = 2;   // no first match (those are 0 or carry kWinFound)
+template <bool kStats, bool kLong>
 __device__ __forceinline__ uint32_t first_match_thread(const uint8_t *__restrict__ blob, const BlobLayout &L,
                                                        uint32_t src, uint32_t dst, uint32_t dport,
                                                        uint32_t in_port, uint32_t sc, uint32_t dc, uint32_t &tests,
@@ -1986,6 +2018,7 @@ __device__ __forceinline__ uint32_t first_match_thread(const uint8_t *__restrict
     const uint32_t *mk = masks + k;
     Candidates cand(__ldg(mk + dc * kBuckets) & __ldg(mk + (kClasses + sc) * kBuckets), __ldg(boff + k), __ldg(boff + k + 1));
     constexpr uint32_t kNone = 0xFFFFu, kOn = 1u;
+    uint32_t pairs = kLanePairs;
     // one candidate: the first match's result, 0 for a table miss, or kOn
     auto decide = [&](uint32_t it, uint4 r) -> uint32_t {
         if (it == kNone) return 0u;   // no candidate left
@@ -2030,7 +2063,28 @@ __device__ __forceinline__ uint32_t first_match_thread(const uint8_t *__restrict
         if (w != kOn) return w;
         w = decide(it1, r1);
         if (w != kOn) return w;
+        if (kLong && --pairs == 0) return kDeep;
     }
+}
+
+// First match of lane j's probe by the whole warp, 32 items a step from L2.
+template <bool kStats>
+__device__ __noinline__ uint32_t first_match_deep(const uint8_t *blob, uint32_t j, uint32_t src, uint32_t dst,
+                                                  uint32_t dport, uint32_t in_port, uint32_t &tests, uint32_t &lookups) {
+    const uint32_t lane = threadIdx.x & 31;
+    blob = reinterpret_cast<const uint8_t *>(__shfl_sync(PV_FULL_MASK, reinterpret_cast<unsigned long long>(blob), j));
+    src = __shfl_sync(PV_FULL_MASK, src, j);
+    dst = __shfl_sync(PV_FULL_MASK, dst, j);
+    dport = __shfl_sync(PV_FULL_MASK, dport, j);
+    in_port = __shfl_sync(PV_FULL_MASK, in_port, j);
+    uint32_t n = 0, l = 0;
+    const uint32_t fm = first_match_indexed<kStats>(blob, 0, __ldg(reinterpret_cast<const uint4 *>(blob)), lane, src, dst,
+                                                    dport, in_port, n, l);
+    if (kStats && lane == j) {
+        tests += n;
+        lookups += l;
+    }
+    return fm;
 }
 
 // Whole walks, or a walk's last hops, in one launch: one thread per probe,
@@ -2051,6 +2105,10 @@ __device__ __forceinline__ uint32_t first_match_thread(const uint8_t *__restrict
 // at work meanwhile.  1,000 probes on the ring: 130 us as 27 launches, 11 us
 // as this one; 100,003 probes on 512 switches: 175 -> 32 us with the filter and
 // the jump blocks.
+// kLong (long_form): a lane gives a first match up after kLanePairs pairs of
+// candidates and its whole warp then finds it, 32 items a step, and a block's
+// probes are spread over all its warps, so that few lanes wait for one another.
+// (One lane tests a list of 6,900 in 3,450 dependent round trips.)
 enum { kSrcProbes = 0, kSrcFlows = 1, kSrcList = 2, kSrcListRec = 3 };
 
 struct ThreadWalkArgs {
@@ -2063,8 +2121,8 @@ struct ThreadWalkArgs {
     unsigned long long *visits;    // [gridDim.x]: visits each block made
 };
 
-template <bool kPolicy, bool kStats, int kSrc>
-__global__ void __launch_bounds__(256, !kStats && kSrc >= kSrcList ? 4 : 1) walk_thread_kernel(HopArgs g, ThreadWalkArgs w) {
+template <bool kPolicy, bool kStats, bool kLong, int kSrc>
+__global__ void __launch_bounds__(256, !kStats && (kLong || kSrc >= kSrcList) ? 4 : 1) walk_thread_kernel(HopArgs g, ThreadWalkArgs w) {
     constexpr bool kList = kSrc == kSrcList || kSrc == kSrcListRec;
     __shared__ uint32_t s_next;
     __shared__ unsigned long long s_visits;
@@ -2089,15 +2147,27 @@ __global__ void __launch_bounds__(256, !kStats && kSrc >= kSrcList ? 4 : 1) walk
     uint4 pr = make_uint4(0, 0, 0, 0);
     uint32_t pid = 0, loc = 0, h = 0, ck = 0, wp = 0, cls = 0;   // cls: source class | destination class << 8
     uint4 ph = make_uint4(0, 0, 0, 0);
+    constexpr uint32_t kUnknown = 1;   // no first match either
+    uint32_t fm = kUnknown;            // kLong: kDeep while the warp is to find it
+    const uint32_t warps = blockDim.x / 32;
+    const bool draws = !kLong || lane < max(1u, (c1 - c0 + warps - 1) / warps);   // the lanes that take probes
     while (true) {
-        const uint32_t idle = __ballot_sync(PV_FULL_MASK, !active);
+        if (kLong)
+            for (uint32_t todo = __ballot_sync(PV_FULL_MASK, fm == kDeep); todo; todo &= todo - 1u) {
+                const uint32_t j = (uint32_t)__ffs(todo) - 1u;
+                const uint32_t x = first_match_deep<kStats>(g.blob + g.blob_offs[(loc >> 8) & 0xFFFFu], j, pr.x, pr.y,
+                                                            pr.z & 0xFFFFu, loc & 0xFFu, stc[kStRuleTests],
+                                                            stc[kStLookups]);
+                if (lane == j) fm = x;
+            }
+        const uint32_t idle = __ballot_sync(PV_FULL_MASK, !active && draws);
         if (idle && more) {
             uint32_t base = 0;
             if (lane == 0) base = atomicAdd(&s_next, (uint32_t)__popc(idle));
             base = __shfl_sync(PV_FULL_MASK, base, 0);
             more = base + (uint32_t)__popc(idle) < c1 - c0;
             const uint32_t k = base + __popc(idle & ((1u << lane) - 1u));
-            if (!active && k < c1 - c0) {
+            if (!active && draws && k < c1 - c0) {
                 const uint32_t i = c0 + k;
                 wp = 0;
                 if (kList) {
@@ -2145,7 +2215,7 @@ __global__ void __launch_bounds__(256, !kStats && kSrc >= kSrcList ? 4 : 1) walk
         }
         if (!active) continue;
         // one visit
-        ++visits;
+        if (!kLong) ++visits;
         const uint32_t s = (loc >> 8) & 0xFFFFu, in_port = loc & 0xFFu, fin = loc_finish(loc);
         uint32_t status = PV_LOOP, hops = g.cap, last = s;   // the walk's end, unless it goes on
         if (fin != 0 && fin - 1 == h) {   // finished at its cycle position
@@ -2154,8 +2224,10 @@ __global__ void __launch_bounds__(256, !kStats && kSrc >= kSrcList ? 4 : 1) walk
             const uint8_t *blob = g.blob + g.blob_offs[s];
             const uint4 hdr = __ldg(reinterpret_cast<const uint4 *>(blob));
             const BlobLayout L(hdr);
-            const uint32_t fm = first_match_thread<kStats>(blob, L, pr.x, pr.y, pr.z & 0xFFFFu, in_port, cls & 0xFFu,
-                                                           cls >> 8, stc[kStRuleTests], stc[kStLookups]);
+            if (!kLong || fm == kUnknown)
+                fm = first_match_thread<kStats, kLong>(blob, L, pr.x, pr.y, pr.z & 0xFFFFu, in_port, cls & 0xFFu, cls >> 8,
+                                                       stc[kStRuleTests], stc[kStLookups]);
+            if (kLong && fm == kDeep) continue;   // the visit goes on with the warp's answer
             if (kStats) {
                 uint32_t depth = 0;
                 const uint32_t ref = scan_first_match(reinterpret_cast<const uint4 *>(blob + L.fa),
@@ -2200,7 +2272,9 @@ __global__ void __launch_bounds__(256, !kStats && kSrc >= kSrcList ? 4 : 1) walk
                 loc = next | (nfin << 24);
                 h = h1;
             }
+            if (kLong) fm = kUnknown;
         }
+        if (kLong) ++visits;
         if (!active) {
             put_result(g.out, pid, status, hops, last);
             if (kPolicy) {
@@ -2538,10 +2612,11 @@ int tables_end(pv_ctx *ctx, pv_table_load &L) {
     if (e == cudaSuccess) {
         for (uint32_t s = 0; s < S; ++s) {
             const uint32_t npad = tab[s + 1] - tab[s];
-            const BlobLayout L(npad, sizes[4 * s + 3], sizes[4 * s], sizes[4 * s + 1], sizes[4 * s + 2]);
+            const BlobLayout L(npad, sizes[4 * s + 3] & 0xFFFFu, sizes[4 * s], sizes[4 * s + 1], sizes[4 * s + 2]);
             boffs[s + 1] = boffs[s] + L.total;
             max_blob = std::max(max_blob, L.fa);             // staged by the indexed kernel
             max_linear = std::max(max_linear, linear_bytes(npad));
+            t.longest_list = std::max(t.longest_list, sizes[4 * s + 3] >> 16);
         }
         e = cudaMemcpyAsync(t.d_blob_offs, boffs.data(), ((size_t)S + 1) * 8, cudaMemcpyHostToDevice, ls);
     }
@@ -2670,10 +2745,15 @@ HopKernel pick_hop(bool indexed, bool pol, bool stats, bool first) {
     return first ? pick_hop_form<kRec, true>(indexed, pol) : pick_hop_form<kRec, false>(indexed, pol);
 }
 
+template <bool kLong, int kSrc>
+ThreadKernel pick_thread_form(bool pol, bool stats) {
+    return pol ? (stats ? walk_thread_kernel<true, true, kLong, kSrc> : walk_thread_kernel<true, false, kLong, kSrc>)
+               : (stats ? walk_thread_kernel<false, true, kLong, kSrc> : walk_thread_kernel<false, false, kLong, kSrc>);
+}
+
 template <int kSrc>
-ThreadKernel pick_thread(bool pol, bool stats) {
-    return pol ? (stats ? walk_thread_kernel<true, true, kSrc> : walk_thread_kernel<true, false, kSrc>)
-               : (stats ? walk_thread_kernel<false, true, kSrc> : walk_thread_kernel<false, false, kSrc>);
+ThreadKernel pick_thread(bool pol, bool stats, bool lng) {
+    return lng ? pick_thread_form<true, kSrc>(pol, stats) : pick_thread_form<false, kSrc>(pol, stats);
 }
 
 // What every walk kernel of a call is given: the loaded tables, the output,
@@ -2709,18 +2789,21 @@ HopArgs walk_args(pv_ctx *ctx, uint32_t hop_cap, const pv_probe *d_probes, pv_re
 
 // Blocks of the thread walk over M probes: one thread per probe up to a full
 // device, in small blocks while they leave SMs idle.
-void thread_walk_grid(pv_ctx *ctx, ThreadKernel fn, uint32_t M, uint32_t *blocks, uint32_t *threads) {
+void thread_walk_grid(pv_ctx *ctx, ThreadKernel fn, uint32_t M, bool lng, uint32_t *blocks, uint32_t *threads) {
     *threads = M < (uint32_t)ctx->num_sms * 256u ? 64u : 256u;
     const uint32_t per_sm = (uint32_t)std::max(1, pv_blocks_per_sm(ctx, (const void *)fn, (int)*threads, 0));
     const uint32_t most = std::min<uint32_t>((uint32_t)ctx->num_sms * per_sm, ctx->walk_visit_slots);
-    *blocks = std::max(1u, (uint32_t)std::min<uint64_t>(((uint64_t)M + *threads - 1) / *threads, most));
+    const uint32_t share = lng ? *threads / 32 : *threads;   // long lists: a warp per probe up to a full device
+    *blocks = std::max(1u, (uint32_t)std::min<uint64_t>(((uint64_t)M + share - 1) / share, most));
 }
 
 // The whole walk in one walk_thread_kernel launch.
 int walk_by_thread(pv_ctx *ctx, uint32_t M, pv_probe *d_probes, uint32_t hop_cap, pv_result *d_out,
                    const PolicyArgs *pa, cudaStream_t st, const BindArgs *ba) {
     const bool stats = ctx->opt_walk_stats != 0;
-    const ThreadKernel fn = ba ? pick_thread<kSrcFlows>(pa != nullptr, stats) : pick_thread<kSrcProbes>(pa != nullptr, stats);
+    const bool lng = long_form(ctx->tb.longest_list, M);
+    const ThreadKernel fn =
+        ba ? pick_thread<kSrcFlows>(pa != nullptr, stats, lng) : pick_thread<kSrcProbes>(pa != nullptr, stats, lng);
     HopArgs g = walk_args(ctx, hop_cap, d_probes, d_out, pa);
     ThreadWalkArgs w = {};
     w.M = M;
@@ -2731,7 +2814,7 @@ int walk_by_thread(pv_ctx *ctx, uint32_t M, pv_probe *d_probes, uint32_t hop_cap
     }
     w.visits = ctx->d_walk_visits;
     uint32_t blocks, threads;
-    thread_walk_grid(ctx, fn, M, &blocks, &threads);
+    thread_walk_grid(ctx, fn, M, lng, &blocks, &threads);
     pv_use_begin(ctx, st);
     if (stats)
         PV_TRY_CUDA(ctx, cudaMemsetAsync(ctx->d_walk_stats, 0, PV_WALK_STATS * sizeof(unsigned long long), st),
@@ -2768,7 +2851,8 @@ int walk_probes(pv_ctx *ctx, uint32_t M, const pv_probe *d_probes, uint32_t hop_
     const bool direct = ba && (!pol || (pa->probe_pol == nullptr && (pa->per == 0 || pa->per % ba->ppg == 0)));
     if (direct && G64 > 0xFFFFFFFFull) return pv_fail(ctx, PV_EINVAL, "pv_verify_flows: too many (group, pod) pairs");
     const uint32_t G = (uint32_t)G64;
-    if (indexed && M <= kThreadWalkMax && ctx->opt_walk_tail_hop < 0 && !ctx->opt_test_stall_staging)
+    const bool one_launch = M <= kThreadWalkMax || t.longest_list >= kThreadWalkList;
+    if (indexed && one_launch && ctx->opt_walk_tail_hop < 0 && !ctx->opt_test_stall_staging)
         return walk_by_thread(ctx, M, const_cast<pv_probe *>(d_probes), hop_cap, d_out, pa, (cudaStream_t)stream, ba);
     const size_t table_smem = indexed ? t.max_blob_bytes : t.max_linear_bytes;
     // the next hop's per-switch counts ride in the hop kernel's shared memory
@@ -2784,7 +2868,8 @@ int walk_probes(pv_ctx *ctx, uint32_t M, const pv_probe *d_probes, uint32_t hop_
     const bool stats = ctx->opt_walk_stats != 0;
     const HopKernel hop_fn = direct ? pick_hop<true>(indexed, pol, stats, false) : pick_hop<false>(indexed, pol, stats, false);
     const HopKernel hop_fn0 = direct ? pick_hop<true>(indexed, pol, stats, true) : pick_hop<false>(indexed, pol, stats, true);
-    const ThreadKernel tail_fn = direct ? pick_thread<kSrcListRec>(pol, stats) : pick_thread<kSrcList>(pol, stats);
+    const bool lng = long_form(t.longest_list, M);
+    const ThreadKernel tail_fn = direct ? pick_thread<kSrcListRec>(pol, stats, lng) : pick_thread<kSrcList>(pol, stats, lng);
     if (int rc = pv_smem_limit(ctx, (const void *)hop_fn, "walk_hop_kernel smem")) return rc;
     if (int rc = pv_smem_limit(ctx, (const void *)hop_fn0, "walk_hop_kernel smem")) return rc;
     hop_blocks_per_sm = pv_blocks_per_sm(ctx, (const void *)hop_fn, kHopThreads, hop_smem);

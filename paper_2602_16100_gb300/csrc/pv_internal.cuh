@@ -45,6 +45,7 @@ struct pv_table_state {
     uint64_t *d_blob_offs = nullptr;  // [S + 1] byte offsets
     uint32_t max_blob_bytes = 0;      // largest stage of the indexed kernel (all but the full rule list)
     uint32_t stage_skip = 0;          // bytes of the candidate filter when the indexed kernel does not stage it
+    uint32_t longest_list = 0;        // most items of one destination-port bucket of one switch
     uint32_t max_linear_bytes = 0;    // largest header + full rule list (linear-scan kernel)
     uint32_t max_ports = 0;           // most ports on one switch
     bool index_fits = false;          // every blob fits shared memory

@@ -12,7 +12,8 @@ import test_gpu_policies as TP
 import test_gpu_walk as TW
 from paper_2602_16100_gb300 import binding as B
 from paper_2602_16100_gb300 import workloads as W
-from netbuild import make_net
+from paper_2602_16100_gb300.validator import empty_device, to_device, to_numpy
+from netbuild import ip, make_net, rule
 
 pytestmark = pytest.mark.gpu
 
@@ -152,3 +153,110 @@ def test_candidate_filter(validator, n, hosts, wide, lane_max, tail):
             validator.set_option(o, x)
     o = oracle.verify_probes(net, pr, 20)
     assert (g == o).all() and (g2 == o).all()
+
+
+def _deep_net(n):
+    """Three switches in a line, two hosts each.  n rules of one port bucket at
+    every switch, each for one source address above every host's or for one
+    port of the hosts (so that the candidate filter keeps most of them), a run
+    of destination rules in their midst and the routes below them."""
+    hosts = [(s, h, ip(10, s, h, 1)) for s in range(3) for h in range(2)]
+    tables = []
+    for s in range(3):
+        t = [rule(1000, hosts[0][2], 32, W.DROP, src_ip=0xF0000000 + i, src_len=32, lo=0, hi=255) for i in range(n)]
+        for i, r in enumerate(t):
+            r["priority"] = 40000 - 2 * i
+            r["action"] = i % 4 if i % 5 else W.DROP
+            r["dst_len"] = 0 if i % 2 else 32
+            if i % 3 == 0:      # and one port of any host
+                r["src_ip"], r["src_len"], r["dst_len"], r["dport_lo"], r["dport_hi"] = ip(10, 0, 0, 0), 8, 0, i % 251, i % 251
+        mid = [rule(40001 - n, ip(99, k, 0, 0), 16, 2 if k % 2 else 3) for k in range(7)]
+        low = [rule(100, a, 32, h if s2 == s else 3 if s2 > s else 2) for s2, h, a in hosts] + [rule(1, 0, 0, 3)]
+        tables.append(t + mid + low)
+    return make_net([4] * 3, [(0, 3, 1, 2), (1, 3, 2, 2)], hosts, [0, 1, 2], tables)
+
+
+def _deep_probes(net, n, m, seed):
+    """Sources of rules at both sides of a lane's and a warp's steps, at the end, of none; a third past the bucket."""
+    r = np.random.default_rng(seed)
+    depth = np.unique(np.clip([0, 1, 15, 16, 17, 31, 32, 33, 63, 64, n // 2 - 1, n // 2, n - 2, n - 1, n], 0, n))
+    pr = np.zeros(m, W.PROBE_DTYPE)
+    pr["src_ip"] = np.where(r.random(m) < 0.7, 0xF0000000 + r.choice(depth, m), 0xF0000000 + r.integers(0, n + 9, m))
+    dst = np.concatenate([net.host_ip, [ip(99, k, 3, 3) for k in range(8)], [5]]).astype(np.uint32)
+    pr["dst_ip"] = r.choice(dst, m)
+    pr["src_host"] = r.integers(0, net.num_hosts + 1, m)
+    pr["dport"] = np.where(r.random(m) < 0.7, r.integers(0, 256, m), r.integers(0, 65536, m))
+    pr["allowed_mask"] = np.where(r.random(m) < 0.8, 7, r.integers(0, 8, m))
+    return pr
+
+
+@pytest.mark.parametrize("n,m", [(95, 3000), (96, 1), (96, 3001), (97, 1 << 17), (97, (1 << 17) + 1), (255, 140_000),
+                                 (256, 140_000), (300, 1500), (2999, 700), (3000, 701), (6000, 900)])
+def test_long_candidate_lists(validator, n, m):
+    """Lists past what a lane tests alone: every depth of the match, interval
+    searches behind it, both sides of the rules on list length and batch size;
+    visit counts add up and no first match differs from a plain scan's."""
+    net = _deep_net(n)
+    pr = _deep_probes(net, n, m, n + m)
+    idx = np.arange(0, m, 1 + m // 20000)
+    o = oracle.verify_probes(net, pr[idx], 20)
+    validator.set_option(B.PV_OPT_WALK_CYCLES, 1)
+    try:
+        g = TW._gpu_walk(validator, net, pr, 20, 2)
+        assert (g[idx] == o).all()
+        ran = g["status"] != W.ST_NOSRC
+        want = int(g["hops"][ran].astype(np.int64).sum()) - int((g["status"] == W.ST_VIOLATION).sum())
+        assert B.pv_get_stat(validator.ctx, B.PV_STAT_WALK_LIVE_TOTAL) == want
+        validator.set_option(B.PV_OPT_WALK_STATS, 1)
+        assert (TW._gpu_walk(validator, net, pr, 20, 2) == g).all()
+        assert B.pv_get_stat(validator.ctx, B.PV_STAT_WALK_INDEX_MISMATCHES) == 0
+    finally:
+        validator.set_option(B.PV_OPT_WALK_CYCLES, 0)
+        validator.set_option(B.PV_OPT_WALK_STATS, 0)
+
+
+@pytest.mark.parametrize("n", [95, 96, 700])
+@pytest.mark.parametrize("policies", [False, True])
+def test_long_candidate_lists_regrouped_and_flows(validator, n, policies):
+    """The same lists in a regrouped walk's last hops (most blocks with no
+    probe left) and for compact flows, with and without path policies."""
+    v, net, ppg, groups = validator, _deep_net(n), 40, 30
+    m = ppg * groups
+    pr = _deep_probes(net, n, m, n)
+    v.load_network(net)
+    pol = W.PathPolicies(1, np.array([0, 1], np.uint32), np.array([1], np.uint16), np.array([0, 2], np.uint32),
+                         np.array([0, 2], np.uint16), np.ones(1, np.uint8)) if policies else None
+    if policies:
+        v.load_policies(pol)
+    r = np.random.default_rng(n)
+    assign = r.integers(0, net.num_hosts + 1, groups).astype(np.uint32)
+    masks = r.choice([7, 7, 5, 3], groups).astype(np.uint32)
+    flows = pr.copy()
+    flows["allowed_mask"] = np.repeat(masks, ppg)
+    bound = oracle.bind_probes(flows, ppg, 1, assign, net.host_ip)
+    d = v.device
+    for tail in (-1, 1, 2):
+        v.set_option(B.PV_OPT_WALK_TAIL_HOP, tail)
+        try:
+            for form, x in (("probes", pr), ("flows", bound)):
+                out, hits = empty_device(4 * m, d), empty_device(4 * m, d)
+                if form == "probes" and policies:
+                    B.pv_verify_probes_constrained(v.ctx, m, to_device(x, d), 20, None, m, out, hits)
+                elif form == "probes":
+                    B.pv_verify_probes(v.ctx, m, to_device(x, d), 20, out)
+                else:
+                    cols = [to_device(np.ascontiguousarray(pr[f]), d) for f in ("dst_ip", "dport")]
+                    a = (v.ctx, m, *cols, ppg, 1, to_device(assign, d), to_device(masks, d), 20)
+                    if policies:
+                        B.pv_verify_flow_columns_constrained(*a, None, m, 0, None, out, hits)
+                    else:
+                        B.pv_verify_flow_columns(*a, None, out)
+                v.sync()
+                if policies:
+                    want, oh = oracle.verify_constrained(net, x, 20, pol, probes_per_policy=m)
+                    assert (to_numpy(hits, np.uint32) == oh).all(), (tail, form)
+                else:
+                    want = oracle.verify_probes(net, x, 20)
+                assert (to_numpy(out, W.RESULT_DTYPE) == want).all(), (tail, form)
+        finally:
+            v.set_option(B.PV_OPT_WALK_TAIL_HOP, -1)
