@@ -694,7 +694,7 @@ void oracle_schedule_paths(uint32_t S, const uint8_t *switch_region, const uint3
         int st = 0;
         if (!ok[cur] || !ok[dst]) st = 2;
         for (uint32_t i = 0; i < nm && !st; ++i)
-            if (!ok[mg[i]]) st = 2;
+            if (mg[i] >= S || !ok[mg[i]]) st = 2;   /* a waypoint that is no switch of this network */
         /* visits: (switch, in_port) with out_port filled when the next link is chosen */
         uint32_t n = 1, vsw[256], vin[256], vout[256];
         vsw[0] = cur; vin[0] = host_port[q->src_host]; vout[0] = 0;

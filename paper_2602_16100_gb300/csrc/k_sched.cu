@@ -68,7 +68,8 @@ __global__ void __launch_bounds__(kSchedThreads) sched_paths_kernel(SchedArgs a)
     uint16_t *g_w = reinterpret_cast<uint16_t *>(g_links + (kStaged ? L : 0u));   // [L] link weights
     __shared__ uint32_t s_st, s_n;
     const uint32_t t = threadIdx.x, nt = blockDim.x;
-    auto allowed = [&](uint32_t s) { return (ok[s >> 5] >> (s & 31)) & 1u; };
+    // (a waypoint of policies loaded for other tables may be no switch of these)
+    auto allowed = [&](uint32_t s) { return s < S && ((ok[s >> 5] >> (s & 31)) & 1u); };
     const uint32_t *in_offs = a.in_offs, *in_links = a.in_links;
     if (kStaged) {
         for (uint32_t v = t; v <= S; v += nt) g_offs[v] = a.in_offs[v];

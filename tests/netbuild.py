@@ -38,6 +38,26 @@ def make_net(nports, links, hosts, region, rules):
                      np.array([h[1] for h in hosts], np.uint16), np.array([h[2] for h in hosts], np.uint32))
 
 
+def ring_net(S, hosts):
+    """Ring of S switches of five regions without rules, `hosts` hosts spread over it."""
+    return make_net([3] * S, [(i, 1, (i + 1) % S, 2) for i in range(S)],
+                    [(i * (S // hosts), 0, ip(10, 0, i, 1)) for i in range(hosts)], [i % 5 for i in range(S)],
+                    [[] for _ in range(S)])
+
+
+# Policies loaded for a ring of 300 and then used on one of 40: waypoints and
+# forbidden switches that the smaller network does not have.
+OUTDATED_FORBID = [[], [280], [], [], [39]]
+OUTDATED_MUST = [[299], [], [5, 64, 7], [135, 3], [7]]
+
+
+def outdated_requests():
+    req = np.zeros(40, W.PATH_REQ_DTYPE)
+    req["src_host"], req["dst_host"] = np.arange(40) % 20, (np.arange(40) * 7 + 1) % 20
+    req["allowed_mask"], req["policy"] = 31, np.arange(40) % 6
+    return req
+
+
 def probe(src_host, src_ip, dst_ip, mask, dport=80):
     p = np.zeros(1, W.PROBE_DTYPE)
     p["src_host"], p["src_ip"], p["dst_ip"], p["allowed_mask"], p["dport"] = src_host, src_ip, dst_ip, mask, dport

@@ -12,7 +12,7 @@ import oracle
 from paper_2602_16100_gb300 import binding as B
 from paper_2602_16100_gb300 import workloads as W
 from paper_2602_16100_gb300.validator import empty_device, to_device, to_numpy
-from netbuild import ip, make_net
+from netbuild import OUTDATED_FORBID, OUTDATED_MUST, ip, make_net, outdated_requests, ring_net
 from test_oracle_policies import _backup_switch_net, _policies
 
 pytestmark = pytest.mark.gpu
@@ -168,3 +168,25 @@ def test_networks_around_the_kernels_shared_memory(validator, S):
     req["src_host"], req["dst_host"] = np.arange(40), (np.arange(40) * 7 + 1) % 50
     req["allowed_mask"], req["policy"] = 31, W.NO_POLICY
     _run(validator, net, req, None, None, 255)
+
+
+@pytest.mark.parametrize("kernel", [0, 1, 2])
+def test_policies_of_a_larger_network(validator, kernel):
+    """Policies stay loaded when a smaller network replaces theirs: a waypoint
+    that is no switch of it blocks the request, a forbidden one means nothing."""
+    net, pol, req = ring_net(40, 20), _policies(OUTDATED_FORBID, OUTDATED_MUST), outdated_requests()
+    validator.load_network(ring_net(300, 20))
+    validator.load_policies(pol)
+    validator.set_option(B.PV_OPT_SCHED_KERNEL, kernel)
+    try:
+        validator.load_network(net)
+        _, vis, ln, st = _gpu_schedule(validator, req, None, 64)
+    finally:
+        validator.set_option(B.PV_OPT_SCHED_KERNEL, 0)
+    o_vis, o_ln, o_st = oracle.schedule_paths(net, req, pol, None, 64)
+    assert (to_numpy(st, np.uint8) == o_st).all() and (to_numpy(ln, np.uint8) == o_ln).all()
+    g_vis = to_numpy(vis, np.uint32, (40, 64))
+    for r in range(40):
+        assert (g_vis[r, : o_ln[r]] == o_vis[r, : o_ln[r]]).all()
+    assert (o_st[np.isin(req["policy"], [0, 2, 3])] == W.PATH_BLOCKED).all()
+    assert (o_st[np.isin(req["policy"], [1, 5])] == W.PATH_OK).all()

@@ -16,7 +16,7 @@ nx = pytest.importorskip("networkx")
 
 import oracle
 from paper_2602_16100_gb300 import workloads as W
-from netbuild import ip, make_net, rule
+from netbuild import OUTDATED_FORBID, OUTDATED_MUST, ip, make_net, outdated_requests, ring_net, rule
 from test_oracle_policies import _backup_switch_net, _policies
 
 
@@ -179,3 +179,12 @@ def test_repeated_state_is_reported():
     req2["policy"] = 0
     h2, l2, s2 = oracle.schedule_paths(net2, req2, pol2)
     assert s2[0] == W.PATH_REPEAT
+
+
+def test_waypoints_that_are_no_switch_block_the_request():
+    net, pol, req = ring_net(40, 20), _policies(OUTDATED_FORBID, OUTDATED_MUST), outdated_requests()
+    vis, ln, st = oracle.schedule_paths(net, req, pol, None, 64)
+    for r in range(len(req)):
+        want, visits = _canonical(net, req[r], pol, None, 64)
+        assert st[r] == want and ln[r] == len(visits), r
+    assert (st[np.isin(req["policy"], [0, 2, 3])] == W.PATH_BLOCKED).all()
