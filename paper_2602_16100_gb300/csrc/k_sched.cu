@@ -68,8 +68,7 @@ __global__ void __launch_bounds__(kSchedThreads) sched_paths_kernel(SchedArgs a)
     uint16_t *g_w = reinterpret_cast<uint16_t *>(g_links + (kStaged ? L : 0u));   // [L] link weights
     __shared__ uint32_t s_st, s_n;
     const uint32_t t = threadIdx.x, nt = blockDim.x;
-    // (a waypoint of policies loaded for other tables may be no switch of these)
-    auto allowed = [&](uint32_t s) { return s < S && ((ok[s >> 5] >> (s & 31)) & 1u); };
+    auto allowed = [&](uint32_t s) { return (ok[s >> 5] >> (s & 31)) & 1u; };
     const uint32_t *in_offs = a.in_offs, *in_links = a.in_links;
     if (kStaged) {
         for (uint32_t v = t; v <= S; v += nt) g_offs[v] = a.in_offs[v];
@@ -112,8 +111,10 @@ __global__ void __launch_bounds__(kSchedThreads) sched_paths_kernel(SchedArgs a)
         __syncthreads();
         const uint32_t src_sw = a.host_switch[q.src_host], dst_sw = a.host_switch[q.dst_host];
         uint32_t st = (allowed(src_sw) && allowed(dst_sw)) ? PV_PATH_OK : PV_PATH_BLOCKED;
-        for (uint32_t i = 0; i < ph.w && st == PV_PATH_OK; ++i)
-            if (!allowed(a.pol_sw[ph.z + i])) st = PV_PATH_BLOCKED;
+        for (uint32_t i = 0; i < ph.w && st == PV_PATH_OK; ++i) {
+            const uint32_t w = a.pol_sw[ph.z + i];   // of policies loaded for other tables: maybe no switch of these
+            if (w >= S || !allowed(w)) st = PV_PATH_BLOCKED;
+        }
         uint32_t n = 1, cur = src_sw;
         if (t == 0) vis[0] = src_sw << 16 | (uint32_t)a.host_port[q.src_host] << 8;
         for (uint32_t i = 0; i <= ph.w && st == PV_PATH_OK; ++i) {
