@@ -306,7 +306,10 @@ int pv_verify_probes(pv_ctx *ctx, uint32_t num_probes, const pv_probe *d_probes,
  * once on a symmetric graph) run on a side stream of the context that
  * `stream` waits for before the call returns (created on the first call).
  * Errors: PV_EINVAL (V == 0, V > 16384, words_per_row too small or not a
- * multiple of 4, NULL pointers); PV_ENOMEM (scratch).
+ * multiple of 4, NULL pointers); PV_ENOMEM (scratch).  Scratch: 4 bytes per
+ * mask and vertex, 4 per row (on graphs without all reverse edges) or up to
+ * 128 MB of component rows; where that cannot be had the sweeps run, which
+ * need 8 bytes per edge and 12 per vertex.
  * ------------------------------------------------------------------------- */
 int pv_compliant_reach(pv_ctx *ctx, uint32_t V, const uint32_t *d_offs, uint32_t num_edges,
                        const uint32_t *d_cols, const uint8_t *d_region, uint32_t num_src, const uint32_t *d_src, uint32_t num_masks,

@@ -300,6 +300,11 @@ __device__ __forceinline__ void uf_union(volatile uint32_t *parent, uint32_t a, 
     pv_device_error(status, PV_ETIMEOUT);
 }
 
+// Component table at most.  Rows past it come from the labels by ballots: 4,096
+// sources on 16,384 vertices, 64 masks and some 2,700 components a mask 364 us
+// with 64 MB, 247 with 128.
+constexpr size_t kTableBytes = (size_t)128 << 20;
+
 constexpr uint16_t kNoLabel = 0xFFFF;
 constexpr uint16_t kSlotNone = 0xFFFF, kSlotOverflow = 0xFFFE, kSlotSingle = 0xFFFD;   // table rows stay below these
 
@@ -945,18 +950,23 @@ extern "C" int pv_compliant_reach(pv_ctx *ctx, uint32_t V, const uint32_t *d_off
     const size_t o_cols = o_cursor + align256((size_t)V * 4);
     const size_t o_pairs = o_cols + align256((size_t)num_edges * 4 + 4);   // undirected pairs
     const size_t o_lab = o_pairs + align256((size_t)num_edges * 4 + 16);   // component labels, or the hubs' sets
-    const bool comp = ctx->opt_reach == 0;
+    bool comp = ctx->opt_reach == 0;
     const size_t set_words = 2 * (((size_t)V + 31) / 32);                  // a hub's two sets
     const size_t o_slots = o_lab + align256((size_t)num_masks * std::max<size_t>((size_t)V * 2, set_words * 4));
     const size_t o_table = o_slots + align256((size_t)num_masks * V * 2);
-    // table rows a mask: every component's when that takes 64 MB or a quarter
-    // of the caller's rows at most
+    // table rows a mask: every component's (of two vertices or more) when they
+    // fit kTableBytes; past the table rows come from the labels
     const size_t mask_row = (size_t)num_masks * words_per_row * 4;
-    const uint32_t cap = (uint32_t)std::min<size_t>(V, std::max<size_t>(((size_t)64 << 20) / mask_row, num_src / 4));
+    const uint32_t cap = (uint32_t)std::min<size_t>(V / 2, kTableBytes / mask_row);
     // search path: the sources to search of every mask and their counts, in the table's place
     const size_t o_rest_n = o_table + align256((size_t)num_masks * num_src * 4);
-    const size_t total = comp ? std::max(o_table + cap * mask_row, o_rest_n + (size_t)num_masks * 8) : o_lab;
-    uint8_t *base = (uint8_t *)pv_scratch(ctx, total);
+    const size_t total = std::max(o_table + cap * mask_row, o_rest_n + (size_t)num_masks * 8);
+    uint8_t *base = (uint8_t *)pv_scratch(ctx, comp ? total : o_lab);
+    if (!base && comp) {   // little memory is left beside the caller's rows: the sweeps need the least
+        ctx->err.clear();
+        comp = false;
+        base = (uint8_t *)pv_scratch(ctx, o_lab);
+    }
     if (!base) return PV_ENOMEM;
     uint32_t *indeg = (uint32_t *)(base + o_indeg), *in_offs = (uint32_t *)(base + o_in_offs);
     uint32_t *cursor = (uint32_t *)(base + o_cursor), *in_cols = (uint32_t *)(base + o_cols);

@@ -4,11 +4,12 @@ blocks fit the GPU at once) and the component table of symmetric ones, against
 the oracle."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
 from paper_2602_16100_gb300 import binding as B
 from paper_2602_16100_gb300 import workloads as W
-from paper_2602_16100_gb300.validator import to_device, to_numpy
+from paper_2602_16100_gb300.validator import Validator, to_device, to_numpy
 
 pytestmark = pytest.mark.gpu
 
@@ -95,7 +96,7 @@ def test_hub_search_malformed(validator, bad):
 @pytest.mark.parametrize("group,num_masks", [(1, 7), (2, 2000), (5, 2000), (2, 7)])
 def test_component_table(validator, group, num_masks):
     """Vertices alone, and components of `group`: fewer and more of them than
-    the mask's table holds (2,000 masks leave it 131 rows)."""
+    the mask's table holds (2,000 masks leave it 262 rows)."""
     V = 2003
     v = np.arange(V)
     a = v[(v % group != group - 1) & (v + 1 < V)] if group > 1 else v[:0]
@@ -103,3 +104,57 @@ def test_component_table(validator, group, num_masks):
     r = np.random.default_rng(group)
     src = np.concatenate([r.integers(0, V, 5), [V - 1, 0, V]])
     _check(validator, g, src, r.integers(0, 8, num_masks), 1)
+
+
+def _pairs_graph(V):
+    """Components of two vertices, one region."""
+    a = np.arange(0, V - 1, 2)
+    return _graph(V, np.concatenate([a, a + 1]), np.concatenate([a + 1, a]), 1, 4)
+
+
+def test_scratch_stays_bounded(validator):
+    """The component table takes 128 MB at most, whatever the caller's rows
+    (1 GB here); components past it are exact."""
+    v, V, masks = Validator(0), 8192, np.ones(64, np.uint32)
+    masks[::3] = 2
+    try:
+        g, src = _pairs_graph(V), np.arange(2 * V) % V
+        out = v.compliant_reach(v.upload_graph(g), len(src), to_device(src.astype(np.uint32), v.device), 64,
+                                to_device(masks, v.device))
+        v.sync()
+        assert B.pv_get_stat(v.ctx, B.PV_STAT_SCRATCH_BYTES) < 180 << 20
+        rows = out.view(torch.int32).view(64, len(src), -1)
+        want = oracle.compliant_reach(g, src.astype(np.uint32), masks[:2])
+        assert (to_numpy(rows[:2].contiguous().view(torch.uint8).flatten(), np.uint32, want.shape) == want).all()
+        for m in range(2, 64):
+            assert torch.equal(rows[m], rows[0 if m % 3 == 0 else 1])
+    finally:
+        v.close()
+
+
+@pytest.mark.parametrize("directed", [False, True])
+def test_little_memory_left(validator, directed):
+    """Beside rows that leave little memory the call still runs (by sweeps)."""
+    v, V = Validator(0), 4096
+    try:
+        if directed:
+            g = _graph(V, *_edges("giant", V, np.random.default_rng(2)), 5, 3)
+        else:
+            g = _pairs_graph(V)
+        src, masks = np.arange(V).astype(np.uint32), np.array([31, 1, 6] * 21 + [2], np.uint32)
+        graph, d_src, d_masks = v.upload_graph(g), to_device(src, v.device), to_device(masks, v.device)
+        out = torch.zeros(len(masks) * V * (V // 8), dtype=torch.uint8, device="cuda")
+        v.sync()
+        torch.cuda.synchronize()
+        hold = torch.empty(torch.cuda.mem_get_info()[0] - (24 << 20), dtype=torch.uint8, device="cuda")
+        try:
+            v.compliant_reach(graph, V, d_src, len(masks), d_masks, d_reach=out)
+            v.sync()
+        finally:
+            del hold
+            torch.cuda.empty_cache()
+        assert B.pv_get_stat(v.ctx, B.PV_STAT_SCRATCH_BYTES) < 24 << 20
+        want = oracle.compliant_reach(g, src, masks[:3])
+        assert (to_numpy(out[: want.size * 4], np.uint32, want.shape) == want).all()
+    finally:
+        v.close()
