@@ -318,11 +318,14 @@ __host__ __device__ inline uint32_t up16u(uint32_t x) { return (x + 15u) & ~15u;
 // root) and copies the pairs inside the permitted subgraph, usually a small
 // share of them, to shared memory; the union pass then runs over that
 // compact list (over the whole list again when it did not fit).  Each
-// component of several vertices then takes the next row of the mask's table,
-// if one is left: slots[m][v] = v's row, kSlotOverflow past the table,
-// kSlotSingle for a vertex alone in its component, kSlotNone for one that is
-// not permitted.
+// component of several vertices then takes a row of the mask's table, if one is
+// left: slots[m][v] = v's row, kSlotOverflow past the table, kSlotSingle for a
+// vertex alone in its component, kSlotNone for one that is not permitted.  With few masks several blocks (parts) label the
+// same mask and each writes a share of its table (4,096 sources on 16,000 vertices
+// of average degree 0.6, one mask: the call takes 101 us with four, 89 with eight,
+// 156 with one).
 constexpr int kLabelThreads = 1024;
+constexpr uint32_t kLabelParts = 8;               // most blocks that label one mask
 constexpr size_t kLabelSmemTarget = 100 * 1024;   // two label blocks per SM
 
 // Layout of the labels kernel's dynamic shared memory for V vertices:
@@ -343,9 +346,9 @@ __global__ void __launch_bounds__(kLabelThreads) reach_labels_kernel(
     uint32_t V, const uint32_t *__restrict__ pairs, const uint8_t *__restrict__ region,
     const uint32_t *__restrict__ masks, uint16_t *__restrict__ lab, uint16_t *__restrict__ slots,
     uint32_t *__restrict__ table, uint32_t cap, uint32_t W, const uint32_t *flags, int32_t *status,
-    uint32_t num_masks, ClearArgs clear) {
-    if (blockIdx.x >= num_masks) {
-        clear_rows(clear, blockIdx.x - num_masks, gridDim.x - num_masks, V, region);
+    uint32_t label_blocks, uint32_t parts, ClearArgs clear) {
+    if (blockIdx.x >= label_blocks) {
+        clear_rows(clear, blockIdx.x - label_blocks, gridDim.x - label_blocks, V, region);
         return;
     }
     if (!component_path(flags)) return;       // the search path runs
@@ -356,7 +359,7 @@ __global__ void __launch_bounds__(kLabelThreads) reach_labels_kernel(
     uint32_t *s_allow = reinterpret_cast<uint32_t *>(s_dyn + L.allow);            // [ceil(V / 32)]
     uint32_t *s_pairs = reinterpret_cast<uint32_t *>(s_dyn + L.pairs);            // [L.cap]
     const uint32_t t = threadIdx.x, lane = t & 31, warp = t >> 5, nt = blockDim.x;
-    const uint32_t m = blockIdx.x, mask = masks[m];
+    const uint32_t m = blockIdx.x / parts, part = blockIdx.x - m * parts, mask = masks[m];
     auto allowed = [&](uint32_t v) { return (s_allow[v >> 5] >> (v & 31)) & 1u; };
     // every vertex its own root; permitted-vertex bitmap
     for (uint32_t v0 = 0; v0 < V; v0 += nt) {
@@ -420,32 +423,64 @@ __global__ void __launch_bounds__(kLabelThreads) reach_labels_kernel(
     }
     __syncthreads();
     uint16_t *s_slot = reinterpret_cast<uint16_t *>(s_pairs);   // [V]: the pairs are done with
+    uint32_t *s_rank = s_pairs + (V + 1) / 2;                   // [ceil(V / 32)]: roots with company before the word
+    const uint32_t words = (V + 31) / 32;
     for (uint32_t v = t; v < V; v += nt) s_slot[v] = 0;
     __syncthreads();
     for (uint32_t v = t; v < V; v += nt) {
         const uint32_t r = uf_find(parent, v);
-        lab[(size_t)m * V + v] = allowed(v) ? (uint16_t)r : kNoLabel;
+        if (part == 0) lab[(size_t)m * V + v] = allowed(v) ? (uint16_t)r : kNoLabel;
         if (r != v) s_slot[r] = 1;   // r has company
     }
     __syncthreads();
-    for (uint32_t v = t; v < V; v += nt)
-        if (parent[v] == v && allowed(v)) {
-            const uint32_t k = s_slot[v] ? atomicAdd(&s_comps, 1u) : 0u;
-            s_slot[v] = !s_slot[v] ? kSlotSingle : k < cap ? (uint16_t)k : kSlotOverflow;
+    if (parts == 1) {
+        for (uint32_t v = t; v < V; v += nt)
+            if (parent[v] == v && allowed(v)) {
+                const uint32_t k = s_slot[v] ? atomicAdd(&s_comps, 1u) : 0u;
+                s_slot[v] = !s_slot[v] ? kSlotSingle : k < cap ? (uint16_t)k : kSlotOverflow;
+            }
+    } else {   // rows in the order of the labels, the same in every part
+        for (uint32_t v0 = warp * 32; v0 < V; v0 += nt) {
+            const uint32_t bal = __ballot_sync(PV_FULL_MASK, v0 + lane < V && s_slot[v0 + lane] != 0);
+            if (lane == 0) s_rank[v0 >> 5] = __popc(bal);
         }
+        __syncthreads();
+        if (warp == 0) {
+            uint32_t run = 0;
+            for (uint32_t w0 = 0; w0 < words; w0 += 32) {
+                const uint32_t c = w0 + lane < words ? s_rank[w0 + lane] : 0u;
+                uint32_t incl = c;
+                for (int d = 1; d < 32; d <<= 1) {
+                    const uint32_t y = __shfl_up_sync(PV_FULL_MASK, incl, d);
+                    if (lane >= (uint32_t)d) incl += y;
+                }
+                if (w0 + lane < words) s_rank[w0 + lane] = run + incl - c;
+                run += __shfl_sync(PV_FULL_MASK, incl, 31);
+            }
+            if (lane == 0) s_comps = run;
+        }
+        __syncthreads();
+        for (uint32_t v0 = warp * 32; v0 < V; v0 += nt) {
+            const uint32_t v = v0 + lane;
+            const bool has = v < V && s_slot[v] != 0;
+            const uint32_t k = s_rank[v0 >> 5] + __popc(__ballot_sync(PV_FULL_MASK, has) & ((1u << lane) - 1u));
+            if (v < V) s_slot[v] = !has ? kSlotSingle : k < cap ? (uint16_t)k : kSlotOverflow;   // (used for roots)
+        }
+    }
     __syncthreads();
-    // the table's rows: cleared, then every word written once, by the first
-    // of the component's vertices among its 32
-    const uint32_t rows = min(s_comps, cap);
+    // the part's rows of the table: cleared, then every word written once, by
+    // the first of the component's vertices among its 32
+    const uint32_t rows = min(s_comps, cap), k0 = rows * part / parts, k1 = rows * (part + 1) / parts;
     uint32_t *tab = table + (size_t)m * cap * W;
-    for (uint32_t q = t; q < rows * (W / 4); q += nt) reinterpret_cast<uint4 *>(tab)[q] = make_uint4(0, 0, 0, 0);
+    for (uint32_t q = t; q < (k1 - k0) * (W / 4); q += nt)
+        reinterpret_cast<uint4 *>(tab + (size_t)k0 * W)[q] = make_uint4(0, 0, 0, 0);
     __syncthreads();
     for (uint32_t v0 = warp * 32; v0 < V; v0 += nt) {
         const uint32_t v = v0 + lane;
         const uint32_t k = v < V && allowed(v) ? s_slot[uf_find(parent, v)] : kSlotNone;
-        if (v < V) slots[(size_t)m * V + v] = (uint16_t)k;
+        if (v < V && part == 0) slots[(size_t)m * V + v] = (uint16_t)k;
         const uint32_t peers = __match_any_sync(PV_FULL_MASK, k);
-        if (k < cap && lane == (uint32_t)(__ffs(peers) - 1)) tab[(size_t)k * W + (v0 >> 5)] = peers;
+        if (k - k0 < k1 - k0 && lane == (uint32_t)(__ffs(peers) - 1)) tab[(size_t)k * W + (v0 >> 5)] = peers;
     }
 }
 
@@ -472,7 +507,7 @@ __device__ __forceinline__ void comp_row(const uint16_t *lab, uint32_t V, uint32
 }
 
 // R(s, m) = the row of s's component (clear_rows writes the rows
-// of the other sources): a warp takes 32 (mask, source) rows, finds their
+// of the other sources): a warp takes per_warp (mask, source) rows, finds their
 // table rows at once and copies them one after the other from L2.
 // Bound by the row writes.  A block per mask and slice of sources used to
 // rebuild the labels and the rows of its components, up to 90 of them, in
@@ -482,14 +517,15 @@ constexpr int kRowThreads = 256;
 __global__ void __launch_bounds__(kRowThreads) reach_rows_kernel(
     uint32_t V, const uint16_t *__restrict__ lab, const uint16_t *__restrict__ slots,
     const uint32_t *__restrict__ table, uint32_t cap, uint32_t num_masks, uint32_t num_src,
-    const uint32_t *__restrict__ src, uint32_t *__restrict__ reach, uint32_t W, const uint32_t *flags) {
+    const uint32_t *__restrict__ src, uint32_t *__restrict__ reach, uint32_t W, uint32_t per_warp,
+    const uint32_t *flags) {
     if (!component_path(flags)) return;
     const uint32_t lane = threadIdx.x & 31, warps = kRowThreads / 32;
-    const uint64_t rows = (uint64_t)num_masks * num_src, step = (uint64_t)gridDim.x * warps * 32;
-    for (uint64_t i0 = ((uint64_t)blockIdx.x * warps + threadIdx.x / 32) * 32; i0 < rows; i0 += step) {
+    const uint64_t rows = (uint64_t)num_masks * num_src, step = (uint64_t)gridDim.x * warps * per_warp;
+    for (uint64_t i0 = ((uint64_t)blockIdx.x * warps + threadIdx.x / 32) * per_warp; i0 < rows; i0 += step) {
         const uint64_t i = i0 + lane;
         const uint32_t m = (uint32_t)(i / num_src);
-        const uint32_t s = i < rows ? src[i - (uint64_t)m * num_src] : V;
+        const uint32_t s = lane < per_warp && i < rows ? src[i - (uint64_t)m * num_src] : V;
         const uint32_t slot = s < V ? __ldg(slots + (size_t)m * V + s) : kSlotNone;
         // four rows in flight
         for (uint32_t todo = __ballot_sync(PV_FULL_MASK, slot < kSlotSingle); todo;) {
@@ -1044,13 +1080,21 @@ extern "C" int pv_compliant_reach(pv_ctx *ctx, uint32_t V, const uint32_t *d_off
         reach_msbfs_kernel<<<(uint32_t)std::min<uint64_t>(items, 0x7FFFFFFFull), kReachThreads, (size_t)V * 8, sw>>>(
             V, in_offs, in_cols, d_region, num_src, d_src, num_masks, d_masks, d_reach, words_per_row, flags);
     }
-    reach_labels_kernel<<<num_masks + sms, kLabelThreads, LabelSmem(V).total, st>>>(
-        V, pairs, d_region, d_masks, lab, slots, table, cap, words_per_row, flags, ctx->d_status, num_masks, clear);
+    // a part for every 1,024 vertices while most SMs are idle (a second one costs
+    // 2 us of 25 at 300 vertices, of 58 on the 4,096-vertex WAN with 64 masks)
+    const uint32_t parts = num_masks * 4 <= sms ? std::max(1u, std::min({kLabelParts, sms / num_masks, V / 1024})) : 1u;
+    reach_labels_kernel<<<num_masks * parts + sms, kLabelThreads, LabelSmem(V).total, st>>>(
+        V, pairs, d_region, d_masks, lab, slots, table, cap, words_per_row, flags, ctx->d_status, num_masks * parts, parts,
+        clear);
     {
-        const uint64_t warps = ((uint64_t)num_masks * num_src + 31) / 32;
+        // rows a warp: 32, fewer while that leaves SMs idle (300 vertices, one
+        // mask: the call takes 28.4 us with 32, 22.2 with one)
+        const uint64_t rows = (uint64_t)num_masks * num_src;
+        const uint32_t per_warp = (uint32_t)std::min<uint64_t>(32, std::max<uint64_t>(1, rows / (sms * 32)));
+        const uint64_t warps = (rows + per_warp - 1) / per_warp;
         const uint32_t rgrid = (uint32_t)std::min<uint64_t>((warps + kRowThreads / 32 - 1) / (kRowThreads / 32), sms * 8);
         reach_rows_kernel<<<rgrid, kRowThreads, 0, st>>>(V, lab, slots, table, cap, num_masks, num_src, d_src, d_reach,
-                                                         words_per_row, flags);
+                                                         words_per_row, per_warp, flags);
     }
     PV_TRY_CUDA(ctx, cudaEventRecord(ctx->reach_join, sw), "reach join");
     PV_TRY_CUDA(ctx, cudaStreamWaitEvent(st, ctx->reach_join, 0), "reach join");

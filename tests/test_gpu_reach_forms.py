@@ -158,3 +158,15 @@ def test_little_memory_left(validator, directed):
         assert (to_numpy(out[: want.size * 4], np.uint32, want.shape) == want).all()
     finally:
         v.close()
+
+
+@pytest.mark.parametrize("V,num_masks", [(1, 1), (31, 3), (1023, 1), (1024, 2), (3001, 1), (3001, 40), (9001, 5),
+                                         (16384, 1), (16384, 17)])
+def test_few_masks_and_rows(validator, V, num_masks):
+    """Several blocks to a mask's table and few rows to a warp: components of
+    one to many vertices, some of them whole regions apart."""
+    r = np.random.default_rng(V)
+    a, b = r.integers(0, V, V // 2), r.integers(0, V, V // 2)
+    g = _graph(V, np.concatenate([a, b]), np.concatenate([b, a]), 4, V)
+    src = np.concatenate([r.integers(0, V, min(V, 700)), [0, V - 1, V]])
+    _check(validator, g, src, np.concatenate([[15], r.integers(0, 16, num_masks - 1)]), 1)
