@@ -580,29 +580,26 @@ __device__ __forceinline__ void block_allow(uint32_t V, const uint8_t *__restric
 }
 
 // Sweeps of up to 64 sources to the fixpoint from the words in s_vis (bit j of
-// s_vis[v]: v is known to be in source j's set; all: the bits in use), then
-// source j's row to row_of(j).
+// s_vis[v]: v is known to be in source j's set), then source j's row to row_of(j)
+// for those in `write`.
+// The loops stay plain: four in-edges at a time made graphs of one or two edges a
+// vertex half as slow again, and a transposition that stops at the last source
+// used in place of 64 unrolled steps cost 6 us of 19 at 1,000 vertices (3,000
+// vertices of one edge each, 24 masks, no cycles: the call 130 us, 104 plain).
 template <typename RowOf>
 __device__ __forceinline__ void msbfs_sweeps(uint32_t V, const uint32_t *__restrict__ in_offs,
-                                             const uint32_t *__restrict__ in_cols, uint32_t nb, uint32_t W,
-                                             uint64_t *s_vis, const uint32_t *s_allow, RowOf row_of) {
+                                             const uint32_t *__restrict__ in_cols, uint64_t write,
+                                             uint32_t W, uint64_t *s_vis, const uint32_t *s_allow, RowOf row_of) {
     const uint32_t t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const uint64_t all = nb == 64 ? ~0ull : (1ull << nb) - 1ull;
     volatile uint64_t *vis = s_vis;
     for (uint32_t iter = 0; iter <= V; ++iter) {
         int changed = 0;
         for (uint32_t v = t; v < V; v += kReachThreads) {
             if (!((s_allow[v >> 5] >> (v & 31)) & 1u)) continue;
             const uint64_t old = vis[v];
-            if (old == all) continue;
             uint64_t acc = old;
             const uint32_t a = __ldg(in_offs + v), b = __ldg(in_offs + v + 1);
-            for (uint32_t e = a; e < b; e += 4) {   // four in-edges in flight (v itself adds nothing)
-                uint32_t x[4];
-#pragma unroll
-                for (uint32_t j = 0; j < 4; ++j) x[j] = e + j < b ? __ldg(in_cols + e + j) : v;
-                acc |= vis[x[0]] | vis[x[1]] | vis[x[2]] | vis[x[3]];
-            }
+            for (uint32_t e = a; e < b; ++e) acc |= vis[__ldg(in_cols + e)];
             if (acc != old) {
                 vis[v] = acc;
                 changed = 1;
@@ -620,7 +617,7 @@ __device__ __forceinline__ void msbfs_sweeps(uint32_t V, const uint32_t *__restr
             x[i] = v < V ? vis[v] : 0ull;
         }
         uint4 lo = make_uint4(0, 0, 0, 0), hi = make_uint4(0, 0, 0, 0);
-        for (uint32_t j = 0; j < nb; ++j) {
+        for (uint32_t j = 0; j < 64; ++j) {   // (unrolled: all 64, used or not)
             uint32_t b[4];
 #pragma unroll
             for (int i = 0; i < 4; ++i) b[i] = __ballot_sync(PV_FULL_MASK, (x[i] >> j) & 1ull);
@@ -629,8 +626,8 @@ __device__ __forceinline__ void msbfs_sweeps(uint32_t V, const uint32_t *__restr
                 else hi = make_uint4(b[0], b[1], b[2], b[3]);
             }
         }
-        if (lane < nb) reinterpret_cast<uint4 *>(row_of(lane))[q] = lo;
-        if (lane + 32 < nb) reinterpret_cast<uint4 *>(row_of(lane + 32))[q] = hi;
+        if ((write >> lane) & 1ull) reinterpret_cast<uint4 *>(row_of(lane))[q] = lo;
+        if ((write >> (lane + 32)) & 1ull) reinterpret_cast<uint4 *>(row_of(lane + 32))[q] = hi;
     }
 }
 
@@ -640,7 +637,7 @@ __global__ void __launch_bounds__(kReachThreads) reach_msbfs_kernel(
     const uint32_t *__restrict__ masks, uint32_t *__restrict__ reach, uint32_t W, const uint32_t *flags) {
     if (flags && component_path(flags)) return;
     extern __shared__ uint64_t s_vis[];                 // [V]
-    __shared__ uint32_t s_allow[kReachMaxV / 32];
+    __shared__ uint32_t s_allow[kReachMaxV / 32], s_on[2];   // s_on: the permitted sources
     const uint32_t nbatch = (num_src + 63) / 64, t = threadIdx.x;
     const uint64_t items = (uint64_t)nbatch * num_masks;   // (mask, source batch) pairs
     for (uint64_t item = blockIdx.x; item < items; item += gridDim.x) {
@@ -649,13 +646,19 @@ __global__ void __launch_bounds__(kReachThreads) reach_msbfs_kernel(
         block_allow(V, region, masks[m], s_allow);
         for (uint32_t v = t; v < V; v += kReachThreads) s_vis[v] = 0;
         __syncthreads();
-        if (t < nb) {
-            const uint32_t s = src[j0 + t];
-            if (s < V && ((s_allow[s >> 5] >> (s & 31)) & 1u)) atomicOr((unsigned long long *)&s_vis[s], 1ull << t);
+        if (t < 64) {
+            const uint32_t s = t < nb ? src[j0 + t] : V;
+            const bool on = s < V && ((s_allow[s >> 5] >> (s & 31)) & 1u);
+            if (on) atomicOr((unsigned long long *)&s_vis[s], 1ull << t);
+            const uint32_t bal = __ballot_sync(PV_FULL_MASK, on);
+            if ((t & 31) == 0) s_on[t >> 5] = bal;
         }
         __syncthreads();
-        msbfs_sweeps(V, in_offs, in_cols, nb, W, s_vis, s_allow,
-                     [&](uint32_t j) { return reach + ((size_t)m * num_src + j0 + j) * W; });
+        // with flags, blocks of other launches write the empty rows
+        const uint64_t on = (uint64_t)s_on[1] << 32 | s_on[0], used = nb == 64 ? ~0ull : (1ull << nb) - 1ull;
+        if (on || !flags)   // (block-uniform)
+            msbfs_sweeps(V, in_offs, in_cols, flags ? on : used, W, s_vis, s_allow,
+                         [&](uint32_t j) { return reach + ((size_t)m * num_src + j0 + j) * W; });
         __syncthreads();
     }
 }
@@ -929,7 +932,9 @@ __global__ void __launch_bounds__(kReachThreads) reach_hub_rows_kernel(
         __syncthreads();
         if (t < nb) atomicOr((unsigned long long *)&s_vis[src[s_list[t]]], 1ull << t);
         __syncthreads();
-        msbfs_sweeps(V, in_offs, in_cols, nb, W, s_vis, s_allow, [&](uint32_t j) { return rows + (size_t)s_list[j] * W; });
+        const uint64_t used = nb == 64 ? ~0ull : (1ull << nb) - 1ull;   // listed sources are permitted
+        msbfs_sweeps(V, in_offs, in_cols, used, W, s_vis, s_allow,
+                     [&](uint32_t j) { return rows + (size_t)s_list[j] * W; });
     }
 }
 
@@ -1088,9 +1093,11 @@ extern "C" int pv_compliant_reach(pv_ctx *ctx, uint32_t V, const uint32_t *d_off
         clear);
     {
         // rows a warp: 32, fewer while that leaves SMs idle (300 vertices, one
-        // mask: the call takes 28.4 us with 32, 22.2 with one)
+        // mask: the call takes 28.4 us with 32, 22 with one), but not more than two
+        // blocks an SM: on other graphs the sweeps' blocks are placed around these
+        // (1,000 vertices, 16 masks, six edges each: 57 us, with four blocks 75)
         const uint64_t rows = (uint64_t)num_masks * num_src;
-        const uint32_t per_warp = (uint32_t)std::min<uint64_t>(32, std::max<uint64_t>(1, rows / (sms * 32)));
+        const uint32_t per_warp = (uint32_t)std::min<uint64_t>(32, std::max<uint64_t>(1, rows / (sms * 16)));
         const uint64_t warps = (rows + per_warp - 1) / per_warp;
         const uint32_t rgrid = (uint32_t)std::min<uint64_t>((warps + kRowThreads / 32 - 1) / (kRowThreads / 32), sms * 8);
         reach_rows_kernel<<<rgrid, kRowThreads, 0, st>>>(V, lab, slots, table, cap, num_masks, num_src, d_src, d_reach,
