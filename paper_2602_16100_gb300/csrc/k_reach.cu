@@ -669,11 +669,18 @@ __global__ void __launch_bounds__(kReachThreads) reach_msbfs_kernel(
 // reached from there, searched level by level, half of the block each way.
 // Any hub is exact; one inside the largest strongly connected component
 // leaves the fewest sources to search, so a second is tried when the first
-// one's component holds less than a quarter of the permitted vertices (and the
-// sets themselves did not both hold one), and the better is kept.  Last, the permitted sources outside the kept component are
-// listed: rest[m][0 .. rest_n[m]), in no particular order.
+// one's component holds less than a quarter of the permitted vertices (unless both
+// sets hold a quarter, or neither a sixteenth: then no large component is near),
+// and the better is kept.  Last, the permitted sources outside the kept component
+// are listed: rest[m][0 .. rest_n[m]), in no particular order.
 constexpr int kHubThreads = 1024;
 constexpr uint32_t kHubTries = 2;
+// Most levels of a search where some permitted vertex has no edge in or none out.
+// There a long search mostly ends without a component (a path of 3,000 vertices, 64
+// masks: the call 13.2 ms without the limit, 5.3 by sweeps alone); a ring, where
+// every level is needed, has no such vertex (1.7 ms, 5.3 by sweeps alone).
+constexpr uint32_t kHubLevels = 256;
+constexpr uint32_t kHubMinV = 1000;   // smallest graph (see the call)
 
 struct HubSmem {   // two visited bitmaps, the permitted bitmap, two queues
     uint32_t allow, queue, total;
@@ -718,6 +725,7 @@ __global__ void __launch_bounds__(kHubThreads) reach_hub_kernel(
     for (uint32_t w = t; w < words; w += kHubThreads)
         if (s_allow[w]) atomicAdd(&s_all, (uint32_t)__popc(s_allow[w]));
     uint32_t tried[kHubTries], kept = 0;
+    bool ends = false;   // this thread has seen a permitted vertex without edges in or out
     for (uint32_t attempt = 0; attempt < kHubTries; ++attempt) {
         if (t == 0) s_best = s_core = 0;
         __syncthreads();
@@ -725,12 +733,15 @@ __global__ void __launch_bounds__(kHubThreads) reach_hub_kernel(
         for (uint32_t v = t; v < V; v += kHubThreads) {
             bool skip = !allowed(v);
             for (uint32_t i = 0; i < attempt; ++i) skip = skip || v == tried[i];
-            if (!skip)
-                best = max(best, (min(min(degree(offs, cols, v), degree(in_offs, in_cols, v)), 0xFFFEu) + 1u) << 16 |
-                                     (0xFFFFu - v));
+            if (!skip) {
+                const uint32_t d = min(min(degree(offs, cols, v), degree(in_offs, in_cols, v)), 0xFFFEu);
+                ends = ends || d == 0;
+                best = max(best, (d + 1u) << 16 | (0xFFFFu - v));
+            }
         }
         best = __reduce_max_sync(PV_FULL_MASK, best);
         if ((t & 31) == 0) atomicMax(&s_best, best);
+        const uint32_t most = __syncthreads_or(ends) ? kHubLevels : V;
         // a vertex that is not permitted counts as seen
         for (uint32_t w = t; w < 2 * words; w += kHubThreads) s_sets[w] = ~s_allow[w < words ? w : w - words];
         __syncthreads();
@@ -744,11 +755,12 @@ __global__ void __launch_bounds__(kHubThreads) reach_hub_kernel(
             }
         }
         __syncthreads();
-        uint32_t head = 0;
+        uint32_t head = 0, levels = 0;
         const uint32_t sub = t % kEdgeLanes, lane8 = t % (kHubThreads / 2) / kEdgeLanes;
         while (true) {
             const uint32_t tail = *(volatile uint32_t *)&s_tail[way];
-            if (!__syncthreads_or(head < tail)) break;   // also: everyone has read the tail before it moves
+            // also: everyone has read the tail before it moves
+            if (!__syncthreads_or(head < tail) || ++levels > most) break;
             for (uint32_t i = head + lane8; i < tail; i += kHubThreads / 2 / kEdgeLanes) {
                 const uint32_t u = queue[i], b = __ldg(o + u + 1);
                 for (uint32_t e = __ldg(o + u) + sub; e < b; e += kEdgeLanes) {
@@ -762,6 +774,12 @@ __global__ void __launch_bounds__(kHubThreads) reach_hub_kernel(
             head = tail;
             __syncthreads();
         }
+        if (levels > most) {   // given up (block-uniform): an earlier hub's sets or none
+            if (attempt == 0)
+                for (uint32_t w = t; w < 2 * words; w += kHubThreads) sets[(size_t)m * 2 * words + w] = 0;
+            __syncthreads();
+            break;
+        }
         for (uint32_t w = t; w < words; w += kHubThreads) {
             const uint32_t n = __popc(s_sets[w] & s_sets[words + w] & s_allow[w]);
             if (n) atomicAdd(&s_core, n);
@@ -774,9 +792,9 @@ __global__ void __launch_bounds__(kHubThreads) reach_hub_kernel(
             kept = core;
         }
         __syncthreads();
-        // (block-uniform) large enough, or both sets large and yet little in
-        // common: no large component is near
-        if (kept * 4 >= s_all || min(s_tail[0], s_tail[1]) * 4 >= s_all) break;
+        // (block-uniform) large enough, both sets large and yet little in common,
+        // or both small: no large component is near
+        if (kept * 4 >= s_all || min(s_tail[0], s_tail[1]) * 4 >= s_all || max(s_tail[0], s_tail[1]) * 16 < s_all) break;
         __syncthreads();
     }
     const uint32_t lane = t & 31;
@@ -822,7 +840,7 @@ __global__ void __launch_bounds__(kReachThreads) reach_hub_rows_kernel(
     const uint32_t *__restrict__ in_offs, const uint32_t *__restrict__ in_cols, const uint8_t *__restrict__ region,
     uint32_t num_src, const uint32_t *__restrict__ src, uint32_t num_masks, const uint32_t *__restrict__ masks,
     const uint32_t *__restrict__ sets, const uint32_t *__restrict__ rest, const uint2 *__restrict__ rest_n,
-    uint32_t *__restrict__ reach, uint32_t W, uint32_t per_block, const uint32_t *flags) {
+    uint32_t *__restrict__ reach, uint32_t W, const uint32_t *flags) {
     if (component_path(flags)) return;
     extern __shared__ uint64_t s_vis[];
     __shared__ uint32_t s_list[64], s_sweep;   // sources (as row numbers) to sweep
@@ -835,8 +853,8 @@ __global__ void __launch_bounds__(kReachThreads) reach_hub_rows_kernel(
     uint32_t *seen = reinterpret_cast<uint32_t *>(s_dyn + L.seen) + warp * words;
     uint16_t *queue = reinterpret_cast<uint16_t *>(s_dyn + L.queue) + warp * kOwnQueue;
     const uint32_t batches = (num_src + 63) / 64;
-    const uint64_t i1 = min((uint64_t)(blockIdx.x + 1) * per_block, (uint64_t)batches * num_masks);
-    for (uint64_t item = (uint64_t)blockIdx.x * per_block; item < i1; ++item) {
+    const uint64_t items = (uint64_t)batches * num_masks;
+    for (uint64_t item = blockIdx.x; item < items; item += gridDim.x) {
         const uint32_t m = (uint32_t)(item / batches), x = (uint32_t)(item % batches);
         __syncthreads();   // the item before is done with the shared state
         uint32_t *rows = reach + (size_t)m * num_src * W;
@@ -1066,21 +1084,24 @@ extern "C" int pv_compliant_reach(pv_ctx *ctx, uint32_t V, const uint32_t *d_off
     reach_scan_kernel<<<1, 1024, 0, sw>>>(V, indeg, in_offs, cursor, flags, flags + kBadOffs);
     reach_fill_kernel<<<egrid, kGridThreads, 0, sw>>>(V, num_edges, d_offs, d_cols, cursor, in_cols, flags,
                                                       flags + kBadOffs);
-    // A hub and its two sets take some 25 us a mask before the first row: more
-    // than sweeps while every (mask, 64 sources) item has a block of its own
-    // (16 masks: 500 vertices 49 us against 66; 3,000, of which no component is
-    // large, 265 against 221; 8,000 with a large one 1,642 against 188).
+    // A hub and its two sets take some 10 to 25 us before the first row: more than
+    // sweeps while every (mask, 64 sources) item has a block of its own, and on
+    // small graphs (sweeps / hub, us; 64 masks: 700 vertices of 1.5 random edges each
+    // 76/98, of 6 82/61; 1,000: 96/116, 116/64; 2,000: 260/237, 318/91; without cycles
+    // and one edge each 43/53, 53/60, 111/110).
     const uint64_t items = (uint64_t)((num_src + 63) / 64) * num_masks;
-    const bool by_hub = items > 4ull * sms;
+    const bool by_hub = items > 4ull * sms && V >= kHubMinV;
     if (by_hub) {
         reach_hub_kernel<<<num_masks, kHubThreads, HubSmem(V).total, sw>>>(V, d_offs, d_cols, in_offs, in_cols, d_region,
                                                                           d_masks, sets, num_src, d_src, rest, rest_n,
                                                                           flags);
-        // at most sixteen blocks an SM: on a symmetric graph they all start and return
-        const uint32_t per = (uint32_t)((items + 16ull * sms - 1) / (16ull * sms));
-        reach_hub_rows_kernel<<<(uint32_t)((items + per - 1) / per), kReachThreads, HubRowSmem(V).total, sw>>>(
+        // at most sixteen blocks an SM: on a symmetric graph they all start and
+        // return.  A block's items lie a grid apart: neighbours are of one mask, and
+        // a mask with long searches would keep its few blocks for twice as long
+        // (8,000 vertices of three edges each, 24 masks: 945 us, 627 a grid apart)
+        reach_hub_rows_kernel<<<(uint32_t)std::min<uint64_t>(items, 16ull * sms), kReachThreads, HubRowSmem(V).total, sw>>>(
             V, d_offs, d_cols, in_offs, in_cols, d_region, num_src, d_src, num_masks, d_masks, sets, rest, rest_n,
-            d_reach, words_per_row, per, flags);
+            d_reach, words_per_row, flags);
     } else {
         reach_msbfs_kernel<<<(uint32_t)std::min<uint64_t>(items, 0x7FFFFFFFull), kReachThreads, (size_t)V * 8, sw>>>(
             V, in_offs, in_cols, d_region, num_src, d_src, num_masks, d_masks, d_reach, words_per_row, flags);

@@ -13,7 +13,12 @@ from paper_2602_16100_gb300.validator import Validator, to_device, to_numpy
 
 pytestmark = pytest.mark.gpu
 
-ITEMS = 4 * 152   # more than this many (mask, 64 sources) items: hub search
+HUB_MIN_V = 1000   # kHubMinV of the library
+
+
+def _items():
+    """More than this many (mask, 64 sources) items on HUB_MIN_V vertices or more: hub search."""
+    return 4 * torch.cuda.get_device_properties(0).multi_processor_count
 
 
 def _graph(V, a, b, regions, seed):
@@ -49,26 +54,31 @@ def _edges(kind, V, r):
         h = V // 3
         return np.concatenate([r.integers(0, h, 8 * h), r.integers(h, V, 5 * (V - h))]), \
             np.concatenate([r.integers(0, h, 8 * h), r.integers(h, V, 5 * (V - h))])
-    a = np.arange(V - 1)         # a long path: as many levels as vertices
+    if kind == "ring":           # as many levels as vertices, each in the component
+        return np.arange(V), (np.arange(V) + 1) % V
+    if kind == "spur":           # the same with a dead end, past the levels that are searched
+        return np.concatenate([np.arange(V - 1), [0]]), np.concatenate([(np.arange(V - 1) + 1) % (V - 1), [V - 1]])
+    a = np.arange(V - 1)         # a long path: searched for some levels only
     return a, a + 1
 
 
-@pytest.mark.parametrize("kind", ["giant", "dag", "tail", "two", "path"])
-@pytest.mark.parametrize("V,num_masks", [(700, 64), (321, 120)])
+@pytest.mark.parametrize("kind", ["giant", "dag", "tail", "two", "path", "ring", "spur"])
+@pytest.mark.parametrize("V,num_masks", [(700, 64), (HUB_MIN_V - 1, 64), (HUB_MIN_V, 64), (1321, 120)])
 def test_hub_search(validator, kind, V, num_masks):
     r = np.random.default_rng(V + len(kind))
     g = _graph(V, *_edges(kind, V, r), 5, 3)
     src = np.concatenate([np.arange(V), [0, V - 1, V, 0xFFFFFFFF]])      # duplicates, out of range
     masks = r.integers(0, 32, num_masks)
     masks[:3] = [31, 0, 1]
-    assert (len(src) + 63) // 64 * num_masks > ITEMS
+    assert (len(src) + 63) // 64 * num_masks > _items()
     _check(validator, g, src, masks, 0)
 
 
-@pytest.mark.parametrize("masks", [ITEMS // 2, ITEMS // 2 + 1])
-def test_either_side_of_the_item_limit(validator, masks):
+@pytest.mark.parametrize("past", [0, 1])
+def test_either_side_of_the_item_limit(validator, past):
+    masks = _items() // 2 + past
     r = np.random.default_rng(masks)
-    g = _graph(130, *_edges("giant", 130, r), 4, 1)
+    g = _graph(1030, *_edges("giant", 1030, r), 4, 1)
     _check(validator, g, np.arange(128), r.integers(1, 16, masks), 0)
 
 
@@ -76,14 +86,14 @@ def test_either_side_of_the_item_limit(validator, masks):
 def test_hub_search_malformed(validator, bad):
     """Malformed offsets (no edges) and columns out of range (skipped), reported by the next sync."""
     r = np.random.default_rng(9)
-    g = _graph(400, *_edges("giant", 400, r), 3, 2)
+    g = _graph(1200, *_edges("giant", 1200, r), 3, 2)
     if bad == "offsets":
         g.offs[200] = g.offs[-1] + 7
     else:
-        g.cols[::9] = 400 + np.arange(len(g.cols[::9]))
-    src, masks = np.arange(400), r.integers(0, 8, 100)
+        g.cols[::9] = 1200 + np.arange(len(g.cols[::9]))
+    src, masks = np.arange(1200), r.integers(0, 8, 100)
     v = validator
-    out = v.compliant_reach(v.upload_graph(g), 400, to_device(src.astype(np.uint32), v.device), 100,
+    out = v.compliant_reach(v.upload_graph(g), 1200, to_device(src.astype(np.uint32), v.device), 100,
                             to_device(masks.astype(np.uint32), v.device))
     with pytest.raises(B.PVError) as e:
         v.sync()
