@@ -119,3 +119,32 @@ def test_malformed_among_well_formed(validator):
         validator.sync()
         o, of = oracle.eval_selector_terms(300, 12, c.labels, pods, bad, ex, assign[:n])
         assert (to_numpy(bits, np.uint32, (n, words)) == o).all() and (to_numpy(flags, np.uint8) == of).all(), (at, to)
+
+
+@pytest.mark.parametrize("n", [161, 5120, 5121, 11000])
+def test_more_expressions_than_lanes(validator, n):
+    """Pods of 31 to 130 expressions in one list, in one term and over several,
+    most of them with nodes left at the end, in rows of one span and more."""
+    r = np.random.default_rng(n)
+    c = _cluster(n, 6)
+    validator.load_cluster(c)
+    lens = np.concatenate([[31, 32, 33, 34, 64, 65, 96, 97, 130, 0, 1], r.integers(0, 70, 60)])
+    offs = _offsets(lens)
+    ex = _exprs(r, int(offs[-1]))
+    ex["op"] = np.where(r.random(len(ex)) < 0.985, 1, ex["op"])
+    ex["nvals"] = np.where(ex["op"] < 2, np.maximum(1, ex["nvals"] // 4), 0)
+    ex["vals"] = np.where(r.random((len(ex), 8)) < 0.97, 10 + np.arange(8), ex["vals"])    # mostly values of no node
+    P, words, d = len(lens), W.words_per_row(n) + 4, validator.device
+    assign = r.integers(0, n + 2, P).astype(np.uint32)
+    g, gf = _lists(validator, c, offs, ex, assign, words)
+    o, of = oracle.eval_selectors(n, 12, c.labels, offs, ex, assign, words=words)
+    assert (g == o).all() and (gf == of).all()
+    assert 5 < (of[lens > 32] & W.F_EMPTY == 0).sum() < (lens > 32).sum()
+    pods = np.unique(np.concatenate([[0, P], r.integers(0, P, 30)])).astype(np.uint32)     # 1 to several terms a pod
+    n_pods = len(pods) - 1
+    bits, flags = empty_device(n_pods * words * 4, d), empty_device(n_pods, d)
+    B.pv_eval_selector_terms(validator.ctx, n_pods, to_device(pods, d), P, to_device(offs, d), len(ex), to_device(ex, d),
+                             to_device(assign[:n_pods], d), bits, words, flags)
+    validator.sync()
+    o, of = oracle.eval_selector_terms(n, 12, c.labels, pods, offs, ex, assign[:n_pods], words=words)
+    assert (to_numpy(bits, np.uint32, (n_pods, words)) == o).all() and (to_numpy(flags, np.uint8) == of).all()
