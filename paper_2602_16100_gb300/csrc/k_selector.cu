@@ -534,7 +534,9 @@ __device__ __forceinline__ bool put_span(uint32_t *row, uint32_t sb, uint32_t la
 // found as it was read, 5,000 pods of 33 to 64 expressions on 5,000 nodes took 253 us,
 // 69 resolved 32 at a time.
 constexpr uint8_t kPodLeft = 0x80;
-template <bool kTerms>
+// kPodWarp: the copy of sel_pods_kernel, which has fewer registers (one copy for both
+// cost sel_rows_kernel 1 to 2%).
+template <bool kTerms, bool kPodWarp>
 __device__ __noinline__ void unresolved_pod(const SelArgs &g, uint32_t p, uint32_t *list) {
     const uint32_t lane = threadIdx.x & 31;
     const uint32_t o0 = g.offs[p], o1 = g.offs[p + 1], W = g.W, N = g.N, a = g.assign ? g.assign[p] : PV_UNPLACED;
@@ -576,6 +578,58 @@ __device__ __noinline__ void unresolved_pod(const SelArgs &g, uint32_t p, uint32
     aok = __any_sync(PV_FULL_MASK, aok);
     if (lane == 0)
         g.flags[p] = pre & 1u ? (uint8_t)PV_F_BAD_EXPR : pod_flags(any, pre & 2u, g.assign != nullptr, aok);
+}
+
+// The term form with one pod to a warp and 40 warps an SM, for as many pods as
+// that many warps and more than sel_rows_kernel has warps for: there some of its
+// warps take two pods and the launch waits for them.  3,700 / 4,500 / 5,400 / 6,000
+// pods, us, a pod a warp against sel_rows_kernel: 5,000 nodes 12.8 / 12.8 / 14.3 /
+// 16.7 against 16.3 / 16.6 / 16.5 / 18.6, 1,000 nodes 12.8 / 12.8 / 12.8 / 14.8 against
+// 14.7 / 16.7 / 16.0 / 16.9, 12,000 29.0 / 29.0 / 29.1 / 35.2 against 31.0 / 35.1 /
+// 33.2 / 39.3.  Bound by one pod's chain of loads; three rows at once are what 48
+// registers hold without spilling in the loop.
+constexpr int kPodThreads = 128;
+__global__ void __launch_bounds__(kPodThreads, 1280 / kPodThreads) sel_pods_kernel(const __grid_constant__ SelArgs g) {
+    __shared__ uint32_t s_list[kPodThreads / 32][kListWords];
+    const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, p = blockIdx.x * (kPodThreads / 32) + warp;
+    if (p >= g.P) return;
+    uint32_t *list = s_list[warp];
+    const uint32_t o0 = g.offs[p], o1 = g.offs[p + 1], n = o1 - o0;
+    const uint32_t a = g.assign ? g.assign[p] : PV_UNPLACED;
+    // lane i: start of term i (lane n: the last one's end); a pod of more than 31
+    // terms, with decreasing offsets or more than 32 expressions is left
+    bool left = o1 < o0 || o1 > g.num_terms || n > 31;
+    uint32_t off = 0, pre = 0, first = 0, count = 0, ends = 0;
+    if (!left && n) {
+        off = g.term_offs[o0 + min(lane, n)];
+        const uint32_t before = __shfl_up_sync(PV_FULL_MASK, off, 1);
+        first = __shfl_sync(PV_FULL_MASK, off, 0);
+        const uint32_t past = __shfl_sync(PV_FULL_MASK, off, n);
+        left = __any_sync(PV_FULL_MASK, lane && off < before) || past > g.num_exprs || past - first > 32;
+        count = past - first;
+        if (!left) ends = __reduce_or_sync(PV_FULL_MASK, lane && off > before ? 1u << (off - first - 1) : 0u);
+    }
+    uint32_t total = 0;
+    if (!left) {
+        total = resolve_list(g, first, count, ends, lane, list, pre);
+        left = pre & 1u;   // a bad expression: validated again, in order
+    }
+    if (left) {   // (warp-uniform, as every condition above)
+        unresolved_pod<true, true>(g, p, list);
+        return;
+    }
+    bool any = false, aok = false;
+    for (uint32_t sb = 0; sb < g.W; sb += 160) {
+        const RowSpan sp = row_span(sb, lane, g.N, g.W, g.row_words);
+        uint4 a0 = sp.m0, r0 = n ? make_uint4(0, 0, 0, 0) : sp.m0;   // no terms: every node
+        uint32_t a1 = sp.m1, r1 = n ? 0u : sp.m1;
+        fold_list<true, 3>(g, list, total, sp, a0, a1, r0, r1);
+        any = any || (r0.x | r0.y | r0.z | r0.w | r1) != 0;
+        aok = put_span(g.bits + (size_t)p * g.W, sb, lane, g.W, g.N, a, r0, r1) || aok;
+    }
+    any = __any_sync(PV_FULL_MASK, any);
+    aok = __any_sync(PV_FULL_MASK, aok);
+    if (lane == 0) g.flags[p] = pod_flags(any, pre & 2u, g.assign != nullptr, aok);
 }
 
 // A pod's row is the AND over its expressions, or, with kTerms (Kubernetes
@@ -830,7 +884,7 @@ __global__ void __launch_bounds__(kRowsThreads<kTerms>, 768 / kRowsThreads<kTerm
         const uint32_t pl = at + lane < end ? (g.pod_list ? g.pod_list[at + lane] : at + lane) : 0u;
         const bool mine = at + lane < end && *(volatile uint8_t *)(g.flags + pl) == kPodLeft;
         for (uint32_t todo = __ballot_sync(PV_FULL_MASK, mine); todo; todo &= todo - 1u)
-            unresolved_pod<kTerms>(g, __shfl_sync(PV_FULL_MASK, pl, __ffs(todo) - 1), s_list[threadIdx.x >> 5]);
+            unresolved_pod<kTerms, false>(g, __shfl_sync(PV_FULL_MASK, pl, __ffs(todo) - 1), s_list[threadIdx.x >> 5]);
     }
 }
 
@@ -1064,6 +1118,15 @@ void launch_rows(pv_ctx *ctx, SelArgs g, cudaStream_t st) {
     const int per_sm = std::max(1, pv_blocks_per_sm(ctx, (const void *)fn, kRowsThreads<kTerms>, 0));
     constexpr uint32_t warps = kRowsThreads<kTerms> / 32;
     const uint32_t blocks = std::min((g.P + warps - 1) / warps, (uint32_t)(ctx->num_sms * per_sm));
+    if (kTerms && g.P > (uint32_t)(ctx->num_sms * per_sm) * warps) {
+        constexpr uint32_t pods = kPodThreads / 32;
+        const uint32_t resident =
+            (uint32_t)(ctx->num_sms * std::max(1, pv_blocks_per_sm(ctx, (const void *)sel_pods_kernel, kPodThreads, 0)));
+        if (g.P <= resident * pods) {
+            sel_pods_kernel<<<(g.P + pods - 1) / pods, kPodThreads, 0, st>>>(g);
+            return;
+        }
+    }
     fn<<<blocks, kRowsThreads<kTerms>, 0, st>>>(g);
 }
 

@@ -4,6 +4,7 @@ among well-formed ones and arrays at the least alignment, against the oracle,
 for expression lists and for terms."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
 from paper_2602_16100_gb300 import binding as B
@@ -148,3 +149,28 @@ def test_more_expressions_than_lanes(validator, n):
     validator.sync()
     o, of = oracle.eval_selector_terms(n, 12, c.labels, pods, offs, ex, assign[:n_pods], words=words)
     assert (to_numpy(bits, np.uint32, (n_pods, words)) == o).all() and (to_numpy(flags, np.uint8) == of).all()
+
+
+@pytest.mark.parametrize("n", [161, 5121])
+@pytest.mark.parametrize("warps,more", [(24, 0), (24, 1), (40, 0), (40, 1)])
+def test_terms_around_a_pod_a_warp(validator, n, warps, more):
+    """As many pods as 24 or 40 warps an SM, and one more (the form with a pod to
+    a warp runs between): 0 to 3 terms a pod and now and then 40, empty terms,
+    more than 32 expressions, bad expressions, offsets that decrease."""
+    P = torch.cuda.get_device_properties(0).multi_processor_count * warps + more
+    r = np.random.default_rng(P + n)
+    c = _cluster(n, 7)
+    validator.load_cluster(c)
+    terms = np.where(r.random(P) < 0.005, 40, r.integers(0, 4, P))
+    pods = _offsets(terms)
+    offs = _offsets(np.where(r.random(pods[-1]) < 0.004, r.integers(25, 60, pods[-1]), r.integers(0, 5, pods[-1])))
+    offs[50:60] = offs[50:60][::-1]
+    ex = _exprs(r, int(offs[-1]), bad=0.002)
+    assign = r.integers(0, n + 2, P).astype(np.uint32)
+    words, d = W.words_per_row(n), validator.device
+    bits, flags = empty_device(P * words * 4, d), empty_device(P, d)
+    B.pv_eval_selector_terms(validator.ctx, P, to_device(pods, d), len(offs) - 1, to_device(offs, d), len(ex),
+                             to_device(ex, d), to_device(assign, d), bits, words, flags)
+    validator.sync()
+    o, of = oracle.eval_selector_terms(n, 12, c.labels, pods, offs, ex, assign)
+    assert (to_numpy(bits, np.uint32, (P, words)) == o).all() and (to_numpy(flags, np.uint8) == of).all()
