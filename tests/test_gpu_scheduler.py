@@ -7,6 +7,7 @@ weights and policies, short max_len, the backup-switch case, invalid calls,
 and the end-to-end network with 10,000 requests."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
 from paper_2602_16100_gb300 import binding as B
@@ -16,6 +17,8 @@ from netbuild import OUTDATED_FORBID, OUTDATED_MUST, ip, make_net, outdated_requ
 from test_oracle_policies import _backup_switch_net, _policies
 
 pytestmark = pytest.mark.gpu
+
+SMS = torch.cuda.get_device_properties(0).multi_processor_count if torch.cuda.is_available() else 1
 
 
 def _gpu_schedule(v, req, weights, max_len):
@@ -146,9 +149,9 @@ def test_end_to_end_network_10000_requests(validator):
 
 
 @pytest.mark.parametrize("requests,must_max,max_len", [(1, 3, 64), (17, 3, 1), (311, 32, 255), (311, 32, 40),
-                                                       (152 * 2 * 16 + 5, 2, 64)])
-def test_warp_per_request_edges(validator, requests, must_max, max_len):
-    """The automatic kernel, a warp per request: one request, paths of one
+                                                       (SMS * 32 + 5, 2, 64)])
+def test_warp_per_segment_edges(validator, requests, must_max, max_len):
+    """The automatic kernel, a warp per segment: one request, paths of one
     visit, requests of up to 33 segments, paths longer than max_len in a later
     segment, and more requests than resident warps."""
     e = W.end_to_end(seed=90, num_switches=70, num_intents=4, probes_per_intent=4, rules_per_switch=80)
@@ -161,7 +164,7 @@ def test_warp_per_request_edges(validator, requests, must_max, max_len):
 
 @pytest.mark.parametrize("S", [700, 1900, 2500, 6000])
 def test_networks_around_the_kernels_shared_memory(validator, S):
-    """Rings of more and more switches: two blocks an SM, one with fewer warps, a block per request."""
+    """Rings of more and more switches: a block of 32 warps an SM, one of fewer warps, a block per request."""
     net = make_net([3] * S, [(i, 1, (i + 1) % S, 2) for i in range(S)], [(i * (S // 50), 0, ip(10, 0, i, 1)) for i in range(50)],
                    [i % 5 for i in range(S)], [[] for _ in range(S)])
     req = np.zeros(40, W.PATH_REQ_DTYPE)

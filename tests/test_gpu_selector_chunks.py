@@ -13,6 +13,8 @@ from paper_2602_16100_gb300.validator import empty_device, to_device, to_numpy
 
 pytestmark = pytest.mark.gpu
 
+SMS = torch.cuda.get_device_properties(0).multi_processor_count if torch.cuda.is_available() else 1
+
 
 def _cluster(n, seed):
     r = np.random.default_rng(seed)
@@ -51,7 +53,7 @@ def _lists(v, c, offs, ex, assign, words):
     return to_numpy(bits, np.uint32, (P, words)), to_numpy(flags, np.uint8)
 
 
-@pytest.mark.parametrize("P", [1, 7, 9, 31, 33, 608 * 8 + 1, 608 * 32 + 5])
+@pytest.mark.parametrize("P", [1, 7, 9, 31, 33, SMS * 32 + 1, SMS * 128 + 5])
 @pytest.mark.parametrize("n", [33, 5121])
 def test_chunk_sizes(validator, P, n):
     if n > 5000 and P > 5000:
@@ -157,7 +159,7 @@ def test_terms_around_a_pod_a_warp(validator, n, warps, more):
     """As many pods as 24 or 40 warps an SM, and one more (the form with a pod to
     a warp runs between): 0 to 3 terms a pod and now and then 40, empty terms,
     more than 32 expressions, bad expressions, offsets that decrease."""
-    P = torch.cuda.get_device_properties(0).multi_processor_count * warps + more
+    P = SMS * warps + more
     r = np.random.default_rng(P + n)
     c = _cluster(n, 7)
     validator.load_cluster(c)

@@ -58,10 +58,12 @@ def test_worked_cases(validator, kernel):
 def test_tiny(validator, kernel, lane_max):
     d = W.tiny()
     validator.set_option(B.PV_OPT_WALK_LANE_MAX, lane_max)
+    validator.set_option(B.PV_OPT_WALK_TAIL_HOP, 0)      # the hop kernels, which the lane limit is for
     try:
         g = _gpu_walk(validator, d["network"], d["probes"].probes, d["probes"].hop_cap, kernel)
     finally:
         validator.set_option(B.PV_OPT_WALK_LANE_MAX, 96)
+        validator.set_option(B.PV_OPT_WALK_TAIL_HOP, -1)
     o = oracle.verify_probes(d["network"], d["probes"].probes, d["probes"].hop_cap)
     assert _same(g, o)
 
@@ -222,13 +224,16 @@ def test_index_stress_tables(validator, seed):
     for kernel in KERNELS:
         g = _gpu_walk(validator, net, pr, 24, kernel)
         assert _same(g, o), kernel
-    # indexed kernel with every batch warp-cooperative, and every batch one probe per lane
+    # indexed hop kernel (every hop regrouped) with every batch warp-cooperative,
+    # and every batch one probe per lane
     for lane_max in (0, 65535):
         validator.set_option(B.PV_OPT_WALK_LANE_MAX, lane_max)
+        validator.set_option(B.PV_OPT_WALK_TAIL_HOP, 0)
         try:
             g = _gpu_walk(validator, net, pr, 24, 2)
         finally:
             validator.set_option(B.PV_OPT_WALK_LANE_MAX, 96)
+            validator.set_option(B.PV_OPT_WALK_TAIL_HOP, -1)
         assert _same(g, o), lane_max
     # every first match along the way also agrees hop by hop with the oracle's
     assert len(np.unique(o["status"])) >= 3

@@ -6,6 +6,7 @@ the thread form runs at the edges of its grid and at the batch size where
 the library changes over."""
 import numpy as np
 import pytest
+import torch
 
 import oracle
 import test_gpu_policies as TP
@@ -18,6 +19,7 @@ from netbuild import ip, make_net, rule
 pytestmark = pytest.mark.gpu
 
 THREAD_WALK_MAX = 1 << 20   # kThreadWalkMax of the library
+SMS = torch.cuda.get_device_properties(0).multi_processor_count if torch.cuda.is_available() else 1
 
 
 @pytest.fixture(params=[0, 1, 6])
@@ -42,6 +44,23 @@ def test_regrouped_policies(regrouped, seed, cap):
     TP.test_random_policies(regrouped, seed, cap, 2)
 
 
+@pytest.mark.parametrize("seed", [1, 2, 3])
+def test_regrouped_index_stress_tables(regrouped, seed):
+    TW.test_index_stress_tables(regrouped, seed)
+
+
+def test_regrouped_long_destination_runs(regrouped):
+    TW.test_long_destination_runs_split_into_segments(regrouped)
+
+
+def test_regrouped_forwarding_cycles(regrouped):
+    TW.test_forwarding_cycles_finish_with_the_full_walk_result(regrouped)
+
+
+def test_regrouped_bounces_on_asymmetric_cabling(regrouped):
+    TW.test_bounces_on_asymmetric_cabling_are_walked_out(regrouped)
+
+
 @pytest.mark.parametrize("form", ["records", "columns"])
 @pytest.mark.parametrize("policy_form", ["per_group", "per_probe", "per_pair_of_groups", "none"])
 def test_regrouped_flows(regrouped, policy_form, form):
@@ -56,7 +75,7 @@ def _random_sources(net, pr, seed):
     return pr
 
 
-@pytest.mark.parametrize("m", [1, 31, 33, 65, 152 * 256 - 1, 152 * 256, 152 * 256 + 1])
+@pytest.mark.parametrize("m", [1, 31, 33, 65, SMS * 256 - 1, SMS * 256, SMS * 256 + 1])
 @pytest.mark.parametrize("cycles", [0, 1])
 def test_thread_walk_grid_edges(validator, m, cycles):
     """One probe, ragged warps and blocks, and both block sizes; visit counts add up."""
