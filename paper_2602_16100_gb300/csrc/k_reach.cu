@@ -1095,20 +1095,21 @@ extern "C" int pv_compliant_reach(pv_ctx *ctx, uint32_t V, const uint32_t *d_off
         reach_hub_kernel<<<num_masks, kHubThreads, HubSmem(V).total, sw>>>(V, d_offs, d_cols, in_offs, in_cols, d_region,
                                                                           d_masks, sets, num_src, d_src, rest, rest_n,
                                                                           flags);
-        // at most sixteen blocks an SM: on a symmetric graph they all start and
-        // return.  A block's items lie a grid apart: neighbours are of one mask, and
+        // at most eight blocks an SM: on a symmetric graph they all start and return
+        // (the 4,096-vertex WAN 57.4 us with sixteen, 55.4 with eight).  A block's items lie a grid apart: neighbours are of one mask, and
         // a mask with long searches would keep its few blocks for twice as long
         // (8,000 vertices of three edges each, 24 masks: 945 us, 627 a grid apart)
-        reach_hub_rows_kernel<<<(uint32_t)std::min<uint64_t>(items, 16ull * sms), kReachThreads, HubRowSmem(V).total, sw>>>(
+        reach_hub_rows_kernel<<<(uint32_t)std::min<uint64_t>(items, 8ull * sms), kReachThreads, HubRowSmem(V).total, sw>>>(
             V, d_offs, d_cols, in_offs, in_cols, d_region, num_src, d_src, num_masks, d_masks, sets, rest, rest_n,
             d_reach, words_per_row, flags);
     } else {
         reach_msbfs_kernel<<<(uint32_t)std::min<uint64_t>(items, 0x7FFFFFFFull), kReachThreads, (size_t)V * 8, sw>>>(
             V, in_offs, in_cols, d_region, num_src, d_src, num_masks, d_masks, d_reach, words_per_row, flags);
     }
-    // a part for every 1,024 vertices while most SMs are idle (a second one costs
-    // 2 us of 25 at 300 vertices, of 58 on the 4,096-vertex WAN with 64 masks)
-    const uint32_t parts = num_masks * 4 <= sms ? std::max(1u, std::min({kLabelParts, sms / num_masks, V / 1024})) : 1u;
+    // a part for every 1,024 vertices of large graphs while most SMs are idle (a
+    // second one costs 2 us of 25 at 300 vertices, of 58 on the 4,096-vertex WAN with
+    // 64 masks)
+    const uint32_t parts = num_masks * 4 <= sms && V >= 4096 ? std::min({kLabelParts, sms / num_masks, V / 1024}) : 1u;
     reach_labels_kernel<<<num_masks * parts + sms, kLabelThreads, LabelSmem(V).total, st>>>(
         V, pairs, d_region, d_masks, lab, slots, table, cap, words_per_row, flags, ctx->d_status, num_masks * parts, parts,
         clear);

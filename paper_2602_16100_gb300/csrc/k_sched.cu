@@ -235,9 +235,10 @@ __global__ void __launch_bounds__(kSchedThreads) sched_paths_kernel(SchedArgs a)
 // canonical walk back's equality.
 // A block per request swept every switch until a sweep changed nothing, and
 // waited at a block barrier each time: 10,000 weighted requests on 512
-// switches took 1,098 us with their rules, 165 us this way.  Bound by
-// instruction issue (about 3,900 warp instructions a segment, 41% of issue
-// slots) and, at a group's end, by its longest segments.  Tried: 32 segments
+// switches took 1,098 us with their rules, 165 us this way.  Bound by the
+// shared-memory latency of a segment's steps (about 3,900 warp instructions a
+// segment, 53% of issue slots) and, at a group's end, by its longest segments.
+// Tried: 32 segments
 // to a warp, one per lane (386 us: the union of their frontiers is every
 // switch), and a warp per whole request (375 us: as long as the requests with
 // the most waypoints).

@@ -534,7 +534,7 @@ __device__ __forceinline__ bool put_span(uint32_t *row, uint32_t sb, uint32_t la
 // found as it was read, 5,000 pods of 33 to 64 expressions on 5,000 nodes took 253 us,
 // 69 resolved 32 at a time.
 constexpr uint8_t kPodLeft = 0x80;
-// kPodWarp: the copy of sel_pods_kernel, which has fewer registers (one copy for both
+// kPodWarp: the copy of pod_terms_kernel, which has fewer registers (one copy for both
 // cost sel_rows_kernel 1 to 2%).
 template <bool kTerms, bool kPodWarp>
 __device__ __noinline__ void unresolved_pod(const SelArgs &g, uint32_t p, uint32_t *list) {
@@ -589,7 +589,7 @@ __device__ __noinline__ void unresolved_pod(const SelArgs &g, uint32_t p, uint32
 // 33.2 / 39.3.  Bound by one pod's chain of loads; three rows at once are what 48
 // registers hold without spilling in the loop.
 constexpr int kPodThreads = 128;
-__global__ void __launch_bounds__(kPodThreads, 1280 / kPodThreads) sel_pods_kernel(const __grid_constant__ SelArgs g) {
+__global__ void __launch_bounds__(kPodThreads, 1280 / kPodThreads) pod_terms_kernel(const __grid_constant__ SelArgs g) {
     __shared__ uint32_t s_list[kPodThreads / 32][kListWords];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, p = blockIdx.x * (kPodThreads / 32) + warp;
     if (p >= g.P) return;
@@ -1121,9 +1121,9 @@ void launch_rows(pv_ctx *ctx, SelArgs g, cudaStream_t st) {
     if (kTerms && g.P > (uint32_t)(ctx->num_sms * per_sm) * warps) {
         constexpr uint32_t pods = kPodThreads / 32;
         const uint32_t resident =
-            (uint32_t)(ctx->num_sms * std::max(1, pv_blocks_per_sm(ctx, (const void *)sel_pods_kernel, kPodThreads, 0)));
+            (uint32_t)(ctx->num_sms * std::max(1, pv_blocks_per_sm(ctx, (const void *)pod_terms_kernel, kPodThreads, 0)));
         if (g.P <= resident * pods) {
-            sel_pods_kernel<<<(g.P + pods - 1) / pods, kPodThreads, 0, st>>>(g);
+            pod_terms_kernel<<<(g.P + pods - 1) / pods, kPodThreads, 0, st>>>(g);
             return;
         }
     }

@@ -46,13 +46,15 @@ constexpr uint32_t kHopShare = 20480;        // probes per hop block before ther
 // about 10 us of launches per hop and a table stage per occupied switch,
 // whatever the batch; the thread walk costs its L2 round trips.  Thread walk
 // against regrouped walk, us, at 1.1M / 1.4M / 1.7M / 2M / 2.5M probes:
-//   mesh of 512, 1,000 rules   91/109 108/123 127/144 142/157 176/173
-//   mesh of 64, 200 rules      58/78   68/84   78/106  91/111 108/127
-//   fat tree, 1,000 rules     135/137 165/157 192/169 222/185 264/216
-//   fat tree, 2,000 rules     161/176 193/200 227/214 257/233 314/274
-//   flows of 512 switches     115/113 143/122 146/137 177/143 199/160
-//   the same with policies    128/135 159/135 162/155 199/165 222/186
-// (a ring of 8 at 1k: 11/126).  The lines cross between 1.1M and 2.4M.
+//   mesh of 512, 1,000 rules   89/111 106/122 125/144 140/157 172/174
+//   mesh of 64, 200 rules      58/78   67/83   77/105  89/112 107/125
+//   fat tree, 1,000 rules     132/137 163/155 189/169 218/186 260/216
+//   fat tree, 2,000 rules     158/174 190/194 223/212 251/233 308/271
+//   flows of 512 switches     113/110 142/121 143/140 174/144 195/161
+//   the same with policies    127/130 158/135 160/155 196/164 220/186
+// (a ring of 8 at 1k: 11/126).  The lines cross at 1.1M for flows and beyond
+// 2.5M on meshes; the limit is the earliest crossing, so meshes between the two
+// are 10 to 25% above what one launch would take them.
 constexpr uint32_t kThreadWalkMax = 1u << 20;
 // Larger batches: the hop from which the probes still walking finish in one
 // thread walk.  Live probes fall about 2.5 times a hop, and the thread walk
@@ -665,8 +667,6 @@ __global__ void __launch_bounds__(kIndexThreads) index_build_kernel(const uint32
     }
     __syncthreads();
 
-    __syncthreads();
-
     // candidate filter: each plain rule's classes once, then a warp per bucket
     // and a lane per group of items, whose class bits are transposed into the
     // sixteen words (two buckets at once; the items were written above by this
@@ -1183,7 +1183,6 @@ __global__ void __launch_bounds__(kGroupInitThreads) walk_init_group_kernel(
     const Slice sb = records ? Slice(ba.dst, 0, 8) : Slice(ba.dport + first, len, 2);
     if (t == 0) {
         mbar_init(&s_bar, 1);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         mbar_arrive_expect_tx(&s_bar, sa.bulk_bytes() + sb.bulk_bytes());
         slice_copy(sa, s_raw, &s_bar);
         slice_copy(sb, s_raw + L.dport, &s_bar);
@@ -1457,8 +1456,6 @@ __device__ __forceinline__ void flush_stats(unsigned long long *stats, const uin
     }
 }
 
-// Linear first match: 32 consecutive rules per warp step.
-// Both first-match routines return kWinFound | action, or 0 for a table miss.
 // A walk reads a probe's header through its list entry's first field: the
 // caller's probe record (pv_verify_probes; the field is the probe id) or,
 // for compact flows placed directly, the walk record the first kernel wrote
@@ -1498,6 +1495,8 @@ __device__ __forceinline__ uint4 header_of(const HopArgs &g, uint4 raw, uint32_t
     return raw;
 }
 
+// Linear first match: 32 consecutive rules per warp step.
+// The first-match routines return kWinFound | action, or 0 for a table miss.
 template <bool kStats>
 __device__ __forceinline__ uint32_t first_match_linear(const uint8_t *sm, uint32_t npad, uint32_t lane, uint32_t src,
                                                        uint32_t dst, uint32_t dport, uint32_t in_port,
@@ -1758,7 +1757,7 @@ __device__ __forceinline__ void hop_outcome(const HopArgs &g, const uint2 *ports
 // in_port is the source host's port (so a live probe never bounces) and no
 // cycle check is due, so all of that is left out.
 template <bool kIndexed, bool kPolicy, bool kStats, bool kRec, bool kFirst>
-__global__ void __launch_bounds__(kHopThreads, kFirst ? 4 : 4) walk_hop_kernel(HopArgs g) {
+__global__ void __launch_bounds__(kHopThreads, 4) walk_hop_kernel(HopArgs g) {
     extern __shared__ __align__(128) uint8_t s_raw[];
     __shared__ uint64_t s_bar;
     __shared__ uint32_t s_count;
@@ -1992,11 +1991,10 @@ __global__ void __launch_bounds__(kHopThreads, kFirst ? 4 : 4) walk_hop_kernel(H
 // First match of one probe by one thread, reading the switch's blob in place
 // (L2-resident tables).  Candidates are taken two at a time, both rules
 // loaded before either is tested: what a walk waits for here is the chain of
-// dependent L2 round trips.  So does a
-// segment's jump block, from kJumpFrom boundaries on: two loads side by side and
-// two or three more where a search of 512 boundaries has ten in a row (100,000
-// probes on 512 switches 41.5 -> 32.3 us, 1 million 112 -> 85, 1 million flows
-// with policies 144 -> 117).
+// dependent L2 round trips.  A segment's jump block shortens that chain too, from
+// kJumpFrom boundaries on: two loads side by side and two or three more where a
+// search of 512 boundaries has ten in a row (100,000 probes on 512 switches 41.5 ->
+// 32.3 us, 1 million 112 -> 85, 1 million flows with policies 144 -> 117).
 // kLong: gives up after kLanePairs pairs, with kDeep as the result (100,000 probes
 // on 512 switches with lists of 337 items: 859 us with 32 pairs, 685 with 16, 625
 // with 8; of 1,932: 1035, 928, 881).
@@ -2101,7 +2099,7 @@ __device__ __noinline__ uint32_t first_match_deep(const uint8_t *blob, uint32_t 
 // walk_hop_kernel; a probe's cycle checkpoint and waypoint bits stay in
 // registers.
 // Bound by the chain of dependent L2 round trips of one first match (about
-// ten) times the visits of a lane; drawing new probes keeps the other lanes
+// six) times the visits of a lane; drawing new probes keeps the other lanes
 // at work meanwhile.  1,000 probes on the ring: 130 us as 27 launches, 11 us
 // as this one; 100,003 probes on 512 switches: 175 -> 32 us with the filter and
 // the jump blocks.
