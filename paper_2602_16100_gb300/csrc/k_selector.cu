@@ -534,7 +534,7 @@ __device__ __forceinline__ bool put_span(uint32_t *row, uint32_t sb, uint32_t la
 // found as it was read, 5,000 pods of 33 to 64 expressions on 5,000 nodes took 253 us,
 // 69 resolved 32 at a time.
 constexpr uint8_t kPodLeft = 0x80;
-// kPodWarp: the copy of pod_terms_kernel, which has fewer registers (one copy for both
+// kPodWarp: the copy of sel_terms_kernel, which has fewer registers (one copy for both
 // cost sel_rows_kernel 1 to 2%).
 template <bool kTerms, bool kPodWarp>
 __device__ __noinline__ void unresolved_pod(const SelArgs &g, uint32_t p, uint32_t *list) {
@@ -589,7 +589,7 @@ __device__ __noinline__ void unresolved_pod(const SelArgs &g, uint32_t p, uint32
 // 33.2 / 39.3.  Bound by one pod's chain of loads; three rows at once are what 48
 // registers hold without spilling in the loop.
 constexpr int kPodThreads = 128;
-__global__ void __launch_bounds__(kPodThreads, 1280 / kPodThreads) pod_terms_kernel(const __grid_constant__ SelArgs g) {
+__global__ void __launch_bounds__(kPodThreads, 1280 / kPodThreads) sel_terms_kernel(const __grid_constant__ SelArgs g) {
     __shared__ uint32_t s_list[kPodThreads / 32][kListWords];
     const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5, p = blockIdx.x * (kPodThreads / 32) + warp;
     if (p >= g.P) return;
@@ -1100,10 +1100,8 @@ extern "C" int pv_load_cluster(pv_ctx *ctx, uint32_t num_nodes, uint32_t num_key
 
 namespace {
 
-// The rows kernel's arguments and grid: a warp per pod until the GPU is full,
-// then the pods shared out.
-template <bool kTerms>
-void launch_rows(pv_ctx *ctx, SelArgs g, cudaStream_t st) {
+// The loaded cluster's part of the kernels' arguments.
+SelArgs cluster_args(const pv_ctx *ctx, SelArgs g) {
     const pv_cluster_state &c = ctx->cl;
     g.N = c.num_nodes;
     g.K = c.num_keys;
@@ -1114,20 +1112,31 @@ void launch_rows(pv_ctx *ctx, SelArgs g, cudaStream_t st) {
     g.row_words = c.row_words;
     g.num_value_rows = c.num_value_rows;
     g.zero_row = (c.num_value_rows + c.num_keys) * c.row_words * 4;
+    return g;
+}
+
+// The rows kernel's grid: a warp per pod until the GPU is full, then the pods
+// shared out.
+template <bool kTerms>
+void launch_rows(pv_ctx *ctx, const SelArgs &g, cudaStream_t st) {
     void (*fn)(SelArgs) = g.W <= 160 ? sel_rows_kernel<kTerms, true> : sel_rows_kernel<kTerms, false>;
     const int per_sm = std::max(1, pv_blocks_per_sm(ctx, (const void *)fn, kRowsThreads<kTerms>, 0));
     constexpr uint32_t warps = kRowsThreads<kTerms> / 32;
     const uint32_t blocks = std::min((g.P + warps - 1) / warps, (uint32_t)(ctx->num_sms * per_sm));
-    if (kTerms && g.P > (uint32_t)(ctx->num_sms * per_sm) * warps) {
-        constexpr uint32_t pods = kPodThreads / 32;
-        const uint32_t resident =
-            (uint32_t)(ctx->num_sms * std::max(1, pv_blocks_per_sm(ctx, (const void *)pod_terms_kernel, kPodThreads, 0)));
-        if (g.P <= resident * pods) {
-            pod_terms_kernel<<<(g.P + pods - 1) / pods, kPodThreads, 0, st>>>(g);
-            return;
-        }
-    }
     fn<<<blocks, kRowsThreads<kTerms>, 0, st>>>(g);
+}
+
+// The term form: a pod to a warp where that many warps fit at once and the rows
+// kernel's do not.
+void launch_terms(pv_ctx *ctx, const SelArgs &g, cudaStream_t st) {
+    constexpr uint32_t pods = kPodThreads / 32, warps = kRowsThreads<true> / 32;
+    const uint32_t sms = (uint32_t)ctx->num_sms;
+    const void *rows = g.W <= 160 ? (const void *)sel_rows_kernel<true, true> : (const void *)sel_rows_kernel<true, false>;
+    if (g.P > sms * warps * (uint32_t)pv_blocks_per_sm(ctx, rows, kRowsThreads<true>, 0) &&
+        g.P <= sms * pods * (uint32_t)pv_blocks_per_sm(ctx, (const void *)sel_terms_kernel, kPodThreads, 0))
+        sel_terms_kernel<<<(g.P + pods - 1) / pods, kPodThreads, 0, st>>>(g);
+    else
+        launch_rows<true>(ctx, g, st);
 }
 
 }  // namespace
@@ -1197,7 +1206,7 @@ extern "C" int pv_eval_selectors(pv_ctx *ctx, uint32_t num_pods, const uint32_t 
         g.flags = d_flags;
         g.pod_list = rep_list;
         g.list_len = rep_count;
-        launch_rows<false>(ctx, g, st);
+        launch_rows<false>(ctx, cluster_args(ctx, g), st);
     } else {
         const size_t smem = (size_t)tile * c.num_keys * 2;
         PV_TRY_CUDA(ctx, cudaFuncSetAttribute(sel_cmp_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem),
@@ -1246,7 +1255,7 @@ extern "C" int pv_eval_selector_terms(pv_ctx *ctx, uint32_t num_pods, const uint
     g.flags = d_flags;
     pv_use_begin(ctx, st);
     const int pr = pv_prof_start(ctx, st, PV_K_SELECTOR);
-    launch_rows<true>(ctx, g, st);
+    launch_terms(ctx, cluster_args(ctx, g), st);
     pv_prof_stop(ctx, st, pr, 1);
     pv_mark_use(ctx, st);
     return pv_check_launch(ctx, "selector kernels");
