@@ -510,9 +510,11 @@ int pv_install_path_rules(pv_ctx *ctx, uint32_t num_slots, const pv_rule *d_rule
  *   same expressions in the same order, unused value slots ignored), such as
  *   the replicas of one deployment or intents sharing a selector, get their
  *   representative's row (the smallest such pod) and flags, with their own
- *   placement check.  Same results and no longer faster where it was tried
- *   (100,000 pods of 10,000 distinct lists 0.111 ms, 0.074 without): for
- *   lists that repeat more than that or are much longer.  2 = the
+ *   placement check.  Same results.  It pays where lists are long or each
+ *   repeats a hundred times or more, and costs time where short lists repeat
+ *   some ten times (100,000 pods on 5,000 nodes, us without / with it, by 10 /
+ *   1,000 / 10,000 distinct lists: 1 to 8 expressions 104/98, 118/113, 110/128;
+ *   20 to 32 expressions 186/103, 235/122, 240/151).  2 = the
  *   same with deliberately weak hashes (tests: every collision is resolved
  *   by comparing the lists).  Not used by pv_eval_selector_terms.
  * PV_OPT_SCHED_KERNEL: pv_schedule_paths' kernel: 0 = automatic (a warp per

@@ -1096,9 +1096,10 @@ extern "C" int pv_compliant_reach(pv_ctx *ctx, uint32_t V, const uint32_t *d_off
                                                                           d_masks, sets, num_src, d_src, rest, rest_n,
                                                                           flags);
         // at most eight blocks an SM: on a symmetric graph they all start and return
-        // (the 4,096-vertex WAN 57.4 us with sixteen, 55.4 with eight).  A block's items lie a grid apart: neighbours are of one mask, and
-        // a mask with long searches would keep its few blocks for twice as long
-        // (8,000 vertices of three edges each, 24 masks: 945 us, 627 a grid apart)
+        // (the 4,096-vertex WAN 57.4 us with sixteen, 55.4 with eight).  A block's items
+        // lie a grid apart: neighbours are of one mask, and a mask with long searches
+        // would keep its few blocks for twice as long (8,000 vertices of three edges
+        // each, 24 masks: 945 us, 627 a grid apart)
         reach_hub_rows_kernel<<<(uint32_t)std::min<uint64_t>(items, 8ull * sms), kReachThreads, HubRowSmem(V).total, sw>>>(
             V, d_offs, d_cols, in_offs, in_cols, d_region, num_src, d_src, num_masks, d_masks, sets, rest, rest_n,
             d_reach, words_per_row, flags);

@@ -645,9 +645,8 @@ __global__ void __launch_bounds__(kPodThreads, 1280 / kPodThreads) sel_terms_ker
 // slots at 100,000 pods, the rows coming from L2), with few the chain offsets
 // -> expressions -> inventory -> rows of one pod.  On 5,000 nodes against a
 // warp per pod that resolved one pod at a time and loaded two rows ahead:
-// 100,000 pods 99.5 -> 69.3 us, 10,000 19.0 -> 15.6, 777 11.6 -> 10.0; in the
-// term form 129.6 -> 96.9, 22.1 -> 18.9 and 14.0 -> 11.1 (6,000 pods, where some
-// warps have two and that kernel had room for a warp each: 17.2 -> 18.6).
+// 100,000 pods 101.8 -> 72.4 us, 10,000 19.0 -> 15.6, 777 12.2 -> 10.3; in the
+// term form 129.6 -> 97, 22.1 -> 18.9 and 14.0 -> 11.1.
 template <bool kTerms, bool kOneSpan>
 __global__ void __launch_bounds__(kRowsThreads<kTerms>, 768 / kRowsThreads<kTerms>)
     sel_rows_kernel(const __grid_constant__ SelArgs g) {

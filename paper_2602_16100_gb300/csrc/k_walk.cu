@@ -59,12 +59,13 @@ constexpr uint32_t kThreadWalkMax = 1u << 20;
 // Larger batches: the hop from which the probes still walking finish in one
 // thread walk.  Live probes fall about 2.5 times a hop, and the thread walk
 // takes over best at some 400,000 of them, so one more hop is regrouped for
-// every factor 2.5 of the batch.  us at tail hop 1 / 2 / 3 / 4 / 5 / 6 / 8 (the hop
-// kernels have become about a tenth faster since, at every tail hop):
-//   mesh of 512, 3M probes    216  199  214  240  274  299  340
-//   fat tree, 10M probes      998  842  744  719  710  711  777
-//   compact flows, 3M         218  206  222  255  280  302  339
-//   compact flows, 50M       2207 1571 1410 1400 1411 1441 1490
+// every factor 2.5 of the batch.  us at tail hop 1 / 2 / 3 / 4 / 5 / 6 / 8:
+//   mesh of 512, 3M probes    194  187  202  229  257  282  328
+//   fat tree, 10M probes     1023  883  765  751  734  732  798
+//   compact flows, 3M         176  171  191  223  252  275  311
+//   compact flows, 50M       1508 1269 1239 1261 1264 1285 1336
+// (Walks that every mask permits live longer and would switch later: mesh of 512,
+// 4.5M probes 836, 724 from hop 5.)
 inline uint32_t auto_tail_hop(uint32_t M) {
     uint32_t hop = 1;
     for (uint64_t most = 1500000; M > most; most = most * 5 / 2) ++hop;
